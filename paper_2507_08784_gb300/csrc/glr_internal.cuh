@@ -335,8 +335,9 @@ struct BjacGroup {
     int nmat;
     BjacMat mat[kBjacGroupMax];
 };
-// J_k^T of every pair of every matrix: one Jacobi sweep on H's 128 x 128 diagonal pair blocks
-cudaError_t bjac_pairs(BjacGroup& g, cudaStream_t st);
+// J_k^T of every pair of every matrix: one Jacobi sweep on H's 128 x 128 diagonal pair blocks, over
+// the pair's two 64-index blocks or (full) over all 128 indices
+cudaError_t bjac_pairs(BjacGroup& g, int full, cudaStream_t st);
 // The start of a solve: H = sum of nparts partials (leading dimension ld; nparts = 0: H given),
 // H_lo = H - trunc_tf32(H), V = I, V_lo = 0 (all n x n row-major)
 struct BjacPrep {

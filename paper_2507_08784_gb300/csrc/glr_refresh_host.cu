@@ -246,7 +246,7 @@ int bjac_run(std::vector<BjItem>& all, glr_handle* h0, cudaStream_t s0) {
                         BjacMat& M = g.mat[g.nmat++];
                         M.n = n; M.H = act[c]->h->Hbuf; M.J = act[c]->h->bjJ; M.Jlo = act[c]->h->bjJlo;
                     }
-                    GLR_LAUNCH(h0, 1, bjac_pairs(g, s0));
+                    GLR_LAUNCH(h0, 1, bjac_pairs(g, round == 0, s0));
                 }
                 for (int mode = 0; mode < 3; ++mode) {
                     for (size_t c0 = 0; c0 < act.size(); c0 += tc::kTcGroupMax) {
