@@ -422,6 +422,10 @@ int glr_create(int64_t m, int64_t n, int32_t r, int32_t N, const glr_schedule* s
         }
     }
     if (rc == GLR_OK && h->tcl) rc = tcl_alloc(h);
+    h->n_state_allocs = h->allocs.size();
+    const int neig = exact ? (int)mp : k;                // scratch, not part of a checkpoint
+    if (!exact) A(&h->eig_ws, eig_ws_floats(k));
+    A(&h->sort_ws, 2 * (size_t)neig);
     if (rc != GLR_OK) {
         g_create_err = h->err;
         free_all(h);
@@ -462,7 +466,6 @@ int glr_create(int64_t m, int64_t n, int32_t r, int32_t N, const glr_schedule* s
     }
     h->iotaJ.resize(r);
     for (int q = 0; q < r; ++q) h->iotaJ[q] = q;
-    h->n_state_allocs = h->allocs.size();
     if (h->tcl && (rc = tcl_maps(h)) != GLR_OK) {
         g_create_err = h->err;
         glr_destroy(h);

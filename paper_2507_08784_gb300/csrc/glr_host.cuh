@@ -50,8 +50,9 @@ struct glr_handle {
     // in mn_scratch (m' x n').
     int tc = 0;
     float* mn_scratch = nullptr;
-    float* jwork = nullptr;      // full basis: the grouped Jacobi's second m' x m' buffer
-    float* jpart = nullptr;      // full basis: its per-CTA norm partials (used by a group's first handle)
+    float* jwork = nullptr;      // full basis: T^T of the blocked Jacobi above m' = 1024
+    float* jpart = nullptr;      // norm partials of the eigen-solver (used by a group's first handle)
+    float *eig_ws = nullptr, *sort_ws = nullptr;   // eigen-solver and eigenpair-order scratch (not checkpointed)
     float* YtJ = nullptr;        // Yt[J, :] (r x k) for P = U[:, J] as a library product
     float* amsv = nullptr;       // AMSGrad: the scalar normaliser and this step's maximum of V
     float* galr = nullptr;       // Algorithm 5: the subspace step direction M / (sqrt(V) + eps), r x n'
@@ -69,8 +70,7 @@ struct glr_handle {
     float *UT = nullptr, *Vbuf2 = nullptr, *bjJ = nullptr, *bjpart = nullptr;
     // ... and the TF32 low parts of the rotations' operands: J^T, H, T^T (in jwork) and both V buffers
     float *bjJlo = nullptr, *Hlo = nullptr, *Ttlo = nullptr, *Vlo = nullptr, *V2lo = nullptr;
-    int bj_sweeps = 0, numeric_failures_host = 0;
-    const float* bj_V = nullptr;       // the blocked Jacobi's final V (after a refresh that used it)
+    int bj_sweeps = 0, bj_vpar = 0, numeric_failures_host = 0;   // bj_vpar: V ended in Vbuf2
     // a data-parallel step in progress (glr_dp_begin / glr_dp_select / glr_dp_finish): 0 idle,
     // 1 begun, 2 selected; the step's plan and the caller's gradient pointers
     int dp_stage = 0, dp_flags = 0;
@@ -206,7 +206,6 @@ enum TcMap { kMapBt, kMapPT0, kMapPT1, kMapP0, kMapP1, kMapRwT, kMapMbarT, kMapY
 const CUtensorMap* tcl_grad_maps(glr_handle* h, const void* const* G, cudaStream_t st, int* rc);
 const CUtensorMap* tcl_x_map(glr_handle* h, const float* X, cudaStream_t st, int* rc);
 bool tcl_eligible(int64_t mp, int64_t np, int r, int N, int k, bool exact, const glr_schedule* s);
-bool tcl_rr_blocked(const glr_handle* h);
 int tcl_alloc(glr_handle* h);         // state buffers (before n_state_allocs is fixed)
 int tcl_maps(glr_handle* h);          // the device map table (after)
 float* tcl_PT_of(const glr_handle* h, const float* P);
@@ -222,13 +221,10 @@ bool encode_map(CUtensorMap* map, CUtensorMapDataType dtype, const void* base, i
 // The Semi-Lazy SVD refresh (glr_refresh_host.cu).
 int cholqr(glr_handle* h, float*& A, float*& tmp, int rows, cudaStream_t st);
 int wy_from_Q(glr_handle* h, cudaStream_t st);
-int refresh_tail(glr_handle* h, cudaStream_t st);
 int refresh_finish(glr_handle* h, cudaStream_t st);
 int refresh_power(glr_handle* h, cudaStream_t st);
 int refresh_trunc_grouped(std::vector<glr_handle*>& hs);
 int refresh_tcl_grouped(std::vector<glr_handle*>& hs);    // tcgen05 path (k <= 256)
-int cholqr(glr_handle* h, float*& A, float*& tmp, int rows, cudaStream_t st);
-int refresh_finish(glr_handle* h, cudaStream_t st);
 int refresh_grouped(std::vector<glr_handle*>& hs);
 int refresh_exact_grouped(std::vector<glr_handle*>& hs);
 int refresh_exact_blocked(std::vector<glr_handle*>& hs);   // m' > 1024, sorted by m'

@@ -226,12 +226,16 @@ cudaError_t materialize_error(int mp, int np, int r, int e_zero, const float* B,
 // Cyclic two-sided Jacobi on the symmetric n x n matrix H (overwritten), one CTA:
 // eigenvalues to evals, eigenvectors (columns) to V; the sweep count to *sweeps.
 cudaError_t jacobi_eig(float* H, int n, float* V, float* evals, int* sweeps, cudaStream_t st);
-// Sort eigenpairs by descending eigenvalue, write the first ncols vectors as columns of Out
-// (rows x ncols, row-major, leading dim ldo), largest-|entry| of each column positive.
-cudaError_t sort_fix_basis(const float* evals, const float* V, int n, int ncols, float* Out,
-                           int ldo, float* evals_sorted, cudaStream_t st);
-// Make the largest-|entry| of each column of A (rows x cols, row-major) positive.
-cudaError_t fix_column_signs(float* A, int rows, int cols, cudaStream_t st);
+// Eigenpairs by descending eigenvalue, several problems at once: V (n x n row-major, column j for
+// evals[j]) -> Out (n x n) with unit columns, the largest-|entry| of each positive, and
+// evals_sorted (may be null).  Two launches; order and scale: n entries of scratch each.
+struct SortMat {
+    int n;
+    const float* evals; const float* V; float* Out; float* evals_sorted;
+    int* order; float* scale;
+};
+struct SortGroup { int nmat; SortMat mat[64]; };
+cudaError_t sort_group(const SortGroup& g, cudaStream_t st);
 // In-place Cholesky of the n x n SPD matrix A (lower factor in the lower triangle); if a
 // pivot is not positive the diagonal is shifted and the factorisation restarted (*flag =
 // number of restarts).  scratch: n*n floats.
@@ -244,13 +248,11 @@ cudaError_t chol_inverse(const float* G, int n, float* S, int* flag, cudaStream_
 struct CholMat { const float* part; int nparts, ld, n; float* out; int* flag; int tri_only; };   // tri_only: (U^T)^{-1} of the upper triangle of part (n x n)
 struct CholGroup { int nmat; CholMat mat[64]; };
 cudaError_t chol_group(const CholGroup& g, cudaStream_t st);
-// The end of a truncated refresh for several matrices, one launch per stage: stage 0 sorts each
-// eigenproblem's pairs by descending value and writes W (k x k, unit columns, signs fixed) and the
-// sorted values; 1 fixes the column signs of Q (m' x k); 2 and 3 the Householder reconstruction
-// (top block into Wtop, Y, T, s; then the rows below).
+// The end of a truncated refresh for several matrices, one launch per stage: stage 1 fixes the
+// column signs of Q (m' x k: the largest-|entry| of each positive); 2 and 3 the Householder
+// reconstruction (top block into Wtop, Y, T, s; then the rows below).
 struct FinishMat {
     int mp, k;
-    const float* evals; const float* V; float* W; float* evals_sorted;
     float* Q; float* Wtop; float* Y; float* T; float* s;
 };
 struct FinishGroup { int nmat; FinishMat mat[64]; };
@@ -287,20 +289,34 @@ struct JacobiGroup {
     int* bar; int* err; float* part;
     JacobiMat mat[kGroupMax];
 };
-// The k x k Rayleigh-Ritz eigenproblems of truncated refreshes (k_eig.cu): one CTA per matrix,
-// H (row-major, n <= 256, read only; summed from partial matrices) -> eigenvalues (unsorted) and eigenvectors V (row-major
-// n x n, column j for evals[j]); sweeps done in *sweeps.
+int jacobi_group_grid();
+cudaError_t jacobi_group(const JacobiGroup& g, int grid, cudaStream_t st);
+// The same iteration (same rotations in the same order, bit for bit) for one matrix of n <= 512 in one
+// thread-block cluster; H is read only.  jacobi_cluster_ok(): whether the device can place it.
+bool jacobi_cluster_ok(int n);
+cudaError_t jacobi_cluster(const JacobiMat& M, int max_sweeps, cudaStream_t st);
+
+// Symmetric eigenproblems of the refresh (k_eig.cu), n <= 1024: H (row-major, read only; the sum of
+// nparts matrices of leading dimension ld, ld * ld apart) -> eigenvalues (unsorted) and eigenvectors
+// V (row-major n x n, column j for evals[j]); sweeps done in *sweeps.  n <= 128: one CTA a problem
+// (eig_small_group).  Larger n: all problems in one cooperative launch (eig_group) that leaves
+// busy_sms SMs free; ws: eig_ws_floats(n) floats a problem, part: 128 floats a problem, bar: two
+// ints, *err counts a barrier that gave up.
+constexpr int kEigSmall = 128;
+constexpr int kEigGroupMax = 64;
 struct EigMat {
     int n; float tol;
-    const float* H; int nparts, ld;       // H = the sum of nparts matrices (leading dimension ld, ld * ld apart)
-    float* V; float* evals; int* sweeps;
+    const float* H; int nparts, ld;
+    float* V; float* evals; int* sweeps; float* ws;
 };
-constexpr int kEigGroupMax = 64;
 struct EigGroup {
     int nmat, max_sweeps;
+    int* bar; int* err; float* part;
     EigMat mat[kEigGroupMax];
 };
-cudaError_t eig_tmem_group(const EigGroup& g, cudaStream_t st);
+size_t eig_ws_floats(int n);
+cudaError_t eig_small_group(const EigGroup& g, cudaStream_t st);
+cudaError_t eig_group(const EigGroup& g, int busy_sms, cudaStream_t st);
 
 // The blocked Jacobi's round-robin tournament over m blocks of 64 indices (circle method: block 0
 // fixed, the others one slot further each round; slots s and m - 1 - s pair up and are stored at
@@ -338,10 +354,9 @@ struct BjacGroup {
 // J_k^T of every pair of every matrix: one Jacobi sweep on H's 128 x 128 diagonal pair blocks, over
 // the pair's two 64-index blocks or (full) over all 128 indices
 cudaError_t bjac_pairs(BjacGroup& g, int full, cudaStream_t st);
-// The start of a solve: H = sum of nparts partials (leading dimension ld; nparts = 0: H given),
-// H_lo = H - trunc_tf32(H), V = I, V_lo = 0 (all n x n row-major)
+// The start of a solve: H_lo = H - trunc_tf32(H), V = I, V_lo = 0 (all n x n row-major)
 struct BjacPrep {
-    const float* part; int nparts, ld, n;
+    int n;
     float *H, *Hlo, *V, *Vlo;
 };
 struct BjacPrepGroup {
@@ -351,11 +366,9 @@ struct BjacPrepGroup {
 cudaError_t bjac_prep(const BjacPrepGroup& g, cudaStream_t st);
 // part[2 (i kBjacNormCtas + c) + {0, 1}]: CTA c's squared diagonal / off-diagonal sums of H_i
 cudaError_t bjac_norms(const BjacGroup& g, float* part, cudaStream_t st);
-cudaError_t bjac_eye(float* V, int n, cudaStream_t st);
 cudaError_t bjac_diag(const float* H, int n, float* evals, cudaStream_t st);
+cudaError_t add_diagonal(float* A, int n, float v, cudaStream_t st);   // A (n x n) += v I
 cudaError_t count_flag(int* flag, int v, cudaStream_t st);   // *flag += v on the device
-int jacobi_group_grid();
-cudaError_t jacobi_group(const JacobiGroup& g, int grid, cudaStream_t st);
 // Q <- Q L^{-T} for the rows x n matrix Q (row-major) and lower-triangular L.
 cudaError_t trsm_right_lt(float* Q, int rows, int n, const float* L, cudaStream_t st);
 // Random Gaussian start block (rows x cols) from Philox with the power-iteration tag.

@@ -1,8 +1,9 @@
 // The Semi-Lazy SVD refresh of Eq. SVD-P1 on the host side: the order of the refresh kernels for
 // a truncated basis (block power iteration with CholeskyQR, Rayleigh-Ritz, the Householder WY
-// form; grouped across matrices through k_power.cu when k <= 32) and for the full basis (the
-// cooperative Jacobi of all refreshing matrices, k_jacobi.cu).  Each handle's refresh runs on its
-// own side stream.
+// form; grouped across matrices through k_power.cu when k <= 32; the larger k x k eigenproblems of
+// all refreshing matrices go to k_eig.cu together) and for the full basis (k_jacobi.cu up to
+// m' = 1024, k_bjac.cu above).
+// Each handle's refresh runs on its own side stream.
 #include "glr_host.cuh"
 
 namespace glr {
@@ -40,22 +41,97 @@ int wy_from_Q(glr_handle* h, cudaStream_t st) {
     return GLR_OK;
 }
 
+// One symmetric eigenproblem of a handle (n = k or m' <= 1024): H as the sum of nparts matrices;
+// eigenvalues to h->evals, eigenvectors to V.
+struct EigItem {
+    glr_handle* h;
+    int n;
+    const float* H; int nparts, ld;
+    float* V;
+};
+
+// The eigenproblems: those of n <= 128 on s1, the larger ones in one cooperative launch on s0 (leaving
+// the small ones' SMs free when s1 is another stream).
+int eig_solve(const std::vector<EigItem>& items, cudaStream_t s0, cudaStream_t s1) {
+    std::vector<const EigItem*> cls[2];
+    for (const EigItem& it : items) cls[it.n > kEigSmall ? 1 : 0].push_back(&it);
+    for (int big = 0; big < 2; ++big)
+        for (size_t c0 = 0; c0 < cls[big].size(); c0 += kGroupMax) {
+            EigGroup g{};
+            glr_handle* h0 = cls[big][c0]->h;
+            g.max_sweeps = 40;
+            g.bar = h0->dflags + 4; g.err = h0->dflags + 2; g.part = h0->jpart;
+            for (size_t i = c0; i < cls[big].size() && i < c0 + (size_t)kGroupMax; ++i) {
+                const EigItem& it = *cls[big][i];
+                EigMat& M = g.mat[g.nmat++];
+                M.n = it.n; M.tol = 4.f * 5.96e-8f * sqrtf(static_cast<float>(it.n)) + 1e-7f;
+                M.H = it.H; M.nparts = it.nparts; M.ld = it.ld; M.V = it.V; M.evals = it.h->evals;
+                M.sweeps = it.h->dflags + 1; M.ws = it.h->eig_ws;
+            }
+            if (big) GLR_LAUNCH(h0, 1, eig_group(g, s0 != s1 ? (int)cls[0].size() : 0, s0));
+            else GLR_LAUNCH(h0, 1, eig_small_group(g, s1));
+        }
+    return GLR_OK;
+}
+
+// A handle's eigenpairs (h->evals, V) sorted into Out.
+SortMat sort_mat(glr_handle* h, int n, const float* V, float* Out) {
+    SortMat S;
+    S.n = n; S.evals = h->evals; S.V = V; S.Out = Out; S.evals_sorted = h->evals_sorted;
+    S.order = reinterpret_cast<int*>(h->sort_ws); S.scale = h->sort_ws + n;
+    return S;
+}
+
 // Rayleigh-Ritz after the k x k eigen-decomposition H = W diag W^T (eigenvalues in evals, W in
 // Vk): Q <- Q W (columns by descending Ritz value, signs fixed), then the WY form.
 int refresh_finish(glr_handle* h, cudaStream_t st) {
     const int mp = h->mp, k = h->k;
-    GLR_LAUNCH(h, 1, sort_fix_basis(h->evals, h->Vk, k, k, h->gram, k, h->evals_sorted, st));
+    SortGroup sg{};
+    sg.mat[sg.nmat++] = sort_mat(h, k, h->Vk, h->gram);
+    GLR_LAUNCH(h, 2, sort_group(sg, st));
     GLR_GEMM(h, gd(mp, k, k, h->Q, k, 1, h->gram, k, 1, h->Qn, k, 1), st);
-    GLR_LAUNCH(h, 1, fix_column_signs(h->Qn, mp, k, st));
+    FinishGroup fg{};
+    FinishMat& F = fg.mat[fg.nmat++];
+    F.mp = mp; F.k = k; F.Q = h->Qn;
+    GLR_LAUNCH(h, 1, finish_group(fg, 1, st));
     std::swap(h->Q, h->Qn);
     return wy_from_Q(h, st);
 }
 
-// End of a truncated refresh, with Q orthonormal and H = Q^T Mbar Mbar^T Q in Hk: the k x k
-// Jacobi in one CTA, then refresh_finish.
+// The end of a truncated refresh with k <= 32, Q orthonormal and H = Q^T Mbar Mbar^T Q in Hk: the
+// k x k Jacobi in one CTA, then refresh_finish.
 int refresh_tail(glr_handle* h, cudaStream_t st) {
     GLR_LAUNCH(h, 1, jacobi_eig(h->Hk, h->k, h->Vk, h->evals, h->dflags + 1, st));
     return refresh_finish(h, st);
+}
+
+// The end of truncated refreshes whose Q is orthonormal and whose H = Q^T Mbar Mbar^T Q is in Hk,
+// each on its own side stream: the eigenproblems together, then each handle's finish.
+int refresh_tails(std::vector<glr_handle*>& hs) {
+    glr_handle* h0 = hs[0];
+    std::vector<EigItem> items;
+    for (glr_handle* h : hs) {
+        if (h != h0) {
+            GLR_CK(h, cudaEventRecord(h->rpow, h->rstream));
+            GLR_CK(h0, cudaStreamWaitEvent(h0->rstream, h->rpow, 0));
+        }
+        items.push_back(EigItem{h, h->k, h->Hk, 1, h->k, h->Vk});
+    }
+    {
+        PhaseScope ps(h0, GLR_PH_REFRESH, h0->rstream);
+        const int rc = eig_solve(items, h0->rstream, h0->rstream);
+        if (rc != GLR_OK) return rc;
+    }
+    GLR_CK(h0, cudaEventRecord(h0->rpow, h0->rstream));
+    for (glr_handle* h : hs) {
+        if (h != h0) GLR_CK(h, cudaStreamWaitEvent(h->rstream, h0->rpow, 0));
+        PhaseScope ps(h, GLR_PH_REFRESH, h->rstream);
+        g_ws = h->gemm_ws;
+        const int rc = refresh_finish(h, h->rstream);
+        g_ws = nullptr;
+        if (rc != GLR_OK) return rc;
+    }
+    return GLR_OK;
 }
 
 // Truncated refreshes of several matrices through the grouped block power iteration
@@ -111,21 +187,45 @@ int refresh_grouped(std::vector<glr_handle*>& hs) {
     return GLR_OK;
 }
 
-// Full-basis refreshes of several matrices: H = Mbar Mbar^T on each handle's side stream, one
-// cooperative Jacobi launch for all of them on the first handle's side stream (k_jacobi.cu), then
-// each handle sorts its eigenvectors by descending eigenvalue and fixes their signs on its own.
+// A full-basis handle's eigenpairs sorted by descending eigenvalue, signs fixed, to U.
+int sort_full_basis(glr_handle* h, cudaStream_t st) {
+    SortGroup sg{};
+    sg.mat[sg.nmat++] = sort_mat(h, h->mp, h->Vbuf, h->U);
+    GLR_LAUNCH(h, 2, sort_group(sg, st));
+    return GLR_OK;
+}
+
+// A full-basis handle's eigenproblem for the Jacobi of k_jacobi.cu.
+JacobiMat jacobi_mat(glr_handle* h) {
+    JacobiMat M{};
+    M.n = h->mp; M.tol = 4.f * 5.96e-8f * sqrtf(static_cast<float>(h->mp)) + 1e-7f;
+    M.H = h->Hbuf; M.H2 = h->jwork; M.V = h->Vbuf; M.evals = h->evals;
+    M.sweeps = h->dflags + 1;
+    return M;
+}
+
+// Full-basis refreshes of several matrices: H = Mbar Mbar^T on each handle's side stream, then the
+// Jacobi: up to m' = 512 a cluster a matrix on its own side stream (the matrices beside each other),
+// up to 1024 one cooperative launch for all of them on the first handle's side stream
+// (k_jacobi.cu); each handle then sorts its eigenvectors and fixes their signs on its own.
 int refresh_exact_grouped(std::vector<glr_handle*>& hs) {
-    {   // above m' = 1024: the blocked solver (tcgen05 path only)
-        std::vector<glr_handle*> big, small;
-        for (glr_handle* h : hs) (h->mp > kMaxFullBasis ? big : small).push_back(h);
-        if (!big.empty()) {
-            std::stable_sort(big.begin(), big.end(), [](const glr_handle* a, const glr_handle* b) { return a->mp < b->mp; });
-            const int rc = refresh_exact_blocked(big);
-            if (rc != GLR_OK) return rc;
-        }
-        if (small.empty()) return GLR_OK;
-        hs.swap(small);
+    std::vector<glr_handle*> huge, rest;
+    for (glr_handle* h : hs) {
+        if (h->mp > kMaxFullBasis) { huge.push_back(h); continue; }    // the tcgen05 path's blocked solver
+        if (!jacobi_cluster_ok(h->mp)) { rest.push_back(h); continue; }
+        PhaseScope ps(h, GLR_PH_REFRESH, h->rstream);
+        const int mp = h->mp, np = h->np;
+        GLR_GEMM(h, gd(mp, mp, np, h->Mbar, np, 1, h->Mbar, 1, np, h->Hbuf, mp, 1), h->rstream);
+        GLR_LAUNCH(h, 1, jacobi_cluster(jacobi_mat(h), 40, h->rstream));
+        const int rc = sort_full_basis(h, h->rstream);
+        if (rc != GLR_OK) return rc;
     }
+    if (!huge.empty()) {
+        std::stable_sort(huge.begin(), huge.end(), [](const glr_handle* a, const glr_handle* b) { return a->mp < b->mp; });
+        const int rc = refresh_exact_blocked(huge);
+        if (rc != GLR_OK) return rc;
+    }
+    hs.swap(rest);
     const int grid = jacobi_group_grid();
     for (size_t c0 = 0, c1 = 0; c0 < hs.size(); c0 = c1) {
         // a group: at most kGroupMax matrices whose rotations fit the kernel's shared memory
@@ -144,7 +244,8 @@ int refresh_exact_grouped(std::vector<glr_handle*>& hs) {
             GLR_GEMM(h, gd(mp, mp, np, h->Mbar, np, 1, h->Mbar, 1, np, h->Hbuf, mp, 1), h->rstream);
             if (!grid) {                                         // no cooperative launch: one CTA each
                 GLR_LAUNCH(h, 1, jacobi_eig(h->Hbuf, mp, h->Vbuf, h->evals, h->dflags + 1, h->rstream));
-                GLR_LAUNCH(h, 1, sort_fix_basis(h->evals, h->Vbuf, mp, mp, h->U, mp, h->evals_sorted, h->rstream));
+                const int rc = sort_full_basis(h, h->rstream);
+                if (rc != GLR_OK) return rc;
                 continue;
             }
             GLR_CK(h, cudaEventRecord(h->rpow, h->rstream));
@@ -158,12 +259,9 @@ int refresh_exact_grouped(std::vector<glr_handle*>& hs) {
         for (size_t i = c0; i < c1; ++i) {
             glr_handle* h = hs[i];
             JacobiMat& M = g.mat[g.nmat++];
-            const int n = h->mp;
-            M.n = n; M.tol = 4.f * 5.96e-8f * sqrtf(static_cast<float>(n)) + 1e-7f;
-            M.H = h->Hbuf; M.H2 = h->jwork; M.V = h->Vbuf; M.evals = h->evals;
-            M.sweeps = h->dflags + 1;
+            M = jacobi_mat(h);
             M.soff = (int)soff;
-            soff += jacobi_rot_floats(n);
+            soff += jacobi_rot_floats(M.n);
         }
         {
             PhaseScope ps(h0, GLR_PH_REFRESH, s0);
@@ -174,15 +272,28 @@ int refresh_exact_grouped(std::vector<glr_handle*>& hs) {
             glr_handle* h = hs[i];
             if (h != h0) GLR_CK(h, cudaStreamWaitEvent(h->rstream, h0->rpow, 0));
             PhaseScope ps(h, GLR_PH_REFRESH, h->rstream);
-            GLR_LAUNCH(h, 1, sort_fix_basis(h->evals, h->Vbuf, h->mp, h->mp, h->U, h->mp, h->evals_sorted, h->rstream));
+            const int rc = sort_full_basis(h, h->rstream);
+            if (rc != GLR_OK) return rc;
         }
     }
     return GLR_OK;
 }
 
-// The blocked Jacobi (k_bjac.cu) for a set of symmetric n x n problems, n a multiple of 128 from
-// 256 to 4096: the full basis's m' x m' eigenproblem, or a truncated refresh's k x k Rayleigh-Ritz
-// problem.  Each problem lives in its handle's buffers (H in Hbuf with its low part in Hlo, T^T in
+// One grouped fp32 product per handle (fill describes it), 64 per launch.
+template <class Fill>
+int fp32_products(std::vector<glr_handle*>& hs, cudaStream_t st, Fill fill) {
+    for (size_t c0 = 0; c0 < hs.size(); c0 += 64) {
+        GemmGroup gg{};
+        for (size_t i = c0; i < hs.size() && i < c0 + 64; ++i) fill(hs[i], gg.mat[gg.nmat++]);
+        PhaseScope ps(hs[c0], GLR_PH_REFRESH, st);
+        GLR_LAUNCH(hs[c0], 1, gemm_group_f32(gg, st));
+    }
+    return GLR_OK;
+}
+
+// The blocked Jacobi (k_bjac.cu) for a set of symmetric n x n problems, n a multiple of 128 above
+// 1024 up to 4096: the full basis's m' x m' eigenproblem on the tcgen05 path.
+// Each problem lives in its handle's buffers (H in Hbuf with its low part in Hlo, T^T in
 // jwork / Ttlo, V in Vbuf / Vbuf2 with Vlo / V2lo, the rotations in bjJ / bjJlo) and the kMapBj*
 // tensor maps over them; bjac_prep has set H, H_lo, V = I, V_lo = 0.  The problems of one size run
 // together, one sweep at a time, each sweep opened by the norm check (per-CTA partials summed on
@@ -196,7 +307,6 @@ struct BjItem {
     glr_handle* h;
     int n, vpar, rd;
     bool done;
-    const float* V() const { return vpar ? h->Vbuf2 : h->Vbuf; }
 };
 
 int bjac_run(std::vector<BjItem>& all, glr_handle* h0, cudaStream_t s0) {
@@ -295,17 +405,14 @@ int bjac_run(std::vector<BjItem>& all, glr_handle* h0, cudaStream_t s0) {
     return GLR_OK;
 }
 
-// bjac_prep over the items (in groups); part(h) gives a problem's partials and their count and
-// leading dimension (count 0: H is already in Hbuf).
-template <class Parts>
-int bjac_prepare(const std::vector<BjItem>& items, glr_handle* h0, cudaStream_t s0, Parts parts) {
+// H's low parts and V = I for the items (in groups).
+int bjac_prepare(const std::vector<BjItem>& items, glr_handle* h0, cudaStream_t s0) {
     for (size_t c0 = 0; c0 < items.size(); c0 += kBjacGroupMax) {
         BjacPrepGroup g{};
         for (size_t c = c0; c < items.size() && c < c0 + kBjacGroupMax; ++c) {
             glr_handle* h = items[c].h;
             BjacPrep& P = g.mat[g.nmat++];
             P.n = items[c].n; P.H = h->Hbuf; P.Hlo = h->Hlo; P.V = h->Vbuf; P.Vlo = h->Vlo;
-            parts(h, P);
         }
         GLR_LAUNCH(h0, 1, bjac_prep(g, s0));
     }
@@ -324,34 +431,49 @@ int refresh_exact_blocked(std::vector<glr_handle*>& hs) {
         GLR_CK(h0, cudaStreamWaitEvent(s0, h->rpow, 0));
     }
     PhaseScope ps(h0, GLR_PH_REFRESH, s0);
-    {   // H = Mbar Mbar^T (Mbar^T is n' x m' row-major)
-        GemmGroup gg{};
-        auto flush = [&]() -> int {
-            if (gg.nmat) GLR_LAUNCH(h0, 1, gemm_group_f32(gg, s0));
-            gg.nmat = 0;
-            return GLR_OK;
-        };
-        for (glr_handle* h : hs) {
-            GemmMat& G = gg.mat[gg.nmat++];
-            G = GemmMat{};
-            G.M = h->mp; G.N = h->mp; G.K = h->np; G.alpha = 1.f;
-            G.A = h->Mbar; G.sAi = 1; G.sAp = h->mp;
-            G.B = h->Mbar; G.sBp = h->mp; G.sBj = 1;
-            G.C = h->Hbuf; G.sCi = h->mp; G.sCj = 1;
-            if (gg.nmat == 64 && flush() != GLR_OK) return GLR_ECUDA;
-        }
-        if (flush() != GLR_OK) return GLR_ECUDA;
-    }
+    // H = Mbar Mbar^T (Mbar^T is n' x m' row-major)
+    int rc = fp32_products(hs, s0, [](glr_handle* h, GemmMat& G) {
+        G.M = h->mp; G.N = h->mp; G.K = h->np;
+        G.A = h->Mbar; G.sAi = 1; G.sAp = h->mp; G.B = h->Mbar; G.sBp = h->mp; G.sBj = 1;
+        G.C = h->Hbuf; G.sCi = h->mp; G.sCj = 1;
+    });
+    if (rc != GLR_OK) return rc;
     std::vector<BjItem> items;
     for (glr_handle* h : hs) items.push_back(BjItem{h, h->mp, 0, 0, false});
-    int rc = bjac_prepare(items, h0, s0, [](glr_handle*, BjacPrep& P) { P.nparts = 0; });
+    rc = bjac_prepare(items, h0, s0);
     if (rc == GLR_OK) rc = bjac_run(items, h0, s0);
     if (rc != GLR_OK) return rc;
+    // V <- V (3/2 I - 1/2 V^T V) in fp32 (a Newton-Schulz step): the rounds' split-TF32 products leave V
+    // orthogonal to a few 1e-5 (1e-4 at m' = 4096), this to fp32 rounding.  It also makes up for the
+    // one or two sweeps more that the cross-only pair sweeps take.
+    hs.clear();
     for (const BjItem& S : items) {
-        glr_handle* h = S.h;
+        hs.push_back(S.h);
+        S.h->bj_vpar = S.vpar;
+    }
+    rc = fp32_products(hs, s0, [](glr_handle* h, GemmMat& G) {
+        const float* V = h->bj_vpar ? h->Vbuf2 : h->Vbuf;
+        G.M = G.N = G.K = h->mp; G.alpha = -0.5f;
+        G.A = V; G.sAi = 1; G.sAp = h->mp; G.B = V; G.sBp = h->mp; G.sBj = 1;
+        G.C = h->jwork; G.sCi = h->mp; G.sCj = 1;
+    });
+    if (rc != GLR_OK) return rc;
+    for (glr_handle* h : hs) {
+        GLR_LAUNCH(h, 1, bjac_diag(h->Hbuf, h->mp, h->evals, s0));
+        GLR_LAUNCH(h, 1, add_diagonal(h->jwork, h->mp, 1.5f, s0));
+    }
+    rc = fp32_products(hs, s0, [](glr_handle* h, GemmMat& G) {
+        G.M = G.N = G.K = h->mp;
+        G.A = h->bj_vpar ? h->Vbuf2 : h->Vbuf; G.sAi = h->mp; G.sAp = 1;
+        G.B = h->jwork; G.sBp = h->mp; G.sBj = 1;
+        G.C = h->bj_vpar ? h->Vbuf : h->Vbuf2; G.sCi = h->mp; G.sCj = 1;
+    });
+    if (rc != GLR_OK) return rc;
+    for (glr_handle* h : hs) {
         const int n = h->mp;
-        GLR_LAUNCH(h, 1, bjac_diag(h->Hbuf, n, h->evals, s0));
-        GLR_LAUNCH(h, 1, sort_fix_basis(h->evals, S.V(), n, n, h->U, n, h->evals_sorted, s0));
+        SortGroup sg{};
+        sg.mat[sg.nmat++] = sort_mat(h, n, h->bj_vpar ? h->Vbuf : h->Vbuf2, h->U);
+        GLR_LAUNCH(h, 2, sort_group(sg, s0));
         GLR_LAUNCH(h, 1, tc::transpose_round(h->UT, n, h->U, n, n, n, s0));
     }
     GLR_CK(h0, cudaEventRecord(h0->rpow, s0));
@@ -386,11 +508,9 @@ int refresh_power(glr_handle* h, cudaStream_t st) {
     return GLR_OK;
 }
 
-// Truncated refreshes of several matrices with large k: each handle's power iteration on its
-// own side stream, then the k x k Rayleigh-Ritz eigen-decompositions of all of them in one
-// cooperative Jacobi launch (k_jacobi.cu: every CTA of the grid works on every matrix, where the
-// one-CTA Jacobi of refresh_tail would take k x k rotations in a single SM), then each handle's
-// finish on its own stream.  Without cooperative launches, refresh_tail per handle.
+// Truncated refreshes of several matrices with large k: each handle's power iteration on its own
+// side stream, then the k x k Rayleigh-Ritz problems of all of them, then each handle's finish on
+// its own stream.
 int refresh_trunc_grouped(std::vector<glr_handle*>& hs) {
     for (glr_handle* h : hs) {
         PhaseScope ps(h, GLR_PH_REFRESH, h->rstream);
@@ -399,98 +519,7 @@ int refresh_trunc_grouped(std::vector<glr_handle*>& hs) {
         g_ws = nullptr;
         if (rc != GLR_OK) return rc;
     }
-    // k <= 256: every matrix's eigenproblem in one launch, one CTA each (k_eig.cu)
-    bool small = true;
-    for (glr_handle* h : hs) small = small && h->k <= 256;
-    if (small) {
-        for (size_t c0 = 0; c0 < hs.size(); c0 += kEigGroupMax) {
-            const size_t c1 = std::min(hs.size(), c0 + (size_t)kEigGroupMax);
-            glr_handle* h0 = hs[c0];
-            cudaStream_t s0 = h0->rstream;
-            EigGroup g{};
-            g.max_sweeps = 40;
-            for (size_t i = c0; i < c1; ++i) {
-                glr_handle* h = hs[i];
-                if (h != h0) {
-                    GLR_CK(h, cudaEventRecord(h->rpow, h->rstream));
-                    GLR_CK(h0, cudaStreamWaitEvent(s0, h->rpow, 0));
-                }
-                EigMat& M = g.mat[g.nmat++];
-                const int n = h->k;
-                M.n = n; M.tol = 4.f * 5.96e-8f * sqrtf(static_cast<float>(n)) + 1e-7f;
-                M.H = h->Hk; M.nparts = 1; M.ld = n; M.V = h->Vk; M.evals = h->evals; M.sweeps = h->dflags + 1;
-            }
-            {
-                PhaseScope ps(h0, GLR_PH_REFRESH, s0);
-                GLR_LAUNCH(h0, 1, eig_tmem_group(g, s0));
-            }
-            GLR_CK(h0, cudaEventRecord(h0->rpow, s0));
-            for (size_t i = c0; i < c1; ++i) {
-                glr_handle* h = hs[i];
-                if (h != h0) GLR_CK(h, cudaStreamWaitEvent(h->rstream, h0->rpow, 0));
-                PhaseScope ps(h, GLR_PH_REFRESH, h->rstream);
-                g_ws = h->gemm_ws;
-                const int rc = refresh_finish(h, h->rstream);
-                g_ws = nullptr;
-                if (rc != GLR_OK) return rc;
-            }
-        }
-        return GLR_OK;
-    }
-    const int grid = jacobi_group_grid();
-    if (!grid) {
-        for (glr_handle* h : hs) {
-            PhaseScope ps(h, GLR_PH_REFRESH, h->rstream);
-            g_ws = h->gemm_ws;
-            const int rc = refresh_tail(h, h->rstream);
-            g_ws = nullptr;
-            if (rc != GLR_OK) return rc;
-        }
-        return GLR_OK;
-    }
-    for (size_t c0 = 0, c1 = 0; c0 < hs.size(); c0 = c1) {
-        size_t rot = 0;
-        for (c1 = c0; c1 < hs.size() && c1 - c0 < (size_t)kGroupMax; ++c1) {
-            const size_t add = jacobi_rot_floats(hs[c1]->k) * sizeof(float);
-            if (c1 > c0 && rot + add > kJacobiMaxSmem) break;
-            rot += add;
-        }
-        glr_handle* h0 = hs[c0];
-        cudaStream_t s0 = h0->rstream;
-        JacobiGroup g{};
-        size_t soff = 0;
-        g.max_sweeps = 40;
-        g.bar = h0->dflags + 4; g.err = h0->dflags + 2; g.part = h0->jpart;
-        for (size_t i = c0; i < c1; ++i) {
-            glr_handle* h = hs[i];
-            if (h != h0) {
-                GLR_CK(h, cudaEventRecord(h->rpow, h->rstream));
-                GLR_CK(h0, cudaStreamWaitEvent(s0, h->rpow, 0));
-            }
-            JacobiMat& M = g.mat[g.nmat++];
-            const int n = h->k;
-            M.n = n; M.tol = 4.f * 5.96e-8f * sqrtf(static_cast<float>(n)) + 1e-7f;
-            M.H = h->Hk; M.H2 = h->scratch; M.V = h->Vk; M.evals = h->evals;
-            M.sweeps = h->dflags + 1;
-            M.soff = (int)soff;
-            soff += jacobi_rot_floats(n);
-        }
-        {
-            PhaseScope ps(h0, GLR_PH_REFRESH, s0);
-            GLR_LAUNCH(h0, 1, jacobi_group(g, grid, s0));
-        }
-        GLR_CK(h0, cudaEventRecord(h0->rpow, s0));
-        for (size_t i = c0; i < c1; ++i) {
-            glr_handle* h = hs[i];
-            if (h != h0) GLR_CK(h, cudaStreamWaitEvent(h->rstream, h0->rpow, 0));
-            PhaseScope ps(h, GLR_PH_REFRESH, h->rstream);
-            g_ws = h->gemm_ws;
-            const int rc = refresh_finish(h, h->rstream);
-            g_ws = nullptr;
-            if (rc != GLR_OK) return rc;
-        }
-    }
-    return GLR_OK;
+    return refresh_tails(hs);
 }
 
 
@@ -531,18 +560,6 @@ int refresh_op(std::vector<glr_handle*>& hs, cudaError_t (*launch)(tc::TcGroup&,
 }
 
 int cdiv(int a, int b) { return (a + b - 1) / b; }
-
-// One grouped fp32 product per handle (fill describes it), 64 per launch.
-template <class Fill>
-int fp32_products(std::vector<glr_handle*>& hs, cudaStream_t st, Fill fill) {
-    for (size_t c0 = 0; c0 < hs.size(); c0 += 64) {
-        GemmGroup gg{};
-        for (size_t i = c0; i < hs.size() && i < c0 + 64; ++i) fill(hs[i], gg.mat[gg.nmat++]);
-        PhaseScope ps(hs[c0], GLR_PH_REFRESH, st);
-        GLR_LAUNCH(hs[c0], 1, gemm_group_f32(gg, st));
-    }
-    return GLR_OK;
-}
 
 // X^T X (Gram partials over row chunks), its factor L^{-1}, then X <- X L^{-T} (and X^T): the
 // CholeskyQR of X = Z (n' rows) or Q (m' rows) in TF32 products.
@@ -678,54 +695,19 @@ int refresh_tcl_grouped(std::vector<glr_handle*>& hs) {
         return true;
     });
     if (rc != GLR_OK) return rc;
-    // the k x k problems: the blocked Jacobi for k a multiple of 128 from 256, else one CTA each
-    std::vector<glr_handle*> small;
-    std::vector<BjItem> big;
-    for (glr_handle* h : hs) {
-        if (tcl_rr_blocked(h)) big.push_back(BjItem{h, h->k, 0, 0, false});
-        else small.push_back(h);
-        h->bj_V = nullptr;
-    }
-    for (size_t c0 = 0; c0 < small.size(); c0 += kEigGroupMax) {
-        EigGroup g{};
-        g.max_sweeps = 40;
-        for (size_t i = c0; i < small.size() && i < c0 + (size_t)kEigGroupMax; ++i) {
-            glr_handle* h = small[i];
-            EigMat& M = g.mat[g.nmat++];
-            const int n = h->k;
-            M.n = n; M.tol = 4.f * 5.96e-8f * sqrtf(static_cast<float>(n)) + 1e-7f;
-            M.H = h->gpart; M.nparts = cdiv(h->np, tc::kGramChunk); M.ld = h->kpad;
-            M.V = h->Vk; M.evals = h->evals; M.sweeps = h->dflags + 1;
-        }
-        PhaseScope ps(small[c0], GLR_PH_REFRESH, s0);
-        GLR_LAUNCH(small[c0], 1, eig_tmem_group(g, s0));
-    }
-    if (!big.empty()) {
-        glr_handle* b0 = big[0].h;
-        PhaseScope ps(b0, GLR_PH_REFRESH, s0);
-        rc = bjac_prepare(big, b0, s0, [](glr_handle* h, BjacPrep& P) {
-            P.part = h->gpart; P.nparts = cdiv(h->np, tc::kGramChunk); P.ld = h->kpad;
-        });
-        if (rc == GLR_OK) rc = bjac_run(big, b0, s0);
-        if (rc != GLR_OK) return rc;
-        for (const BjItem& S : big) {
-            GLR_LAUNCH(S.h, 1, bjac_diag(S.h->Hbuf, S.n, S.h->evals, s0));
-            S.h->bj_V = S.V();
-        }
+    std::vector<EigItem> items;                             // H is the sum of the Gram partials
+    for (glr_handle* h : hs) items.push_back(EigItem{h, h->k, h->gpart, cdiv(h->np, tc::kGramChunk), h->kpad, h->Vk});
+    {
+        PhaseScope ps(h0, GLR_PH_REFRESH, s0);
+        if ((rc = eig_solve(items, s0, s0)) != GLR_OK) return rc;
     }
     // the finish, grouped: sorted Ritz pairs, Q <- Q W, column signs, the Householder WY form,
     // Yt = Y T^T, then Y^T for the W = Y^T Mbar products
     for (size_t c0 = 0; c0 < hs.size(); c0 += 64) {
-        FinishGroup fg{};
-        for (size_t i = c0; i < hs.size() && i < c0 + 64; ++i) {
-            glr_handle* h = hs[i];
-            FinishMat& F = fg.mat[fg.nmat++];
-            F.mp = h->mp; F.k = h->k; F.evals = h->evals; F.V = h->bj_V ? h->bj_V : h->Vk; F.W = h->gram;
-            F.evals_sorted = h->evals_sorted;
-            F.Wtop = h->scratch; F.Y = h->Y; F.T = h->T; F.s = h->dsign;
-        }
+        SortGroup sg{};
+        for (size_t i = c0; i < hs.size() && i < c0 + 64; ++i) sg.mat[sg.nmat++] = sort_mat(hs[i], hs[i]->k, hs[i]->Vk, hs[i]->gram);
         PhaseScope ps(hs[c0], GLR_PH_REFRESH, s0);
-        GLR_LAUNCH(hs[c0], 1, finish_group(fg, 0, s0));
+        GLR_LAUNCH(hs[c0], 2, sort_group(sg, s0));
     }
     if ((rc = fp32_products(hs, s0, [](glr_handle* h, GemmMat& G) {          // Qn = Q W
              G.M = h->mp; G.N = h->k; G.K = h->k;

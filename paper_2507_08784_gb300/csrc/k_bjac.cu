@@ -17,7 +17,7 @@
 //      round's storage order;
 // and a sweep ends with the off-diagonal norm, checked on the host against tol^2 of the total.
 // V starts as the identity, so its columns follow H's storage order; at the end diag(H) and V
-// are sorted by descending eigenvalue with the sign rule of the small solvers (sort_fix_basis).
+// orthogonalised once more in fp32 and sorted by descending eigenvalue with the sign rule of the small solvers (sort_group).
 //
 // Every product keeps its output's TF32 low part beside it (H_lo, T^T_lo, V_lo; J_lo from the
 // pair sweep), so each operand enters the MMAs as hi + lo.
@@ -99,21 +99,13 @@ __global__ void __launch_bounds__(pair::PTHREADS, 1) bjac_pair_kernel(const __gr
     }
 }
 
-// Before the first round, per problem: H = the sum of nparts partial matrices (leading dimension
-// ld; none when H is already formed), H's TF32 low part, V = I and V's low part 0.
+// Before the first round, per problem: H's TF32 low part, V = I and V's low part 0.
 __global__ void bjac_prep_kernel(const __grid_constant__ BjacPrepGroup g) {
     const BjacPrep& P = g.mat[blockIdx.y];
     const int n = P.n;
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < (int64_t)n * n; q += (int64_t)gridDim.x * blockDim.x) {
         const int r = (int)(q / n), c = (int)(q % n);
-        float h;
-        if (P.nparts > 0) {
-            h = 0.f;
-            for (int p = 0; p < P.nparts; ++p) h += P.part[(int64_t)p * P.ld * P.ld + (int64_t)r * P.ld + c];
-            P.H[q] = h;
-        } else {
-            h = P.H[q];
-        }
+        const float h = P.H[q];
         P.Hlo[q] = h - __uint_as_float(__float_as_uint(h) & 0xffffe000u);
         P.V[q] = r == c ? 1.f : 0.f;
         P.Vlo[q] = 0.f;
@@ -122,14 +114,12 @@ __global__ void bjac_prep_kernel(const __grid_constant__ BjacPrepGroup g) {
 
 __global__ void count_flag_kernel(int* flag, int v) { atomicAdd(flag, v); }
 
-__global__ void bjac_eye_kernel(float* V, int n) {
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < (int64_t)n * n; q += (int64_t)gridDim.x * blockDim.x)
-        V[q] = (q / n == q % n) ? 1.f : 0.f;
-}
 __global__ void bjac_diag_kernel(const float* H, int n, float* evals) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) evals[i] = H[(int64_t)i * n + i];
 }
-
+__global__ void add_diagonal_kernel(float* A, int n, float v) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) A[(int64_t)i * n + i] += v;
+}
 
 }  // namespace
 
@@ -166,8 +156,8 @@ cudaError_t count_flag(int* flag, int v, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t bjac_eye(float* V, int n, cudaStream_t st) {
-    bjac_eye_kernel<<<1024, 256, 0, st>>>(V, n);
+cudaError_t add_diagonal(float* A, int n, float v, cudaStream_t st) {
+    add_diagonal_kernel<<<(n + 255) / 256, 256, 0, st>>>(A, n, v);
     return cudaGetLastError();
 }
 

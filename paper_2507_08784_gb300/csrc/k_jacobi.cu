@@ -13,6 +13,16 @@
 // keeps every CTA resident, which is what makes the barrier safe to wait on.  Data written by one
 // CTA and read by another (H, V, the norm partials) is read through L2 (__ldcg), so no stale L1
 // line survives a barrier.
+//
+// For n <= 512 a matrix fits the shared memory of one thread-block cluster and is solved there
+// (jacobi_cluster_kernel), a launch a matrix: the rows of H (two buffers) and V are spread over up to
+// 16 CTAs, a round's rotations and the partner rows come over distributed shared memory, and a round
+// ends with one hardware cluster barrier.  The rotations, their order and every product and sum are
+// those of the grid-wide kernel, so the results are the same bits.  Bound by shared-memory
+// instructions and the cluster's barrier and remote loads; the grid-wide kernel pays
+// 14 us a round for its barrier in global memory and the L2 round trips.
+#include <cooperative_groups.h>
+
 #include "glr_internal.cuh"
 
 namespace glr {
@@ -215,7 +225,237 @@ __global__ void __launch_bounds__(JT) jacobi_group_kernel(const __grid_constant_
     }
 }
 
+// ---- n <= 512: one cluster a matrix ------------------------------------------------------------
+constexpr int CT = 512;
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() { cluster_arrive(); cluster_wait(); }
+template <class T> __device__ __forceinline__ T* peer(T* p, int cta) {       // p in another CTA of the cluster
+    return cooperative_groups::this_cluster().map_shared_rank(p, cta);
+}
+// c x - s y and s x + c y, rounded as the grid-wide kernel's expressions are (checked bit for bit)
+__device__ __forceinline__ float rot_dif(float c, float x, float s, float y) { return __fmaf_rn(c, x, -__fmul_rn(s, y)); }
+__device__ __forceinline__ float rot_sum(float s, float x, float c, float y) { return __fmaf_rn(s, x, __fmul_rn(c, y)); }
+// Slots (row pairs) a CTA and CTAs a matrix; V's rows a CTA.
+__host__ __device__ __forceinline__ int cluster_slots(int half) { return half > 128 ? (half + 15) / 16 : 8; }
+__host__ __device__ __forceinline__ int cluster_ctas(int n) {
+    const int half = (n + 1) / 2, S = cluster_slots(half);
+    return (half + S - 1) / S;
+}
+size_t cluster_smem(int n) {
+    const size_t half = (n + 1) / 2, S = cluster_slots((int)half), C = cluster_ctas(n);
+    const size_t rows = (2 * S + 3) + (n + C - 1) / C;
+    return sizeof(float) * (4 * half + rows * n);
+}
+
+// The round's pairs sit in npad / 2 slots (T, B); slot 0's T is index 0, the others move by one slot a
+// round: T to the left, B to the right, T of slot 1 to B of slot 0, B of the last slot to its T.  A
+// CTA holds the H rows of S consecutive slots, in two rings of row buffers with a spare each, so
+// that only one T and one B row a round go to a neighbour's spare, written there in place of the
+// row itself.  A row pair's 2 x 2 blocks are then one thread's and are updated in place.
+__global__ void __launch_bounds__(CT, 1) jacobi_cluster_kernel(const __grid_constant__ JacobiMat M, int max_sweeps) {
+    extern __shared__ __align__(16) float csm[];
+    __shared__ float red[2][CT / 32], part[2];
+    __shared__ int stop;
+    const int n = M.n, C = gridDim.x, b = blockIdx.x, t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int npad = n + (n & 1), half = npad / 2, nm1 = npad - 1, Smax = cluster_slots(half);
+    const int s0 = b * Smax, S = half - s0 < Smax ? half - s0 : Smax;          // own slots s0 .. s0 + S - 1
+    const int slast = half - (C - 1) * Smax;                                // the last CTA's slots
+    const int ST = b == 0 ? S - 1 : S, LT = ST + 1, LB = S + 1;             // rings (slot 0's T is apart)
+    const int R = (n + C - 1) / C, v0 = b * R, vrows = n - v0 < R ? (n - v0 > 0 ? n - v0 : 0) : R;
+    float2* const scs = reinterpret_cast<float2*>(csm);                     // 2 x half: cos, sin
+    float* const F = csm + 4 * half;                                        // index 0's row
+    float* const Tr = F + n;
+    float* const Br = Tr + (size_t)(Smax + 1) * n;
+    float* const V = Br + (size_t)(Smax + 1) * n;
+    // the buffer of the first ring T and of the first B: own, of the left and of the right neighbour
+    const int LTl = b == 1 ? Smax : Smax + 1, LBr = (b + 1 == C - 1 ? slast : Smax) + 1;
+    int tb = 0, bb = 0, tbl = 0, bbr = 0, par = 0;
+    auto wrap = [](int x, int L) { return x >= L ? x - L : x; };
+    auto trow = [&](int i) -> float* {                                      // T, B of own slot s0 + i
+        return b == 0 ? (i == 0 ? F : Tr + (size_t)wrap(tb + i - 1, LT) * n) : Tr + (size_t)wrap(tb + i, LT) * n;
+    };
+    auto brow = [&](int i) -> float* { return Br + (size_t)wrap(bb + i, LB) * n; };
+    auto tidx = [&](int slot, int rd) { return slot == 0 ? 0 : 1 + (rd + slot < nm1 ? rd + slot : rd + slot - nm1); };
+    auto bidx = [&](int slot, int rd) { return 1 + (rd - slot < 0 ? rd - slot + nm1 : rd - slot); };
+    for (int e = t; e < 2 * S * n; e += CT) {
+        const int i = (e / n) >> 1, c = e % n, low = (e / n) & 1;
+        const int r = low ? bidx(s0 + i, 0) : tidx(s0 + i, 0);
+        (low ? brow(i) : trow(i))[c] = r < n ? M.H[(size_t)r * n + c] : 0.f;
+    }
+    for (int e = t; e < vrows * n; e += CT) V[e] = v0 + e / n == e % n ? 1.f : 0.f;
+    cluster_sync();
+    // the columns' rotations in this thread's share of the work: warps share a slot when there are few
+    const int G = S > 8 ? 1 : S > 4 ? 2 : S > 2 ? 4 : S > 1 ? 8 : 16;
+    const int myslot = warp / G, sub = warp % G, JU = (half + 31) / 32;
+    int sweep = 0;
+    for (;; ++sweep) {
+        float off = 0.f, tot = 0.f;
+        for (int e = t; e < 2 * S * n; e += CT) {
+            const int i = (e / n) >> 1, c = e % n, low = (e / n) & 1;
+            const float h = (low ? brow(i) : trow(i))[c];
+            tot += h * h;
+            if ((low ? bidx(s0 + i, 0) : tidx(s0 + i, 0)) != c) off += h * h;
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            off += __shfl_xor_sync(0xffffffffu, off, o);
+            tot += __shfl_xor_sync(0xffffffffu, tot, o);
+        }
+        if (lane == 0) { red[0][warp] = off; red[1][warp] = tot; }
+        __syncthreads();
+        if (t == 0) {
+            float o2 = 0.f, t2 = 0.f;
+            for (int w = 0; w < CT / 32; ++w) { o2 += red[0][w]; t2 += red[1][w]; }
+            part[0] = o2; part[1] = t2;
+        }
+        cluster_sync();
+        if (t == 0) {                                   // the same sums, the same decision in every CTA
+            float o2 = 0.f, t2 = 0.f;
+            for (int c = 0; c < C; ++c) { o2 += peer(part, c)[0]; t2 += peer(part, c)[1]; }
+            stop = (o2 <= M.tol * M.tol * t2 || sweep >= max_sweeps) ? 1 : 0;
+        }
+        cluster_sync();                                 // part is read before anyone writes it again
+        if (stop) break;
+        for (int rd = 0; rd < nm1; ++rd) {
+            float2* cs = scs + par * half;
+            for (int e = t; e < S * C; e += CT) {       // own slots' rotations, to every CTA
+                const int i = e % S, to = e / S, x = tidx(s0 + i, rd), y = bidx(s0 + i, rd);
+                const int p = x < y ? x : y, q = x < y ? y : x;
+                float c = 1.f, s = 0.f;
+                if (q < n) {
+                    const float* rp = x < y ? trow(i) : brow(i);
+                    const float* rq = x < y ? brow(i) : trow(i);
+                    const float hpq = rp[q], hpp = rp[p], hqq = rq[q];
+                    if (fabsf(hpq) > 1e-30f && fabsf(hpq) > 1e-9f * sqrtf(fabsf(hpp * hqq))) {
+                        const float theta = (hqq - hpp) / (2.f * hpq);
+                        float tt;
+                        if (fabsf(theta) > 1e15f) tt = 0.5f / theta;
+                        else tt = copysignf(1.f, theta) / (fabsf(theta) + sqrtf(theta * theta + 1.f));
+                        c = 1.f / sqrtf(tt * tt + 1.f);
+                        s = tt * c;
+                    }
+                }
+                peer(cs, to)[s0 + i] = make_float2(c, s);
+            }
+            cluster_sync();
+            // own row pair: its rows, and where each goes
+            const float *hp = nullptr, *hq = nullptr;
+            float *op = nullptr, *oq = nullptr;
+            float2 ri = make_float2(1.f, 0.f);
+            const bool mine = myslot < S;
+            if (mine) {
+                const int i = myslot, slot = s0 + i;
+                float *tr = trow(i), *br = brow(i), *to = tr, *bo = br;
+                if (slot > 0 && i == (b == 0 ? 1 : 0)) {                    // the first ring T leaves
+                    if (b == 0) to = Br + (size_t)wrap(bb + S, LB) * n;
+                    else to = peer(Tr, b - 1) + (size_t)wrap(tbl + LTl - 1, LTl) * n;
+                }
+                if (i == S - 1 && half > 1) {                               // the last B leaves
+                    if (b == C - 1) bo = Tr + (size_t)wrap(tb + ST, LT) * n;
+                    else bo = peer(Br, b + 1) + (size_t)wrap(bbr + LBr - 1, LBr) * n;
+                }
+                const bool up = tidx(slot, rd) < bidx(slot, rd);
+                hp = up ? tr : br; hq = up ? br : tr;
+                op = up ? to : bo; oq = up ? bo : to;
+                ri = cs[slot];
+            }
+            for (int u = sub; u < JU; u += G) {
+                const int j = lane + 32 * u;
+                if (!mine || j >= half) continue;
+                const int x = tidx(j, rd), y = bidx(j, rd);
+                const int pj = x < y ? x : y, qj = x < y ? y : x;
+                const float2 rj = cs[j];
+                const bool vq = qj < n;
+                const float h00 = hp[pj], h10 = hq[pj], h01 = vq ? hp[qj] : 0.f, h11 = vq ? hq[qj] : 0.f;
+                const float a00 = rot_dif(ri.x, h00, ri.y, h10), a01 = rot_dif(ri.x, h01, ri.y, h11);
+                const float a10 = rot_sum(ri.y, h00, ri.x, h10), a11 = rot_sum(ri.y, h01, ri.x, h11);
+                const bool diag = j == s0 + myslot && ri.y != 0.f;
+                op[pj] = rot_dif(rj.x, a00, rj.y, a01);
+                oq[pj] = diag ? 0.f : rot_dif(rj.x, a10, rj.y, a11);
+                if (vq) {
+                    op[qj] = diag ? 0.f : rot_sum(rj.y, a00, rj.x, a01);
+                    oq[qj] = rot_sum(rj.y, a10, rj.x, a11);
+                }
+            }
+            cluster_arrive();
+            for (int r = warp; r < vrows; r += 2 * (CT / 32)) {              // V <- V J, in place, two rows at a time
+                float* w0 = V + (size_t)r * n;
+                const bool two = r + CT / 32 < vrows;
+                float* w1 = two ? w0 + (CT / 32) * n : w0;
+                for (int j = lane; j < half; j += 32) {
+                    const float2 rj = cs[j];
+                    if (rj.y == 0.f) continue;
+                    const int x = tidx(j, rd), y = bidx(j, rd);
+                    const int pj = x < y ? x : y, qj = x < y ? y : x;
+                    const float x0 = w0[pj], y0 = w0[qj], x1 = w1[pj], y1 = w1[qj];
+                    w0[pj] = rot_dif(rj.x, x0, rj.y, y0);
+                    w0[qj] = rot_sum(rj.y, x0, rj.x, y0);
+                    if (two) {
+                        w1[pj] = rot_dif(rj.x, x1, rj.y, y1);
+                        w1[qj] = rot_sum(rj.y, x1, rj.x, y1);
+                    }
+                }
+            }
+            cluster_wait();
+            par ^= 1;
+            if (half > 1) {
+                tb = wrap(tb + 1, LT); tbl = wrap(tbl + 1, LTl);
+                bb = bb == 0 ? LB - 1 : bb - 1; bbr = bbr == 0 ? LBr - 1 : bbr - 1;
+            }
+        }
+    }
+    for (int e = t; e < vrows * n; e += CT) M.V[(size_t)v0 * n + e] = V[e];
+    for (int e = t; e < 2 * S; e += CT) {
+        const int i = e >> 1, r = (e & 1) ? bidx(s0 + i, 0) : tidx(s0 + i, 0);
+        if (r < n) M.evals[r] = ((e & 1) ? brow(i) : trow(i))[r];
+    }
+    if (b == 0 && t == 0 && M.sweeps) *M.sweeps = sweep;
+}
+
+cudaLaunchConfig_t cluster_config(int n, cudaLaunchAttribute* attr, cudaStream_t st) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(cluster_ctas(n));
+    cfg.blockDim = dim3(CT);
+    cfg.dynamicSmemBytes = cluster_smem(n);
+    cfg.stream = st;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = cluster_ctas(n); attr->val.clusterDim.y = 1; attr->val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+// per device: set on every call (cheap next to the launch)
+cudaError_t cluster_attributes() {
+    const void* k = reinterpret_cast<const void*>(jacobi_cluster_kernel);
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem(512));
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+}
+
 }  // namespace
+
+bool jacobi_cluster_ok(int n) {
+    if (n < 1 || n > 512) return false;
+    cudaLaunchAttribute attr{};
+    const cudaLaunchConfig_t cfg = cluster_config(n, &attr, nullptr);
+    int clusters = 0;
+    if (cluster_attributes() != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&clusters, reinterpret_cast<const void*>(jacobi_cluster_kernel), &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return clusters > 0;
+}
+
+cudaError_t jacobi_cluster(const JacobiMat& M, int max_sweeps, cudaStream_t st) {
+    if (M.n < 1 || M.n > 512) return cudaErrorInvalidValue;
+    const cudaError_t e = cluster_attributes();
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute attr{};
+    const cudaLaunchConfig_t cfg = cluster_config(M.n, &attr, st);
+    return cudaLaunchKernelEx(&cfg, jacobi_cluster_kernel, M, max_sweeps);
+}
 
 int jacobi_group_grid() {
     static int grid = 0;

@@ -1,5 +1,6 @@
 // One sweep of parallel two-sided Jacobi on a 128 x 128 symmetric block, held in the registers of
-// one 512-thread CTA: the inner solver of the blocked Jacobi (k_bjac.cu).
+// one 512-thread CTA: the inner solver of the blocked Jacobis (k_bjac.cu, k_eig.cu), and for 128
+// indices or fewer, repeated, the whole solver.
 //
 // The 128 indices are split into groups of 2 g consecutive ones, each group into a half A and a
 // half B of g.  A level of g rounds rotates every A index once against every B index of its group
@@ -123,12 +124,16 @@ struct Block {
 
     // The g rounds of level g.  S and W hold the block in shared memory and the registers its
     // level-g arrangement; on return only the registers are current (B back in its own order).
-    // xch: 2 x 16 x 128 floats, apq: 2 x 64 floats of shared memory.
-    __device__ __forceinline__ void level(const float* S, int g, float* xch, float* apq, int warp, int lane) {
+    // xch: 2 x 16 x 128 floats, apq: 2 x 64 floats of shared memory.  A block of 2 lim < 128 indices
+    // takes lim / 4 warps and levels up to lim; the columns past it hold zeros.
+    __device__ __forceinline__ void level(const float* S, int g, float* xch, float* apq, int warp, int lane, int lim = 64) {
         const int j0 = 2 * lane, j1 = 2 * lane + 1;
-        float app0 = S[posA(j0, g) * (PLD + 1)], app1 = S[posA(j1, g) * (PLD + 1)];
-        float aqq0 = S[posB(j0, g) * (PLD + 1)], aqq1 = S[posB(j1, g) * (PLD + 1)];
-        float apq0 = S[posA(j0, g) * PLD + posB(j0, g)], apq1 = S[posA(j1, g) * PLD + posB(j1, g)];
+        float app0 = 0.f, app1 = 0.f, aqq0 = 0.f, aqq1 = 0.f, apq0 = 0.f, apq1 = 0.f;
+        if (j0 < lim) {
+            app0 = S[posA(j0, g) * (PLD + 1)]; app1 = S[posA(j1, g) * (PLD + 1)];
+            aqq0 = S[posB(j0, g) * (PLD + 1)]; aqq1 = S[posB(j1, g) * (PLD + 1)];
+            apq0 = S[posA(j0, g) * PLD + posB(j0, g)]; apq1 = S[posA(j1, g) * PLD + posB(j1, g)];
+        }
         const int hg = g > 1 ? g / 2 : 1;
         const int src = (lane & ~(hg - 1)) | ((lane + 1) & (hg - 1));
         const int row = 4 * warp;                              // next warp's first row in the group
@@ -171,8 +176,10 @@ struct Block {
                 *reinterpret_cast<float2*>(ab + 2 * lane) = make_float2(x, y);
             }
             __syncthreads();
-            const float2 nx = *reinterpret_cast<const float2*>(ab + 2 * lane);
-            apq0 = nx.x; apq1 = nx.y;
+            if (j0 < lim) {
+                const float2 nx = *reinterpret_cast<const float2*>(ab + 2 * lane);
+                apq0 = nx.x; apq1 = nx.y;
+            }
             if (g > 2) {
                 BA[0] = BA[1]; BA[1] = BA[2]; BA[2] = BA[3];
                 BB[0] = BB[1]; BB[1] = BB[2]; BB[2] = BB[3];

@@ -1,7 +1,6 @@
-// Refresh kernels: the Semi-Lazy SVD step of Eq. SVD-P1 on the device.
-//  * full basis: eigen-decomposition of H = Mbar Mbar^T by parallel cyclic Jacobi;
-//  * truncated basis: block power iteration with CholeskyQR2, Rayleigh-Ritz (Jacobi on the
-//    k x k projected Gram matrix) and the Householder reconstruction of the complement.
+// Refresh kernels (the Semi-Lazy SVD step of Eq. SVD-P1): the order and sign rule of the
+// eigenpairs, the CholeskyQR factors, and the Householder reconstruction of a truncated basis's
+// complement (the eigenproblems are in k_eig.cu and k_bjac.cu).
 #include "glr_internal.cuh"
 
 namespace glr {
@@ -123,80 +122,95 @@ __device__ __forceinline__ uint32_t float_order(float f) {
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// argmax |column| (first index on ties) of one column, by one warp; returns the sign there.
-__device__ float warp_column_sign(const float* A, int rows, int ld, int col) {
-    const int lane = threadIdx.x & 31;
-    float best = -1.f;
-    int bidx = 0x7fffffff;
-    for (int a = lane; a < rows; a += 32) {
-        const float v = fabsf(A[(size_t)a * ld + col]);
-        if (v > best) { best = v; bidx = a; }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bidx, o);
-        if (ob > best || (ob == best && oi < bidx)) { best = ob; bidx = oi; }
-    }
-    return (bidx < rows && A[(size_t)bidx * ld + col] < 0.f) ? -1.f : 1.f;
-}
-
-__device__ __forceinline__ void sort_fix_body(const float* evals, const float* V, int n, int ncols, float* Out,
-                                              int ldo, float* evals_sorted, int npow2) {
-    extern __shared__ unsigned long long keys[];
-    const int tid = threadIdx.x;
-    for (int i = tid; i < npow2; i += blockDim.x)
-        keys[i] = (i < n) ? ((static_cast<unsigned long long>(float_order(evals[i])) << 32) |
-                             (0xFFFFFFFFull - static_cast<unsigned long long>(i)))
-                          : 0ull;
-    __syncthreads();
-    for (int size = 2; size <= npow2; size <<= 1)
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int i = tid; i < npow2; i += blockDim.x) {
-                const int partner = i ^ stride;
-                if (partner > i) {
-                    const bool desc = (i & size) == 0;
-                    const unsigned long long x = keys[i], y = keys[partner];
-                    if ((x < y) == desc) { keys[i] = y; keys[partner] = x; }
-                }
-            }
-            __syncthreads();
+// Column statistics of 32 columns from col0 of A (rows x cols, leading dimension ld) by a CTA of 32 x
+// 32 threads, lanes along the columns: the sign of the largest-magnitude entry (first row on
+// ties) and the sum of squares, both valid in row ty = 0.
+__device__ __forceinline__ void column_stats(const float* A, int rows, int64_t ld, int col, bool in, float& sign, float& ss) {
+    __shared__ float sbest[32][33], sval[32][33], ssum[32][33];
+    __shared__ int sidx[32][33];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    float best = -1.f, val = 0.f, sum = 0.f;
+    int idx = 0x7fffffff;
+    if (in)
+        for (int a = ty; a < rows; a += 32) {
+            const float v = A[a * ld + col], m = fabsf(v);
+            sum = fmaf(v, v, sum);
+            if (m > best) { best = m; val = v; idx = a; }
         }
-    const int warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
-    for (int c = warp; c < ncols; c += nw) {
-        const int src = static_cast<int>(0xFFFFFFFFull - (keys[c] & 0xFFFFFFFFull));
-        const float sg = warp_column_sign(V, n, n, src);
-        // renormalise: thousands of plane rotations let the column norms drift by a few ulp each
-        float ss = 0.f;
-        for (int a = lane; a < n; a += 32) { const float v = V[(size_t)a * n + src]; ss = fmaf(v, v, ss); }
-        for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        const float scale = sg / sqrtf(ss);
-        for (int a = lane; a < n; a += 32) Out[(size_t)a * ldo + c] = scale * V[(size_t)a * n + src];
-        if (lane == 0 && evals_sorted) evals_sorted[c] = evals[src];
+    __syncthreads();
+    sbest[ty][tx] = best; sval[ty][tx] = val; ssum[ty][tx] = sum; sidx[ty][tx] = idx;
+    __syncthreads();
+    if (ty == 0) {
+        for (int o = 16; o > 0; o >>= 1)                   // pairwise: what a warp's xor reduction gives
+            for (int q = 0; q < o; ++q) ssum[q][tx] += ssum[q + o][tx];
+        sum = ssum[0][tx];
+        for (int q = 0; q < 32; ++q) {
+            if (sbest[q][tx] > best || (sbest[q][tx] == best && sidx[q][tx] < idx)) {
+                best = sbest[q][tx]; val = sval[q][tx]; idx = sidx[q][tx];
+            }
+        }
+        sign = val < 0.f ? -1.f : 1.f;
+        ss = sum;
     }
 }
-__global__ void __launch_bounds__(1024) sort_fix_kernel(const float* evals, const float* V, int n, int ncols,
-                                                        float* Out, int ldo, float* evals_sorted, int npow2) {
-    sort_fix_body(evals, V, n, ncols, Out, ldo, evals_sorted, npow2);
+
+// Eigenpairs by descending value (ties by index; NaN ordered as its bits), in two launches: a CTA per
+// 32 columns counts each one's rank and writes the column's number and its scale (sign rule, unit
+// norm: thousands of plane rotations let the norms drift by a few ulp each) there, then a CTA per
+// row gathers the row.  One CTA sorting and moving everything took 10.3 ms for n = 2048.
+__global__ void __launch_bounds__(1024) sort_rank_kernel(const __grid_constant__ SortGroup g) {
+    const SortMat& M = g.mat[blockIdx.y];
+    const int n = M.n, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    if ((int)blockIdx.x * 32 >= n) return;
+    const int col = blockIdx.x * 32 + tx;
+    __shared__ int cnt[32][33];
+    int c = 0;
+    if (col < n) {
+        const uint32_t mine = float_order(M.evals[col]);
+        for (int j = ty; j < n; j += 32) {
+            const uint32_t other = float_order(M.evals[j]);
+            c += (other > mine || (other == mine && j < col)) ? 1 : 0;
+        }
+    }
+    cnt[ty][tx] = c;
+    float sign = 1.f, ss = 1.f;
+    column_stats(M.V, n, n, col, col < n, sign, ss);       // its barriers cover cnt
+    if (ty == 0 && col < n) {
+        int rank = 0;
+        for (int q = 0; q < 32; ++q) rank += cnt[q][tx];
+        M.order[rank] = col;
+        M.scale[rank] = sign / sqrtf(ss);
+        if (M.evals_sorted) M.evals_sorted[rank] = M.evals[col];
+    }
+    if (n > 32) return;
+    __syncthreads();                                       // one CTA holds it all: no second launch
+    if (col < n && ty < n) M.Out[(size_t)ty * n + col] = M.scale[col] * M.V[(size_t)ty * n + M.order[col]];
 }
-__global__ void __launch_bounds__(1024) sort_fix_group_kernel(const __grid_constant__ FinishGroup g, int npow2) {
-    const FinishMat& M = g.mat[blockIdx.x];
-    sort_fix_body(M.evals, M.V, M.k, M.k, M.W, M.k, M.evals_sorted, npow2);
+__global__ void __launch_bounds__(256) sort_gather_kernel(const __grid_constant__ SortGroup g) {
+    extern __shared__ float srow[];
+    const SortMat& M = g.mat[blockIdx.y];
+    const int n = M.n;
+    if (n <= 32) return;
+    for (int r = blockIdx.x; r < n; r += gridDim.x) {
+        __syncthreads();
+        for (int c = threadIdx.x; c < n; c += 256) srow[c] = M.V[(size_t)r * n + c];
+        __syncthreads();
+        for (int c = threadIdx.x; c < n; c += 256) M.Out[(size_t)r * n + c] = M.scale[c] * srow[M.order[c]];
+    }
 }
 
-__global__ void fix_signs_group_kernel(const __grid_constant__ FinishGroup g) {
+// The largest-magnitude entry of each column of Q (m' x k) positive; a CTA per 32 columns.
+__global__ void __launch_bounds__(1024) fix_signs_group_kernel(const __grid_constant__ FinishGroup g) {
     const FinishMat& M = g.mat[blockIdx.y];
-    const int col = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (col >= M.k) return;
-    const float sg = warp_column_sign(M.Q, M.mp, M.k, col);
-    if (sg < 0.f)
-        for (int a = threadIdx.x & 31; a < M.mp; a += 32) M.Q[(size_t)a * M.k + col] = -M.Q[(size_t)a * M.k + col];
-}
-__global__ void fix_signs_kernel(float* A, int rows, int cols) {
-    const int col = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (col >= cols) return;
-    const float sg = warp_column_sign(A, rows, cols, col);
-    if (sg < 0.f)
-        for (int a = threadIdx.x & 31; a < rows; a += 32) A[(size_t)a * cols + col] = -A[(size_t)a * cols + col];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, col = blockIdx.x * 32 + tx;
+    if ((int)blockIdx.x * 32 >= M.k) return;
+    __shared__ float sg[32];
+    float sign = 1.f, ss;
+    column_stats(M.Q, M.mp, M.k, col, col < M.k, sign, ss);
+    if (ty == 0) sg[tx] = sign;
+    __syncthreads();
+    if (col < M.k && sg[tx] < 0.f)
+        for (int a = ty; a < M.mp; a += 32) M.Q[(size_t)a * M.k + col] = -M.Q[(size_t)a * M.k + col];
 }
 
 // Right-looking Cholesky (one CTA) with a diagonal shift retry on breakdown.
@@ -381,17 +395,13 @@ cudaError_t jacobi_eig(float* H, int n, float* V, float* evals, int* sweeps, cud
     return cudaGetLastError();
 }
 
-cudaError_t sort_fix_basis(const float* evals, const float* V, int n, int ncols, float* Out, int ldo,
-                           float* evals_sorted, cudaStream_t st) {
-    int npow2 = 1;
-    while (npow2 < n) npow2 <<= 1;
-    sort_fix_kernel<<<1, 1024, sizeof(unsigned long long) * npow2, st>>>(evals, V, n, ncols, Out, ldo,
-                                                                         evals_sorted, npow2);
-    return cudaGetLastError();
-}
-
-cudaError_t fix_column_signs(float* A, int rows, int cols, cudaStream_t st) {
-    fix_signs_kernel<<<(cols + 7) / 8, 256, 0, st>>>(A, rows, cols);
+cudaError_t sort_group(const SortGroup& g, cudaStream_t st) {
+    if (g.nmat <= 0) return cudaSuccess;
+    int n = 0;
+    for (int i = 0; i < g.nmat; ++i) n = g.mat[i].n > n ? g.mat[i].n : n;
+    sort_rank_kernel<<<dim3((n + 31) / 32, g.nmat), 1024, 0, st>>>(g);
+    if (n <= 32) return cudaGetLastError();
+    sort_gather_kernel<<<dim3(n < 1024 ? n : 1024, g.nmat), 256, sizeof(float) * n, st>>>(g);
     return cudaGetLastError();
 }
 
@@ -402,12 +412,8 @@ cudaError_t finish_group(const FinishGroup& g, int stage, cudaStream_t st) {
         kmax = g.mat[i].k > kmax ? g.mat[i].k : kmax;
         rows_max = g.mat[i].mp - g.mat[i].k > rows_max ? g.mat[i].mp - g.mat[i].k : rows_max;
     }
-    if (stage == 0) {                                   // sort the eigenpairs, normalise, fix signs
-        int npow2 = 1;
-        while (npow2 < kmax) npow2 <<= 1;
-        sort_fix_group_kernel<<<g.nmat, 1024, sizeof(unsigned long long) * npow2, st>>>(g, npow2);
-    } else if (stage == 1) {                            // column signs of Q
-        fix_signs_group_kernel<<<dim3((kmax + 7) / 8, g.nmat), 256, 0, st>>>(g);
+    if (stage == 1) {                                   // column signs of Q
+        fix_signs_group_kernel<<<dim3((kmax + 31) / 32, g.nmat), 1024, 0, st>>>(g);
     } else if (stage == 2) {                            // Householder top block
         hh_top_group_kernel<<<g.nmat, 1024, 0, st>>>(g);
     } else {                                            // Householder rows below
