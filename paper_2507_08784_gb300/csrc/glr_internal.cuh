@@ -245,15 +245,18 @@ cudaError_t cholesky(float* A, int n, float* scratch, int* flag, cudaStream_t st
 cudaError_t chol_inverse(const float* G, int n, float* S, int* flag, cudaStream_t st);
 // The same factor and inverse for several Gram matrices (one CTA each), each given as the sum of
 // nparts partial matrices (leading dimension ld, ld * ld apart); writes L^{-1} row-major ld x ld.
-struct CholMat { const float* part; int nparts, ld, n; float* out; int* flag; int tri_only; };   // tri_only: (U^T)^{-1} of the upper triangle of part (n x n)
+// tri_only: the inverse alone, of U^T for the upper triangle U of part (n x n), or of its unit lower one.
+enum : int { kTriUpper = 1, kTriUnitLower = 2 };
+struct CholMat { const float* part; int nparts, ld, n; float* out; int* flag; int tri_only; };
 struct CholGroup { int nmat; CholMat mat[64]; };
 cudaError_t chol_group(const CholGroup& g, cudaStream_t st);
 // The end of a truncated refresh for several matrices, one launch per stage: stage 1 fixes the
-// column signs of Q (m' x k: the largest-|entry| of each positive); 2 and 3 the Householder
-// reconstruction (top block into Wtop, Y, T, s; then the rows below).
+// column signs of Q (m' x k: the largest-|entry| of each positive); 2 the Householder
+// reconstruction's top block (k <= 256, a multiple of 4): L1 \ U into Wtop, Y's first k rows, the signs
+// s, and Us = U diag(s), with T = Us L1^{-T}.
 struct FinishMat {
     int mp, k;
-    float* Q; float* Wtop; float* Y; float* T; float* s;
+    float* Q; float* Wtop; float* Y; float* Us; float* s;
 };
 struct FinishGroup { int nmat; FinishMat mat[64]; };
 cudaError_t finish_group(const FinishGroup& g, int stage, cudaStream_t st);

@@ -722,24 +722,33 @@ int refresh_tcl_grouped(std::vector<glr_handle*>& hs) {
             for (size_t i = c0; i < hs.size() && i < c0 + 64; ++i) {
                 glr_handle* h = hs[i];
                 FinishMat& F = fg.mat[fg.nmat++];
-                F.mp = h->mp; F.k = h->k; F.Q = h->Q; F.Wtop = h->scratch; F.Y = h->Y; F.T = h->T; F.s = h->dsign;
+                F.mp = h->mp; F.k = h->k; F.Q = h->Q; F.Wtop = h->scratch; F.Y = h->Y; F.Us = h->gram; F.s = h->dsign;
             }
             PhaseScope ps(hs[c0], GLR_PH_REFRESH, s0);
             GLR_LAUNCH(hs[c0], 1, finish_group(fg, stage, s0));
         }
     }
-    // rows a >= k of Y: Y[a, :] Utilde = -Q[a, :] with Utilde the upper triangle the top-block
-    // LU left in scratch: Utilde^{-1} (as the inverse of its transpose), then one product
-    for (size_t c0 = 0; c0 < hs.size(); c0 += 64) {
+    // rows a >= k of Y: Y[a, :] U = -Q[a, :] with U the upper triangle the top-block LU left in scratch:
+    // U^{-1} (as the inverse of its transpose), then one product; T = Us L1^{-T} with L1^{-1} in Hk
+    for (size_t c0 = 0; c0 < hs.size(); c0 += 32) {
         CholGroup cg{};
-        for (size_t i = c0; i < hs.size() && i < c0 + 64; ++i) {
+        for (size_t i = c0; i < hs.size() && i < c0 + 32; ++i) {
             glr_handle* h = hs[i];
             CholMat& C = cg.mat[cg.nmat++];
-            C.part = h->scratch; C.nparts = 1; C.ld = h->k; C.n = h->k; C.out = h->Linv; C.tri_only = 1;
+            C.part = h->scratch; C.nparts = 1; C.ld = h->k; C.n = h->k; C.out = h->Linv; C.tri_only = kTriUpper;
+            CholMat& D = cg.mat[cg.nmat++];
+            D = C;
+            D.out = h->Hk; D.tri_only = kTriUnitLower;
         }
         PhaseScope ps(hs[c0], GLR_PH_REFRESH, s0);
         GLR_LAUNCH(hs[c0], 1, chol_group(cg, s0));
     }
+    if ((rc = fp32_products(hs, s0, [](glr_handle* h, GemmMat& G) {          // T = Us L1^{-T}
+             G.M = h->k; G.N = h->k; G.K = h->k;
+             G.A = h->gram; G.sAi = h->k; G.sAp = 1; G.B = h->Hk; G.sBp = 1; G.sBj = h->k;
+             G.C = h->T; G.sCi = h->k; G.sCj = 1;
+         })) != GLR_OK)
+        return rc;
     if ((rc = fp32_products(hs, s0, [](glr_handle* h, GemmMat& G) {          // Y[k:] = -Q[k:] Utilde^{-1}
              G.M = h->mp - h->k; G.N = h->k; G.K = h->k; G.alpha = -1.f;
              G.A = h->Q + (size_t)h->k * h->k; G.sAi = h->k; G.sAp = 1;

@@ -335,11 +335,6 @@ __global__ void __launch_bounds__(1024) hh_top_kernel(const float* Q, int k, flo
                                                       float* s) {
     hh_top_body(Q, k, W, Y, T, s);
 }
-__global__ void __launch_bounds__(1024) hh_top_group_kernel(const __grid_constant__ FinishGroup g) {
-    const FinishMat& M = g.mat[blockIdx.x];
-    hh_top_body(M.Q, M.k, M.Wtop, M.Y, M.T, M.s);
-}
-
 // Rows a >= k: Y[a, :] Utilde = -Q[a, :], one warp per row (forward substitution).
 __device__ __forceinline__ void hh_rows_body(const float* Q, int mp, int k, const float* W, float* Y, int warp) {
     const int lane = threadIdx.x & 31;
@@ -360,11 +355,6 @@ __device__ __forceinline__ void hh_rows_body(const float* Q, int mp, int k, cons
 __global__ void hh_rows_kernel(const float* Q, int mp, int k, const float* W, float* Y) {
     hh_rows_body(Q, mp, k, W, Y, blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
 }
-__global__ void hh_rows_group_kernel(const __grid_constant__ FinishGroup g) {
-    const FinishMat& M = g.mat[blockIdx.y];
-    hh_rows_body(M.Q, M.mp, M.k, M.Wtop, M.Y, blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
-}
-
 __global__ void wy_basis_kernel(int mp, int k, const float* Y, const float* Yt, const float* dsign, float* U) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)mp * mp) return;
@@ -405,24 +395,6 @@ cudaError_t sort_group(const SortGroup& g, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t finish_group(const FinishGroup& g, int stage, cudaStream_t st) {
-    if (g.nmat <= 0) return cudaSuccess;
-    int kmax = 0, rows_max = 0;
-    for (int i = 0; i < g.nmat; ++i) {
-        kmax = g.mat[i].k > kmax ? g.mat[i].k : kmax;
-        rows_max = g.mat[i].mp - g.mat[i].k > rows_max ? g.mat[i].mp - g.mat[i].k : rows_max;
-    }
-    if (stage == 1) {                                   // column signs of Q
-        fix_signs_group_kernel<<<dim3((kmax + 31) / 32, g.nmat), 1024, 0, st>>>(g);
-    } else if (stage == 2) {                            // Householder top block
-        hh_top_group_kernel<<<g.nmat, 1024, 0, st>>>(g);
-    } else {                                            // Householder rows below
-        if (rows_max <= 0) return cudaSuccess;
-        hh_rows_group_kernel<<<dim3((rows_max + 7) / 8, g.nmat), 256, 0, st>>>(g);
-    }
-    return cudaGetLastError();
-}
-
 namespace {
 // Packed lower triangle: element (i, l), l <= i, at i (i + 1) / 2 + l.
 __device__ __forceinline__ int tri(int i, int l) { return i * (i + 1) / 2 + l; }
@@ -436,11 +408,7 @@ __device__ __forceinline__ int tri(int i, int l) { return i * (i + 1) / 2 + l; }
 // copies the column it reads into a contiguous array (a column of the packed triangle is strided
 // by the row lengths, which would make the lanes' reads collide in the banks).  S (row-major
 // n x n) is the transpose of L^{-1}.
-// The Gram matrix is the sum of `nparts` partial matrices (leading dimension ld, spaced ld * ld
-// apart).  Output: S = L^{-T} (row-major n x n), or with out_linv L^{-1} (row-major ld x ld, zero
-// above the diagonal and outside n x n).
-__device__ __forceinline__ void chol_inverse_body(const float* G, int nparts, int ld, int n, float* S, int out_linv,
-                                                  int* flag) {
+__global__ void __launch_bounds__(1024) chol_inverse_kernel(const float* G, int n, float* S, int* flag) {
     extern __shared__ float L[];                       // n (n + 1) / 2 packed, then n + n temporaries
     float* col = L + n * (n + 1) / 2;
     float* tmp = col + n;
@@ -449,11 +417,7 @@ __device__ __forceinline__ void chol_inverse_body(const float* G, int nparts, in
     __shared__ float shift, trace;
     if (warp == 0) {                                   // trace: a warp sum in a fixed order
         float tr = 0.f;
-        for (int i = lane; i < n; i += 32) {
-            float gi = 0.f;
-            for (int p = 0; p < nparts; ++p) gi += G[(size_t)p * ld * ld + (size_t)i * ld + i];
-            tr += gi;
-        }
+        for (int i = lane; i < n; i += 32) tr += G[(size_t)i * n + i];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
         if (lane == 0) { trace = tr; shift = 0.f; }
@@ -462,11 +426,7 @@ __device__ __forceinline__ void chol_inverse_body(const float* G, int nparts, in
     int attempt = 0;
     for (; attempt < 6; ++attempt) {
         for (int i = warp; i < n; i += nw)
-            for (int l = lane; l <= i; l += 32) {
-                float gil = 0.f;
-                for (int p = 0; p < nparts; ++p) gil += G[(size_t)p * ld * ld + (size_t)i * ld + l];
-                L[tri(i, l)] = gil + (l == i ? shift : 0.f);
-            }
+            for (int l = lane; l <= i; l += 32) L[tri(i, l)] = G[(size_t)i * n + l] + (l == i ? shift : 0.f);
         if (tid == 0) fail = 0;
         __syncthreads();
         const float thresh = 1e-12f * fmaxf(trace / n, 1e-30f);
@@ -515,60 +475,354 @@ __device__ __forceinline__ void chol_inverse_body(const float* G, int nparts, in
         if (tid == 0) L[tri(j, j)] = ajj;
         __syncthreads();
     }
-    if (out_linv) {
-        for (int e = tid; e < ld * ld; e += blockDim.x) {
-            const int r = e / ld, c = e % ld;
-            S[e] = (c <= r && r < n) ? L[tri(r, c)] : 0.f;
-        }
-        return;
-    }
     for (int e = tid; e < n * n; e += blockDim.x) {
         const int r = e / n, c = e % n;
         S[e] = c >= r ? L[tri(c, r)] : 0.f;
     }
 }
 
-__global__ void __launch_bounds__(1024) chol_inverse_kernel(const float* G, int n, float* S, int* flag) {
-    chol_inverse_body(G, 1, n, n, S, 0, flag);
-}
-// L^{-1} of the lower-triangular L = U^T, U the upper triangle of the n x n matrix at A (leading
-// dimension lda): the inverse stage of chol_inverse_body alone.  Output row-major ld x ld.
-__device__ __forceinline__ void tri_inverse_body(const float* A, int lda, int n, float* out, int ld) {
-    extern __shared__ float L[];
-    float* col = L + n * (n + 1) / 2;
-    float* tmp = col + n;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-    for (int i = warp; i < n; i += nw)
-        for (int l = lane; l <= i; l += 32) L[tri(i, l)] = A[(size_t)l * lda + i];
-    __syncthreads();
-    for (int j = n - 1; j >= 0; --j) {
-        for (int l = j + 1 + tid; l < n; l += blockDim.x) col[l] = L[tri(l, j)];
-        __syncthreads();
-        for (int i = j + 1 + warp; i < n; i += nw) {
-            float t = 0.f;
-            for (int l = j + 1 + lane; l <= i; l += 32) t += L[tri(i, l)] * col[l];
+// ---- blocked factor and inverse of the grouped refreshes, n <= 256 --------------------------------
+// One CTA of 16 warps a matrix, the lower triangle as 32 x 32 blocks in shared memory (block (i, j) at
+// i (i + 1) / 2 + j, pitch 36: rows 16-byte aligned, the products' reads free of bank conflicts),
+// padded to whole blocks with the identity.  A panel: one warp factors the diagonal block with a row
+// a lane, a warp per block below solves against it by substitution, then the trailing blocks are
+// 32 x 32 x 32 products, a warp each.  The inverse goes block column by block column from the last,
+// in place: T_i = sum_{j < k <= i} X_ik L_kj, X_ij = -T_i X_jj.  Bound by the diagonal blocks' chain of
+// square roots, quotients and shuffles and by shared-memory reads; factoring and inverting column by
+// column, four barriers each, took 0.80 ms for n = 256 and 0.22 ms for n = 128.
+constexpr int CB = 32, CP = 36, CBLK = CB * CP, CWARPS = 16;
+constexpr int kCholMaxBlocks = 8;
+constexpr size_t kCholSmem = sizeof(float) * CBLK * (kCholMaxBlocks * (kCholMaxBlocks + 1) / 2 + kCholMaxBlocks - 1);
+
+__device__ __forceinline__ float* cblk(float* L, int i, int j) { return L + (size_t)(i * (i + 1) / 2 + j) * CBLK; }
+
+// acc += A B or A B^T over a 32 x 32 block: rows r0 + lane / 4 + 8 i, columns as cmm_col.
+template <int ROWS, bool TB>
+__device__ __forceinline__ void cmm(const float* A, const float* B, int r0, int lane, float (&acc)[ROWS][8]) {
+    const float* a = A + (r0 + (lane >> 2)) * CP;
+    const float* b = TB ? B + (lane & 3) * CP : B + 8 * (lane & 3);
+#pragma unroll 4
+    for (int k = 0; k < CB; ++k) {
+        float av[ROWS], bv[8];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (lane == 0) tmp[i] = t;
+        for (int i = 0; i < ROWS; ++i) av[i] = a[8 * i * CP + k];
+        if (TB) {
+#pragma unroll
+            for (int c = 0; c < 8; ++c) bv[c] = b[4 * c * CP + k];
+        } else {
+            const float4 x = *reinterpret_cast<const float4*>(b + k * CP), y = *reinterpret_cast<const float4*>(b + k * CP + 4);
+            bv[0] = x.x; bv[1] = x.y; bv[2] = x.z; bv[3] = x.w; bv[4] = y.x; bv[5] = y.y; bv[6] = y.z; bv[7] = y.w;
         }
-        __syncthreads();
-        const float ajj = 1.0f / L[tri(j, j)];
-        for (int i = j + 1 + tid; i < n; i += blockDim.x) L[tri(i, j)] = -tmp[i] * ajj;
-        if (tid == 0) L[tri(j, j)] = ajj;
-        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) acc[i][c] = fmaf(av[i], bv[c], acc[i][c]);
     }
-    for (int e = tid; e < ld * ld; e += blockDim.x) {
-        const int r = e / ld, c = e % ld;
-        out[e] = (c <= r && r < n) ? L[tri(r, c)] : 0.f;
+}
+template <bool TB> __device__ __forceinline__ int cmm_col(int lane, int c) { return TB ? (lane & 3) + 4 * c : 8 * (lane & 3) + c; }
+
+// A diagonal block's Cholesky factor in place (upper part zeroed), one warp, lane = row; false when a
+// pivot is not above thresh.
+__device__ __forceinline__ bool chol_diag(float* D, float thresh, int lane) {
+    float a[CB];
+#pragma unroll
+    for (int c = 0; c < CB; c += 4) {
+        const float4 x = *reinterpret_cast<const float4*>(D + lane * CP + c);
+        a[c] = x.x; a[c + 1] = x.y; a[c + 2] = x.z; a[c + 3] = x.w;
     }
+    bool ok = true;
+#pragma unroll
+    for (int c = 0; c < CB; ++c) {
+        const float d = __shfl_sync(0xffffffffu, a[c], c);
+        ok = ok && d > thresh;
+        const float l = sqrtf(d);
+        a[c] = lane == c ? l : lane > c ? a[c] / l : 0.f;
+#pragma unroll
+        for (int q = c + 1; q < CB; ++q) a[q] = fmaf(-a[c], __shfl_sync(0xffffffffu, a[c], q), a[q]);
+    }
+#pragma unroll
+    for (int c = 0; c < CB; c += 4) *reinterpret_cast<float4*>(D + lane * CP + c) = make_float4(a[c], a[c + 1], a[c + 2], a[c + 3]);
+    return ok;
 }
 
-__global__ void __launch_bounds__(1024) chol_group_kernel(const __grid_constant__ CholGroup g) {
+// A panel block's rows against the factor D: y_c = (a_c - sum_{k < c} y_k D_ck) / D_cc, lane = row.
+__device__ __forceinline__ void chol_panel(float* A, const float* D, int lane) {
+    float y[CB];
+#pragma unroll
+    for (int c = 0; c < CB; c += 4) {
+        const float4 x = *reinterpret_cast<const float4*>(A + lane * CP + c);
+        y[c] = x.x; y[c + 1] = x.y; y[c + 2] = x.z; y[c + 3] = x.w;
+    }
+#pragma unroll
+    for (int c = 0; c < CB; ++c) {
+        float s0 = y[c], s1 = 0.f;
+#pragma unroll
+        for (int k = 0; k < c; ++k) {
+            if (k & 1) s1 = fmaf(-y[k], D[c * CP + k], s1);
+            else s0 = fmaf(-y[k], D[c * CP + k], s0);
+        }
+        y[c] = (s0 + s1) / D[c * CP + c];
+    }
+#pragma unroll
+    for (int c = 0; c < CB; c += 4) *reinterpret_cast<float4*>(A + lane * CP + c) = make_float4(y[c], y[c + 1], y[c + 2], y[c + 3]);
+}
+
+// A lower-triangular block's inverse in place, one warp, lane = column of the inverse.
+__device__ __forceinline__ void tri_diag(float* D, int lane) {
+    float x[CB];
+#pragma unroll
+    for (int i = 0; i < CB; ++i) {
+        float s0 = lane == i ? 1.f : 0.f, s1 = 0.f;
+#pragma unroll
+        for (int k = 0; k < i; ++k) {
+            if (k & 1) s1 = fmaf(-D[i * CP + k], x[k], s1);
+            else s0 = fmaf(-D[i * CP + k], x[k], s0);
+        }
+        x[i] = (s0 + s1) / D[i * CP + i];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < CB; ++i) D[i * CP + lane] = x[i];
+}
+
+__global__ void __launch_bounds__(CWARPS * 32) chol_group_kernel(const __grid_constant__ CholGroup g) {
+    extern __shared__ __align__(16) float csm[];
     const CholMat& M = g.mat[blockIdx.x];
-    if (M.tri_only) tri_inverse_body(M.part, M.n, M.n, M.out, M.ld);
-    else chol_inverse_body(M.part, M.nparts, M.ld, M.n, M.out, 1, M.flag);
+    const int n = M.n, nb = (n + CB - 1) / CB, t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    float* L = csm;
+    float* T = L + (size_t)(nb * (nb + 1) / 2) * CBLK;
+    __shared__ int fail;
+    __shared__ float shift, trace;
+    auto entry = [&](int i, int l) {
+        if (M.tri_only == kTriUpper) return M.part[(size_t)l * M.n + i];           // L = U^T
+        if (M.tri_only == kTriUnitLower) return i == l ? 1.f : M.part[(size_t)i * M.n + l];
+        float v = 0.f;
+        for (int p = 0; p < M.nparts; ++p) v += M.part[(size_t)p * M.ld * M.ld + (size_t)i * M.ld + l];
+        return v;
+    };
+    if (warp == 0) {                                   // trace: a warp sum in a fixed order
+        float tr = 0.f;
+        if (!M.tri_only)
+            for (int i = lane; i < n; i += 32) tr += entry(i, i);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
+        if (lane == 0) { trace = tr; shift = 0.f; }
+    }
+    int attempt = 0;
+    for (; attempt < 6; ++attempt) {
+        __syncthreads();
+        for (int q = warp; q < nb * (nb + 1) / 2 * CB; q += CWARPS) {    // a block row a warp
+            int i = 0, j = q / CB;                                       // j = i (i + 1) / 2 + block column
+            while (j > i) { j -= i + 1; ++i; }
+            const int r = i * CB + q % CB, c = j * CB + lane;
+            float v = r == c ? 1.f : 0.f;
+            if (r < n && c < n) {
+                v = c <= r ? entry(r, c) : 0.f;
+                if (r == c && !M.tri_only) v += shift;
+            }
+            cblk(L, i, j)[(q % CB) * CP + lane] = v;
+        }
+        if (t == 0) fail = 0;
+        __syncthreads();
+        if (M.tri_only) break;
+        const float thresh = 1e-12f * fmaxf(trace / n, 1e-30f);
+        for (int p = 0; p < nb; ++p) {
+            if (warp == 0 && !chol_diag(cblk(L, p, p), thresh, lane) && lane == 0) fail = 1;
+            __syncthreads();
+            if (fail) break;                           // uniform: read after the barrier, written before it
+            for (int i = p + 1 + warp; i < nb; i += CWARPS) chol_panel(cblk(L, i, p), cblk(L, p, p), lane);
+            __syncthreads();
+            const int m = nb - p - 1;
+            for (int q = warp; q < m * (m + 1) / 2; q += CWARPS) {       // A_ij -= L_ip L_jp^T
+                int i = 0, j = q;
+                while (j > i) { j -= i + 1; ++i; }
+                i += p + 1; j += p + 1;
+                float acc[4][8] = {};
+                cmm<4, true>(cblk(L, i, p), cblk(L, j, p), 0, lane, acc);
+                float* C = cblk(L, i, j);
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) C[((lane >> 2) + 8 * r) * CP + cmm_col<true>(lane, c)] -= acc[r][c];
+            }
+            __syncthreads();
+        }
+        if (!fail) break;
+        __syncthreads();
+        if (t == 0) shift = (attempt == 0 ? 1e-7f : shift * 100.f) * fmaxf(trace / n, 1e-30f);
+    }
+    __syncthreads();
+    if (t == 0 && !M.tri_only && M.flag) {
+        *M.flag = attempt;
+        // no factorisation after every shift, or a Gram matrix with no positive trace (a zero or
+        // non-finite block): the refresh cannot orthonormalise it (flag + 6 counts these)
+        if (attempt == 6 || !(trace > 0.f) || !isfinite(trace)) atomicAdd(M.flag + 6, 1);
+    }
+    for (int j = warp; j < nb; j += CWARPS) tri_diag(cblk(L, j, j), lane);
+    __syncthreads();
+    for (int j = nb - 2; j >= 0; --j) {
+        const int m = nb - 1 - j;                      // half a block (16 rows) a task
+        for (int q = warp; q < 2 * m; q += CWARPS) {
+            const int i = nb - 1 - (q >> 1), r0 = 16 * (q & 1);          // the longest sums first
+            float acc[2][8] = {};
+            for (int k = j + 1; k <= i; ++k) cmm<2, false>(cblk(L, i, k), cblk(L, k, j), r0, lane, acc);
+            float* C = T + (size_t)(i - j - 1) * CBLK;
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+#pragma unroll
+                for (int c = 0; c < 8; ++c) C[(r0 + (lane >> 2) + 8 * r) * CP + cmm_col<false>(lane, c)] = -acc[r][c];
+        }
+        __syncthreads();
+        for (int q = warp; q < 2 * m; q += CWARPS) {
+            const int i = j + 1 + (q >> 1), r0 = 16 * (q & 1);
+            float acc[2][8] = {};
+            cmm<2, false>(T + (size_t)(i - j - 1) * CBLK, cblk(L, j, j), r0, lane, acc);
+            float* C = cblk(L, i, j);
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+#pragma unroll
+                for (int c = 0; c < 8; ++c) C[(r0 + (lane >> 2) + 8 * r) * CP + cmm_col<false>(lane, c)] = acc[r][c];
+        }
+        __syncthreads();
+    }
+    for (int e = t; e < M.ld * M.ld; e += CWARPS * 32) {
+        const int r = e / M.ld, c = e % M.ld;
+        M.out[e] = (c <= r && r < n) ? cblk(L, r / CB, c / CB)[(r % CB) * CP + c % CB] : 0.f;
+    }
+}
+// Householder reconstruction, top blocks of the grouped refreshes: the modified LU of hh_top_kernel
+// (pivots W_jj + s_j, s_j = -sign of the current Schur complement of Q) in 32-column panels: the
+// panel's column and row blocks in shared memory, the diagonal block by one warp with a row a lane,
+// the others by substitution, a warp each, the trailing blocks as 32 x 32 x 32 products on the matrix
+// in L2.  W ends holding L1 \ U, Y's top the unit lower L1, and Us = U diag(s) (zero below), from
+// which T = Us L1^{-T}.  Column by column, with T by a thread per row: 2.1 ms for k = 256.
+constexpr size_t kHhSmem = sizeof(float) * CBLK * (2 * kCholMaxBlocks - 1);
+
+__global__ void __launch_bounds__(CWARPS * 32) hh_lu_group_kernel(const __grid_constant__ FinishGroup g) {
+    extern __shared__ __align__(16) float hsm[];
+    const FinishMat& M = g.mat[blockIdx.x];
+    const int k = M.k, nb = (k + CB - 1) / CB, t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    float* const W = M.Wtop;
+    for (int e = t; e < k * k; e += CWARPS * 32) W[e] = -M.Q[e];         // rows 0..k-1 of Q (ld = k)
+    __syncthreads();
+    for (int p = 0; p < nb; ++p) {
+        const int m = nb - p;                          // column blocks p .., then row blocks p + 1 ..
+        for (int q = warp; q < (2 * m - 1) * CB; q += CWARPS) {
+            const int blk = q / CB, r = (blk < m ? p + blk : p) * CB + q % CB, c = (blk < m ? p : p + 1 + blk - m) * CB + lane;
+            hsm[(size_t)blk * CBLK + (q % CB) * CP + lane] = r < k && c < k ? W[(size_t)r * k + c] : r == c ? 1.f : 0.f;
+        }
+        __syncthreads();
+        float* D = hsm;
+        if (warp == 0) {
+            float a[CB];
+#pragma unroll
+            for (int c = 0; c < CB; c += 4) {
+                const float4 x = *reinterpret_cast<const float4*>(D + lane * CP + c);
+                a[c] = x.x; a[c + 1] = x.y; a[c + 2] = x.z; a[c + 3] = x.w;
+            }
+#pragma unroll
+            for (int c = 0; c < CB; ++c) {
+                const float d = __shfl_sync(0xffffffffu, a[c], c), sj = d <= 0.f ? -1.f : 1.f, piv = d + sj;
+                if (lane == c && p * CB + c < k) M.s[p * CB + c] = sj;
+                a[c] = lane == c ? piv : lane > c ? a[c] / piv : a[c];
+#pragma unroll
+                for (int q = c + 1; q < CB; ++q) {
+                    const float u = __shfl_sync(0xffffffffu, a[q], c);
+                    if (lane > c) a[q] = fmaf(-a[c], u, a[q]);
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < CB; c += 4)
+                *reinterpret_cast<float4*>(D + lane * CP + c) = make_float4(a[c], a[c + 1], a[c + 2], a[c + 3]);
+        }
+        __syncthreads();
+        for (int blk = 1 + warp; blk < 2 * m - 1; blk += CWARPS) {
+            float* A = hsm + (size_t)blk * CBLK;
+            float y[CB];
+            if (blk < m) {                             // L = A U^{-1}, lane = row
+#pragma unroll
+                for (int c = 0; c < CB; ++c) y[c] = A[lane * CP + c];
+#pragma unroll
+                for (int c = 0; c < CB; ++c) {
+                    float s0 = y[c], s1 = 0.f;
+#pragma unroll
+                    for (int q = 0; q < c; ++q) {
+                        if (q & 1) s1 = fmaf(-y[q], D[q * CP + c], s1);
+                        else s0 = fmaf(-y[q], D[q * CP + c], s0);
+                    }
+                    y[c] = (s0 + s1) / D[c * CP + c];
+                }
+                __syncwarp();
+#pragma unroll
+                for (int c = 0; c < CB; ++c) A[lane * CP + c] = y[c];
+            } else {                                   // U = L1^{-1} A, lane = column
+#pragma unroll
+                for (int c = 0; c < CB; ++c) y[c] = A[c * CP + lane];
+#pragma unroll
+                for (int c = 0; c < CB; ++c) {
+                    float s0 = y[c], s1 = 0.f;
+#pragma unroll
+                    for (int q = 0; q < c; ++q) {
+                        if (q & 1) s1 = fmaf(-D[c * CP + q], y[q], s1);
+                        else s0 = fmaf(-D[c * CP + q], y[q], s0);
+                    }
+                    y[c] = s0 + s1;
+                }
+                __syncwarp();
+#pragma unroll
+                for (int c = 0; c < CB; ++c) A[c * CP + lane] = y[c];
+            }
+        }
+        __syncthreads();
+        for (int q = warp; q < (2 * m - 1) * CB; q += CWARPS) {
+            const int blk = q / CB, r = (blk < m ? p + blk : p) * CB + q % CB, c = (blk < m ? p : p + 1 + blk - m) * CB + lane;
+            if (r < k && c < k) W[(size_t)r * k + c] = hsm[(size_t)blk * CBLK + (q % CB) * CP + lane];
+        }
+        for (int q = warp; q < (m - 1) * (m - 1); q += CWARPS) {
+            const int i = q / (m - 1), j = q % (m - 1);
+            float acc[4][8] = {};
+            cmm<4, false>(hsm + (size_t)(1 + i) * CBLK, hsm + (size_t)(m + j) * CBLK, 0, lane, acc);
+            const int c0 = (p + 1 + j) * CB + 8 * (lane & 3);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int row = (p + 1 + i) * CB + (lane >> 2) + 8 * r;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {          // k is a multiple of 4
+                    if (row >= k || c0 + 4 * h >= k) continue;
+                    float4* C = reinterpret_cast<float4*>(W + (size_t)row * k + c0 + 4 * h);
+                    float4 x = *C;
+                    x.x -= acc[r][4 * h]; x.y -= acc[r][4 * h + 1]; x.z -= acc[r][4 * h + 2]; x.w -= acc[r][4 * h + 3];
+                    *C = x;
+                }
+            }
+        }
+        __syncthreads();
+    }
+    for (int e = t; e < k * k; e += CWARPS * 32) {
+        const int i = e / k, l = e % k;
+        const float w = W[e];
+        M.Y[e] = i > l ? w : i == l ? 1.f : 0.f;
+        M.Us[e] = i <= l ? w * M.s[l] : 0.f;
+    }
 }
 }  // namespace
+
+cudaError_t finish_group(const FinishGroup& g, int stage, cudaStream_t st) {
+    if (g.nmat <= 0) return cudaSuccess;
+    int kmax = 0;
+    for (int i = 0; i < g.nmat; ++i) {
+        kmax = g.mat[i].k > kmax ? g.mat[i].k : kmax;
+        if (stage == 2 && (g.mat[i].k > CB * kCholMaxBlocks || g.mat[i].k % 4)) return cudaErrorInvalidValue;
+    }
+    if (stage == 1) {                                   // column signs of Q
+        fix_signs_group_kernel<<<dim3((kmax + 31) / 32, g.nmat), 1024, 0, st>>>(g);
+    } else {                                            // Householder top block
+        const cudaError_t ea = cudaFuncSetAttribute(hh_lu_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHhSmem);
+        if (ea != cudaSuccess) return ea;
+        hh_lu_group_kernel<<<g.nmat, CWARPS * 32, kHhSmem, st>>>(g);
+    }
+    return cudaGetLastError();
+}
 
 cudaError_t chol_group(const CholGroup& g, cudaStream_t st) {
     if (g.nmat <= 0) return cudaSuccess;
@@ -577,13 +831,14 @@ cudaError_t chol_group(const CholGroup& g, cudaStream_t st) {
         if (g.mat[i].n < 1 || g.mat[i].n > 256 || g.mat[i].ld < g.mat[i].n) return cudaErrorInvalidValue;
         nmax = g.mat[i].n > nmax ? g.mat[i].n : nmax;
     }
-    const size_t smem = sizeof(float) * ((size_t)nmax * (nmax + 1) / 2 + 2 * nmax);
+    const int nb = (nmax + CB - 1) / CB;
+    const size_t smem = sizeof(float) * CBLK * (nb * (nb + 1) / 2 + nb - 1);
     {   // per device: set on every call (cheap next to the launch)
         const cudaError_t ea = cudaFuncSetAttribute(chol_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)(sizeof(float) * (256 * 257 / 2 + 2 * 256)));
+                                                   (int)kCholSmem);
         if (ea != cudaSuccess) return ea;
     }
-    chol_group_kernel<<<g.nmat, 1024, smem, st>>>(g);
+    chol_group_kernel<<<g.nmat, CWARPS * 32, smem, st>>>(g);
     return cudaGetLastError();
 }
 
