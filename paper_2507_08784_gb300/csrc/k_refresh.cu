@@ -132,6 +132,7 @@ __device__ __forceinline__ void column_stats(const float* A, int rows, int64_t l
     float best = -1.f, val = 0.f, sum = 0.f;
     int idx = 0x7fffffff;
     if (in)
+#pragma unroll 8
         for (int a = ty; a < rows; a += 32) {
             const float v = A[a * ld + col], m = fabsf(v);
             sum = fmaf(v, v, sum);
@@ -492,7 +493,8 @@ __global__ void __launch_bounds__(1024) chol_inverse_kernel(const float* G, int 
 // column, four barriers each, took 0.80 ms for n = 256 and 0.22 ms for n = 128.
 constexpr int CB = 32, CP = 36, CBLK = CB * CP, CWARPS = 16;
 constexpr int kCholMaxBlocks = 8;
-constexpr size_t kCholSmem = sizeof(float) * CBLK * (kCholMaxBlocks * (kCholMaxBlocks + 1) / 2 + kCholMaxBlocks - 1);
+// a block more than the triangle and T: the eliminations' dead reads
+constexpr size_t kCholSmem = sizeof(float) * CBLK * (kCholMaxBlocks * (kCholMaxBlocks + 1) / 2 + kCholMaxBlocks);
 
 __device__ __forceinline__ float* cblk(float* L, int i, int j) { return L + (size_t)(i * (i + 1) / 2 + j) * CBLK; }
 
@@ -521,68 +523,52 @@ __device__ __forceinline__ void cmm(const float* A, const float* B, int r0, int 
 }
 template <bool TB> __device__ __forceinline__ int cmm_col(int lane, int c) { return TB ? (lane & 3) + 4 * c : 8 * (lane & 3) + c; }
 
+// The 32-step eliminations below keep a lane's 32 values in registers and shift them down by one a step, so
+// that the step's code is the same every time: unrolled over the steps they are ten thousand
+// instructions run once, and the instruction fetches took ten times the arithmetic (k = 256 top
+// block 1.93 ms).  Reads past the block (dead values) stay inside the padded shared memory.
+
+__device__ __forceinline__ void load_row(float (&a)[CB], const float* row) {
+#pragma unroll
+    for (int c = 0; c < CB; c += 4) {
+        const float4 x = *reinterpret_cast<const float4*>(row + c);
+        a[c] = x.x; a[c + 1] = x.y; a[c + 2] = x.z; a[c + 3] = x.w;
+    }
+}
+
+// Substitution against the triangular block D: x_c = a_c (/ D_cc), a_q -= x_c D(c, q) for q > c, the
+// coefficients dq apart from the diagonal on; x_c to out[c * os].  One warp, a system a lane.
+template <bool DIV>
+__device__ __forceinline__ void eliminate(float (&a)[CB], const float* D, int dq, float* out, int os) {
+#pragma unroll 1
+    for (int c = 0; c < CB; ++c) {
+        const float* d = D + c * (CP + 1);
+        const float x = DIV ? a[0] / d[0] : a[0];
+#pragma unroll
+        for (int q = 1; q < CB; ++q) a[q - 1] = fmaf(-x, d[q * dq], a[q]);
+        a[CB - 1] = 0.f;
+        __syncwarp();                                  // out may be D's row c, read by now
+        out[c * os] = x;
+    }
+}
+
 // A diagonal block's Cholesky factor in place (upper part zeroed), one warp, lane = row; false when a
 // pivot is not above thresh.
 __device__ __forceinline__ bool chol_diag(float* D, float thresh, int lane) {
     float a[CB];
-#pragma unroll
-    for (int c = 0; c < CB; c += 4) {
-        const float4 x = *reinterpret_cast<const float4*>(D + lane * CP + c);
-        a[c] = x.x; a[c + 1] = x.y; a[c + 2] = x.z; a[c + 3] = x.w;
-    }
+    load_row(a, D + lane * CP);
     bool ok = true;
-#pragma unroll
+#pragma unroll 1
     for (int c = 0; c < CB; ++c) {
-        const float d = __shfl_sync(0xffffffffu, a[c], c);
+        const float d = __shfl_sync(0xffffffffu, a[0], c);
         ok = ok && d > thresh;
-        const float l = sqrtf(d);
-        a[c] = lane == c ? l : lane > c ? a[c] / l : 0.f;
+        const float l = sqrtf(d), v = lane == c ? l : lane > c ? a[0] / l : 0.f;
 #pragma unroll
-        for (int q = c + 1; q < CB; ++q) a[q] = fmaf(-a[c], __shfl_sync(0xffffffffu, a[c], q), a[q]);
+        for (int q = 1; q < CB; ++q) a[q - 1] = fmaf(-v, __shfl_sync(0xffffffffu, v, (c + q) & 31), a[q]);
+        a[CB - 1] = 0.f;
+        D[lane * CP + c] = v;
     }
-#pragma unroll
-    for (int c = 0; c < CB; c += 4) *reinterpret_cast<float4*>(D + lane * CP + c) = make_float4(a[c], a[c + 1], a[c + 2], a[c + 3]);
     return ok;
-}
-
-// A panel block's rows against the factor D: y_c = (a_c - sum_{k < c} y_k D_ck) / D_cc, lane = row.
-__device__ __forceinline__ void chol_panel(float* A, const float* D, int lane) {
-    float y[CB];
-#pragma unroll
-    for (int c = 0; c < CB; c += 4) {
-        const float4 x = *reinterpret_cast<const float4*>(A + lane * CP + c);
-        y[c] = x.x; y[c + 1] = x.y; y[c + 2] = x.z; y[c + 3] = x.w;
-    }
-#pragma unroll
-    for (int c = 0; c < CB; ++c) {
-        float s0 = y[c], s1 = 0.f;
-#pragma unroll
-        for (int k = 0; k < c; ++k) {
-            if (k & 1) s1 = fmaf(-y[k], D[c * CP + k], s1);
-            else s0 = fmaf(-y[k], D[c * CP + k], s0);
-        }
-        y[c] = (s0 + s1) / D[c * CP + c];
-    }
-#pragma unroll
-    for (int c = 0; c < CB; c += 4) *reinterpret_cast<float4*>(A + lane * CP + c) = make_float4(y[c], y[c + 1], y[c + 2], y[c + 3]);
-}
-
-// A lower-triangular block's inverse in place, one warp, lane = column of the inverse.
-__device__ __forceinline__ void tri_diag(float* D, int lane) {
-    float x[CB];
-#pragma unroll
-    for (int i = 0; i < CB; ++i) {
-        float s0 = lane == i ? 1.f : 0.f, s1 = 0.f;
-#pragma unroll
-        for (int k = 0; k < i; ++k) {
-            if (k & 1) s1 = fmaf(-D[i * CP + k], x[k], s1);
-            else s0 = fmaf(-D[i * CP + k], x[k], s0);
-        }
-        x[i] = (s0 + s1) / D[i * CP + i];
-    }
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < CB; ++i) D[i * CP + lane] = x[i];
 }
 
 __global__ void __launch_bounds__(CWARPS * 32) chol_group_kernel(const __grid_constant__ CholGroup g) {
@@ -630,7 +616,12 @@ __global__ void __launch_bounds__(CWARPS * 32) chol_group_kernel(const __grid_co
             if (warp == 0 && !chol_diag(cblk(L, p, p), thresh, lane) && lane == 0) fail = 1;
             __syncthreads();
             if (fail) break;                           // uniform: read after the barrier, written before it
-            for (int i = p + 1 + warp; i < nb; i += CWARPS) chol_panel(cblk(L, i, p), cblk(L, p, p), lane);
+            for (int i = p + 1 + warp; i < nb; i += CWARPS) {            // L_ip = A_ip L_pp^{-T}, lane = row
+                float a[CB];
+                float* A = cblk(L, i, p) + lane * CP;
+                load_row(a, A);
+                eliminate<true>(a, cblk(L, p, p), CP, A, 1);
+            }
             __syncthreads();
             const int m = nb - p - 1;
             for (int q = warp; q < m * (m + 1) / 2; q += CWARPS) {       // A_ij -= L_ip L_jp^T
@@ -658,7 +649,12 @@ __global__ void __launch_bounds__(CWARPS * 32) chol_group_kernel(const __grid_co
         // non-finite block): the refresh cannot orthonormalise it (flag + 6 counts these)
         if (attempt == 6 || !(trace > 0.f) || !isfinite(trace)) atomicAdd(M.flag + 6, 1);
     }
-    for (int j = warp; j < nb; j += CWARPS) tri_diag(cblk(L, j, j), lane);
+    for (int j = warp; j < nb; j += CWARPS) {          // X_jj in place, lane = column
+        float a[CB];
+#pragma unroll
+        for (int i = 0; i < CB; ++i) a[i] = lane == i ? 1.f : 0.f;
+        eliminate<true>(a, cblk(L, j, j), CP, cblk(L, j, j) + lane, CP);
+    }
     __syncthreads();
     for (int j = nb - 2; j >= 0; --j) {
         const int m = nb - 1 - j;                      // half a block (16 rows) a task
@@ -696,7 +692,7 @@ __global__ void __launch_bounds__(CWARPS * 32) chol_group_kernel(const __grid_co
 // the others by substitution, a warp each, the trailing blocks as 32 x 32 x 32 products on the matrix
 // in L2.  W ends holding L1 \ U, Y's top the unit lower L1, and Us = U diag(s) (zero below), from
 // which T = Us L1^{-T}.  Column by column, with T by a thread per row: 2.1 ms for k = 256.
-constexpr size_t kHhSmem = sizeof(float) * CBLK * (2 * kCholMaxBlocks - 1);
+constexpr size_t kHhSmem = sizeof(float) * CBLK * (2 * kCholMaxBlocks);
 
 __global__ void __launch_bounds__(CWARPS * 32) hh_lu_group_kernel(const __grid_constant__ FinishGroup g) {
     extern __shared__ __align__(16) float hsm[];
@@ -715,62 +711,29 @@ __global__ void __launch_bounds__(CWARPS * 32) hh_lu_group_kernel(const __grid_c
         float* D = hsm;
         if (warp == 0) {
             float a[CB];
-#pragma unroll
-            for (int c = 0; c < CB; c += 4) {
-                const float4 x = *reinterpret_cast<const float4*>(D + lane * CP + c);
-                a[c] = x.x; a[c + 1] = x.y; a[c + 2] = x.z; a[c + 3] = x.w;
-            }
-#pragma unroll
+            load_row(a, D + lane * CP);
+#pragma unroll 1
             for (int c = 0; c < CB; ++c) {
-                const float d = __shfl_sync(0xffffffffu, a[c], c), sj = d <= 0.f ? -1.f : 1.f, piv = d + sj;
+                const float d = __shfl_sync(0xffffffffu, a[0], c), sj = d <= 0.f ? -1.f : 1.f, piv = d + sj;
                 if (lane == c && p * CB + c < k) M.s[p * CB + c] = sj;
-                a[c] = lane == c ? piv : lane > c ? a[c] / piv : a[c];
+                const float v = lane > c ? a[0] / piv : 0.f;
+                D[lane * CP + c] = lane > c ? v : lane == c ? piv : a[0];
 #pragma unroll
-                for (int q = c + 1; q < CB; ++q) {
-                    const float u = __shfl_sync(0xffffffffu, a[q], c);
-                    if (lane > c) a[q] = fmaf(-a[c], u, a[q]);
-                }
+                for (int q = 1; q < CB; ++q) a[q - 1] = fmaf(-v, __shfl_sync(0xffffffffu, a[q], c), a[q]);
+                a[CB - 1] = 0.f;
             }
-#pragma unroll
-            for (int c = 0; c < CB; c += 4)
-                *reinterpret_cast<float4*>(D + lane * CP + c) = make_float4(a[c], a[c + 1], a[c + 2], a[c + 3]);
         }
         __syncthreads();
         for (int blk = 1 + warp; blk < 2 * m - 1; blk += CWARPS) {
             float* A = hsm + (size_t)blk * CBLK;
-            float y[CB];
+            float a[CB];
             if (blk < m) {                             // L = A U^{-1}, lane = row
-#pragma unroll
-                for (int c = 0; c < CB; ++c) y[c] = A[lane * CP + c];
-#pragma unroll
-                for (int c = 0; c < CB; ++c) {
-                    float s0 = y[c], s1 = 0.f;
-#pragma unroll
-                    for (int q = 0; q < c; ++q) {
-                        if (q & 1) s1 = fmaf(-y[q], D[q * CP + c], s1);
-                        else s0 = fmaf(-y[q], D[q * CP + c], s0);
-                    }
-                    y[c] = (s0 + s1) / D[c * CP + c];
-                }
-                __syncwarp();
-#pragma unroll
-                for (int c = 0; c < CB; ++c) A[lane * CP + c] = y[c];
+                load_row(a, A + lane * CP);
+                eliminate<true>(a, D, 1, A + lane * CP, 1);
             } else {                                   // U = L1^{-1} A, lane = column
 #pragma unroll
-                for (int c = 0; c < CB; ++c) y[c] = A[c * CP + lane];
-#pragma unroll
-                for (int c = 0; c < CB; ++c) {
-                    float s0 = y[c], s1 = 0.f;
-#pragma unroll
-                    for (int q = 0; q < c; ++q) {
-                        if (q & 1) s1 = fmaf(-D[c * CP + q], y[q], s1);
-                        else s0 = fmaf(-D[c * CP + q], y[q], s0);
-                    }
-                    y[c] = s0 + s1;
-                }
-                __syncwarp();
-#pragma unroll
-                for (int c = 0; c < CB; ++c) A[c * CP + lane] = y[c];
+                for (int c = 0; c < CB; ++c) a[c] = A[c * CP + lane];
+                eliminate<false>(a, D, CP, A + lane, CP);
             }
         }
         __syncthreads();
@@ -832,7 +795,7 @@ cudaError_t chol_group(const CholGroup& g, cudaStream_t st) {
         nmax = g.mat[i].n > nmax ? g.mat[i].n : nmax;
     }
     const int nb = (nmax + CB - 1) / CB;
-    const size_t smem = sizeof(float) * CBLK * (nb * (nb + 1) / 2 + nb - 1);
+    const size_t smem = sizeof(float) * CBLK * (nb * (nb + 1) / 2 + nb);
     {   // per device: set on every call (cheap next to the launch)
         const cudaError_t ea = cudaFuncSetAttribute(chol_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)kCholSmem);
