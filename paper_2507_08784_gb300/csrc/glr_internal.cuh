@@ -268,7 +268,8 @@ struct GemmMat {
     const float* A; int64_t sAi, sAp;
     const float* B; int64_t sBp, sBj;
     float* C; int64_t sCi, sCj;
-    int tile0;
+    float* ws;                            // kGemmWsFloats of scratch for K slices (null: none)
+    int tile0, splits;                    // set by gemm_group_f32
 };
 struct GemmGroup { int nmat, total_tiles; GemmMat mat[64]; };
 cudaError_t gemm_group_f32(GemmGroup& g, cudaStream_t st);

@@ -284,7 +284,10 @@ template <class Fill>
 int fp32_products(std::vector<glr_handle*>& hs, cudaStream_t st, Fill fill) {
     for (size_t c0 = 0; c0 < hs.size(); c0 += 64) {
         GemmGroup gg{};
-        for (size_t i = c0; i < hs.size() && i < c0 + 64; ++i) fill(hs[i], gg.mat[gg.nmat++]);
+        for (size_t i = c0; i < hs.size() && i < c0 + 64; ++i) {
+            gg.mat[gg.nmat].ws = hs[i]->gemm_ws;
+            fill(hs[i], gg.mat[gg.nmat++]);
+        }
         PhaseScope ps(hs[c0], GLR_PH_REFRESH, st);
         GLR_LAUNCH(hs[c0], 1, gemm_group_f32(gg, st));
     }

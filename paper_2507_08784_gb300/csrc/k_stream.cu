@@ -13,47 +13,78 @@ namespace glr {
 namespace {
 constexpr int GB_M = 64, GB_N = 64, GB_K = 16;
 
-__global__ void __launch_bounds__(256) gemm_f32_kernel(GemmDesc d, int kchunk) {
-    __shared__ float As[GB_K][GB_M + 4];
-    __shared__ float Bs[GB_K][GB_N + 4];
-    const bool split = kchunk > 0;                  // blockIdx.z = K slice (batch == 1)
-    const int z = split ? 0 : blockIdx.z;
-    const float* A = d.A + z * d.sAz;
-    const float* B = d.B + z * d.sBz;
-    float* C = d.C + z * d.sCz;
-    const int i0 = blockIdx.y * GB_M, j0 = blockIdx.x * GB_N;
-    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    float acc[4][4] = {};
-    const bool a_i_unit = d.sAi == 1;
-    const bool b_j_unit = d.sBj == 1;
-    const int kbeg = split ? blockIdx.z * kchunk : 0;
-    const int kend = split ? min(d.K, kbeg + kchunk) : d.K;
-    for (int p0 = kbeg; p0 < kend; p0 += GB_K) {
-        for (int e = tid; e < GB_M * GB_K; e += 256) {
-            int ii, pp;
-            if (a_i_unit) { ii = e % GB_M; pp = e / GB_M; } else { pp = e % GB_K; ii = e / GB_K; }
-            const int gi = i0 + ii, gp = p0 + pp;
-            As[pp][ii] = (gi < d.M && gp < kend) ? A[gi * d.sAi + gp * d.sAp] : 0.f;
+// 64 x 64 tile (i0, j0) of A B over [kbeg, kend): the next slab's elements are on their way to
+// registers while the current one is multiplied (one barrier a slab); every output is one fma chain
+// over k ascending.  Without the prefetch a slab of 16 waited out the whole load latency (3.4 us).
+struct GemmTile {
+    const float* A; int64_t sAi, sAp;
+    const float* B; int64_t sBp, sBj;
+    int M, N;
+};
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void gemm_tile(const GemmTile& g, int i0, int j0, int kbeg, int kend, float (&acc)[4][4]) {
+    __shared__ __align__(16) float As[2][GB_K][GB_M + 4], Bs[2][GB_K][GB_N + 4];
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const bool ai = g.sAi == 1, bj = g.sBj == 1;            // consecutive threads along the contiguous index
+    const int aii = ai ? tid & 63 : tid / GB_K, app = ai ? tid >> 6 : tid % GB_K;
+    const int bjj = bj ? tid & 63 : tid / GB_K, bpp = bj ? tid >> 6 : tid % GB_K;
+    constexpr int NL = GB_K / 4, IS = 256 / GB_K;           // elements a thread; index step along i or j
+    float ra[NL], rb[NL];
+    f32x2 c[4][2] = {};
+    auto load = [&](int p0) {
+#pragma unroll
+        for (int u = 0; u < NL; ++u) {
+            const int ii = ai ? aii : aii + IS * u, pa = p0 + (ai ? app + 4 * u : app);
+            ra[u] = i0 + ii < g.M && pa < kend ? g.A[(int64_t)(i0 + ii) * g.sAi + (int64_t)pa * g.sAp] : 0.f;
+            const int jj = bj ? bjj : bjj + IS * u, pb = p0 + (bj ? bpp + 4 * u : bpp);
+            rb[u] = j0 + jj < g.N && pb < kend ? g.B[(int64_t)pb * g.sBp + (int64_t)(j0 + jj) * g.sBj] : 0.f;
         }
-        for (int e = tid; e < GB_N * GB_K; e += 256) {
-            int jj, pp;
-            if (b_j_unit) { jj = e % GB_N; pp = e / GB_N; } else { pp = e % GB_K; jj = e / GB_K; }
-            const int gj = j0 + jj, gp = p0 + pp;
-            Bs[pp][jj] = (gj < d.N && gp < kend) ? B[gp * d.sBp + gj * d.sBj] : 0.f;
+    };
+    if (kbeg < kend) load(kbeg);
+    int s = 0;
+    for (int p0 = kbeg; p0 < kend; p0 += GB_K, s ^= 1) {
+#pragma unroll
+        for (int u = 0; u < NL; ++u) {
+            As[s][ai ? app + 4 * u : app][ai ? aii : aii + IS * u] = ra[u];
+            Bs[s][bj ? bpp + 4 * u : bpp][bj ? bjj : bjj + IS * u] = rb[u];
         }
-        __syncthreads();
+        __syncthreads();                                    // the other buffer is read up to here
+        if (p0 + GB_K < kend) load(p0 + GB_K);
 #pragma unroll
         for (int p = 0; p < GB_K; ++p) {
-            float a[4], b[4];
+            const float4 a = *reinterpret_cast<const float4*>(&As[s][p][ty * 4]);
+            const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(&Bs[s][p][tx * 4]);
+            const float av[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
-            for (int u = 0; u < 4; ++u) { a[u] = As[p][ty * 4 + u]; b[u] = Bs[p][tx * 4 + u]; }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
+            for (int u = 0; u < 4; ++u) {
+                const f32x2 aa = pack2(av[u], av[u]);
+                asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c[u][0]) : "l"(aa), "l"(b.x));
+                asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c[u][1]) : "l"(aa), "l"(b.y));
+            }
         }
-        __syncthreads();
     }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 2; ++v) asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[u][2 * v]), "=f"(acc[u][2 * v + 1]) : "l"(c[u][v]));
+}
+
+__global__ void __launch_bounds__(256) gemm_f32_kernel(GemmDesc d, int kchunk) {
+    const bool split = kchunk > 0;                  // blockIdx.z = K slice (batch == 1)
+    const int z = split ? 0 : blockIdx.z;
+    float* C = d.C + z * d.sCz;
+    const int i0 = blockIdx.y * GB_M, j0 = blockIdx.x * GB_N;
+    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+    const int kbeg = split ? blockIdx.z * kchunk : 0;
+    const int kend = split ? min(d.K, kbeg + kchunk) : d.K;
+    const GemmTile g{d.A + z * d.sAz, d.sAi, d.sAp, d.B + z * d.sBz, d.sBp, d.sBj, d.M, d.N};
+    float acc[4][4];
+    gemm_tile(g, i0, j0, kbeg, kend, acc);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         const int gi = i0 + ty * 4 + u;
@@ -304,8 +335,12 @@ cudaError_t materialize_error(int mp, int np, int r, int e_zero, const float* B,
 namespace glr {
 namespace {
 
+// K elements of a slice: whole slabs.
+__host__ __device__ __forceinline__ int gemm_chunk(const GemmMat& M) {
+    return ((M.K + M.splits - 1) / M.splits + GB_K - 1) / GB_K * GB_K;
+}
+
 __global__ void __launch_bounds__(256) gemm_group_kernel(const __grid_constant__ GemmGroup g) {
-    __shared__ float As[16][68], Bs[16][68];
     const int tile = blockIdx.x;
     int lo = 0, hi = g.nmat - 1;
     while (lo < hi) {
@@ -313,55 +348,63 @@ __global__ void __launch_bounds__(256) gemm_group_kernel(const __grid_constant__
         if (g.mat[mid].tile0 <= tile) lo = mid; else hi = mid - 1;
     }
     const GemmMat& M = g.mat[lo];
-    const int lt = tile - M.tile0, tn = (M.N + 63) / 64;
+    const int tn = (M.N + 63) / 64, tiles = tn * ((M.M + 63) / 64);
+    const int lt = (tile - M.tile0) % tiles, z = (tile - M.tile0) / tiles;
     const int i0 = (lt / tn) * 64, j0 = (lt % tn) * 64;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    float acc[4][4] = {};
-    for (int p0 = 0; p0 < M.K; p0 += 16) {
-        for (int e = threadIdx.x; e < 16 * 64; e += 256) {
-            // consecutive threads along the operand's contiguous index
-            const bool pa = M.sAp == 1;
-            const int pp = pa ? (e & 15) : (e >> 6), ii = pa ? (e >> 4) : (e & 63);
-            const int i = i0 + ii, p = p0 + pp;
-            As[pp][ii] = (i < M.M && p < M.K) ? M.A[(int64_t)i * M.sAi + (int64_t)p * M.sAp] : 0.f;
-            const bool jb = M.sBj == 1;
-            const int jj = jb ? (e & 63) : (e >> 4), pq = jb ? (e >> 6) : (e & 15);
-            const int j = j0 + jj, q = p0 + pq;
-            Bs[pq][jj] = (j < M.N && q < M.K) ? M.B[(int64_t)q * M.sBp + (int64_t)j * M.sBj] : 0.f;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int pp = 0; pp < 16; ++pp) {
-            float a[4], b[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) { a[u] = As[pp][ty * 4 + u]; b[u] = Bs[pp][tx * 4 + u]; }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
-        }
-        __syncthreads();
-    }
+    const int chunk = gemm_chunk(M), kend = min(M.K, (z + 1) * chunk);
+    const GemmTile t{M.A, M.sAi, M.sAp, M.B, M.sBp, M.sBj, M.M, M.N};
+    float acc[4][4];
+    gemm_tile(t, i0, j0, z * chunk, kend, acc);
+    const float alpha = M.alpha != 0.f ? M.alpha : 1.f;
 #pragma unroll
     for (int u = 0; u < 4; ++u)
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             const int i = i0 + ty * 4 + u, j = j0 + tx * 4 + v;
-            if (i < M.M && j < M.N) M.C[(int64_t)i * M.sCi + (int64_t)j * M.sCj] = (M.alpha != 0.f ? M.alpha : 1.f) * acc[u][v];
+            if (i >= M.M || j >= M.N) continue;
+            if (M.splits > 1) M.ws[((int64_t)z * M.M + i) * M.N + j] = acc[u][v];
+            else M.C[(int64_t)i * M.sCi + (int64_t)j * M.sCj] = alpha * acc[u][v];
         }
+}
+
+// C = alpha times the sum of the K slices, added in order.
+__global__ void __launch_bounds__(256) gemm_group_reduce(const __grid_constant__ GemmGroup g) {
+    const GemmMat& M = g.mat[blockIdx.y];
+    if (M.splits <= 1) return;
+    const float alpha = M.alpha != 0.f ? M.alpha : 1.f;
+    const int64_t mn = (int64_t)M.M * M.N;
+    for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < mn; e += (int64_t)gridDim.x * 256) {
+        float acc = 0.f;
+        for (int z = 0; z < M.splits; ++z) acc += M.ws[z * mn + e];
+        M.C[(e / M.N) * M.sCi + (e % M.N) * M.sCj] = alpha * acc;
+    }
 }
 
 }  // namespace
 
 cudaError_t gemm_group_f32(GemmGroup& g, cudaStream_t st) {
     g.total_tiles = 0;
+    bool reduce = false;
     for (int i = 0; i < g.nmat; ++i) {
         GemmMat& M = g.mat[i];
+        const int tiles = ((M.M + 63) / 64) * ((M.N + 63) / 64);
+        // long products with few tiles (a Gram matrix: 16 tiles, K = 4096) in K slices of at least 256, by
+        // the product's own sizes so that its sums do not depend on the group: 677 -> about 60 us there
+        M.splits = 1;
+        if (M.ws && tiles <= 16 && M.K >= 512) {
+            M.splits = M.K / 256 < 16 ? M.K / 256 : 16;
+            while ((int64_t)M.splits * M.M * M.N > kGemmWsFloats) --M.splits;
+            if (M.splits < 1) M.splits = 1;
+        }
+        if (M.splits > 1) M.splits = (M.K + gemm_chunk(M) - 1) / gemm_chunk(M);
+        reduce = reduce || M.splits > 1;
         M.tile0 = g.total_tiles;
-        g.total_tiles += ((M.M + 63) / 64) * ((M.N + 63) / 64);
+        g.total_tiles += tiles * M.splits;
     }
     if (g.total_tiles <= 0) return cudaSuccess;
     gemm_group_kernel<<<g.total_tiles, 256, 0, st>>>(g);
+    if (reduce) gemm_group_reduce<<<dim3(64, g.nmat), 256, 0, st>>>(g);
     return cudaGetLastError();
 }
 
