@@ -196,41 +196,69 @@ int fail_cuda(glr_handle* h, cudaError_t e, const char* file, int line) {
 
 namespace {
 
-// Rbar = P^T Mbar; Ghat = P Rbar; optimizer.
-int project_and_update(glr_handle* h, float* X, cudaStream_t st) {
+// Plain fp32 products of several handles gathered into one launch (the same sums as one by one).  A
+// product that gemm() sends to the library (2^26 flops and more) is run at once instead.
+struct ProductQueue {
+    GemmGroup g{};
+    glr_handle* h0 = nullptr;
+    int phase;
+    cudaStream_t st;
+    ProductQueue(int phase_, cudaStream_t st_) : phase(phase_), st(st_) {}
+    int add(glr_handle* h, const GemmDesc& d) {
+        if (2.0 * d.M * d.N * (double)d.K * d.batch >= 67108864.0) {
+            PhaseScope ps(h, phase, st);
+            return gemm(h, d, st);
+        }
+        if (!h0) h0 = h;
+        for (int z = 0; z < d.batch; ++z) {
+            GemmMat& M = g.mat[g.nmat++];
+            M = GemmMat{};
+            M.M = d.M; M.N = d.N; M.K = d.K; M.alpha = d.alpha;
+            M.A = d.A + z * d.sAz; M.sAi = d.sAi; M.sAp = d.sAp;
+            M.B = d.B + z * d.sBz; M.sBp = d.sBp; M.sBj = d.sBj;
+            M.C = d.C + z * d.sCz; M.sCi = d.sCi; M.sCj = d.sCj;
+            if (g.nmat == 64) {
+                const int rc = flush();
+                if (rc != GLR_OK) return rc;
+                h0 = h;
+            }
+        }
+        return GLR_OK;
+    }
+    int flush() {
+        if (g.nmat == 0) return GLR_OK;
+        PhaseScope ps(h0, phase, st);
+        GLR_LAUNCH(h0, 1, gemm_group_f32(g, st));
+        g.nmat = 0;
+        h0 = nullptr;
+        return GLR_OK;
+    }
+};
+
+UpdateArgs update_args(glr_handle* h, float* X, bool compressed) {
+    UpdateArgs u{};
+    u.mp = h->mp; u.np = h->np; u.r = h->r; u.transposed = h->transposed; u.compressed = compressed ? 1 : 0;
+    u.optimizer = h->s.optimizer; u.lr = h->s.lr; u.beta1 = h->s.beta1; u.beta2 = h->s.beta2; u.eps = h->s.eps;
+    u.P = h->P; u.Rbar = h->Rbar; u.Mbar = h->Mbar; u.X = X; u.Mo = h->Mo; u.Vo = h->Vo;
+    return u;
+}
+
+// Rbar = P^T Mbar, Ghat = P Rbar as a library product written straight into X's layout (transposed
+// when m > n), then one elementwise optimizer pass.
+int project_and_update_tc(glr_handle* h, float* X, cudaStream_t st) {
     const int mp = h->mp, np = h->np, r = h->r;
     {
         PhaseScope ps(h, GLR_PH_PROJECT, st);
         GLR_GEMM(h, gd(r, np, mp, h->P, 1, r, h->Mbar, np, 1, h->Rbar, np, 1), st);
     }
     PhaseScope ps(h, GLR_PH_UPDATE, st);
-    UpdateArgs u{};
-    u.mp = mp; u.np = np; u.r = r; u.transposed = h->transposed; u.compressed = 1;
-    if (h->tc) {
-        // Ghat = P Rbar as a library product written straight into X's layout (transposed when
-        // m > n), then one elementwise optimizer pass
-        if (h->transposed)
-            GLR_GEMM(h, gd(mp, np, r, h->P, r, 1, h->Rbar, np, 1, h->mn_scratch, 1, mp), st);
-        else
-            GLR_GEMM(h, gd(mp, np, r, h->P, r, 1, h->Rbar, np, 1, h->mn_scratch, np, 1), st);
-        u.compressed = 0;
-        u.optimizer = h->s.optimizer; u.lr = h->s.lr; u.beta1 = h->s.beta1; u.beta2 = h->s.beta2; u.eps = h->s.eps;
-        u.P = h->P; u.Rbar = h->Rbar; u.Mbar = h->mn_scratch; u.X = X; u.Mo = h->Mo; u.Vo = h->Vo;
-        GLR_LAUNCH(h, 1, update_streamed_flat(u, st));
-        return GLR_OK;
-    }
-    u.optimizer = h->s.optimizer; u.lr = h->s.lr; u.beta1 = h->s.beta1; u.beta2 = h->s.beta2; u.eps = h->s.eps;
-    u.P = h->P; u.Rbar = h->Rbar; u.Mbar = h->Mbar; u.X = X; u.Mo = h->Mo; u.Vo = h->Vo;
-    GLR_LAUNCH(h, 1, update(u, st));
-    return GLR_OK;
-}
-
-int uncompressed_update(glr_handle* h, float* X, cudaStream_t st) {
-    UpdateArgs u{};
-    u.mp = h->mp; u.np = h->np; u.r = h->r; u.transposed = h->transposed; u.compressed = 0;
-    u.optimizer = h->s.optimizer; u.lr = h->s.lr; u.beta1 = h->s.beta1; u.beta2 = h->s.beta2; u.eps = h->s.eps;
-    u.P = h->P; u.Rbar = h->Rbar; u.Mbar = h->Mbar; u.X = X; u.Mo = h->Mo; u.Vo = h->Vo;
-    GLR_LAUNCH(h, 1, update(u, st));
+    if (h->transposed)
+        GLR_GEMM(h, gd(mp, np, r, h->P, r, 1, h->Rbar, np, 1, h->mn_scratch, 1, mp), st);
+    else
+        GLR_GEMM(h, gd(mp, np, r, h->P, r, 1, h->Rbar, np, 1, h->mn_scratch, np, 1), st);
+    UpdateArgs u = update_args(h, X, false);
+    u.Mbar = h->mn_scratch;
+    GLR_LAUNCH(h, 1, update_streamed_flat(u, st));
     return GLR_OK;
 }
 
@@ -283,11 +311,6 @@ int separate_optimizer_update(glr_handle* h, float* X, bool compressed, bool ref
     }
     GLR_LAUNCH(h, 3, amsgrad_update(Gh, mp, np, h->transposed, X, h->Mo, h->Vo, h->amsv, h->s.lr, h->s.beta1,
                                     h->s.beta2, h->s.eps, st));
-    return GLR_OK;
-}
-
-int build_selection_P(glr_handle* h, cudaStream_t st) {
-    GLR_LAUNCH(h, 1, build_P(h->exact ? 0 : 1, h->mp, h->r, h->k, h->J, h->U, h->Y, h->Yt, h->dsign, h->P, st));
     return GLR_OK;
 }
 
@@ -536,32 +559,67 @@ void plan_step(StepPlan& p) {
     h->forced_this_step = p.forced;
 }
 
-// K1 with the first-path kernels: R_w,i = P_prev^T B_i, then compose.
-int compose_unfused(StepPlan& p, cudaStream_t st) {
+ComposeArgs compose_args(const StepPlan& p) {
     glr_handle* h = p.h;
-    const int mp = h->mp, np = h->np, r = h->r, N = h->N;
-    if (!h->e_zero) {
-        PhaseScope ps(h, GLR_PH_PREV_PROJECT, st);
-        GemmDesc d = gd(r, np, mp, h->Pprev, 1, r, h->B, np, 1, h->Rw, np, 1);
-        d.batch = N; d.sAz = 0; d.sBz = (int64_t)mp * np; d.sCz = (int64_t)r * np;
-        GLR_GEMM(h, d, st);
-        if (h->tc) {
-            // B_i <- E_i = B_i - P_prev R_w,i in place (one batched library product); the
-            // compose pass below then only adds G_i
-            GemmDesc e = gd(mp, np, r, h->Pprev, r, 1, h->Rw, np, 1, h->B, np, 1, -1.f, 1.f);
-            e.batch = N; e.sAz = 0; e.sBz = (int64_t)r * np; e.sCz = (int64_t)mp * np;
-            GLR_GEMM(h, e, st);
-        }
-    }
-    PhaseScope ps(h, GLR_PH_COMPOSE, st);
     ComposeArgs ca{};
-    for (int i = 0; i < N; ++i) ca.G[i] = p.G[i];
+    for (int i = 0; i < h->N; ++i) ca.G[i] = p.G[i];
     ca.grad_dtype = h->s.grad_dtype; ca.transposed = h->transposed;
-    ca.mp = mp; ca.np = np; ca.N = N; ca.r = h->tc ? 0 : r; ca.e_zero = h->e_zero ? 1 : 0;
+    ca.mp = h->mp; ca.np = h->np; ca.N = h->N; ca.r = h->tc ? 0 : h->r; ca.e_zero = h->e_zero ? 1 : 0;
     ca.write_B = (p.warm || h->s.no_error_feedback) ? 0 : 1;   // B feeds only the error
     ca.B = h->B; ca.Pprev = h->Pprev; ca.Rw = h->Rw; ca.Mbar = h->Mbar; ca.nonfinite = h->dflags + 3;
-    if (h->tc) GLR_LAUNCH(h, 1, compose_streamed(ca, st));
-    else GLR_LAUNCH(h, 1, compose(ca, st));
+    return ca;
+}
+
+// R_w,i = P_prev^T B_i for every node.
+GemmDesc prev_project(glr_handle* h) {
+    GemmDesc d = gd(h->r, h->np, h->mp, h->Pprev, 1, h->r, h->B, h->np, 1, h->Rw, h->np, 1);
+    d.batch = h->N; d.sAz = 0; d.sBz = (int64_t)h->mp * h->np; d.sCz = (int64_t)h->r * h->np;
+    return d;
+}
+
+// K1 with library products: R_w,i, then E_i = B_i - P_prev R_w,i in place (one batched product; the
+// compose pass then only adds G_i).
+int compose_tc(StepPlan& p, cudaStream_t st) {
+    glr_handle* h = p.h;
+    const int mp = h->mp, np = h->np, r = h->r;
+    if (!h->e_zero) {
+        PhaseScope ps(h, GLR_PH_PREV_PROJECT, st);
+        GLR_GEMM(h, prev_project(h), st);
+        GemmDesc e = gd(mp, np, r, h->Pprev, r, 1, h->Rw, np, 1, h->B, np, 1, -1.f, 1.f);
+        e.batch = h->N; e.sAz = 0; e.sBz = (int64_t)r * np; e.sCz = (int64_t)mp * np;
+        GLR_GEMM(h, e, st);
+    }
+    PhaseScope ps(h, GLR_PH_COMPOSE, st);
+    GLR_LAUNCH(h, 1, compose_streamed(compose_args(p), st));
+    return GLR_OK;
+}
+
+// K1 with the first-path kernels, grouped: the R_w,i of every plan, then one compose launch.  (A
+// launch of each per matrix: 27 launches and 425 us for four ragged matrices of 0.26 M elements.)
+int compose_unfused(std::vector<StepPlan*>& plans, cudaStream_t st) {
+    ProductQueue q(GLR_PH_PREV_PROJECT, st);
+    int rc;
+    for (StepPlan* p : plans) {
+        if (p->h->tc) {
+            if ((rc = compose_tc(*p, st)) != GLR_OK) return rc;
+        } else if (!p->h->e_zero && (rc = q.add(p->h, prev_project(p->h))) != GLR_OK) {
+            return rc;
+        }
+    }
+    if ((rc = q.flush()) != GLR_OK) return rc;
+    static thread_local ComposeGroup g;          // ~20 KiB: kept off the stack
+    for (size_t i = 0; i < plans.size();) {
+        g.nmat = 0;
+        glr_handle* h0 = nullptr;
+        for (; i < plans.size() && g.nmat < kGroupMax; ++i) {
+            if (plans[i]->h->tc) continue;
+            if (!h0) h0 = plans[i]->h;
+            g.mat[g.nmat++] = compose_args(*plans[i]);
+        }
+        if (!h0) continue;
+        PhaseScope ps(h0, GLR_PH_COMPOSE, st);
+        GLR_LAUNCH(h0, 1, compose(g, st));
+    }
     return GLR_OK;
 }
 
@@ -874,8 +932,33 @@ int tcl_project_update(std::vector<StepPlan*>& plans, cudaStream_t st) {
     return rc != GLR_OK ? rc : tcl_update(plans, st);
 }
 
-// Between K1 and K3: refresh, or Approx-Top-r selection and P.
-int select_phase(StepPlan& p, cudaStream_t st) {
+// The scores' partial sums of the matrices outside the fused kernels, gathered for grouped launches:
+// W = Y^T Mbar where the basis is truncated, then the bilinear forms.
+struct ScoreQueue {
+    ProductQueue W;
+    LambdaGroup g;
+    glr_handle* h0 = nullptr;
+    explicit ScoreQueue(cudaStream_t st) : W(GLR_PH_LAMBDA, st) { g.nmat = 0; }
+    int add(glr_handle* h, const LambdaArgs& la) {
+        if (!h0) h0 = h;
+        g.mat[g.nmat++] = la;
+        return g.nmat == kGroupMax ? flush() : GLR_OK;
+    }
+    int flush() {
+        const int rc = W.flush();
+        if (rc != GLR_OK || g.nmat == 0) return rc;
+        PhaseScope ps(h0, GLR_PH_LAMBDA, W.st);
+        int modes = 0;
+        for (int i = 0; i < g.nmat; ++i) modes |= 1 << g.mat[i].mode;
+        GLR_LAUNCH(h0, (modes & 1) + (modes >> 1), lambda_partials(g, W.st));
+        g.nmat = 0;
+        h0 = nullptr;
+        return GLR_OK;
+    }
+};
+
+// Between K1 and K3: refresh, or Approx-Top-r selection (the scores' work queued on q) and P.
+int select_phase(StepPlan& p, ScoreQueue& q, cudaStream_t st) {
     glr_handle* h = p.h;
     const int mp = h->mp, np = h->np, r = h->r;
     int rc = GLR_OK;
@@ -896,7 +979,6 @@ int select_phase(StepPlan& p, cudaStream_t st) {
     } else if (h->tcl) {
         h->comm += (int64_t)r * np + mp;           // the scores come from tcl_lambda
     } else if (!p.lam_fused) {
-        PhaseScope ps(h, GLR_PH_LAMBDA, st);
         LambdaArgs la{};
         la.mp = mp; la.np = np; la.seed = h->s.seed; la.t = static_cast<uint32_t>(h->t);
         la.part = h->lam_part; la.ntiles = h->ntiles;
@@ -904,16 +986,20 @@ int select_phase(StepPlan& p, cudaStream_t st) {
             la.mode = 0; la.K = mp; la.A = h->U; la.Bm = h->Mbar; la.Mbar = h->Mbar;
         } else {
             const int k = h->k;
-            GLR_GEMM(h, gd(k, np, mp, h->Y, 1, k, h->Mbar, np, 1, h->Wbar, np, 1), st);  // Wbar = Y^T Mbar
+            const GemmDesc w = gd(k, np, mp, h->Y, 1, k, h->Mbar, np, 1, h->Wbar, np, 1);    // Wbar = Y^T Mbar
             la.mode = 1; la.K = k; la.A = h->Yt; la.Bm = h->Wbar; la.Mbar = h->Mbar;
             if (h->tc) {
                 // Yt Wbar as a library product into the scratch; the score kernel then forms the
                 // row sums of (Mbar - scratch) against v_j (K = 0)
+                PhaseScope ps(h, GLR_PH_LAMBDA, st);
+                GLR_GEMM(h, w, st);
                 GLR_GEMM(h, gd(mp, np, k, h->Yt, k, 1, h->Wbar, np, 1, h->mn_scratch, np, 1), st);
                 la.K = 0; la.Csub = h->mn_scratch;
+            } else if ((rc = q.W.add(h, w)) != GLR_OK) {
+                return rc;
             }
         }
-        GLR_LAUNCH(h, 1, lambda_partials(la, st));
+        if ((rc = q.add(h, la)) != GLR_OK) return rc;
         h->comm += (int64_t)r * np + mp;
     } else {
         h->comm += (int64_t)r * np + mp;
@@ -971,12 +1057,35 @@ int select_P_grouped(std::vector<StepPlan>& plans, cudaStream_t st, int stages =
     return GLR_OK;
 }
 
-int update_unfused(StepPlan& p, cudaStream_t st) {
-    if (!p.compressed) {
-        PhaseScope ps(p.h, GLR_PH_UPDATE, st);
-        return uncompressed_update(p.h, p.X, st);
+// K3 with the first-path kernels, grouped: Rbar = P^T Mbar of every compressed plan, then one launch for
+// Ghat = P Rbar (or Mbar) and the optimizers.
+int update_unfused(std::vector<StepPlan*>& plans, cudaStream_t st) {
+    ProductQueue q(GLR_PH_PROJECT, st);
+    int rc;
+    for (StepPlan* p : plans) {
+        glr_handle* h = p->h;
+        if (!p->compressed) continue;
+        if (h->tc) {
+            if ((rc = project_and_update_tc(h, p->X, st)) != GLR_OK) return rc;
+        } else if ((rc = q.add(h, gd(h->r, h->np, h->mp, h->P, 1, h->r, h->Mbar, h->np, 1, h->Rbar, h->np, 1))) != GLR_OK) {
+            return rc;
+        }
     }
-    return project_and_update(p.h, p.X, st);
+    if ((rc = q.flush()) != GLR_OK) return rc;
+    for (size_t i = 0; i < plans.size();) {
+        UpdateTileGroup g;
+        g.nmat = 0;
+        glr_handle* h0 = nullptr;
+        for (; i < plans.size() && g.nmat < kGroupMax; ++i) {
+            if (plans[i]->compressed && plans[i]->h->tc) continue;
+            if (!h0) h0 = plans[i]->h;
+            g.mat[g.nmat++] = update_args(plans[i]->h, plans[i]->X, plans[i]->compressed);
+        }
+        if (!h0) continue;
+        PhaseScope ps(h0, GLR_PH_UPDATE, st);
+        GLR_LAUNCH(h0, 1, update(g, st));
+    }
+    return GLR_OK;
 }
 
 void finish_step(StepPlan& p) {
@@ -1005,8 +1114,7 @@ int step_group(std::vector<StepPlan>& plans, cudaStream_t st) {
     int rc;
     if (!fused.empty() && (rc = compose_fused(fused, st)) != GLR_OK) return rc;
     if (!tcl.empty() && (rc = tcl_compose(tcl, st)) != GLR_OK) return rc;
-    for (StepPlan* p : unfused)
-        if ((rc = compose_unfused(*p, st)) != GLR_OK) return rc;
+    if (!unfused.empty() && (rc = compose_unfused(unfused, st)) != GLR_OK) return rc;
     // Refreshes (Semi-Lazy SVD) of different matrices are independent: each runs on its
     // handle's side stream after the compose pass, overlapping the others and the selection
     // work of the non-refreshing matrices; the main stream joins them before P is built.
@@ -1024,8 +1132,10 @@ int step_group(std::vector<StepPlan>& plans, cudaStream_t st) {
     if (!trunc.empty() && (rc = refresh_trunc_grouped(trunc)) != GLR_OK) return rc;
     if (!tclr.empty() && (rc = refresh_tcl_grouped(tclr)) != GLR_OK) return rc;
     for (glr_handle* h : refreshing) GLR_CK(h, cudaEventRecord(h->rdone, h->rstream));
+    ScoreQueue scores(st);
     for (StepPlan& p : plans)
-        if ((rc = select_phase(p, st)) != GLR_OK) return rc;
+        if ((rc = select_phase(p, scores, st)) != GLR_OK) return rc;
+    if ((rc = scores.flush()) != GLR_OK) return rc;
     if (!tcl.empty() && (rc = tcl_lambda(tcl, st)) != GLR_OK) return rc;
     for (glr_handle* h : refreshing) GLR_CK(h, cudaStreamWaitEvent(st, h->rdone, 0));
     if ((rc = select_P_grouped(plans, st)) != GLR_OK) return rc;
@@ -1043,8 +1153,9 @@ int step_group(std::vector<StepPlan>& plans, cudaStream_t st) {
     }
     if (!streamed.empty() && (rc = update_streamed(streamed, st)) != GLR_OK) return rc;
     if (!strips.empty() && (rc = update_fused(strips, st)) != GLR_OK) return rc;
-    for (StepPlan* p : unfused)
-        if (!separate_optimizer(p->h) && (rc = update_unfused(*p, st)) != GLR_OK) return rc;
+    unfused.erase(std::remove_if(unfused.begin(), unfused.end(), [](StepPlan* p) { return separate_optimizer(p->h); }),
+                  unfused.end());
+    if (!unfused.empty() && (rc = update_unfused(unfused, st)) != GLR_OK) return rc;
     for (StepPlan& p : plans)
         if (separate_optimizer(p.h) && (rc = separate_optimizer_update(p.h, p.X, p.compressed, p.refresh, st)) != GLR_OK)
             return rc;
@@ -1084,7 +1195,8 @@ int dp_begin(glr_handle* h, const void* const* G, cudaStream_t st, glr_dp_exchan
         dp_expose(ex, h->Mbar, (int64_t)h->mp * h->np);
         return GLR_OK;
     }
-    if ((rc = select_phase(p, st)) != GLR_OK) return rc;     // J of a forced / fixed selection
+    ScoreQueue scores(st);                     // the tcgen05 path queues nothing on it
+    if ((rc = select_phase(p, scores, st)) != GLR_OK) return rc;     // J of a forced / fixed selection
     if (tc_needs_lambda(p)) {                  // this shard's lambda-bar (linear in Mbar)
         if ((rc = tcl_lambda(v, st)) != GLR_OK) return rc;
         if ((rc = select_P_grouped(plans, st, 1)) != GLR_OK) return rc;
@@ -1108,7 +1220,8 @@ int dp_select(glr_handle* h, cudaStream_t st, glr_dp_exchange* ex) {
         if (rc != GLR_OK) return rc;
         GLR_CK(h, cudaEventRecord(h->rdone, h->rstream));
         GLR_CK(h, cudaStreamWaitEvent(st, h->rdone, 0));
-        if ((rc = select_phase(p, st)) != GLR_OK) return rc;
+        ScoreQueue scores(st);
+        if ((rc = select_phase(p, scores, st)) != GLR_OK) return rc;
     }
     if (!p.compressed) return GLR_OK;          // Ghat = Mbar: nothing more to average
     if ((rc = select_P_grouped(plans, st, 2)) != GLR_OK) return rc;   // lambda-bar came from glr_dp_begin

@@ -137,7 +137,8 @@ struct ComposeArgs {
     float* Mbar;            // m' x n'
     int* nonfinite;         // counts warps that found a NaN / Inf in Mbar (may be null)
 };
-cudaError_t compose(const ComposeArgs& a, cudaStream_t st);
+struct ComposeGroup { int nmat; ComposeArgs mat[kGroupMax]; int tile0[kGroupMax]; };
+cudaError_t compose(ComposeGroup& g, cudaStream_t st);
 
 // Approx-Top-r partial sums: part[tb * m' + j] = sum_{b in tile tb} C(j, b) v_j[b] where
 //   dense:  C = U^T Mbar                  (A(j, p) = U[p * m' + j], K = m')
@@ -153,7 +154,8 @@ struct LambdaArgs {
     float* part; int ntiles;
 };
 constexpr int kLambdaTile = 64;
-cudaError_t lambda_partials(const LambdaArgs& a, cudaStream_t st);
+struct LambdaGroup { int nmat; LambdaArgs mat[kGroupMax]; int tile0[kGroupMax]; };
+cudaError_t lambda_partials(const LambdaGroup& g, cudaStream_t st);      // at most one launch per mode
 
 // Reduce the partials in fixed order, apply the column signs d (k entries, may be null),
 // pick J = the r largest lambda^2 (ties -> lower index), J ascending.
@@ -186,10 +188,6 @@ cudaError_t select_group(const SelectGroup& g, cudaStream_t st, int stages = 3);
 cudaError_t wy_columns_gather(const float* Yt, const int32_t* J, int r, int k, float* YtJ, cudaStream_t st);
 cudaError_t wy_columns_fix(float* P, const int32_t* J, const float* dsign, int mp, int r, int k, cudaStream_t st);
 
-// P(:, q) = column J[q] of U: dense U (mode 0) or U = (I - Y Yt^T) D (mode 1).
-cudaError_t build_P(int mode, int mp, int r, int k, const int32_t* J, const float* U,
-                    const float* Y, const float* Yt, const float* dsign, float* P, cudaStream_t st);
-
 // K3 -- decompress + optimizer: Ghat(a, b) = sum_q P(a, q) Rbar(q, b) (compressed) or
 // Mbar(a, b), mapped back to X's layout (transposed when m > n), then MSGD / Adam.
 struct UpdateArgs {
@@ -198,7 +196,8 @@ struct UpdateArgs {
     const float* P; const float* Rbar; const float* Mbar;
     float* X; float* Mo; float* Vo;
 };
-cudaError_t update(const UpdateArgs& a, cudaStream_t st);
+struct UpdateTileGroup { int nmat; UpdateArgs mat[kGroupMax]; int tile0[kGroupMax]; };
+cudaError_t update(UpdateTileGroup& g, cudaStream_t st);
 // The first path's streaming passes when its products run as library GEMMs (k_big.cu):
 // compose_streamed takes B holding E_i (the correction already applied; r unused) and needs
 // m' % 4 == n' % 4 == 0; update_streamed_flat takes Ghat in Mbar laid out like X (a.mp x a.np =

@@ -67,10 +67,12 @@ extern "C" int glr_select_noalloc(int32_t mp, int32_t np, int32_t r, const float
         part = g_scratch_addr[dev];
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    glr::LambdaArgs la{};
+    glr::LambdaGroup lg{};
+    lg.nmat = 1;
+    glr::LambdaArgs& la = lg.mat[0];
     la.mode = 0; la.mp = mp; la.np = np; la.K = mp; la.A = U; la.Bm = Mbar; la.Mbar = Mbar;
     la.seed = seed; la.t = static_cast<uint32_t>(t); la.part = part; la.ntiles = ntiles;
-    cudaError_t e = glr::lambda_partials(la, st);
+    cudaError_t e = glr::lambda_partials(lg, st);
     if (e == cudaSuccess) e = glr::select_top_r(part, ntiles, mp, r, nullptr, mp, lambda_out, J_out, st);
     if (e != cudaSuccess) {
         snprintf(msg, sizeof(msg), "glr_select_noalloc: launch failed: %s", cudaGetErrorString(e));

@@ -11,10 +11,14 @@ constexpr int LK = 16;
 
 // C(j, b) = sum_p A(j, p) B(p, b) for a 64 x 64 tile; then for each row j the partial
 // sum over the tile's columns of C'(j, b) v_j[b], with C' = C (dense) or Mbar - C (wy).
-__global__ void __launch_bounds__(256) lambda_kernel(LambdaArgs a) {
+__global__ void __launch_bounds__(256) lambda_kernel(const __grid_constant__ LambdaGroup lg) {
+    int mi = 0;
+    while (mi + 1 < lg.nmat && lg.tile0[mi + 1] <= (int)blockIdx.x) ++mi;
+    const LambdaArgs& a = lg.mat[mi];
+    const int bx = ((int)blockIdx.x - lg.tile0[mi]) % a.ntiles, by = ((int)blockIdx.x - lg.tile0[mi]) / a.ntiles;
     __shared__ float As[LK][LT + 4];
     __shared__ float Bs[LK][LT + 4];
-    const int j0 = blockIdx.y * LT, b0 = blockIdx.x * LT;
+    const int j0 = by * LT, b0 = bx * LT;
     const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
     // A(j, p): dense U^T -> U[p * m' + j] (unit stride along j); wy Yt -> Yt[j * K + p]
     const int64_t sAj = a.mode == 0 ? 1 : a.K;
@@ -69,7 +73,7 @@ __global__ void __launch_bounds__(256) lambda_kernel(LambdaArgs a) {
         // fixed-order reduction over the 16 column groups (lanes with equal ty share a half-warp)
 #pragma unroll
         for (int off = 8; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        if (tx == 0 && j < a.mp) a.part[(int64_t)blockIdx.x * a.mp + j] = s;
+        if (tx == 0 && j < a.mp) a.part[(int64_t)bx * a.mp + j] = s;
     }
 }
 
@@ -94,11 +98,15 @@ __device__ __forceinline__ void lm_mma(float (&d)[4], uint32_t a0, uint32_t a1, 
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-__global__ void __launch_bounds__(256) lambda_mma_kernel(LambdaArgs a) {
+__global__ void __launch_bounds__(256) lambda_mma_kernel(const __grid_constant__ LambdaGroup lg) {
+    int mi = 0;
+    while (mi + 1 < lg.nmat && lg.tile0[mi + 1] <= (int)blockIdx.x) ++mi;
+    const LambdaArgs& a = lg.mat[mi];
+    const int bx = ((int)blockIdx.x - lg.tile0[mi]) % a.ntiles, by = ((int)blockIdx.x - lg.tile0[mi]) / a.ntiles;
     __shared__ __align__(16) float As[LMK][LMP];             // U[p][j0 + jj]
     __shared__ __align__(16) float Bs[LMK][LMP];             // Mbar[p][b0 + bb]
     __shared__ float half_sum[2][LT];
-    const int j0 = blockIdx.y * LT, b0 = blockIdx.x * LT;
+    const int j0 = by * LT, b0 = bx * LT;
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     const int mt = w & 3, nh = w >> 2;                        // m-tile (16 rows j), column half
     const int mp = a.mp, np = a.np, K = a.K;
@@ -179,15 +187,30 @@ __global__ void __launch_bounds__(256) lambda_mma_kernel(LambdaArgs a) {
     __syncthreads();
     for (int jj = tid; jj < LT; jj += 256) {
         const int j = j0 + jj;
-        if (j < mp) a.part[(int64_t)blockIdx.x * mp + j] = half_sum[0][jj] + half_sum[1][jj];
+        if (j < mp) a.part[(int64_t)bx * mp + j] = half_sum[0][jj] + half_sum[1][jj];
     }
 }
 }  // namespace
 
-cudaError_t lambda_partials(const LambdaArgs& a, cudaStream_t st) {
-    dim3 grid(a.ntiles, (a.mp + LT - 1) / LT);
-    if (a.mode == 0) lambda_mma_kernel<<<grid, 256, 0, st>>>(a);   // dense U: a dense contraction
-    else lambda_kernel<<<grid, 256, 0, st>>>(a);
+// All matrices of a step in one launch per mode: one launch a matrix left most SMs idle in each
+// (conv stack, dense bases: 8 launches, 179 us).
+cudaError_t lambda_partials(const LambdaGroup& all, cudaStream_t st) {
+    for (int mode = 0; mode < 2; ++mode) {
+        LambdaGroup g;
+        int tiles = 0;
+        g.nmat = 0;
+        for (int order = 0; order < 2; ++order)            // the longer products first, so that the grid ends evenly
+            for (int i = 0; i < all.nmat; ++i) {
+                const LambdaArgs& a = all.mat[i];
+                if (a.mode != mode || (a.K > 128) != (order == 0)) continue;
+                g.mat[g.nmat] = a;
+                g.tile0[g.nmat++] = tiles;
+                tiles += a.ntiles * ((a.mp + LT - 1) / LT);
+            }
+        if (!tiles) continue;
+        if (mode == 0) lambda_mma_kernel<<<tiles, 256, 0, st>>>(g);   // dense U: a dense contraction
+        else lambda_kernel<<<tiles, 256, 0, st>>>(g);
+    }
     return cudaGetLastError();
 }
 
@@ -241,21 +264,6 @@ __global__ void __launch_bounds__(1024) select_kernel(const float* part, int nti
     }
 }
 
-__global__ void build_P_kernel(int mode, int mp, int r, int k, const int32_t* J, const float* U,
-                               const float* Y, const float* Yt, const float* dsign, float* P) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (int64_t)mp * r) return;
-    const int aa = static_cast<int>(e / r), q = static_cast<int>(e % r);
-    const int j = J[q];
-    if (mode == 0) { P[e] = U[(int64_t)aa * mp + j]; return; }
-    // column j of (I - Y Yt^T), times d_j for the spectral columns j < k
-    float v = (aa == j) ? 1.f : 0.f;
-    const float* ya = Y + (int64_t)aa * k;
-    const float* yj = Yt + (int64_t)j * k;
-    for (int c = 0; c < k; ++c) v = fmaf(-ya[c], yj[c], v);
-    if (j < k) v *= dsign[j];
-    P[e] = v;
-}
 }  // namespace
 
 // ------------------------------------------------------------------------------------------
@@ -498,13 +506,6 @@ cudaError_t select_top_r(const float* part, int ntiles, int mp, int r, const flo
         if (ea != cudaSuccess) return ea;
     }
     select_kernel<<<1, 1024, smem, st>>>(part, ntiles, mp, r, dsign, k, lam, J, npow2);
-    return cudaGetLastError();
-}
-
-cudaError_t build_P(int mode, int mp, int r, int k, const int32_t* J, const float* U, const float* Y,
-                    const float* Yt, const float* dsign, float* P, cudaStream_t st) {
-    const int64_t total = (int64_t)mp * r;
-    build_P_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(mode, mp, r, k, J, U, Y, Yt, dsign, P);
     return cudaGetLastError();
 }
 

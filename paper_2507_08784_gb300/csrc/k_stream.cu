@@ -152,12 +152,16 @@ cudaError_t gemm_f32(const GemmDesc& d, cudaStream_t st) {
 namespace {
 constexpr int CT = 32;
 
-__global__ void __launch_bounds__(256) compose_kernel(ComposeArgs a) {
+__global__ void __launch_bounds__(256) compose_kernel(const __grid_constant__ ComposeGroup g) {
+    int mi = 0;
+    while (mi + 1 < g.nmat && g.tile0[mi + 1] <= (int)blockIdx.x) ++mi;
+    const ComposeArgs& a = g.mat[mi];
+    const int tiles_b = (a.np + CT - 1) / CT, lt = (int)blockIdx.x - g.tile0[mi];
     extern __shared__ float sm[];
     float* Ps = sm;                       // CT x r
     float* Rs = Ps + CT * a.r;            // r x CT
     float* Gs = Rs + a.r * CT;            // CT x (CT + 1)
-    const int a0 = blockIdx.y * CT, b0 = blockIdx.x * CT;
+    const int a0 = lt / tiles_b * CT, b0 = lt % tiles_b * CT;
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * CT + tx;
     const bool corr = !a.e_zero;
     if (corr) {
@@ -169,6 +173,15 @@ __global__ void __launch_bounds__(256) compose_kernel(ComposeArgs a) {
     float sum[4] = {0.f, 0.f, 0.f, 0.f};
     for (int i = 0; i < a.N; ++i) {
         const void* G = a.G[i];
+        float* Bi = a.B + (int64_t)i * a.mp * a.np;
+        float old[4] = {0.f, 0.f, 0.f, 0.f};     // in flight together with the tiles below
+        if (corr) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int aa = a0 + ty + 8 * u, b = b0 + tx;
+                if (aa < a.mp && b < a.np) old[u] = Bi[(int64_t)aa * a.np + b];
+            }
+        }
         if (a.transposed) {       // G_i(a, b) = G_i[b * m' + a]: read along a
             for (int rr = ty; rr < CT; rr += 8) {
                 const int b = b0 + rr, aa = a0 + tx;
@@ -188,7 +201,6 @@ __global__ void __launch_bounds__(256) compose_kernel(ComposeArgs a) {
             }
         }
         __syncthreads();
-        float* Bi = a.B + (int64_t)i * a.mp * a.np;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int rr = ty + 8 * u, aa = a0 + rr, b = b0 + tx;
@@ -198,7 +210,7 @@ __global__ void __launch_bounds__(256) compose_kernel(ComposeArgs a) {
             if (corr) {
                 float c = 0.f;
                 for (int q = 0; q < a.r; ++q) c = fmaf(Ps[rr * a.r + q], Rs[q * CT + tx], c);
-                mval += Bi[idx] - c;
+                mval += old[u] - c;
             }
             if (a.write_B) Bi[idx] = mval;
             sum[u] += mval;
@@ -219,14 +231,21 @@ __global__ void __launch_bounds__(256) compose_kernel(ComposeArgs a) {
 }
 }  // namespace
 
-cudaError_t compose(const ComposeArgs& a, cudaStream_t st) {
-    dim3 grid((a.np + CT - 1) / CT, (a.mp + CT - 1) / CT);
-    const size_t smem = sizeof(float) * (2 * CT * a.r + CT * (CT + 1));
+cudaError_t compose(ComposeGroup& g, cudaStream_t st) {
+    if (g.nmat <= 0) return cudaSuccess;
+    int tiles = 0, r = 0;
+    for (int i = 0; i < g.nmat; ++i) {
+        const auto& a = g.mat[i];
+        g.tile0[i] = tiles;
+        tiles += ((a.np + CT - 1) / CT) * ((a.mp + CT - 1) / CT);
+        r = a.r > r ? a.r : r;
+    }
+    const size_t smem = sizeof(float) * (2 * CT * r + CT * (CT + 1));
     {   // per device: set on every call (cheap next to the launch)
         const cudaError_t ea = cudaFuncSetAttribute(compose_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
         if (ea != cudaSuccess) return ea;
     }
-    compose_kernel<<<grid, dim3(CT, 8), smem, st>>>(a);
+    compose_kernel<<<tiles, dim3(CT, 8), smem, st>>>(g);
     return cudaGetLastError();
 }
 
@@ -235,12 +254,16 @@ cudaError_t compose(const ComposeArgs& a, cudaStream_t st) {
 // into shared memory, then X / M / V are updated in X's own layout (transposed when m > n).
 // ------------------------------------------------------------------------------------------
 namespace {
-__global__ void __launch_bounds__(256) update_kernel(UpdateArgs a) {
+__global__ void __launch_bounds__(256) update_kernel(const __grid_constant__ UpdateTileGroup grp) {
+    int mi = 0;
+    while (mi + 1 < grp.nmat && grp.tile0[mi + 1] <= (int)blockIdx.x) ++mi;
+    const UpdateArgs& a = grp.mat[mi];
+    const int tiles_b = (a.np + CT - 1) / CT, lt = (int)blockIdx.x - grp.tile0[mi];
     extern __shared__ float sm[];
     float* Ps = sm;                       // CT x r
     float* Rs = Ps + CT * a.r;            // r x CT
     float* Gt = Rs + a.r * CT;            // CT x (CT + 1)
-    const int a0 = blockIdx.y * CT, b0 = blockIdx.x * CT;
+    const int a0 = lt / tiles_b * CT, b0 = lt % tiles_b * CT;
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * CT + tx;
     if (a.compressed) {
         for (int e = tid; e < CT * a.r; e += 256) {
@@ -307,14 +330,21 @@ __global__ void __launch_bounds__(256) error_kernel(int mp, int np, int r, int e
 }
 }  // namespace
 
-cudaError_t update(const UpdateArgs& a, cudaStream_t st) {
-    dim3 grid((a.np + CT - 1) / CT, (a.mp + CT - 1) / CT);
-    const size_t smem = sizeof(float) * (2 * CT * a.r + CT * (CT + 1));
+cudaError_t update(UpdateTileGroup& g, cudaStream_t st) {
+    if (g.nmat <= 0) return cudaSuccess;
+    int tiles = 0, r = 0;
+    for (int i = 0; i < g.nmat; ++i) {
+        const auto& a = g.mat[i];
+        g.tile0[i] = tiles;
+        tiles += ((a.np + CT - 1) / CT) * ((a.mp + CT - 1) / CT);
+        r = a.r > r ? a.r : r;
+    }
+    const size_t smem = sizeof(float) * (2 * CT * r + CT * (CT + 1));
     {   // per device: set on every call (cheap next to the launch)
         const cudaError_t ea = cudaFuncSetAttribute(update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
         if (ea != cudaSuccess) return ea;
     }
-    update_kernel<<<grid, dim3(CT, 8), smem, st>>>(a);
+    update_kernel<<<tiles, dim3(CT, 8), smem, st>>>(g);
     return cudaGetLastError();
 }
 
