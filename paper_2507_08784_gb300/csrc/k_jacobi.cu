@@ -18,9 +18,10 @@
 // (jacobi_cluster_kernel), a launch a matrix: the rows of H (two buffers) and V are spread over up to
 // 16 CTAs, a round's rotations and the partner rows come over distributed shared memory, and a round
 // ends with one hardware cluster barrier.  The rotations, their order and every product and sum are
-// those of the grid-wide kernel, so the results are the same bits.  Bound by shared-memory
-// instructions and the cluster's barrier and remote loads; the grid-wide kernel pays
-// 14 us a round for its barrier in global memory and the L2 round trips.
+// those of the grid-wide kernel, so the results are the same bits.  A round takes 3.7 us at n = 512
+// (bound by instruction issue) and 2 us below n = 128 (the rotation's chain of quotients and roots,
+// two cluster barriers); the grid-wide kernel pays 6 us at n = 512 alone and 14 us for the eight
+// matrices of a conv stack, its barrier in global memory and the L2 round trips.
 #include <cooperative_groups.h>
 
 #include "glr_internal.cuh"
@@ -254,6 +255,9 @@ size_t cluster_smem(int n) {
 // CTA holds the H rows of S consecutive slots, in two rings of row buffers with a spare each, so
 // that only one T and one B row a round go to a neighbour's spare, written there in place of the
 // row itself.  A row pair's 2 x 2 blocks are then one thread's and are updated in place.
+// JU: the rotations a lane looks at (n <= 64 JU), whose indices it carries from round to round; ODD: n odd
+// (index n of the padded problem has no column).
+template <int JU, bool ODD>
 __global__ void __launch_bounds__(CT, 1) jacobi_cluster_kernel(const __grid_constant__ JacobiMat M, int max_sweeps) {
     extern __shared__ __align__(16) float csm[];
     __shared__ float red[2][CT / 32], part[2];
@@ -288,7 +292,13 @@ __global__ void __launch_bounds__(CT, 1) jacobi_cluster_kernel(const __grid_cons
     cluster_sync();
     // the columns' rotations in this thread's share of the work: warps share a slot when there are few
     const int G = S > 8 ? 1 : S > 4 ? 2 : S > 2 ? 4 : S > 1 ? 8 : 16;
-    const int myslot = warp / G, sub = warp % G, JU = (half + 31) / 32;
+    int jx[JU], jy[JU];                                                     // T, B of slot lane + 32 u in this round
+#pragma unroll
+    for (int u = 0; u < JU; ++u) {
+        const int j = lane + 32 * u < half ? lane + 32 * u : 0;
+        jx[u] = tidx(j, 0);
+        jy[u] = bidx(j, 0);
+    }
     int sweep = 0;
     for (;; ++sweep) {
         float off = 0.f, tot = 0.f;
@@ -323,7 +333,7 @@ __global__ void __launch_bounds__(CT, 1) jacobi_cluster_kernel(const __grid_cons
                 const int i = e % S, to = e / S, x = tidx(s0 + i, rd), y = bidx(s0 + i, rd);
                 const int p = x < y ? x : y, q = x < y ? y : x;
                 float c = 1.f, s = 0.f;
-                if (q < n) {
+                if (!ODD || q < n) {
                     const float* rp = x < y ? trow(i) : brow(i);
                     const float* rq = x < y ? brow(i) : trow(i);
                     const float hpq = rp[q], hpp = rp[p], hqq = rq[q];
@@ -339,13 +349,18 @@ __global__ void __launch_bounds__(CT, 1) jacobi_cluster_kernel(const __grid_cons
                 peer(cs, to)[s0 + i] = make_float2(c, s);
             }
             cluster_sync();
-            // own row pair: its rows, and where each goes
-            const float *hp = nullptr, *hq = nullptr;
-            float *op = nullptr, *oq = nullptr;
-            float2 ri = make_float2(1.f, 0.f);
-            const bool mine = myslot < S;
-            if (mine) {
-                const int i = myslot, slot = s0 + i;
+            int pj[JU], qj[JU];
+            float2 rj[JU];
+#pragma unroll
+            for (int u = 0; u < JU; ++u) {
+                pj[u] = jx[u] < jy[u] ? jx[u] : jy[u];
+                qj[u] = jx[u] < jy[u] ? jy[u] : jx[u];
+                rj[u] = cs[lane + 32 * u < half ? lane + 32 * u : 0];
+                jx[u] = jx[u] == 0 ? 0 : jx[u] == nm1 ? 1 : jx[u] + 1;
+                jy[u] = jy[u] == nm1 ? 1 : jy[u] + 1;
+            }
+            if (warp / G < S) {                                             // a row pair (S <= 16): its rows, and where each goes
+                const int i = warp / G, slot = s0 + i;
                 float *tr = trow(i), *br = brow(i), *to = tr, *bo = br;
                 if (slot > 0 && i == (b == 0 ? 1 : 0)) {                    // the first ring T leaves
                     if (b == 0) to = Br + (size_t)wrap(bb + S, LB) * n;
@@ -356,45 +371,39 @@ __global__ void __launch_bounds__(CT, 1) jacobi_cluster_kernel(const __grid_cons
                     else bo = peer(Br, b + 1) + (size_t)wrap(bbr + LBr - 1, LBr) * n;
                 }
                 const bool up = tidx(slot, rd) < bidx(slot, rd);
-                hp = up ? tr : br; hq = up ? br : tr;
-                op = up ? to : bo; oq = up ? bo : to;
-                ri = cs[slot];
-            }
-            for (int u = sub; u < JU; u += G) {
-                const int j = lane + 32 * u;
-                if (!mine || j >= half) continue;
-                const int x = tidx(j, rd), y = bidx(j, rd);
-                const int pj = x < y ? x : y, qj = x < y ? y : x;
-                const float2 rj = cs[j];
-                const bool vq = qj < n;
-                const float h00 = hp[pj], h10 = hq[pj], h01 = vq ? hp[qj] : 0.f, h11 = vq ? hq[qj] : 0.f;
-                const float a00 = rot_dif(ri.x, h00, ri.y, h10), a01 = rot_dif(ri.x, h01, ri.y, h11);
-                const float a10 = rot_sum(ri.y, h00, ri.x, h10), a11 = rot_sum(ri.y, h01, ri.x, h11);
-                const bool diag = j == s0 + myslot && ri.y != 0.f;
-                op[pj] = rot_dif(rj.x, a00, rj.y, a01);
-                oq[pj] = diag ? 0.f : rot_dif(rj.x, a10, rj.y, a11);
-                if (vq) {
-                    op[qj] = diag ? 0.f : rot_sum(rj.y, a00, rj.x, a01);
-                    oq[qj] = rot_sum(rj.y, a10, rj.x, a11);
+                const float *hp = up ? tr : br, *hq = up ? br : tr;
+                float *op = up ? to : bo, *oq = up ? bo : to;
+                const float2 ri = cs[slot];
+#pragma unroll
+                for (int u = 0; u < JU; ++u) {
+                    if ((G > 1 && (u % G) != warp % G) || lane + 32 * u >= half) continue;
+                    const bool vq = !ODD || qj[u] < n;
+                    const float h00 = hp[pj[u]], h10 = hq[pj[u]], h01 = vq ? hp[qj[u]] : 0.f, h11 = vq ? hq[qj[u]] : 0.f;
+                    const float a00 = rot_dif(ri.x, h00, ri.y, h10), a01 = rot_dif(ri.x, h01, ri.y, h11);
+                    const float a10 = rot_sum(ri.y, h00, ri.x, h10), a11 = rot_sum(ri.y, h01, ri.x, h11);
+                    const bool diag = lane + 32 * u == slot && ri.y != 0.f;
+                    op[pj[u]] = rot_dif(rj[u].x, a00, rj[u].y, a01);
+                    oq[pj[u]] = diag ? 0.f : rot_dif(rj[u].x, a10, rj[u].y, a11);
+                    if (vq) {
+                        op[qj[u]] = diag ? 0.f : rot_sum(rj[u].y, a00, rj[u].x, a01);
+                        oq[qj[u]] = rot_sum(rj[u].y, a10, rj[u].x, a11);
+                    }
                 }
             }
             cluster_arrive();
-            for (int r = warp; r < vrows; r += 2 * (CT / 32)) {              // V <- V J, in place, two rows at a time
-                float* w0 = V + (size_t)r * n;
-                const bool two = r + CT / 32 < vrows;
-                float* w1 = two ? w0 + (CT / 32) * n : w0;
-                for (int j = lane; j < half; j += 32) {
-                    const float2 rj = cs[j];
-                    if (rj.y == 0.f) continue;
-                    const int x = tidx(j, rd), y = bidx(j, rd);
-                    const int pj = x < y ? x : y, qj = x < y ? y : x;
-                    const float x0 = w0[pj], y0 = w0[qj], x1 = w1[pj], y1 = w1[qj];
-                    w0[pj] = rot_dif(rj.x, x0, rj.y, y0);
-                    w0[qj] = rot_sum(rj.y, x0, rj.x, y0);
-                    if (two) {
-                        w1[pj] = rot_dif(rj.x, x1, rj.y, y1);
-                        w1[qj] = rot_sum(rj.y, x1, rj.x, y1);
-                    }
+            for (int r = warp; r < vrows; r += CT / 32) {                    // V <- V J, in place
+                float* w = V + (size_t)r * n;
+                float v[JU][2];
+#pragma unroll
+                for (int u = 0; u < JU; ++u) {
+                    v[u][0] = w[pj[u]];
+                    v[u][1] = !ODD || qj[u] < n ? w[qj[u]] : 0.f;
+                }
+#pragma unroll
+                for (int u = 0; u < JU; ++u) {
+                    if (lane + 32 * u >= half) continue;
+                    w[pj[u]] = rot_dif(rj[u].x, v[u][0], rj[u].y, v[u][1]);
+                    if (!ODD || qj[u] < n) w[qj[u]] = rot_sum(rj[u].y, v[u][0], rj[u].x, v[u][1]);
                 }
             }
             cluster_wait();
@@ -413,6 +422,13 @@ __global__ void __launch_bounds__(CT, 1) jacobi_cluster_kernel(const __grid_cons
     if (b == 0 && t == 0 && M.sweeps) *M.sweeps = sweep;
 }
 
+using ClusterKernel = void (*)(const JacobiMat, int);
+template <bool ODD> ClusterKernel cluster_kernel_of(int n) {
+    return n <= 64 ? jacobi_cluster_kernel<1, ODD> : n <= 128 ? jacobi_cluster_kernel<2, ODD>
+           : n <= 256 ? jacobi_cluster_kernel<4, ODD> : jacobi_cluster_kernel<8, ODD>;
+}
+ClusterKernel cluster_kernel(int n) { return n & 1 ? cluster_kernel_of<true>(n) : cluster_kernel_of<false>(n); }
+
 cudaLaunchConfig_t cluster_config(int n, cudaLaunchAttribute* attr, cudaStream_t st) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(cluster_ctas(n));
@@ -427,8 +443,8 @@ cudaLaunchConfig_t cluster_config(int n, cudaLaunchAttribute* attr, cudaStream_t
 }
 
 // per device: set on every call (cheap next to the launch)
-cudaError_t cluster_attributes() {
-    const void* k = reinterpret_cast<const void*>(jacobi_cluster_kernel);
+cudaError_t cluster_attributes(int n) {
+    const void* k = reinterpret_cast<const void*>(cluster_kernel(n));
     const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem(512));
     return e != cudaSuccess ? e : cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }
@@ -440,8 +456,8 @@ bool jacobi_cluster_ok(int n) {
     cudaLaunchAttribute attr{};
     const cudaLaunchConfig_t cfg = cluster_config(n, &attr, nullptr);
     int clusters = 0;
-    if (cluster_attributes() != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&clusters, reinterpret_cast<const void*>(jacobi_cluster_kernel), &cfg) != cudaSuccess) {
+    if (cluster_attributes(n) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&clusters, reinterpret_cast<const void*>(cluster_kernel(n)), &cfg) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -450,11 +466,11 @@ bool jacobi_cluster_ok(int n) {
 
 cudaError_t jacobi_cluster(const JacobiMat& M, int max_sweeps, cudaStream_t st) {
     if (M.n < 1 || M.n > 512) return cudaErrorInvalidValue;
-    const cudaError_t e = cluster_attributes();
+    const cudaError_t e = cluster_attributes(M.n);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr{};
     const cudaLaunchConfig_t cfg = cluster_config(M.n, &attr, st);
-    return cudaLaunchKernelEx(&cfg, jacobi_cluster_kernel, M, max_sweeps);
+    return cudaLaunchKernelEx(&cfg, cluster_kernel(M.n), M, max_sweeps);
 }
 
 int jacobi_group_grid() {

@@ -289,7 +289,7 @@ constexpr int TCH = 1024;              // threads of pow_chol_kernel
 template <int KM>
 __global__ void __launch_bounds__(TCH) pow_chol_kernel(const __grid_constant__ PowGroup g, int use_t_tiles, int mode) {
     __shared__ float Gs[KM][KM + 1];
-    __shared__ float Ls[KM][KM + 1];
+    __shared__ float Ls[2 * KM][KM + 1];                       // rows past k: read for values nobody uses
     __shared__ float Xi[KM][KM + 1];                           // L^{-1}, column c by lane c
     __shared__ double Gq[4][KM * KM];
     const PowMat& M = g.mat[blockIdx.x];
@@ -303,6 +303,7 @@ __global__ void __launch_bounds__(TCH) pow_chol_kernel(const __grid_constant__ P
         const float* p = M.G + a * KM + b;
         double s0 = 0.0, s1 = 0.0;
         int t = j;
+#pragma unroll 4
         for (; t + 4 < nt; t += 8) {
             s0 += static_cast<double>(p[(int64_t)t * KM * KM]);
             s1 += static_cast<double>(p[(int64_t)(t + 4) * KM * KM]);
@@ -324,32 +325,35 @@ __global__ void __launch_bounds__(TCH) pow_chol_kernel(const __grid_constant__ P
     if (lane == 0 && M.flag && (!(tr > 0.f) || !isfinite(tr))) atomicAdd(M.flag + 6, 1);   // degenerate block
     float shift = 0.f;
     for (int attempt = 0; attempt < 6; ++attempt) {
-        for (int o = lane; o < k * k; o += 32) Ls[o / k][o % k] = Gs[o / k][o % k] + (o / k == o % k ? shift : 0.f);
-        __syncwarp();
+        // right-looking factor with lane = row: the row's entries in registers, moved down by one a column,
+        // so that every column runs the same few instructions; a row past k stays zero
+        float a[KM];
+#pragma unroll
+        for (int c = 0; c < KM; ++c) a[c] = lane < k && c < k ? Gs[lane < KM ? lane : 0][c] + (lane == c ? shift : 0.f) : 0.f;
         bool ok = true;
-        for (int j = 0; j < k && ok; ++j) {                    // right-looking, column j
-            const float d = Ls[j][j];
+#pragma unroll 1
+        for (int j = 0; j < k && ok; ++j) {
+            const float d = __shfl_sync(0xffffffffu, a[0], j);
             ok = d > 0.f;                                      // same value in every lane
-            if (ok) {
-                const float ljj = sqrtf(d);
-                __syncwarp();
-                for (int i = j + lane; i < k; i += 32) Ls[i][j] = i == j ? ljj : Ls[i][j] / ljj;
-                __syncwarp();
-                const int w = k - j - 1;
-                for (int o = lane; o < w * w; o += 32) {
-                    const int i = j + 1 + o / w, l = j + 1 + o % w;
-                    if (l <= i) Ls[i][l] -= Ls[i][j] * Ls[l][j];
-                }
-                __syncwarp();
-            }
+            const float ljj = sqrtf(d);
+            const float v = lane == j ? ljj : lane > j ? a[0] / ljj : 0.f;
+#pragma unroll
+            for (int q = 1; q < KM; ++q) a[q - 1] = fmaf(-v, __shfl_sync(0xffffffffu, v, (j + q) & 31), a[q]);
+            a[KM - 1] = 0.f;
+            if (lane < KM) Ls[lane][j] = v;
         }
         if (ok) {
-            if (lane < k) {                                    // column c = lane of L^{-1}
-                const int c = lane;
-                for (int i = 0; i < k; ++i) {
-                    float v = i == c ? 1.f : 0.f;
-                    for (int l = c; l < i; ++l) v -= Ls[i][l] * Xi[l][c];
-                    Xi[i][c] = i < c ? 0.f : v / Ls[i][i];
+            __syncwarp();
+            // column c = lane of L^{-1}, by substitution along the columns of L (the same sums, row by row)
+            if (lane < KM) {
+#pragma unroll
+                for (int i = 0; i < KM; ++i) a[i] = i == lane ? 1.f : 0.f;
+#pragma unroll 1
+                for (int l = 0; l < k; ++l) {
+                    const float x = a[0] / Ls[l][l];
+#pragma unroll
+                    for (int q = 1; q < KM; ++q) a[q - 1] = fmaf(-x, Ls[l + q][l], a[q]);
+                    Xi[l][lane] = x;
                 }
             }
             __syncwarp();
