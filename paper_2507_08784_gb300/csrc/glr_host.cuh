@@ -63,6 +63,7 @@ struct glr_handle {
     // refresh scratch of the tcgen05 path (not checkpointed): Mbar row-major and its TF32 low parts,
     // TF32 transposes of Q and Z, Gram partials, L^{-1}
     float *Mrow = nullptr, *Mlo = nullptr, *QTt = nullptr, *ZTt = nullptr, *gpart = nullptr, *Linv = nullptr;
+    float* pow_ws = nullptr;                      // the power-iteration products' K slices
     float* Qbuf0 = nullptr;                       // Q's first allocation (Q and Qn trade places)
     // the full basis on the tcgen05 path (m' > 1024): U^T rounded to TF32 (the score operand, part
     // of the state), and the blocked Jacobi's scratch (not checkpointed): the second V buffer, the

@@ -529,8 +529,11 @@ struct TcMat {
     // refresh products (PowT, PowN, Gram, Apply): a second A operand (PowN split), the rows of the
     // operand they stream, their outputs (fp32, leading dimension ld_out) and TF32 transposes
     const CUtensorMap* mA2;
-    int rows, ld_out, split, chunk;
+    int rows, ld_out, split;
     float* out; float* outT;
+    // Pow: K in `splits` slices of `chunk` 32-element steps; their partials, splits x rows x kpad
+    int splits, chunk;
+    float* pws;
     float* MbarRow;                                   // Compose on a refresh step: Mbar row-major too
     // BjacMul (the blocked Jacobi's rotations): the second B operand (B's TF32 low parts; mA2 holds
     // A's), the output mode and the tournament round, the output's low parts
@@ -553,6 +556,8 @@ cudaError_t launch_compose(TcGroup& g, cudaStream_t st);
 cudaError_t launch_wbar(TcGroup& g, cudaStream_t st);
 cudaError_t launch_lambda(TcGroup& g, cudaStream_t st);
 cudaError_t launch_lambda_u(TcGroup& g, cudaStream_t st);   // full basis: the scores from U^T Mbar
+// Slices of a power-iteration product over kdim with k columns, and the 32-element steps of each.
+int pow_splits(int kdim, int k, int* chunk);
 // The blocked Jacobi's rotations in the split TF32 form (k_tc.cu, BjacMul; modes in k_tc.cu)
 cudaError_t launch_bjac(TcGroup& g, cudaStream_t st);
 cudaError_t launch_pbuild(TcGroup& g, cudaStream_t st);

@@ -301,8 +301,8 @@ int fp32_products(std::vector<glr_handle*>& hs, cudaStream_t st, Fill fill) {
 // tensor maps over them; bjac_prep has set H, H_lo, V = I, V_lo = 0.  The problems of one size run
 // together, one sweep at a time, each sweep opened by the norm check (per-CTA partials summed on
 // the host in a fixed order, so that the decision does not depend on the grouping); a round is the
-// pair sweeps (J_k^T and its low part), then the three split-TF32 products of tc_kernel<BjacMul>:
-// T^T = (H J)^T, H <- T^T J, V' <- V J.  A problem that has not converged after kBjacMaxSweeps
+// pair sweeps (J_k^T and its low part), then the three split-TF32 products of tc_kernel<BjacMul> in
+// two launches: T^T = (H J)^T and V' <- V J, then H <- T^T J.  A problem that has not converged after kBjacMaxSweeps
 // sweeps keeps its last V and counts a numeric failure (GLR_ENUMERIC from glr_get_stats).
 constexpr int kBjacMaxSweeps = 30;
 
@@ -361,31 +361,35 @@ int bjac_run(std::vector<BjItem>& all, glr_handle* h0, cudaStream_t s0) {
                     }
                     GLR_LAUNCH(h0, 1, bjac_pairs(g, round == 0, s0));
                 }
-                for (int mode = 0; mode < 3; ++mode) {
-                    for (size_t c0 = 0; c0 < act.size(); c0 += tc::kTcGroupMax) {
+                // T^T and V' in one launch (both need only J), then H
+                for (int pass = 0; pass < 2; ++pass) {
+                    constexpr size_t kEach = tc::kTcGroupMax / 2;
+                    for (size_t c0 = 0; c0 < act.size(); c0 += kEach) {
                         tg.nmat = 0; tg.total_tiles = 0; tg.err = h0->dflags + 2;
-                        for (size_t c = c0; c < act.size() && c < c0 + tc::kTcGroupMax; ++c) {
-                            const BjItem* S = act[c];
-                            glr_handle* h = S->h;
-                            tc::TcMat M{};
-                            M.mp = n; M.ntiles = P * P; M.tile0 = tg.total_tiles; M.bjmode = mode; M.bjround = S->rd;
-                            const int vin = S->vpar ? kMapBjV1 : kMapBjV0;
-                            if (mode == 0) {
-                                M.mA = tcl_map(h, kMapBjH); M.mA2 = tcl_map(h, kMapBjHlo);
-                                M.mB = tcl_map(h, kMapBjJ); M.mB2 = tcl_map(h, kMapBjJlo);
-                                M.out = h->jwork; M.out_lo = h->Ttlo;
-                            } else if (mode == 1) {
-                                M.mA = tcl_map(h, kMapBjT); M.mA2 = tcl_map(h, kMapBjTlo);
-                                M.mB = tcl_map(h, kMapBjJ); M.mB2 = tcl_map(h, kMapBjJlo);
-                                M.out = h->Hbuf; M.out_lo = h->Hlo;
-                            } else {
-                                M.mA = tcl_map(h, kMapBjJ); M.mA2 = tcl_map(h, kMapBjJlo);
-                                M.mB = tcl_map(h, vin); M.mB2 = tcl_map(h, vin + 1);
-                                M.out = S->vpar ? h->Vbuf : h->Vbuf2; M.out_lo = S->vpar ? h->Vlo : h->V2lo;
+                        for (int mode = pass ? 1 : 2; mode >= 0; mode -= 2)
+                            for (size_t c = c0; c < act.size() && c < c0 + kEach; ++c) {
+                                const BjItem* S = act[c];
+                                glr_handle* h = S->h;
+                                tc::TcMat M{};
+                                M.mp = n; M.ntiles = mode == 2 ? P * P : P * (P + 1) / 2;
+                                M.tile0 = tg.total_tiles; M.bjmode = mode; M.bjround = S->rd;
+                                const int vin = S->vpar ? kMapBjV1 : kMapBjV0;
+                                if (mode == 0) {
+                                    M.mA = tcl_map(h, kMapBjH); M.mA2 = tcl_map(h, kMapBjHlo);
+                                    M.mB = tcl_map(h, kMapBjJ); M.mB2 = tcl_map(h, kMapBjJlo);
+                                    M.out = h->jwork; M.out_lo = h->Ttlo;
+                                } else if (mode == 1) {
+                                    M.mA = tcl_map(h, kMapBjT); M.mA2 = tcl_map(h, kMapBjTlo);
+                                    M.mB = tcl_map(h, kMapBjJ); M.mB2 = tcl_map(h, kMapBjJlo);
+                                    M.out = h->Hbuf; M.out_lo = h->Hlo;
+                                } else {
+                                    M.mA = tcl_map(h, kMapBjJ); M.mA2 = tcl_map(h, kMapBjJlo);
+                                    M.mB = tcl_map(h, vin); M.mB2 = tcl_map(h, vin + 1);
+                                    M.out = S->vpar ? h->Vbuf : h->Vbuf2; M.out_lo = S->vpar ? h->Vlo : h->V2lo;
+                                }
+                                tg.total_tiles += M.ntiles;
+                                tg.mat[tg.nmat++] = M;
                             }
-                            tg.total_tiles += M.ntiles;
-                            tg.mat[tg.nmat++] = M;
-                        }
                         GLR_LAUNCH(h0, 1, tc::launch_bjac(tg, s0));
                     }
                 }
@@ -564,6 +568,13 @@ int refresh_op(std::vector<glr_handle*>& hs, cudaError_t (*launch)(tc::TcGroup&,
 
 int cdiv(int a, int b) { return (a + b - 1) / b; }
 
+// Z = Mbar^T Q (and Z^T).
+void pow_t(glr_handle* h, tc::TcMat& M) {
+    M.rows = h->np; M.mA = tcl_map(h, kMapMbarT); M.mB = tcl_map(h, kMapQTtB);
+    M.out = h->Z; M.outT = h->ZTt; M.ld_out = h->k; M.pws = h->pow_ws;
+    M.splits = tc::pow_splits(h->mp, h->k, &M.chunk); M.ntiles = cdiv(h->np, 256) * M.splits;
+}
+
 // X^T X (Gram partials over row chunks), its factor L^{-1}, then X <- X L^{-T} (and X^T): the
 // CholeskyQR of X = Z (n' rows) or Q (m' rows) in TF32 products.
 int cholqr_tc(std::vector<glr_handle*>& hs, bool zside, cudaStream_t st, const std::vector<int>& active) {
@@ -629,8 +640,7 @@ int refresh_tcl_grouped(std::vector<glr_handle*>& hs) {
         // Z = Mbar^T Q
         rc = refresh_op(hs, tc::launch_powt, s0, [&](glr_handle* h, tc::TcMat& M) {
             if (!is_active(h)) return false;
-            M.rows = h->np; M.mA = tcl_map(h, kMapMbarT); M.mB = tcl_map(h, kMapQTtB);
-            M.out = h->Z; M.outT = h->ZTt; M.ld_out = h->k; M.ntiles = cdiv(h->np, 256);
+            pow_t(h, M);
             return true;
         });
         if (rc != GLR_OK) return rc;
@@ -646,7 +656,8 @@ int refresh_tcl_grouped(std::vector<glr_handle*>& hs) {
             if (!is_active(h)) return false;
             M.rows = h->mp; M.mA = tcl_map(h, kMapMrow); M.mA2 = tcl_map(h, kMapMlo); M.mB = tcl_map(h, kMapZTtB);
             M.split = it == h->s.power_iters - 1 ? 1 : 0;
-            M.out = h->Q; M.outT = h->QTt; M.ld_out = h->k; M.ntiles = cdiv(h->mp, 256);
+            M.out = h->Q; M.outT = h->QTt; M.ld_out = h->k; M.pws = h->pow_ws;
+            M.splits = tc::pow_splits(h->np, h->k, &M.chunk); M.ntiles = cdiv(h->mp, 256) * M.splits;
             return true;
         });
         if (rc != GLR_OK) return rc;
@@ -687,8 +698,7 @@ int refresh_tcl_grouped(std::vector<glr_handle*>& hs) {
     }
     // Rayleigh-Ritz: Z = Mbar^T Q, H = Z^T Z (Gram partials), the eigenproblems
     rc = refresh_op(hs, tc::launch_powt, s0, [&](glr_handle* h, tc::TcMat& M) {
-        M.rows = h->np; M.mA = tcl_map(h, kMapMbarT); M.mB = tcl_map(h, kMapQTtB);
-        M.out = h->Z; M.outT = h->ZTt; M.ld_out = h->k; M.ntiles = cdiv(h->np, 256);
+        pow_t(h, M);
         return true;
     });
     if (rc != GLR_OK) return rc;

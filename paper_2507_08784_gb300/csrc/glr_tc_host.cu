@@ -74,6 +74,8 @@ int tcl_maps(glr_handle* h) {
             A(&h->Mrow, mp * np); A(&h->Mlo, mp * np);
             A(&h->QTt, kp * mp); A(&h->ZTt, kp * np);
             A(&h->gpart, std::max<size_t>(nch, 1) * kp * kp); A(&h->Linv, kp * kp);
+            int chunk;
+            A(&h->pow_ws, kp * std::max(np * tc::pow_splits((int)mp, (int)k, &chunk), mp * tc::pow_splits((int)np, (int)k, &chunk)));
         }
         if (rc != GLR_OK) return rc;
     }

@@ -12,9 +12,10 @@
 //      a sweep's first round over the indices inside each block too), so that J_k stays close to
 //      the identity and no reordering inside the pair is needed;
 //   2. applies the block-diagonal J = diag(J_k) on the tensor cores (tc_kernel<BjacMul>, k_tc.cu,
-//      split TF32: A B + A_lo B + A B_lo): T^T = (H J)^T, then H <- T^T J = J^T H J (H symmetric)
-//      and V <- V J, the last two writing every 64-block straight to its place in the next
-//      round's storage order;
+//      split TF32: A B + A_lo B + A B_lo): T^T = (H J)^T, then H <- T^T J = J^T H J and V <- V J, the
+//      last two writing every 64-block straight to its place in the next round's storage order.
+//      H is symmetric: after the first round only its 128 x 128 blocks on and below the diagonal
+//      hold values;
 // and a sweep ends with the off-diagonal norm, checked on the host against tol^2 of the total.
 // V starts as the identity, so its columns follow H's storage order; at the end diag(H) and V
 // orthogonalised once more in fp32 and sorted by descending eigenvalue with the sign rule of the small solvers (sort_group).
@@ -27,16 +28,19 @@ namespace glr {
 
 namespace {
 
-// Per matrix, per CTA: the squared diagonal and off-diagonal sums of H (part[2 (mat G + cta)]).
+// Per matrix, per CTA: the squared diagonal and off-diagonal sums of H (part[2 (mat G + cta)]), from its
+// 128 x 128 blocks on and below the diagonal.
 __global__ void __launch_bounds__(256) bjac_norms_kernel(const __grid_constant__ BjacGroup g, float* part) {
     const BjacMat& M = g.mat[blockIdx.y];
     const int n = M.n;
     float d = 0.f, o = 0.f;
     for (int r = blockIdx.x; r < n; r += gridDim.x) {
         const float* row = M.H + (int64_t)r * n;
-        for (int c = threadIdx.x; c < n; c += 256) {
+        const int c0 = r & ~127;
+        for (int c = threadIdx.x; c < c0 + 128; c += 256) {
             const float v = row[c];
-            if (c == r) d += v * v; else o += v * v;
+            if (c == r) d += v * v;
+            else o += (c < c0 ? 2.f : 1.f) * (v * v);
         }
     }
     __shared__ float red[2][8];

@@ -699,22 +699,34 @@ struct LambdaU : NoData {
 // ------------------------------------------------------------------------------------------
 // BjacMul (the blocked Jacobi of the full-basis refresh, k_bjac.cu): Y = X J_l over the 128
 // columns of pair l, as three products per K slice (A B + A_lo B + A B_lo: the split TF32 form,
-// about as accurate as fp32 FFMA); tile = (128-row block rt, pair l), K = 128.  Modes:
-//   0: A = H rows, B = J_l^T:    D(i, c) = (H J)(i, 128 l + c), written to T^T (row 128 l + c)
-//   1: A = T^T rows, B = J_l^T:  D(r, c) = (T^T J)(r, 128 l + c) = (J^T H J)(r, 128 l + c),
-//      written transposed (the matrix is symmetric) at the next round's rows and columns
+// about as accurate as fp32 FFMA); tile = (128-row block rt, pair l), K = 128.  Of H (symmetric) only
+// the 128 x 128 blocks on and below the diagonal are kept, so modes 0 and 1 have half the tiles (n =
+// 2048: one wave of 136 instead of two).  Modes:
+//   0: A = H rows, B = J_l^T:    D(i, c) = (H J)(i, 128 l + c), rt >= l, written to T^T (row 128 l + c)
+//   1: A = T^T rows, B = J_l^T:  D(r, c) = (T^T J)(r, 128 l + c) = (J^T H J)(r, 128 l + c), rt <= l,
+//      written at the next round's rows and columns, each 64 x 64 piece on the side of the diagonal
+//      that is kept there (both sides where it meets a diagonal block)
 //   2: A = J_l^T, B = V rows:    D(c, r) = (V J)(r, 128 l + c), written to V' at row r and the
 //      next round's column of 128 l + c
-// With these orientations a warp's stores are 128 contiguous bytes.  Each output goes out with
-// its TF32 low part x - trunc_tf32(x), the next product's second operand.
+// Each output goes out with its TF32 low part x - trunc_tf32(x), the next product's second operand.
 // ------------------------------------------------------------------------------------------
 struct BjacMul : NoData {
     static constexpr int kEpi = 16;
     static __device__ __forceinline__ int nk(const TcGroup&, const Tile&) { return 4; }
     static __device__ __forceinline__ uint32_t tx_bytes(const TcGroup&, const Tile&, int) { return 4u * 16384u; }
+    static __device__ __forceinline__ void decode(const TcMat& M, int lt, int& rt, int& l) {
+        if (M.bjmode == 2) { rt = lt / (M.mp / 128); l = lt % (M.mp / 128); return; }
+        int hi = (int)((sqrtf(8.f * lt + 1.f) - 1.f) * 0.5f);               // lt = hi (hi + 1) / 2 + lo, lo <= hi
+        while (hi * (hi + 1) / 2 > lt) --hi;
+        while ((hi + 1) * (hi + 2) / 2 <= lt) ++hi;
+        const int lo = lt - hi * (hi + 1) / 2;
+        rt = M.bjmode == 0 ? hi : lo;
+        l = M.bjmode == 0 ? lo : hi;
+    }
     static __device__ __forceinline__ void load(const TcGroup& g, const Tile& t, int kc, uint32_t st, uint32_t bar) {
         const TcMat& M = g.mat[t.mat];
-        const int P = M.mp / 128, rt = t.lt / P, l = t.lt % P;
+        int rt, l;
+        decode(M, t.lt, rt, l);
         int ax, ay, bx, by;
         if (M.bjmode < 2) { ax = 128 * l + 32 * kc; ay = 128 * rt; bx = 32 * kc; by = 128 * l; }
         else { ax = 32 * kc; ay = 128 * l; bx = 128 * l + 32 * kc; by = 128 * rt; }
@@ -728,34 +740,45 @@ struct BjacMul : NoData {
         mma_slice(d, st + 16384u, st + 32768u, 128, false);    // A_lo B
         mma_slice(d, st, st + 49152u, 128, false);             // A B_lo
     }
+    static __device__ __forceinline__ float low_part(float v) { return v - __uint_as_float(__float_as_uint(v) & 0xffffe000u); }
     static __device__ __forceinline__ int dest(int x, int m, int rd) {
         return 64 * bjac_dest_of(x >> 6, m, rd) + (x & 63);
     }
     static __device__ __forceinline__ bool epilogue(const TcGroup& g, const Tile& t, uint32_t tl, int warp, int lane,
                                                     DataRing&) {
         const TcMat& M = g.mat[t.mat];
-        const int n = M.mp, P = n / 128, m = n / 64, rt = t.lt / P, l = t.lt % P;
-        const int row = 32 * (warp & 3) + lane, h = warp >> 2;
-        // per-thread parts of the output index: a stride for the tile's columns, a fixed offset;
-        // mode 1: a warp's 32 columns lie in one 64-block, whose next place is found once
-        int64_t base = 0, step = 0;
-        if (M.bjmode == 0) { base = (int64_t)(128 * l) * n + 128 * rt + row; step = n; }
-        else if (M.bjmode == 1) {
-            const int x0 = 128 * l + 32 * h;
-            base = (int64_t)(64 * bjac_dest_of(x0 >> 6, m, M.bjround) + (x0 & 63)) * n + dest(128 * rt + row, m, M.bjround);
-            step = n;
-        } else { base = dest(128 * l + row, m, M.bjround); step = n; }
+        const int n = M.mp, m = n / 64, row = 32 * (warp & 3) + lane, h = warp >> 2;
+        int rt, l;
+        decode(M, t.lt, rt, l);
+        // this thread's row and its warp's 32 columns: the row's stride-1 place and the columns', one of
+        // which is the storage row
+        int64_t normal = -1, turned = -1;                     // element (row, col): [row][col] / [col][row]
+        if (M.bjmode == 0) turned = (int64_t)(128 * l + 32 * h) * n + 128 * rt + row;
+        else if (M.bjmode == 2) turned = (int64_t)(128 * rt + 32 * h) * n + dest(128 * l + row, m, M.bjround);
+        else {
+            const int dr = dest(128 * rt + row, m, M.bjround), dc = dest(128 * l + 32 * h, m, M.bjround);
+            const int pr = dr >> 7, pc = dc >> 7;             // (warp-uniform: 32 rows of one 64-block)
+            if (pr >= pc) normal = (int64_t)dr * n + dc;
+            if (rt != l && pr <= pc) turned = (int64_t)dc * n + dr;
+        }
         for (int cc = 0; cc < 32; cc += 16) {
             float d[16];
             tmem_ld16(tl + (uint32_t)(32 * h + cc), d);
+            if (turned >= 0) {
 #pragma unroll
-            for (int e = 0; e < 16; ++e) {
-                const int col = 32 * h + cc + e;
-                const int64_t a = M.bjmode == 2 ? base + (int64_t)(128 * rt + col) * step
-                                                : base + (int64_t)(cc + e + (M.bjmode == 0 ? 32 * h : 0)) * step;
-                const float v = d[e];
-                M.out[a] = v;
-                M.out_lo[a] = v - __uint_as_float(__float_as_uint(v) & 0xffffe000u);
+                for (int e = 0; e < 16; ++e) {
+                    const int64_t a = turned + (int64_t)(cc + e) * n;
+                    M.out[a] = d[e];
+                    M.out_lo[a] = low_part(d[e]);
+                }
+            }
+            if (normal >= 0) {
+#pragma unroll
+                for (int e = 0; e < 16; e += 4) {
+                    *reinterpret_cast<float4*>(M.out + normal + cc + e) = make_float4(d[e], d[e + 1], d[e + 2], d[e + 3]);
+                    *reinterpret_cast<float4*>(M.out_lo + normal + cc + e) =
+                        make_float4(low_part(d[e]), low_part(d[e + 1]), low_part(d[e + 2]), low_part(d[e + 3]));
+                }
             }
         }
         return true;
@@ -987,11 +1010,19 @@ struct Update {
 // exact to fp32 level for the TF32 value of B.  The epilogue writes out[row][q] (fp32, leading
 // dimension ld_out, q < k) and outT[q][row] (TF32).
 // ------------------------------------------------------------------------------------------
+// K is cut into `splits` slices of `chunk` 32-element steps (pow_splits, by the matrix's own sizes): a
+// 4096 x 11008 matrix alone has 16 tiles of 344 steps for 152 SMs, each bound by what one SM loads
+// (216 us).  The slices' fp32 partial products go to pws and are added in order by
+// pow_reduce_kernel, which writes out and outT.  At most one slice per 48 steps and per 16 k of K, so
+// that the partials stay below an eighth of the operand's bytes: with three slices of K = 4096 at k = 256
+// the seven matrices of a d = 4096 layer got slower (13.7 -> 14.0 ms), k = 128 gains (5.1 -> 4.4 ms).
 template <int kDir>
 struct Pow : NoData {
+    static __device__ __forceinline__ int steps(const TcMat& M) { return ((kDir == 0 ? M.mp : M.np) + 31) / 32; }
     static __device__ __forceinline__ int nk(const TcGroup& g, const Tile& t) {
         const TcMat& M = g.mat[t.mat];
-        return ((kDir == 0 ? M.mp : M.np) + 31) / 32;
+        const int k0 = (t.lt % M.splits) * M.chunk, left = steps(M) - k0;
+        return left < M.chunk ? left : M.chunk;
     }
     static __device__ __forceinline__ uint32_t tx_bytes(const TcGroup& g, const Tile& t, int) {
         const TcMat& M = g.mat[t.mat];
@@ -999,15 +1030,16 @@ struct Pow : NoData {
     }
     static __device__ __forceinline__ void load(const TcGroup& g, const Tile& t, int kc, uint32_t st, uint32_t bar) {
         const TcMat& M = g.mat[t.mat];
-        tma_load_2d(st, M.mA, kc * 32, t.lt * 256, bar);
-        tma_load_2d(st + 16384u, M.mA, kc * 32, t.lt * 256 + 128, bar);
+        const int x = ((t.lt % M.splits) * M.chunk + kc) * 32, y = t.lt / M.splits * 256;
+        tma_load_2d(st, M.mA, x, y, bar);
+        tma_load_2d(st + 16384u, M.mA, x, y + 128, bar);
         uint32_t o = 32768u;
         if (M.split) {
-            tma_load_2d(st + o, M.mA2, kc * 32, t.lt * 256, bar);
-            tma_load_2d(st + o + 16384u, M.mA2, kc * 32, t.lt * 256 + 128, bar);
+            tma_load_2d(st + o, M.mA2, x, y, bar);
+            tma_load_2d(st + o + 16384u, M.mA2, x, y + 128, bar);
             o += 32768u;
         }
-        tma_load_2d(st + o, M.mB, kc * 32, 0, bar);
+        tma_load_2d(st + o, M.mB, x, 0, bar);
     }
     static __device__ __forceinline__ void mma(const TcGroup& g, const Tile& t, int kc, uint32_t st, uint32_t d) {
         const TcMat& M = g.mat[t.mat];
@@ -1022,11 +1054,18 @@ struct Pow : NoData {
     static __device__ __forceinline__ bool epilogue(const TcGroup& g, const Tile& t, uint32_t tl, int warp, int lane, DataRing&) {
         const TcMat& M = g.mat[t.mat];
         const int h = warp >> 2;
-        const int c = t.lt * 256 + h * 128 + 32 * (warp & 3) + lane;
+        const int c = t.lt / M.splits * 256 + h * 128 + 32 * (warp & 3) + lane;
+        float* part = M.splits > 1 ? M.pws + ((int64_t)(t.lt % M.splits) * M.rows + c) * M.kpad : nullptr;
         for (int q = 0; q < M.kpad; q += 16) {
             float v[16];
             tmem_ld16(tl + (uint32_t)(h * M.kpad + q), v);
             if (c >= M.rows) continue;
+            if (part) {
+#pragma unroll
+                for (int j = 0; j < 16; j += 4)
+                    *reinterpret_cast<float4*>(part + q + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                continue;
+            }
 #pragma unroll
             for (int j = 0; j < 16; j += 4)
                 if (q + j < M.k)
@@ -1222,8 +1261,49 @@ cudaError_t launch_bjac(TcGroup& g, cudaStream_t st) { return launch<BjacMul>(g,
 cudaError_t launch_pbuild(TcGroup& g, cudaStream_t st) { return launch<PBuild>(g, st); }
 cudaError_t launch_rbar(TcGroup& g, cudaStream_t st) { return launch<RBar>(g, st); }
 cudaError_t launch_update(TcGroup& g, cudaStream_t st) { return launch<Update>(g, st); }
-cudaError_t launch_powt(TcGroup& g, cudaStream_t st) { return launch<PowT>(g, st); }
-cudaError_t launch_pown(TcGroup& g, cudaStream_t st) { return launch<PowN>(g, st); }
+namespace {
+// The K slices of Pow added in order: out (rows x k, fp32) and outT (kpad x rows, TF32).
+__global__ void __launch_bounds__(256) pow_reduce_kernel(const __grid_constant__ TcGroup g) {
+    __shared__ float tile[32][33];
+    const TcMat& M = g.mat[blockIdx.y];
+    const int r0 = blockIdx.x * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    if (M.splits <= 1 || r0 >= M.rows) return;
+    for (int q0 = 0; q0 < M.kpad; q0 += 32) {
+        __syncthreads();
+        for (int y = ty; y < 32; y += 8) {
+            float v = 0.f;
+            if (r0 + y < M.rows) {
+                const float* p = M.pws + (int64_t)(r0 + y) * M.kpad + q0 + tx;
+                for (int z = 0; z < M.splits; ++z) v += p[(int64_t)z * M.rows * M.kpad];
+                if (q0 + tx < M.k) M.out[(int64_t)(r0 + y) * M.ld_out + q0 + tx] = v;
+            }
+            tile[y][tx] = v;
+        }
+        __syncthreads();
+        for (int y = ty; y < 32; y += 8)
+            if (r0 + tx < M.rows) M.outT[(int64_t)(q0 + y) * M.rows + r0 + tx] = rna_tf32(tile[tx][y]);
+    }
+}
+template <class Op>
+cudaError_t launch_pow(TcGroup& g, cudaStream_t st) {
+    const cudaError_t e = launch<Op>(g, st);
+    int rows = 0;
+    for (int i = 0; i < g.nmat; ++i)
+        if (g.mat[i].splits > 1) rows = std::max(rows, g.mat[i].rows);
+    if (e != cudaSuccess || !rows) return e;
+    pow_reduce_kernel<<<dim3((rows + 31) / 32, g.nmat), 256, 0, st>>>(g);
+    return cudaGetLastError();
+}
+}  // namespace
+
+int pow_splits(int kdim, int k, int* chunk) {
+    const int steps = (kdim + 31) / 32, splits = std::max(1, std::min((steps + 47) / 48, kdim / (16 * k)));
+    *chunk = (steps + splits - 1) / splits;
+    return (steps + *chunk - 1) / *chunk;
+}
+
+cudaError_t launch_powt(TcGroup& g, cudaStream_t st) { return launch_pow<PowT>(g, st); }
+cudaError_t launch_pown(TcGroup& g, cudaStream_t st) { return launch_pow<PowN>(g, st); }
 cudaError_t launch_gram(TcGroup& g, cudaStream_t st) { return launch<Gram>(g, st); }
 cudaError_t launch_apply(TcGroup& g, cudaStream_t st) { return launch<Apply>(g, st); }
 
