@@ -313,13 +313,13 @@ struct EigMat {
     float* V; float* evals; int* sweeps; float* ws;
 };
 struct EigGroup {
-    int nmat, max_sweeps;
+    int nmat, max_sweeps, parts;            // parts: CTAs a pair, set by eig_group
     int* bar; int* err; float* part;
     EigMat mat[kEigGroupMax];
 };
 size_t eig_ws_floats(int n);
 cudaError_t eig_small_group(const EigGroup& g, cudaStream_t st);
-cudaError_t eig_group(const EigGroup& g, int busy_sms, cudaStream_t st);
+cudaError_t eig_group(EigGroup& g, int busy_sms, cudaStream_t st);
 
 // The blocked Jacobi's round-robin tournament over m blocks of 64 indices (circle method: block 0
 // fixed, the others one slot further each round; slots s and m - 1 - s pair up and are stored at

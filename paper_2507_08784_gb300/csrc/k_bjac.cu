@@ -64,42 +64,28 @@ __global__ void __launch_bounds__(256) bjac_norms_kernel(const __grid_constant__
 // block meet once a sweep too) all 127 rounds.  J_k^T is written row-major with its TF32 low part.
 // On the 2048 x 2048 problem the cross-only rounds take as many sweeps as 127 rounds in each pairing
 // do or one or two more, at half the work of a round.
+// Where the pairs leave most SMs idle (n = 2048: 16 pairs), four CTAs share one, each with a quarter
+// of W's rows (WR = 2): the same bits.
+template <int WR>
 __global__ void __launch_bounds__(pair::PTHREADS, 1) bjac_pair_kernel(const __grid_constant__ BjacGroup g, int full) {
     using namespace pair;
+    constexpr int PARTS = 8 / WR, ROWS = 16 * WR;
     extern __shared__ __align__(16) float psm[];
-    float* S = psm;
-    float* W = S + PN * PLD;
-    float* xch = W + PN * PLD;
-    float* apq = xch + 2 * 16 * 128;
+    const int tile = blockIdx.x / PARTS, w0 = blockIdx.x % PARTS * ROWS;
     int mi = 0;
-    while (mi + 1 < g.nmat && g.mat[mi + 1].tile0p <= (int)blockIdx.x) ++mi;
+    while (mi + 1 < g.nmat && g.mat[mi + 1].tile0p <= tile) ++mi;
     const BjacMat& M = g.mat[mi];
-    const int n = M.n, k = blockIdx.x - M.tile0p, t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const float* S0 = M.H + (int64_t)(PN * k) * (n + 1);
-    for (int e = t; e < PN * PN / 2; e += PTHREADS) {
-        const int r = e >> 6, c = 2 * (e & 63);
-        *reinterpret_cast<float2*>(S + r * PLD + c) = *reinterpret_cast<const float2*>(S0 + (int64_t)r * n + c);
-        *reinterpret_cast<float2*>(W + r * PLD + c) = make_float2(r == c ? 1.f : 0.f, r == c + 1 ? 1.f : 0.f);
-    }
-    __syncthreads();
-    Block b;
-    const int last = full ? 1 : 64;
-    for (int lv = 64;; lv >>= 1) {
-        b.load(S, W, lv, warp, lane);
-        b.level(S, lv, xch, apq, warp, lane);
-        __syncthreads();
-        if (lv == last) { b.storeW(W, lv, warp, lane); break; }
-        b.store(S, W, lv, warp, lane);
-        __syncthreads();
-    }
-    __syncthreads();
+    const int n = M.n, k = tile - M.tile0p;
+    const float* W = sweep<WR>(M.H + (int64_t)(PN * k) * (n + 1), n, w0, full, psm,
+                               [](const float* p) { return *reinterpret_cast<const float2*>(p); });
     // J_k^T (row c = column c of W) and its TF32 low part: the rotations' MMA operands
-    float* Jt = M.J + (int64_t)k * PN * PN;
-    float* Jl = M.Jlo + (int64_t)k * PN * PN;
-    for (int e = t; e < PN * PN; e += PTHREADS) {
-        const float v = W[(e & 127) * PLD + (e >> 7)];
-        Jt[e] = v;
-        Jl[e] = v - __uint_as_float(__float_as_uint(v) & 0xffffe000u);
+    float* Jt = M.J + (int64_t)k * PN * PN + w0;
+    float* Jl = M.Jlo + (int64_t)k * PN * PN + w0;
+    for (int e = threadIdx.x; e < PN * ROWS; e += PTHREADS) {
+        const int c = e / ROWS, r = e % ROWS;
+        const float v = W[r * PLD + c];
+        Jt[c * PN + r] = v;
+        Jl[c * PN + r] = v - __uint_as_float(__float_as_uint(v) & 0xffffe000u);
     }
 }
 
@@ -136,10 +122,17 @@ cudaError_t bjac_pairs(BjacGroup& g, int full, cudaStream_t st) {
         M.tile0p = tiles;
         tiles += M.n / 128;
     }
-    // per device: set on every call (cheap next to the launch)
-    cudaError_t e = cudaFuncSetAttribute(bjac_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair::kSmem);
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    bjac_pair_kernel<<<tiles, pair::PTHREADS, pair::kSmem, st>>>(g, full);
+    const bool parts = 4 * tiles <= sms;
+    // per device: set on every call (cheap next to the launch)
+    e = parts ? cudaFuncSetAttribute(bjac_pair_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair::kSmem)
+              : cudaFuncSetAttribute(bjac_pair_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair::kSmem);
+    if (e != cudaSuccess) return e;
+    if (parts) bjac_pair_kernel<2><<<4 * tiles, pair::PTHREADS, pair::kSmem, st>>>(g, full);
+    else bjac_pair_kernel<8><<<tiles, pair::PTHREADS, pair::kSmem, st>>>(g, full);
     return cudaGetLastError();
 }
 

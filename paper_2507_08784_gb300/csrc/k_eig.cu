@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(8 * LIM, 1) eig_small_kernel(const __grid_cons
         W[e] = r == c ? 1.f : 0.f;
     }
     __syncthreads();
-    Block b;
+    Block<8> b;
     int sweep = 0;
     for (;; ++sweep) {
         float off = 0.f, tot = 0.f;
@@ -270,36 +270,19 @@ struct Work {                       // the parts of a problem's workspace
     }
 };
 
-// J_k of pair k, row-major in J and transposed in Jt.
-__device__ void pair_job(const Work& w, const float* H, int k, int full, float* sm) {
-    float* S = sm;
-    float* W = S + PN * PLD;
-    float* xch = W + PN * PLD;
-    float* apq = xch + 2 * 16 * 128;
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const float* S0 = H + (int64_t)(PN * k) * (w.np + 1);
-    for (int e = t; e < PN * PN / 2; e += PTHREADS) {
-        const int r = e >> 6, c = 2 * (e & 63);
-        *reinterpret_cast<float2*>(S + r * PLD + c) = __ldcg(reinterpret_cast<const float2*>(S0 + (int64_t)r * w.np + c));
-        *reinterpret_cast<float2*>(W + r * PLD + c) = make_float2(r == c ? 1.f : 0.f, r == c + 1 ? 1.f : 0.f);
-    }
-    __syncthreads();
-    Block b;
-    const int last = full ? 1 : 64;
-    for (int lv = 64;; lv >>= 1) {
-        b.load(S, W, lv, warp, lane);
-        b.level(S, lv, xch, apq, warp, lane);
-        __syncthreads();
-        if (lv == last) { b.storeW(W, lv, warp, lane); break; }
-        b.store(S, W, lv, warp, lane);
-        __syncthreads();
-    }
-    __syncthreads();
+// J_k of pair k, row-major in J and transposed in Jt: all of it, or with WR = 2 the quarter `part` of
+// its rows.
+template <int WR>
+__device__ void pair_job(const Work& w, const float* H, int k, int part, int full, float* sm) {
+    constexpr int ROWS = 16 * WR;
+    const int w0 = part * ROWS;
+    const float* W = pair::sweep<WR>(H + (int64_t)(PN * k) * (w.np + 1), w.np, w0, full, sm,
+                                     [](const float* p) { return __ldcg(reinterpret_cast<const float2*>(p)); });
     float* J = w.J + (int64_t)k * PN * PN;
     float* Jt = w.Jt + (int64_t)k * PN * PN;
-    for (int e = t; e < PN * PN; e += PTHREADS) {
-        J[e] = W[(e >> 7) * PLD + (e & 127)];
-        Jt[e] = W[(e & 127) * PLD + (e >> 7)];
+    for (int e = threadIdx.x; e < PN * ROWS; e += PTHREADS) {
+        J[(w0 + e / PN) * PN + e % PN] = W[e / PN * PLD + e % PN];
+        Jt[e / ROWS * PN + w0 + e % ROWS] = W[e % ROWS * PLD + e / ROWS];
     }
     __syncthreads();
 }
@@ -518,8 +501,11 @@ __global__ void __launch_bounds__(PTHREADS, 1) eig_group_kernel(const __grid_con
                 }
                 item += kNormChunks;
             } else if (state == kPair) {
-                for (int k = (b - item % G + G) % G; k < w.P; k += G) pair_job(w, Hc, k, rd == 0, gsm);
-                item += w.P;
+                for (int k = (b - item % G + G) % G; k < w.P * g.parts; k += G) {
+                    if (g.parts == 4) pair_job<2>(w, Hc, k >> 2, k & 3, rd == 0, gsm);
+                    else pair_job<8>(w, Hc, k, 0, rd == 0, gsm);
+                }
+                item += w.P * g.parts;
             } else if (state == kApply) {
                 const int nh = w.P * (w.P + 1), nv = w.m * w.P;
                 float* Hn = sflip[mi] ? w.H0 : w.H1;
@@ -613,10 +599,13 @@ cudaError_t eig_small_group(const EigGroup& g, cudaStream_t st) {
     return cudaSuccess;
 }
 
-cudaError_t eig_group(const EigGroup& g, int busy_sms, cudaStream_t st) {
+cudaError_t eig_group(EigGroup& g, int busy_sms, cudaStream_t st) {
     if (g.nmat <= 0) return cudaSuccess;
-    for (int i = 0; i < g.nmat; ++i)
+    int pairs = 0;
+    for (int i = 0; i < g.nmat; ++i) {
         if (g.mat[i].n <= kEigSmall || g.mat[i].n > 1024 || !g.mat[i].ws) return cudaErrorInvalidValue;
+        pairs += pad128(g.mat[i].n) / 128;
+    }
     int dev = 0, sms = 0, coop = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -625,12 +614,13 @@ cudaError_t eig_group(const EigGroup& g, int busy_sms, cudaStream_t st) {
         e = cudaFuncSetAttribute(eig_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGroupSmem);
     if (e == cudaSuccess) e = cudaMemsetAsync(g.bar, 0, 2 * sizeof(int), st);    // arrivals and generation
     if (e != cudaSuccess) return e;
+    const int grid = busy_sms < sms / 2 ? sms - busy_sms : sms;
+    g.parts = 4 * pairs <= grid ? 4 : 1;      // four CTAs a pair where they are to spare (the same bits)
     if (!coop) {               // one CTA: the barriers wait for nobody
         eig_group_kernel<<<1, PTHREADS, kGroupSmem, st>>>(g);
         return cudaGetLastError();
     }
-    const int grid = busy_sms < sms / 2 ? sms - busy_sms : sms;
-    void* args[] = {const_cast<EigGroup*>(&g)};
+    void* args[] = {&g};
     return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(eig_group_kernel), dim3(grid), dim3(PTHREADS), args,
                                        kGroupSmem, st);
 }

@@ -10,7 +10,7 @@
 // B is kept in its rotated order, so a round always pairs position j of A with position j of B and
 // the 2 x 2 block of rotations i, j is (AA, AB, BA, BB)[i][j]: four values of one thread.  Warp w
 // holds rows 4 w .. + 3 of the four 64 x 64 quadrants and lane l columns 2 l and 2 l + 1 as packed
-// fp32 pairs (fma.rn.f32x2), and the eigenvector block W the same way (8 rows a warp).  After a
+// fp32 pairs (fma.rn.f32x2), and the eigenvector block W the same way (8 rows a warp, or 2).  After a
 // round B moves on by one position: columns by one shuffle per value pair, rows inside the warp's
 // registers with the last one from the next warp through shared memory (double-buffered, one
 // barrier a round).  Every warp forms all 64 rotations itself, two a lane, from the diagonal, which
@@ -18,8 +18,9 @@
 // pairs, which their owners publish with the boundary rows.  W trails the rotations by a round, so
 // that its updates fill the latency of the next rotations.
 //
-// Bound by instruction issue (16 warps, about 240 instructions a round, one CTA an SM); a sweep
-// that keeps S and W in shared memory and updates them through indices takes 2.4 us a round.
+// Bound by instruction issue (16 warps, 340 instructions each a round, 0.58 of the issue slots; 96
+// packed fmas at two cycles): 1.15 us a round.  A sweep that keeps S and W in shared memory and
+// updates them through indices takes 2.4 us a round.
 #pragma once
 
 #include "glr_internal.cuh"
@@ -67,8 +68,11 @@ __device__ __forceinline__ void rotation(float app, float aqq, float apq, float&
     s = t * c;
 }
 
+// WR: rows of W a warp (8: all 128 in this CTA; 2: a quarter of them, where four CTAs share a pair, each
+// with all of S: the rotations are the same in every one).
+template <int WR>
 struct Block {
-    u64 AA[4], AB[4], BA[4], BB[4], WA[8], WB[8];
+    u64 AA[4], AB[4], BA[4], BB[4], WA[WR], WB[WR];
 
     // Position j of half A / B at level g -> index in the block.
     static __device__ __forceinline__ int posA(int j, int g) { return 2 * (j & ~(g - 1)) + (j & (g - 1)); }
@@ -95,8 +99,8 @@ struct Block {
             BA[r] = row2(rb, a0, a1, v2); BB[r] = row2(rb, a0 + g, a1 + g, v2);
         }
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            const float* rw = W + (8 * warp + r) * PLD;
+        for (int r = 0; r < WR; ++r) {
+            const float* rw = W + (WR * warp + r) * PLD;
             WA[r] = row2(rw, a0, a1, v2); WB[r] = row2(rw, a0 + g, a1 + g, v2);
         }
     }
@@ -116,8 +120,8 @@ struct Block {
         const bool v2 = g > 1;
         const int a0 = posA(2 * lane, g), a1 = posA(2 * lane + 1, g);
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            float* rw = W + (8 * warp + r) * PLD;
+        for (int r = 0; r < WR; ++r) {
+            float* rw = W + (WR * warp + r) * PLD;
             put2(rw, a0, a1, v2, WA[r]); put2(rw, a0 + g, a1 + g, v2, WB[r]);
         }
     }
@@ -206,13 +210,44 @@ private:
         unpk(s, s0, s1);
         const u64 n = pk(-s0, -s1);
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
+        for (int r = 0; r < WR; ++r) {
             const u64 x = fma2(c, WA[r], mul2(n, WB[r])), y = fma2(s, WA[r], mul2(c, WB[r]));
             WA[r] = x;
             WB[r] = g > 1 ? turn(y, src) : y;
         }
     }
 };
+
+// The sweep of one pair block: S from S0 (row pitch ld), the CTA's rows w0 .. w0 + 16 WR - 1 of W from
+// the identity; the 64 cross rounds, or with `full` all 127.  On return W holds those rows (pitch PLD).
+// sm: kSmem bytes.
+template <int WR, class Load>
+__device__ __forceinline__ float* sweep(const float* S0, int64_t ld, int w0, int full, float* sm, Load load2) {
+    float* S = sm;
+    float* W = S + PN * PLD;
+    float* xch = W + PN * PLD;
+    float* apq = xch + 2 * 16 * 128;
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    for (int e = t; e < PN * PN / 2; e += PTHREADS) {
+        const int r = e >> 6, c = 2 * (e & 63);
+        *reinterpret_cast<float2*>(S + r * PLD + c) = load2(S0 + (int64_t)r * ld + c);
+        if (r < 16 * WR)
+            *reinterpret_cast<float2*>(W + r * PLD + c) = make_float2(w0 + r == c ? 1.f : 0.f, w0 + r == c + 1 ? 1.f : 0.f);
+    }
+    __syncthreads();
+    Block<WR> b;
+    const int last = full ? 1 : 64;
+    for (int lv = 64;; lv >>= 1) {
+        b.load(S, W, lv, warp, lane);
+        b.level(S, lv, xch, apq, warp, lane);
+        __syncthreads();
+        if (lv == last) { b.storeW(W, lv, warp, lane); break; }
+        b.store(S, W, lv, warp, lane);
+        __syncthreads();
+    }
+    __syncthreads();
+    return W;
+}
 
 }  // namespace pair
 }  // namespace glr
