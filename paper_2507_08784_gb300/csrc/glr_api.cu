@@ -448,6 +448,7 @@ int glr_create(int64_t m, int64_t n, int32_t r, int32_t N, const glr_schedule* s
     h->n_state_allocs = h->allocs.size();
     const int neig = exact ? (int)mp : k;                // scratch, not part of a checkpoint
     if (!exact) A(&h->eig_ws, eig_ws_floats(k));
+    else if (mp > 256 && mp <= 512) A(&h->jlog, jacobi_log_floats((int)mp, kJacobiSweeps));
     A(&h->sort_ws, 2 * (size_t)neig);
     if (rc != GLR_OK) {
         g_create_err = h->err;

@@ -52,6 +52,7 @@ struct glr_handle {
     float* mn_scratch = nullptr;
     float* jwork = nullptr;      // full basis: T^T of the blocked Jacobi above m' = 1024
     float* jpart = nullptr;      // norm partials of the eigen-solver (used by a group's first handle)
+    float* jlog = nullptr;       // full basis up to m' = 512: the Jacobi's rotations (not checkpointed)
     float *eig_ws = nullptr, *sort_ws = nullptr;   // eigen-solver and eigenpair-order scratch (not checkpointed)
     float* YtJ = nullptr;        // Yt[J, :] (r x k) for P = U[:, J] as a library product
     float* amsv = nullptr;       // AMSGrad: the scalar normaliser and this step's maximum of V

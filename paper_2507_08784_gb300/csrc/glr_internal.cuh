@@ -283,7 +283,10 @@ struct JacobiMat {
     float* H; float* H2; float* V; float* evals;   // H2: a second n x n buffer (rounds alternate)
     int* sweeps;
     int soff;               // first float of this matrix's rotations in shared memory (see jacobi_rot_floats)
+    float* log;             // jacobi_cluster: jacobi_log_floats(n, max_sweeps) floats, every round's rotations
 };
+constexpr int kJacobiSweeps = 40;
+size_t jacobi_log_floats(int n, int max_sweeps);     // 0 up to n = 256 and above 512
 constexpr int kJacobiMaxGrid = 1024;
 constexpr size_t kJacobiMaxSmem = 96 * 1024;     // the group's rotations; groups are split to fit
 size_t jacobi_rot_floats(int n);
@@ -295,7 +298,7 @@ struct JacobiGroup {
 int jacobi_group_grid();
 cudaError_t jacobi_group(const JacobiGroup& g, int grid, cudaStream_t st);
 // The same iteration (same rotations in the same order, bit for bit) for one matrix of n <= 512 in one
-// thread-block cluster; H is read only.  jacobi_cluster_ok(): whether the device can place it.
+// thread-block cluster (above n = 256 V from the logged rotations by a second launch); H is read only.  jacobi_cluster_ok(): whether the device can place it.
 bool jacobi_cluster_ok(int n);
 cudaError_t jacobi_cluster(const JacobiMat& M, int max_sweeps, cudaStream_t st);
 

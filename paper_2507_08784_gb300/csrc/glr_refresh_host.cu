@@ -200,7 +200,7 @@ JacobiMat jacobi_mat(glr_handle* h) {
     JacobiMat M{};
     M.n = h->mp; M.tol = 4.f * 5.96e-8f * sqrtf(static_cast<float>(h->mp)) + 1e-7f;
     M.H = h->Hbuf; M.H2 = h->jwork; M.V = h->Vbuf; M.evals = h->evals;
-    M.sweeps = h->dflags + 1;
+    M.sweeps = h->dflags + 1; M.log = h->jlog;
     return M;
 }
 
@@ -216,7 +216,7 @@ int refresh_exact_grouped(std::vector<glr_handle*>& hs) {
         PhaseScope ps(h, GLR_PH_REFRESH, h->rstream);
         const int mp = h->mp, np = h->np;
         GLR_GEMM(h, gd(mp, mp, np, h->Mbar, np, 1, h->Mbar, 1, np, h->Hbuf, mp, 1), h->rstream);
-        GLR_LAUNCH(h, 1, jacobi_cluster(jacobi_mat(h), 40, h->rstream));
+        GLR_LAUNCH(h, mp > 256 ? 2 : 1, jacobi_cluster(jacobi_mat(h), kJacobiSweeps, h->rstream));
         const int rc = sort_full_basis(h, h->rstream);
         if (rc != GLR_OK) return rc;
     }
@@ -254,7 +254,7 @@ int refresh_exact_grouped(std::vector<glr_handle*>& hs) {
         if (!grid) continue;
         JacobiGroup g{};
         size_t soff = 0;
-        g.max_sweeps = 40;
+        g.max_sweeps = kJacobiSweeps;
         g.bar = h0->dflags + 4; g.err = h0->dflags + 2; g.part = h0->jpart;
         for (size_t i = c0; i < c1; ++i) {
             glr_handle* h = hs[i];

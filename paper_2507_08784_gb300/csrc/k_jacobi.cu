@@ -15,10 +15,9 @@
 // line survives a barrier.
 //
 // For n <= 512 a matrix fits the shared memory of one thread-block cluster and is solved there
-// (jacobi_cluster_kernel), a launch a matrix: the rows of H (two buffers) and V are spread over up to
-// 16 CTAs, a round's rotations and the partner rows come over distributed shared memory, and a round
-// ends with one hardware cluster barrier.  The rotations, their order and every product and sum are
-// those of the grid-wide kernel, so the results are the same bits.  A round takes 3.7 us at n = 512
+// (jacobi_cluster_kernel): the row pairs of H are spread over up to 16 CTAs, a round's rotations go to
+// all of them over distributed shared memory; two hardware cluster barriers a round.  The rotations, their order and every product and sum are
+// those of the grid-wide kernel, so the results are the same bits.  A round takes 3.2 us at n = 512
 // (bound by instruction issue) and 2 us below n = 128 (the rotation's chain of quotients and roots,
 // two cluster barriers); the grid-wide kernel pays 6 us at n = 512 alone and 14 us for the eight
 // matrices of a conv stack, its barrier in global memory and the L2 round trips.
@@ -238,7 +237,9 @@ template <class T> __device__ __forceinline__ T* peer(T* p, int cta) {       // 
 // c x - s y and s x + c y, rounded as the grid-wide kernel's expressions are (checked bit for bit)
 __device__ __forceinline__ float rot_dif(float c, float x, float s, float y) { return __fmaf_rn(c, x, -__fmul_rn(s, y)); }
 __device__ __forceinline__ float rot_sum(float s, float x, float c, float y) { return __fmaf_rn(s, x, __fmul_rn(c, y)); }
-// Slots (row pairs) a CTA and CTAs a matrix; V's rows a CTA.
+// Rotations of a round in the log: whole 16-byte units.
+__host__ __device__ __forceinline__ int log_stride(int half) { return (half + 1) & ~1; }
+// Slots (row pairs) a CTA and CTAs a matrix.
 __host__ __device__ __forceinline__ int cluster_slots(int half) { return half > 128 ? (half + 15) / 16 : 8; }
 __host__ __device__ __forceinline__ int cluster_ctas(int n) {
     const int half = (n + 1) / 2, S = cluster_slots(half);
@@ -246,8 +247,8 @@ __host__ __device__ __forceinline__ int cluster_ctas(int n) {
 }
 size_t cluster_smem(int n) {
     const size_t half = (n + 1) / 2, S = cluster_slots((int)half), C = cluster_ctas(n);
-    const size_t rows = (2 * S + 3) + (n + C - 1) / C;
-    return sizeof(float) * (4 * half + rows * n);
+    const size_t rows = (2 * S + 3) + (n > 256 ? 0 : (n + C - 1) / C);
+    return sizeof(float) * (4 * (size_t)log_stride((int)half) + rows * n);
 }
 
 // The round's pairs sit in npad / 2 slots (T, B); slot 0's T is index 0, the others move by one slot a
@@ -256,9 +257,12 @@ size_t cluster_smem(int n) {
 // that only one T and one B row a round go to a neighbour's spare, written there in place of the
 // row itself.  A row pair's 2 x 2 blocks are then one thread's and are updated in place.
 // JU: the rotations a lane looks at (n <= 64 JU), whose indices it carries from round to round; ODD: n odd
-// (index n of the padded problem has no column).
+// (index n of the padded problem has no column).  V <- V J: up to n = 256 by the same CTAs, each its share
+// of the rows, while the round's second barrier completes; above (LOG) from the log afterwards (n = 512:
+// 3.5 -> 3.2 us a round; n = 128: 1.8 us a round here, 2.1 with the log).
 template <int JU, bool ODD>
 __global__ void __launch_bounds__(CT, 1) jacobi_cluster_kernel(const __grid_constant__ JacobiMat M, int max_sweeps) {
+    constexpr bool LOG = JU > 4;
     extern __shared__ __align__(16) float csm[];
     __shared__ float red[2][CT / 32], part[2];
     __shared__ int stop;
@@ -267,12 +271,15 @@ __global__ void __launch_bounds__(CT, 1) jacobi_cluster_kernel(const __grid_cons
     const int s0 = b * Smax, S = half - s0 < Smax ? half - s0 : Smax;          // own slots s0 .. s0 + S - 1
     const int slast = half - (C - 1) * Smax;                                // the last CTA's slots
     const int ST = b == 0 ? S - 1 : S, LT = ST + 1, LB = S + 1;             // rings (slot 0's T is apart)
-    const int R = (n + C - 1) / C, v0 = b * R, vrows = n - v0 < R ? (n - v0 > 0 ? n - v0 : 0) : R;
-    float2* const scs = reinterpret_cast<float2*>(csm);                     // 2 x half: cos, sin
-    float* const F = csm + 4 * half;                                        // index 0's row
+    const int lstride = log_stride(half);
+    float2* const scs = reinterpret_cast<float2*>(csm);                     // 2 x lstride: cos, sin
+    float* const F = csm + 4 * lstride;                                        // index 0's row
     float* const Tr = F + n;
     float* const Br = Tr + (size_t)(Smax + 1) * n;
-    float* const V = Br + (size_t)(Smax + 1) * n;
+    const int R = (n + C - 1) / C, v0 = b * R, vrows = LOG ? 0 : n - v0 < R ? (n - v0 > 0 ? n - v0 : 0) : R;
+    float* const V = Br + (size_t)(Smax + 1) * n;                           // own rows of V (unless LOG)
+    for (int e = t; e < vrows * n; e += CT) V[e] = v0 + e / n == e % n ? 1.f : 0.f;
+    float2* log = reinterpret_cast<float2*>(M.log);                         // this round's rotations
     // the buffer of the first ring T and of the first B: own, of the left and of the right neighbour
     const int LTl = b == 1 ? Smax : Smax + 1, LBr = (b + 1 == C - 1 ? slast : Smax) + 1;
     int tb = 0, bb = 0, tbl = 0, bbr = 0, par = 0;
@@ -288,7 +295,6 @@ __global__ void __launch_bounds__(CT, 1) jacobi_cluster_kernel(const __grid_cons
         const int r = low ? bidx(s0 + i, 0) : tidx(s0 + i, 0);
         (low ? brow(i) : trow(i))[c] = r < n ? M.H[(size_t)r * n + c] : 0.f;
     }
-    for (int e = t; e < vrows * n; e += CT) V[e] = v0 + e / n == e % n ? 1.f : 0.f;
     cluster_sync();
     // the columns' rotations in this thread's share of the work: warps share a slot when there are few
     const int G = S > 8 ? 1 : S > 4 ? 2 : S > 2 ? 4 : S > 1 ? 8 : 16;
@@ -328,7 +334,7 @@ __global__ void __launch_bounds__(CT, 1) jacobi_cluster_kernel(const __grid_cons
         cluster_sync();                                 // part is read before anyone writes it again
         if (stop) break;
         for (int rd = 0; rd < nm1; ++rd) {
-            float2* cs = scs + par * half;
+            float2* cs = scs + par * lstride;
             for (int e = t; e < S * C; e += CT) {       // own slots' rotations, to every CTA
                 const int i = e % S, to = e / S, x = tidx(s0 + i, rd), y = bidx(s0 + i, rd);
                 const int p = x < y ? x : y, q = x < y ? y : x;
@@ -349,6 +355,16 @@ __global__ void __launch_bounds__(CT, 1) jacobi_cluster_kernel(const __grid_cons
                 peer(cs, to)[s0 + i] = make_float2(c, s);
             }
             cluster_sync();
+            if (LOG && b == 0 && t == 0) {
+                // the round's rotations to the log, as an asynchronous copy: the cluster barrier's release
+                // would wait for plain stores to global memory (0.4 us a round).  The copy before this one
+                // has read its buffer by the time its rows of shared memory are written again.
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
+                             ::"l"(log), "r"(static_cast<uint32_t>(__cvta_generic_to_shared(cs))), "r"(lstride * 8) : "memory");
+                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+            }
             int pj[JU], qj[JU];
             float2 rj[JU];
 #pragma unroll
@@ -391,7 +407,7 @@ __global__ void __launch_bounds__(CT, 1) jacobi_cluster_kernel(const __grid_cons
                 }
             }
             cluster_arrive();
-            for (int r = warp; r < vrows; r += CT / 32) {                    // V <- V J, in place
+            for (int r = warp; r < vrows; r += CT / 32) {
                 float* w = V + (size_t)r * n;
                 float v[JU][2];
 #pragma unroll
@@ -407,6 +423,7 @@ __global__ void __launch_bounds__(CT, 1) jacobi_cluster_kernel(const __grid_cons
                 }
             }
             cluster_wait();
+            log += lstride;
             par ^= 1;
             if (half > 1) {
                 tb = wrap(tb + 1, LT); tbl = wrap(tbl + 1, LTl);
@@ -414,15 +431,70 @@ __global__ void __launch_bounds__(CT, 1) jacobi_cluster_kernel(const __grid_cons
             }
         }
     }
-    for (int e = t; e < vrows * n; e += CT) M.V[(size_t)v0 * n + e] = V[e];
     for (int e = t; e < 2 * S; e += CT) {
         const int i = e >> 1, r = (e & 1) ? bidx(s0 + i, 0) : tidx(s0 + i, 0);
         if (r < n) M.evals[r] = ((e & 1) ? brow(i) : trow(i))[r];
     }
-    if (b == 0 && t == 0 && M.sweeps) *M.sweeps = sweep;
+    for (int e = t; e < vrows * n; e += CT) M.V[(size_t)v0 * n + e] = V[e];
+    if (b == 0 && t == 0) {
+        *M.sweeps = sweep;
+        if (LOG) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // the log is complete before the CTA ends
+    }
+}
+
+// V, the product of the logged rotations in their order, a warp a row: its rows depend on nothing else, so
+// they are spread over the whole GPU afterwards (n = 512: 0.5 ms, against 1.1 us of the 3.5 us of every
+// round in the cluster).
+template <int JU, bool ODD>
+__global__ void __launch_bounds__(128) jacobi_rows_kernel(const __grid_constant__ JacobiMat M) {
+    extern __shared__ __align__(16) float vsm[];
+    const int n = M.n, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = blockIdx.x * 4 + warp;
+    const int npad = n + (n & 1), half = npad / 2, nm1 = npad - 1;
+    if (r >= n) return;
+    float* w = vsm + (size_t)warp * n;
+    for (int c = lane; c < n; c += 32) w[c] = r == c ? 1.f : 0.f;
+    int jx[JU], jy[JU];
+    float2 next[JU];
+    const float2* log = reinterpret_cast<const float2*>(M.log);
+    const int rounds = *M.sweeps * nm1;
+#pragma unroll
+    for (int u = 0; u < JU; ++u) {
+        const int j = lane + 32 * u;
+        jx[u] = j == 0 ? 0 : 1 + j % nm1;                   // circle(0 + j), circle(0 - j)
+        jy[u] = j == 0 || j >= half ? 1 : 1 + nm1 - j;
+        next[u] = j < half && rounds > 0 ? log[j] : make_float2(1.f, 0.f);
+    }
+    __syncwarp();
+    for (int rd = 0; rd < rounds; ++rd) {
+        log += log_stride(half);
+        float2 cs[JU];
+        float v[JU][2];
+        int p[JU], q[JU];
+#pragma unroll
+        for (int u = 0; u < JU; ++u) {
+            cs[u] = next[u];
+            if (lane + 32 * u < half && rd + 1 < rounds) next[u] = log[lane + 32 * u];
+            p[u] = jx[u] < jy[u] ? jx[u] : jy[u];
+            q[u] = jx[u] < jy[u] ? jy[u] : jx[u];
+            jx[u] = jx[u] == 0 ? 0 : jx[u] == nm1 ? 1 : jx[u] + 1;
+            jy[u] = jy[u] == nm1 ? 1 : jy[u] + 1;
+            if (lane + 32 * u >= half) continue;
+            v[u][0] = w[p[u]];
+            v[u][1] = !ODD || q[u] < n ? w[q[u]] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < JU; ++u) {
+            if (lane + 32 * u >= half) continue;
+            w[p[u]] = rot_dif(cs[u].x, v[u][0], cs[u].y, v[u][1]);
+            if (!ODD || q[u] < n) w[q[u]] = rot_sum(cs[u].y, v[u][0], cs[u].x, v[u][1]);
+        }
+        __syncwarp();
+    }
+    for (int c = lane; c < n; c += 32) M.V[(size_t)r * n + c] = w[c];
 }
 
 using ClusterKernel = void (*)(const JacobiMat, int);
+
 template <bool ODD> ClusterKernel cluster_kernel_of(int n) {
     return n <= 64 ? jacobi_cluster_kernel<1, ODD> : n <= 128 ? jacobi_cluster_kernel<2, ODD>
            : n <= 256 ? jacobi_cluster_kernel<4, ODD> : jacobi_cluster_kernel<8, ODD>;
@@ -465,12 +537,22 @@ bool jacobi_cluster_ok(int n) {
 }
 
 cudaError_t jacobi_cluster(const JacobiMat& M, int max_sweeps, cudaStream_t st) {
-    if (M.n < 1 || M.n > 512) return cudaErrorInvalidValue;
+    if (M.n < 1 || M.n > 512 || (M.n > 256 && !M.log) || !M.sweeps) return cudaErrorInvalidValue;
     const cudaError_t e = cluster_attributes(M.n);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr{};
     const cudaLaunchConfig_t cfg = cluster_config(M.n, &attr, st);
-    return cudaLaunchKernelEx(&cfg, cluster_kernel(M.n), M, max_sweeps);
+    const cudaError_t le = cudaLaunchKernelEx(&cfg, cluster_kernel(M.n), M, max_sweeps);
+    if (le != cudaSuccess || M.n <= 256) return le;
+    if (M.n & 1) jacobi_rows_kernel<8, true><<<(M.n + 3) / 4, 128, sizeof(float) * 4 * M.n, st>>>(M);
+    else jacobi_rows_kernel<8, false><<<(M.n + 3) / 4, 128, sizeof(float) * 4 * M.n, st>>>(M);
+    return cudaGetLastError();
+}
+
+size_t jacobi_log_floats(int n, int max_sweeps) {
+    if (n <= 256 || n > 512) return 0;
+    const size_t npad = n + (n & 1);
+    return (size_t)max_sweeps * (npad - 1) * 2 * log_stride((int)npad / 2);
 }
 
 int jacobi_group_grid() {
