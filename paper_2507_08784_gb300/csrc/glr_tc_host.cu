@@ -140,8 +140,8 @@ int tcl_maps(glr_handle* h) {
     };
     {
         const uint64_t d3[3] = {mp, np, N}, s3[2] = {mp * 4, mp * np * 4};
-        const uint32_t b3[3] = {128, 64, 1};
-        plain(kMapBtD, h->B, 3, d3, s3, b3, CU_TENSOR_MAP_SWIZZLE_NONE);          // B_i^T tiles, 128 x 64
+        const uint32_t b3[3] = {64, 64, 1};
+        plain(kMapBtD, h->B, 3, d3, s3, b3, CU_TENSOR_MAP_SWIZZLE_NONE);          // B_i^T tiles, 64 x 64
         const uint64_t d2[2] = {mp, np}, s2[1] = {mp * 4};
         const uint32_t bl[2] = {128, 128}, bu[2] = {128, 32};
         plain(kMapMbarL, h->Mbar, 2, d2, s2, bl, CU_TENSOR_MAP_SWIZZLE_NONE);     // Mbar^T tiles, 128 x 128
@@ -169,7 +169,7 @@ int tcl_maps(glr_handle* h) {
     return GLR_OK;
 }
 
-// The maps of this step's N gradients (bf16 tiles of 128 rows x 64 columns, read in the caller's
+// The maps of this step's N gradients (bf16 tiles of 64 rows x 64 columns, read in the caller's
 // layout): one of two slots, re-encoded and copied to the device (stream-ordered) only when the
 // set of pointers differs from both.
 const CUtensorMap* tcl_grad_maps(glr_handle* h, const void* const* G, cudaStream_t st, int* rc) {
@@ -186,11 +186,11 @@ const CUtensorMap* tcl_grad_maps(glr_handle* h, const void* const* G, cudaStream
         bool ok;
         if (h->transposed) {                       // G is n' x m' row-major: G(a, c) = G[c m' + a]
             const uint64_t d[2] = {mp, np}, s[1] = {mp * 2};
-            const uint32_t b[2] = {128, 64};
+            const uint32_t b[2] = {64, 64};
             ok = encode_map(&maps[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, G[i], 2, d, s, b, CU_TENSOR_MAP_SWIZZLE_NONE);
         } else {
             const uint64_t d[2] = {np, mp}, s[1] = {np * 2};
-            const uint32_t b[2] = {64, 128};
+            const uint32_t b[2] = {64, 64};
             ok = encode_map(&maps[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, G[i], 2, d, s, b, CU_TENSOR_MAP_SWIZZLE_128B);
         }
         if (!ok) {

@@ -45,7 +45,7 @@ namespace {
 // Epilogue warps per op (Op::kEpi); the three role warps follow them.
 template <class Op> constexpr int threads_of() { return (Op::kEpi + 3) * 32; }
 constexpr int kMaxStages = 8;
-constexpr int kMaxDStages = 4;
+constexpr int kMaxDStages = 6;
 constexpr uint32_t kTmemCols = 512;      // every op keeps more than half of shared memory, so one CTA per SM
 constexpr size_t kSmemBudget = 220 * 1024;
 constexpr size_t kMinSmem = 120 * 1024;  // above half of an SM's 228 KiB: one CTA, one allocation per SM
@@ -191,6 +191,7 @@ struct DataRing {
     volatile int* abort;
     int* err;
     int pend;                                         // stage whose group may still be reading (leader)
+    int step;                                         // stages a warp moves on by (2: it takes every second one)
     // warp-uniform: every lane gets the stage, or none (the CTA aborted)
     __device__ __forceinline__ uint8_t* acquire() {
         const bool ok = wait_phase(smem_u32(&full[s]), use, abort, err);
@@ -204,7 +205,7 @@ struct DataRing {
         if (leader) {
             if (wait_phase(smem_u32(&done[s]), use, abort, err)) store(smem_u32(base + (size_t)s * bytes));
             bulk_commit();                            // one group per stage (empty when nothing is stored)
-            if (n < 3) {                              // two stages: hand this one back at once
+            if (n < 3 * step) {                       // two stages (a half): hand this one back at once
                 bulk_wait_read();
                 mbar_arrive(smem_u32(&empty[s]));
             } else {
@@ -215,7 +216,8 @@ struct DataRing {
                 pend = s;
             }
         }
-        if (++s == n) { s = 0; use ^= 1u; }
+        s += step;
+        if (s >= n) { s -= n; use ^= 1u; }
     }
     __device__ __forceinline__ void finish(bool leader) {
         if (!leader) return;
@@ -230,6 +232,7 @@ struct NoStore { __device__ bool operator()(uint32_t) const { return false; } };
 // Ops without epilogue data.
 struct NoData {
     static constexpr int kEpi = 8;
+    static constexpr int kHalves = 1;                 // 2: a data stage is 64 rows of the tile, even ones the upper
     static __device__ __forceinline__ int ndata(const TcGroup&, const Tile&) { return 0; }
     static __device__ __forceinline__ uint32_t data_tx(const TcGroup&, const Tile&, int) { return 0; }
     static __device__ __forceinline__ void data_load(const TcGroup&, const Tile&, int, uint32_t, uint32_t) {}
@@ -257,7 +260,7 @@ __global__ void __launch_bounds__(threads_of<Op>(), 1) tc_kernel(const __grid_co
         for (int q = 0; q < D; ++q) {
             mbar_init(smem_u32(&dfull_bar[q]), 1);
             mbar_init(smem_u32(&dempty_bar[q]), 1);
-            mbar_init(smem_u32(&ddone_bar[q]), kEpiWarps * 32);
+            mbar_init(smem_u32(&ddone_bar[q]), kEpiWarps * 32 / Op::kHalves);
         }
         for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&tfull_bar[b]), 1); mbar_init(smem_u32(&tempty_bar[b]), kEpiWarps); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -343,7 +346,9 @@ __global__ void __launch_bounds__(threads_of<Op>(), 1) tc_kernel(const __grid_co
     } else {
         uint32_t tuse[2] = {0, 0};
         int b = 0;
-        DataRing dr{dring, DB, D, 0, 0u, dfull_bar, dempty_bar, ddone_bar, abort, g.err, -1};
+        // with two halves the warps of lanes 0-63 take the even stages, those of 64-127 the odd ones
+        const int half = Op::kHalves == 2 ? (warp & 3) >> 1 : 0;
+        DataRing dr{dring, DB, D, half, 0u, dfull_bar, dempty_bar, ddone_bar, abort, g.err, -1, Op::kHalves};
         for (int tile = blockIdx.x; tile < g.total_tiles; tile += gridDim.x) {
             Tile t = find_tile(g, tile);
             t.nk = Op::nk(g, t);
@@ -358,7 +363,7 @@ __global__ void __launch_bounds__(threads_of<Op>(), 1) tc_kernel(const __grid_co
             tuse[b] ^= 1u;
             if (nbuf == 2) b ^= 1;
         }
-        if (D > 0) dr.finish(warp == 0 && lane == 0);
+        if (D > 0) dr.finish((warp == 0 || (Op::kHalves == 2 && warp == 2)) && lane == 0);
     }
     fence_before();
     __syncthreads();
@@ -435,14 +440,17 @@ struct PrevProj : NoData {
 // Compose: tile = (128 rows a, 64 columns c).  D_i (128 x 64) = P_prev[a, :] R_w,i[:, c] (K = r)
 // for every node; the epilogue forms M_i = G_i + B_i - D_i, writes B_i^T, and Mbar^T = mean_i M_i.
 // A = P_prev (m' x r), B = R_w^T (3-D map rpad x n' x N).  Error reset (e_zero): no MMAs, M_i = G_i.
-// Data stage of node i: B_i^T tile (64 columns x 128 rows fp32, 512 bytes a column, 32 KiB) and
-// G_i's tile (bf16; 128 rows x 128 bytes with the 128-byte swizzle, or for m > n 64 columns x 256
-// bytes), 16 KiB.  B_i^T is stored back from the stage.
+// Data stage of node i and a half of the tile's rows: B_i^T tile (64 columns x 64 rows fp32, 256 bytes
+// a column, 16 KiB) and G_i's tile (bf16; 64 rows x 128 bytes with the 128-byte swizzle, or for m > n
+// 64 columns x 128 bytes), 8 KiB; the halves' warps work on different stages at a time.  B_i^T is
+// stored back from the stage.  Whole tiles a stage (48 KiB, two stages) leave one stage's copies in
+// flight while the other is worked on.
 // ------------------------------------------------------------------------------------------
 struct Compose {
     static constexpr int kEpi = 16;
     static constexpr int BN = 64;
-    static constexpr uint32_t kG = 32768;             // offset of the gradient tile in a data stage
+    static constexpr int kHalves = 2;
+    static constexpr uint32_t kG = 16384;             // offset of the gradient tile in a data stage
     static __device__ __forceinline__ int nk(const TcGroup& g, const Tile& t) {
         const TcMat& M = g.mat[t.mat];
         return M.e_zero ? 0 : M.rpad / 32;
@@ -460,16 +468,16 @@ struct Compose {
         const TcMat& M = g.mat[t.mat];
         for (int i = 0; i < M.N; ++i) mma_slice(d + (uint32_t)(i * BN), st, st + 16384u + i * (BN * 128u), BN, kc == 0);
     }
-    static __device__ __forceinline__ int ndata(const TcGroup& g, const Tile& t) { return g.mat[t.mat].N; }
+    static __device__ __forceinline__ int ndata(const TcGroup& g, const Tile& t) { return 2 * g.mat[t.mat].N; }
     static __device__ __forceinline__ uint32_t data_tx(const TcGroup& g, const Tile& t, int) {
-        return (g.mat[t.mat].e_zero ? 0u : 32768u) + 16384u;
+        return (g.mat[t.mat].e_zero ? 0u : 16384u) + 8192u;
     }
-    static __device__ __forceinline__ void data_load(const TcGroup& g, const Tile& t, int i, uint32_t st, uint32_t bar) {
+    static __device__ __forceinline__ void data_load(const TcGroup& g, const Tile& t, int u, uint32_t st, uint32_t bar) {
         const TcMat& M = g.mat[t.mat];
-        const int rt = t.lt / M.tn, ct = t.lt % M.tn;
-        if (!M.e_zero) tma_load_3d(st, M.mD0, rt * 128, ct * BN, i, bar);
-        if (M.transposed) tma_load_2d(st + kG, M.mD1 + i, rt * 128, ct * BN, bar);
-        else tma_load_2d(st + kG, M.mD1 + i, ct * BN, rt * 128, bar);
+        const int rt = t.lt / M.tn, ct = t.lt % M.tn, i = u >> 1, row0 = rt * 128 + 64 * (u & 1);
+        if (!M.e_zero) tma_load_3d(st, M.mD0, row0, ct * BN, i, bar);
+        if (M.transposed) tma_load_2d(st + kG, M.mD1 + i, row0, ct * BN, bar);
+        else tma_load_2d(st + kG, M.mD1 + i, ct * BN, row0, bar);
     }
     static __device__ __forceinline__ bool epilogue(const TcGroup& g, const Tile& t, uint32_t tl, int warp, int lane,
                                                     DataRing& dr) {
@@ -479,20 +487,21 @@ struct Compose {
         const int a = rt * 128 + al;
         const int cw = (warp >> 2) * 16;                  // this warp's 16 columns of the tile
         const int c0 = ct * BN + cw;
-        const bool leader = warp == 0 && lane == 0;
+        const int hl = al & 63, row0 = rt * 128 + (al & 64);  // row within the data stage, the stage's first row
+        const bool leader = (warp == 0 || warp == 2) && lane == 0;
         float acc[16];
 #pragma unroll
         for (int j = 0; j < 16; ++j) acc[j] = 0.f;
         for (int i = 0; i < M.N; ++i) {
             uint8_t* sm = dr.acquire();
             if (!sm) return false;
-            float* Bs = reinterpret_cast<float*>(sm) + al;    // B^T tile: column c at Bs[128 c]
+            float* Bs = reinterpret_cast<float*>(sm) + hl;    // B^T tile: column c at Bs[64 c]
             float m[16];
             if (!M.transposed) {
-                const uint8_t* row = sm + kG + al * 128;
+                const uint8_t* row = sm + kG + hl * 128;
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
-                    const uint4 u = *reinterpret_cast<const uint4*>(row + ((((cw >> 3) + q) ^ (al & 7)) << 4));
+                    const uint4 u = *reinterpret_cast<const uint4*>(row + ((((cw >> 3) + q) ^ (hl & 7)) << 4));
                     const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
                     for (int h = 0; h < 4; ++h) {
@@ -502,25 +511,25 @@ struct Compose {
                     }
                 }
             } else {
-                const __nv_bfloat16* col = reinterpret_cast<const __nv_bfloat16*>(sm + kG) + al;
+                const __nv_bfloat16* col = reinterpret_cast<const __nv_bfloat16*>(sm + kG) + hl;
 #pragma unroll
-                for (int j = 0; j < 16; ++j) m[j] = __bfloat162float(col[(cw + j) * 128]);
+                for (int j = 0; j < 16; ++j) m[j] = __bfloat162float(col[(cw + j) * 64]);
             }
             if (!M.e_zero) {
                 float d[16];
                 tmem_ld16(tl + (uint32_t)(i * BN + cw), d);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) m[j] += Bs[(cw + j) * 128] - d[j];
+                for (int j = 0; j < 16; ++j) m[j] += Bs[(cw + j) * 64] - d[j];
             }
             if (M.write_B) {
 #pragma unroll
-                for (int j = 0; j < 16; ++j) Bs[(cw + j) * 128] = m[j];
+                for (int j = 0; j < 16; ++j) Bs[(cw + j) * 64] = m[j];
             }
 #pragma unroll
             for (int j = 0; j < 16; ++j) acc[j] += m[j];
             dr.release(leader, [&](uint32_t st) {
-                if (!M.write_B) return false;
-                tma_store_3d(M.mD0, rt * 128, ct * BN, i, st);
+                if (!M.write_B || row0 >= M.mp) return false;
+                tma_store_3d(M.mD0, row0, ct * BN, i, st);
                 return true;
             });
         }
@@ -595,6 +604,7 @@ struct WBar : NoData {
 // ------------------------------------------------------------------------------------------
 struct Lambda {
     static constexpr int kEpi = 16;
+    static constexpr int kHalves = 1;
     static __device__ __forceinline__ int nk(const TcGroup& g, const Tile& t) { return g.mat[t.mat].kpad / 32; }
     static __device__ __forceinline__ uint32_t tx_bytes(const TcGroup&, const Tile&, int) { return 2u * 16384u; }
     static __device__ __forceinline__ void load(const TcGroup& g, const Tile& t, int kc, uint32_t st, uint32_t bar) {
@@ -879,6 +889,7 @@ struct RBar : NoData {
 // ------------------------------------------------------------------------------------------
 struct Update {
     static constexpr int kEpi = 16;
+    static constexpr int kHalves = 1;
     static __device__ __forceinline__ int nk(const TcGroup& g, const Tile& t) {
         const TcMat& M = g.mat[t.mat];
         return M.compressed ? M.rpad / 32 : 0;
@@ -1200,7 +1211,7 @@ template <> int acc_cols_of<Apply>(const TcMat& M) { return M.kpad; }
 
 // Data-stage bytes of an op (0: no data ring).
 template <class Op> size_t dstage_bytes_of(const TcGroup&, const TcMat&) { return 0; }
-template <> size_t dstage_bytes_of<Compose>(const TcGroup&, const TcMat&) { return 49152; }
+template <> size_t dstage_bytes_of<Compose>(const TcGroup&, const TcMat&) { return 24576; }
 template <> size_t dstage_bytes_of<Lambda>(const TcGroup&, const TcMat&) { return 65536; }
 template <> size_t dstage_bytes_of<Update>(const TcGroup& g, const TcMat& M) {
     return 16384 * (2 + (g.optimizer != GLR_MSGD ? 1 : 0) + (M.compressed ? 0 : 1));
@@ -1220,13 +1231,14 @@ cudaError_t launch(TcGroup& g, cudaStream_t st) {
     }
     if (cols > (int)kTmemCols) return cudaErrorInvalidValue;
     // without epilogue data: as many operand stages as fit; with it: two operand stages (one if
-    // two leave no room for two data stages), then as many data stages as fit (at most four)
+    // two leave no room for two data stages of every half), then as many data stages as fit
     int stages, dstages = 0;
     if (!db) {
         stages = std::min(static_cast<int>(kSmemBudget / sb), kMaxStages);
     } else {
-        stages = kSmemBudget >= 2 * sb + 2 * db ? 2 : 1;
+        stages = kSmemBudget >= 2 * sb + 2 * Op::kHalves * db ? 2 : 1;
         dstages = std::min(static_cast<int>((kSmemBudget - stages * sb) / db), kMaxDStages);
+        dstages -= dstages % Op::kHalves;
         if (dstages < 1) return cudaErrorInvalidValue;
     }
     if (stages < 1) return cudaErrorInvalidValue;
