@@ -82,7 +82,9 @@ __global__ void __launch_bounds__(256) lambda_kernel(const __grid_constant__ Lam
 // TF32 rounding of x, lo the TF32 truncation of x - hi; a b ~ a_hi b_hi + a_hi b_lo + a_lo b_hi),
 // then part[tile][j] = sum over the tile's 64 columns b of C(j, b) v_j[b].  CTA tile 64 j x 64 b,
 // K = m' in chunks of 32 staged in shared memory (row pitch 72: conflict-free fragment loads);
-// 8 warps = 4 m-tiles x 2 column halves of 4 n-tiles each.
+// 4 warps = 2 row halves of 2 m-tiles x 2 column halves of 4 n-tiles: splitting the operands, not the
+// MMAs, fills the issue slots, and each B fragment serves two m-tiles (8 warps of one m-tile each:
+// conv stack 145 us).
 constexpr int LMK = 32;                 // K chunk
 constexpr int LMP = 72;                 // shared row pitch (floats)
 
@@ -98,7 +100,7 @@ __device__ __forceinline__ void lm_mma(float (&d)[4], uint32_t a0, uint32_t a1, 
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-__global__ void __launch_bounds__(256) lambda_mma_kernel(const __grid_constant__ LambdaGroup lg) {
+__global__ void __launch_bounds__(128) lambda_mma_kernel(const __grid_constant__ LambdaGroup lg) {
     int mi = 0;
     while (mi + 1 < lg.nmat && lg.tile0[mi + 1] <= (int)blockIdx.x) ++mi;
     const LambdaArgs& a = lg.mat[mi];
@@ -108,29 +110,25 @@ __global__ void __launch_bounds__(256) lambda_mma_kernel(const __grid_constant__
     __shared__ float half_sum[2][LT];
     const int j0 = by * LT, b0 = bx * LT;
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-    const int mt = w & 3, nh = w >> 2;                        // m-tile (16 rows j), column half
+    const int mh = w & 1, nh = w >> 1;                        // row half (two m-tiles of 16), column half
     const int mp = a.mp, np = a.np, K = a.K;
-    constexpr int EPT = LMK * LT / 256;                       // 8 entries of each chunk per thread
+    constexpr int EPT = LMK * LT / 128;                       // 16 entries of each chunk per thread
     float na[EPT], nb[EPT];
     auto fetch = [&](int p0) {
 #pragma unroll
         for (int l = 0; l < EPT; ++l) {
-            const int e = tid + l * 256, pp = e / LT, cc = e % LT, gp = p0 + pp;
+            const int e = tid + l * 128, pp = e / LT, cc = e % LT, gp = p0 + pp;
             na[l] = gp < K && j0 + cc < mp ? a.A[(int64_t)gp * mp + j0 + cc] : 0.f;
             nb[l] = gp < K && b0 + cc < np ? a.Bm[(int64_t)gp * np + b0 + cc] : 0.f;
         }
     };
-    float acc[4][4];
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) acc[nt][e] = 0.f;
+    float acc[2][4][4] = {};
     fetch(0);
     for (int p0 = 0; p0 < K; p0 += LMK) {
         __syncthreads();
 #pragma unroll
         for (int l = 0; l < EPT; ++l) {
-            const int e = tid + l * 256, pp = e / LT, cc = e % LT;
+            const int e = tid + l * 128, pp = e / LT, cc = e % LT;
             As[pp][cc] = na[l];
             Bs[pp][cc] = nb[l];
         }
@@ -139,11 +137,15 @@ __global__ void __launch_bounds__(256) lambda_mma_kernel(const __grid_constant__
 #pragma unroll
         for (int k0 = 0; k0 < LMK; k0 += 8) {
             // A (16 j x 8 p): a0 (g, t), a1 (g + 8, t), a2 (g, t + 4), a3 (g + 8, t + 4)
-            uint32_t ah[4], al[4];
-            lm_split(As[k0 + t][mt * 16 + g], ah[0], al[0]);
-            lm_split(As[k0 + t][mt * 16 + g + 8], ah[1], al[1]);
-            lm_split(As[k0 + t + 4][mt * 16 + g], ah[2], al[2]);
-            lm_split(As[k0 + t + 4][mt * 16 + g + 8], ah[3], al[3]);
+            uint32_t ah[2][4], al[2][4];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int j = mh * 32 + i * 16 + g;
+                lm_split(As[k0 + t][j], ah[i][0], al[i][0]);
+                lm_split(As[k0 + t][j + 8], ah[i][1], al[i][1]);
+                lm_split(As[k0 + t + 4][j], ah[i][2], al[i][2]);
+                lm_split(As[k0 + t + 4][j + 8], ah[i][3], al[i][3]);
+            }
 #pragma unroll
             for (int nt = 0; nt < 4; ++nt) {
                 // B (8 p x 8 b): b0 (t, g), b1 (t + 4, g)
@@ -151,41 +153,47 @@ __global__ void __launch_bounds__(256) lambda_mma_kernel(const __grid_constant__
                 uint32_t bh0, bl0, bh1, bl1;
                 lm_split(Bs[k0 + t][bc], bh0, bl0);
                 lm_split(Bs[k0 + t + 4][bc], bh1, bl1);
-                lm_mma(acc[nt], al[0], al[1], al[2], al[3], bh0, bh1);
-                lm_mma(acc[nt], ah[0], ah[1], ah[2], ah[3], bl0, bl1);
-                lm_mma(acc[nt], ah[0], ah[1], ah[2], ah[3], bh0, bh1);
-            }
-        }
-    }
-    // C fragment: c0 (g, 2t), c1 (g, 2t + 1), c2 (g + 8, 2t), c3 (g + 8, 2t + 1) of each n-tile
-    float s[2] = {0.f, 0.f};
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int j = j0 + mt * 16 + g + 8 * h;
-        if (j < mp) {
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                const int bq = b0 + nh * 32 + nt * 8 + 4 * (t >> 1);   // the quad holding 2t, 2t + 1
-                if (bq < np) {
-                    const float4 v = gauss4_fast(a.seed, a.t, static_cast<uint32_t>(j), static_cast<uint32_t>(bq >> 2),
-                                                 kTagLambdaV);
-                    const bool upper = (t & 1) != 0;            // columns 2, 3 of the quad
-                    const float v0 = upper ? v.z : v.x, v1 = upper ? v.w : v.y;
-                    const int b = bq + 2 * (t & 1);
-                    if (b < np) s[h] = fmaf(acc[nt][2 * h], v0, s[h]);
-                    if (b + 1 < np) s[h] = fmaf(acc[nt][2 * h + 1], v1, s[h]);
+                for (int i = 0; i < 2; ++i) {
+                    lm_mma(acc[i][nt], al[i][0], al[i][1], al[i][2], al[i][3], bh0, bh1);
+                    lm_mma(acc[i][nt], ah[i][0], ah[i][1], ah[i][2], ah[i][3], bl0, bl1);
+                    lm_mma(acc[i][nt], ah[i][0], ah[i][1], ah[i][2], ah[i][3], bh0, bh1);
                 }
             }
         }
     }
+    // C fragment: c0 (g, 2t), c1 (g, 2t + 1), c2 (g + 8, 2t), c3 (g + 8, 2t + 1) of each n-tile
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {                             // the four lanes of a row, in order
-        s[h] += __shfl_xor_sync(0xffffffffu, s[h], 1);
-        s[h] += __shfl_xor_sync(0xffffffffu, s[h], 2);
-        if (t == 0) half_sum[nh][mt * 16 + g + 8 * h] = s[h];
+    for (int i = 0; i < 2; ++i) {
+        float s[2] = {0.f, 0.f};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int j = j0 + mh * 32 + i * 16 + g + 8 * h;
+            if (j < mp) {
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt) {
+                    const int bq = b0 + nh * 32 + nt * 8 + 4 * (t >> 1);   // the quad holding 2t, 2t + 1
+                    if (bq < np) {
+                        const float4 v = gauss4_fast(a.seed, a.t, static_cast<uint32_t>(j), static_cast<uint32_t>(bq >> 2),
+                                                     kTagLambdaV);
+                        const bool upper = (t & 1) != 0;            // columns 2, 3 of the quad
+                        const float v0 = upper ? v.z : v.x, v1 = upper ? v.w : v.y;
+                        const int b = bq + 2 * (t & 1);
+                        if (b < np) s[h] = fmaf(acc[i][nt][2 * h], v0, s[h]);
+                        if (b + 1 < np) s[h] = fmaf(acc[i][nt][2 * h + 1], v1, s[h]);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {                             // the four lanes of a row, in order
+            s[h] += __shfl_xor_sync(0xffffffffu, s[h], 1);
+            s[h] += __shfl_xor_sync(0xffffffffu, s[h], 2);
+            if (t == 0) half_sum[nh][mh * 32 + i * 16 + g + 8 * h] = s[h];
+        }
     }
     __syncthreads();
-    for (int jj = tid; jj < LT; jj += 256) {
+    for (int jj = tid; jj < LT; jj += 128) {
         const int j = j0 + jj;
         if (j < mp) a.part[(int64_t)bx * mp + j] = half_sum[0][jj] + half_sum[1][jj];
     }
@@ -208,7 +216,7 @@ cudaError_t lambda_partials(const LambdaGroup& all, cudaStream_t st) {
                 tiles += a.ntiles * ((a.mp + LT - 1) / LT);
             }
         if (!tiles) continue;
-        if (mode == 0) lambda_mma_kernel<<<tiles, 256, 0, st>>>(g);   // dense U: a dense contraction
+        if (mode == 0) lambda_mma_kernel<<<tiles, 128, 0, st>>>(g);   // dense U: a dense contraction
         else lambda_kernel<<<tiles, 256, 0, st>>>(g);
     }
     return cudaGetLastError();
@@ -320,47 +328,69 @@ __device__ __forceinline__ void select_top_r_block(const SelectMat& M, unsigned 
         }
         return;
     }
-    int npow2 = 1;
-    while (npow2 < mp) npow2 <<= 1;
-    for (int j = tid; j < npow2; j += nth) keys[j] = key_of(j);
-    __syncthreads();
-    if (mp <= 1024) {
-        // keys are distinct: j is among the r largest iff fewer than r keys exceed it
-        __shared__ unsigned char win[1024];
-        for (int j = tid; j < mp; j += nth) {
-            const unsigned long long kj = keys[j];
-            int above = 0;
-            for (int w = 0; w < mp; ++w) above += keys[w] > kj;
-            win[j] = above < r ? 1 : 0;
-        }
+    // The r-th largest score by its bits, a byte a pass (histogram of the scores that share the bytes found
+    // so far), then every score above it and the first of those equal to it, ranked by index.  (A bitonic
+    // sort of the keys, 78 barriers for m' = 4096: 64 us a launch.)
+    uint32_t* sc = reinterpret_cast<uint32_t*>(keys);
+    __shared__ int hist[256], wsum[32], found[2];
+    const int lane = tid & 31, w = tid >> 5;
+    for (int j = tid; j < mp; j += nth) {
+        const float l = M.lam[j];
+        sc[j] = __float_as_uint(l * l);
+    }
+    uint32_t prefix = 0;
+    int want = r;                                            // still to be found at or below the prefix
+    for (int sh = 24; sh >= 0; sh -= 8) {
+        if (tid < 256) hist[tid] = 0;
         __syncthreads();
-        for (int j = tid; j < mp; j += nth) {
-            if (!win[j]) continue;
-            int pos = 0;
-            for (int w = 0; w < j; ++w) pos += win[w];
-            M.J[pos] = j;
-        }
-    } else {
-        for (int size = 2; size <= npow2; size <<= 1) {
-            for (int stride = size >> 1; stride > 0; stride >>= 1) {
-                for (int i = tid; i < npow2; i += nth) {
-                    const int partner = i ^ stride;
-                    if (partner > i) {
-                        const bool desc = (i & size) == 0;
-                        const unsigned long long x = keys[i], y = keys[partner];
-                        if ((x < y) == desc) { keys[i] = y; keys[partner] = x; }
-                    }
-                }
-                __syncthreads();
+        for (int j = tid; j < mp; j += nth)
+            if (sh == 24 || (sc[j] >> (sh + 8)) == prefix) atomicAdd(&hist[(sc[j] >> sh) & 255], 1);
+        __syncthreads();
+        if (w == 0) {                                        // lane 0 the highest bins
+            int c[8], sum = 0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) { c[q] = hist[255 - (8 * lane + q)]; sum += c[q]; }
+            int before = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int x = __shfl_up_sync(0xffffffffu, before, o);
+                if (lane >= o) before += x;
+            }
+            before -= sum;
+            if (before < want && before + sum >= want) {
+                int q = 0;
+                while (before + c[q] < want) before += c[q++];
+                found[0] = 255 - (8 * lane + q);
+                found[1] = want - before;
             }
         }
-        for (int q = tid; q < r; q += nth) {
-            const int32_t jq = index_of(keys[q]);
-            int rank = 0;
-            for (int w = 0; w < r; ++w) rank += index_of(keys[w]) < jq;
-            M.J[rank] = jq;
-        }
+        __syncthreads();
+        prefix = (prefix << 8) | (uint32_t)found[0];
+        want = found[1];
     }
+    // prefix: the r-th largest score; `want` of those equal to it are taken, the lowest indices first
+    const int chunk = (mp + nth - 1) / nth, j0 = tid * chunk, j1 = j0 + chunk < mp ? j0 + chunk : mp;
+    auto block_before = [&](int mine) {                      // sum over the threads before this one
+        int incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += x;
+        }
+        __syncthreads();
+        if (lane == 31) wsum[w] = incl;
+        __syncthreads();
+        int base = 0;
+        for (int q = 0; q < w; ++q) base += wsum[q];
+        return base + incl - mine;
+    };
+    int eq = 0;
+    for (int j = j0; j < j1; ++j) eq += sc[j] == prefix;
+    int rank = block_before(eq), win = 0;
+    for (int j = j0, e = rank; j < j1; ++j) win += sc[j] > prefix || (sc[j] == prefix && e++ < want);
+    int pos = block_before(win);
+    for (int j = j0; j < j1; ++j)
+        if (sc[j] > prefix || (sc[j] == prefix && rank++ < want)) M.J[pos++] = j;
 }
 
 __global__ void __launch_bounds__(1024) select_group_kernel(const __grid_constant__ SelectGroup g) {
@@ -371,11 +401,11 @@ __global__ void __launch_bounds__(1024) select_group_kernel(const __grid_constan
     // YtJ = Yt[J, :] (r x k) for the tcgen05 path's P and Rbar products
     __syncthreads();
     const int r = M.r, k = M.k;
-    for (int e = threadIdx.x; e < r * k; e += blockDim.x) {
-        const int q = e / k, c = e - q * k;
-        M.YtJ[e] = M.Yt[(int64_t)M.J[q] * k + c];
+    const int k4 = k / 4;                                    // k is a multiple of 4 on that path
+    for (int e = threadIdx.x; e < r * k4; e += blockDim.x) {
+        const int q = e / k4, c = e - q * k4;
+        reinterpret_cast<float4*>(M.YtJ)[e] = reinterpret_cast<const float4*>(M.Yt + (int64_t)M.J[q] * k)[c];
     }
-
 }
 
 // Output o of the group: matrix i owns [out0, out0 + m' r) for P (row-major m' x r) and, when
