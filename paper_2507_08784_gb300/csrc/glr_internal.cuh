@@ -242,11 +242,11 @@ cudaError_t cholesky(float* A, int n, float* scratch, int* flag, cudaStream_t st
 // S = L^{-T} for L L^T = G (n x n SPD, n <= 256), one CTA with the factor in shared memory; the
 // same shifted retries as cholesky(), attempts counted in *flag.
 cudaError_t chol_inverse(const float* G, int n, float* S, int* flag, cudaStream_t st);
-// The same factor and inverse for several Gram matrices (one CTA each), each given as the sum of
-// nparts partial matrices (leading dimension ld, ld * ld apart); writes L^{-1} row-major ld x ld.
+// The same factor and inverse for several Gram matrices (one CTA each; leading dimension ld); writes
+// L^{-1} row-major ld x ld.
 // tri_only: the inverse alone, of U^T for the upper triangle U of part (n x n), or of its unit lower one.
 enum : int { kTriUpper = 1, kTriUnitLower = 2 };
-struct CholMat { const float* part; int nparts, ld, n; float* out; int* flag; int tri_only; };
+struct CholMat { const float* part; int ld, n; float* out; int* flag; int tri_only; };
 struct CholGroup { int nmat; CholMat mat[64]; };
 cudaError_t chol_group(const CholGroup& g, cudaStream_t st);
 // The end of a truncated refresh for several matrices, one launch per stage: stage 1 fixes the
@@ -302,8 +302,8 @@ cudaError_t jacobi_group(const JacobiGroup& g, int grid, cudaStream_t st);
 bool jacobi_cluster_ok(int n);
 cudaError_t jacobi_cluster(const JacobiMat& M, int max_sweeps, cudaStream_t st);
 
-// Symmetric eigenproblems of the refresh (k_eig.cu), n <= 1024: H (row-major, read only; the sum of
-// nparts matrices of leading dimension ld, ld * ld apart) -> eigenvalues (unsorted) and eigenvectors
+// Symmetric eigenproblems of the refresh (k_eig.cu), n <= 1024: H (row-major, leading dimension ld,
+// read only) -> eigenvalues (unsorted) and eigenvectors
 // V (row-major n x n, column j for evals[j]); sweeps done in *sweeps.  n <= 128: one CTA a problem
 // (eig_small_group).  Larger n: all problems in one cooperative launch (eig_group) that leaves
 // busy_sms SMs free; ws: eig_ws_floats(n) floats a problem, part: 128 floats a problem, bar: two
@@ -312,7 +312,7 @@ constexpr int kEigSmall = 128;
 constexpr int kEigGroupMax = 64;
 struct EigMat {
     int n; float tol;
-    const float* H; int nparts, ld;
+    const float* H; int ld;
     float* V; float* evals; int* sweeps; float* ws;
 };
 struct EigGroup {

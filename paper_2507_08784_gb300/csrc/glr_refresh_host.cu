@@ -41,12 +41,12 @@ int wy_from_Q(glr_handle* h, cudaStream_t st) {
     return GLR_OK;
 }
 
-// One symmetric eigenproblem of a handle (n = k or m' <= 1024): H as the sum of nparts matrices;
-// eigenvalues to h->evals, eigenvectors to V.
+// One symmetric eigenproblem of a handle (H of leading dimension ld): eigenvalues to h->evals,
+// eigenvectors to V.
 struct EigItem {
     glr_handle* h;
     int n;
-    const float* H; int nparts, ld;
+    const float* H; int ld;
     float* V;
 };
 
@@ -65,7 +65,7 @@ int eig_solve(const std::vector<EigItem>& items, cudaStream_t s0, cudaStream_t s
                 const EigItem& it = *cls[big][i];
                 EigMat& M = g.mat[g.nmat++];
                 M.n = it.n; M.tol = 4.f * 5.96e-8f * sqrtf(static_cast<float>(it.n)) + 1e-7f;
-                M.H = it.H; M.nparts = it.nparts; M.ld = it.ld; M.V = it.V; M.evals = it.h->evals;
+                M.H = it.H; M.ld = it.ld; M.V = it.V; M.evals = it.h->evals;
                 M.sweeps = it.h->dflags + 1; M.ws = it.h->eig_ws;
             }
             if (big) GLR_LAUNCH(h0, 1, eig_group(g, s0 != s1 ? (int)cls[0].size() : 0, s0));
@@ -115,7 +115,7 @@ int refresh_tails(std::vector<glr_handle*>& hs) {
             GLR_CK(h, cudaEventRecord(h->rpow, h->rstream));
             GLR_CK(h0, cudaStreamWaitEvent(h0->rstream, h->rpow, 0));
         }
-        items.push_back(EigItem{h, h->k, h->Hk, 1, h->k, h->Vk});
+        items.push_back(EigItem{h, h->k, h->Hk, h->k, h->Vk});
     }
     {
         PhaseScope ps(h0, GLR_PH_REFRESH, h0->rstream);
@@ -575,7 +575,7 @@ void pow_t(glr_handle* h, tc::TcMat& M) {
     M.splits = tc::pow_splits(h->mp, h->k, &M.chunk); M.ntiles = cdiv(h->np, 256) * M.splits;
 }
 
-// X^T X (Gram partials over row chunks), its factor L^{-1}, then X <- X L^{-T} (and X^T): the
+// X^T X, its factor L^{-1}, then X <- X L^{-T} (and X^T): the
 // CholeskyQR of X = Z (n' rows) or Q (m' rows) in TF32 products.
 int cholqr_tc(std::vector<glr_handle*>& hs, bool zside, cudaStream_t st, const std::vector<int>& active) {
     std::vector<glr_handle*> act;
@@ -592,7 +592,7 @@ int cholqr_tc(std::vector<glr_handle*>& hs, bool zside, cudaStream_t st, const s
         for (size_t i = c0; i < act.size() && i < c0 + 64; ++i) {
             glr_handle* h = act[i];
             CholMat& C = cg.mat[cg.nmat++];
-            C.part = h->gpart; C.nparts = cdiv(zside ? h->np : h->mp, tc::kGramChunk); C.ld = h->kpad; C.n = h->k;
+            C.part = h->gpart; C.ld = h->kpad; C.n = h->k;
             C.out = h->Linv; C.flag = h->dflags + 0;
         }
         PhaseScope ps(act[c0], GLR_PH_REFRESH, st);
@@ -679,7 +679,7 @@ int refresh_tcl_grouped(std::vector<glr_handle*>& hs) {
             for (size_t i = c0; i < hs.size() && i < c0 + 64; ++i) {
                 glr_handle* h = hs[i];
                 CholMat& C = cg.mat[cg.nmat++];
-                C.part = h->gram; C.nparts = 1; C.ld = h->k; C.n = h->k; C.out = h->Linv; C.flag = h->dflags + 0;
+                C.part = h->gram; C.ld = h->k; C.n = h->k; C.out = h->Linv; C.flag = h->dflags + 0;
             }
             PhaseScope ps(hs[c0], GLR_PH_REFRESH, s0);
             GLR_LAUNCH(hs[c0], 1, chol_group(cg, s0));
@@ -708,8 +708,8 @@ int refresh_tcl_grouped(std::vector<glr_handle*>& hs) {
         return true;
     });
     if (rc != GLR_OK) return rc;
-    std::vector<EigItem> items;                             // H is the sum of the Gram partials
-    for (glr_handle* h : hs) items.push_back(EigItem{h, h->k, h->gpart, cdiv(h->np, tc::kGramChunk), h->kpad, h->Vk});
+    std::vector<EigItem> items;
+    for (glr_handle* h : hs) items.push_back(EigItem{h, h->k, h->gpart, h->kpad, h->Vk});
     {
         PhaseScope ps(h0, GLR_PH_REFRESH, s0);
         if ((rc = eig_solve(items, s0, s0)) != GLR_OK) return rc;
@@ -748,7 +748,7 @@ int refresh_tcl_grouped(std::vector<glr_handle*>& hs) {
         for (size_t i = c0; i < hs.size() && i < c0 + 32; ++i) {
             glr_handle* h = hs[i];
             CholMat& C = cg.mat[cg.nmat++];
-            C.part = h->scratch; C.nparts = 1; C.ld = h->k; C.n = h->k; C.out = h->Linv; C.tri_only = kTriUpper;
+            C.part = h->scratch; C.ld = h->k; C.n = h->k; C.out = h->Linv; C.tri_only = kTriUpper;
             CholMat& D = cg.mat[cg.nmat++];
             D = C;
             D.out = h->Hk; D.tri_only = kTriUnitLower;

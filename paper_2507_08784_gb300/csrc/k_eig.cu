@@ -39,10 +39,8 @@ using namespace pair;
 
 constexpr int kNormChunks = 64;
 
-__device__ __forceinline__ float part_sum(const EigMat& M, int r, int c) {
-    float h = 0.f;
-    for (int p = 0; p < M.nparts; ++p) h += M.H[(size_t)p * M.ld * M.ld + (size_t)r * M.ld + c];
-    return h;
+__device__ __forceinline__ float h_entry(const EigMat& M, int r, int c) {
+    return r < M.n && c < M.n ? M.H[(size_t)r * M.ld + c] : 0.f;
 }
 
 // E_ij of the polish from (V^T V)_ij and S_ij, i < j, for both sides of the diagonal: half of R_ij and
@@ -85,7 +83,7 @@ __global__ void __launch_bounds__(8 * LIM, 1) eig_small_kernel(const __grid_cons
     const int n = M.n, t = threadIdx.x, warp = t >> 5, lane = t & 31;
     for (int e = t; e < R * PLD; e += NT) {
         const int r = e / PLD, c = e - r * PLD;
-        S[e] = (r < n && c < n) ? part_sum(M, r, c) : 0.f;
+        S[e] = h_entry(M, r, c);
         W[e] = r == c ? 1.f : 0.f;
     }
     __syncthreads();
@@ -126,7 +124,7 @@ __global__ void __launch_bounds__(8 * LIM, 1) eig_small_kernel(const __grid_cons
     float* lam = xch;
     for (int e = t; e < R * PLD; e += NT) {
         const int r = e / PLD, c = e - r * PLD;
-        S[e] = (r < n && c < n) ? part_sum(M, r, c) : 0.f;
+        S[e] = h_entry(M, r, c);
     }
     __syncthreads();
     u64 x[8][2], y[8][2];
@@ -433,7 +431,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) eig_group_kernel(const __grid_con
         const Work w(M);
         for (int64_t e = gtid; e < (int64_t)w.np * w.np; e += gsz) {
             const int r = (int)(e / w.np), c = (int)(e % w.np);
-            w.H0[e] = (r < M.n && c < M.n) ? part_sum(M, r, c) : 0.f;
+            w.H0[e] = h_entry(M, r, c);
             w.V0[e] = r == c ? 1.f : 0.f;
         }
     }
@@ -528,7 +526,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) eig_group_kernel(const __grid_con
                     if (state == kCopy) {
                         for (int e = t; e < 64 * w.np; e += PTHREADS) {
                             const int r = 64 * j + e / w.np, c = e % w.np;
-                            Ha[(int64_t)r * w.np + c] = (r < M.n && c < M.n) ? part_sum(M, r, c) : 0.f;
+                            Ha[(int64_t)r * w.np + c] = h_entry(M, r, c);
                         }
                     } else if (state == kProducts) {
                         if (j < tiles) tn_job(w, Ha, Vc, Hb, i0, j0, gsm);

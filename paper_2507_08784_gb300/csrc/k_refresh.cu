@@ -582,9 +582,7 @@ __global__ void __launch_bounds__(CWARPS * 32) chol_group_kernel(const __grid_co
     auto entry = [&](int i, int l) {
         if (M.tri_only == kTriUpper) return M.part[(size_t)l * M.n + i];           // L = U^T
         if (M.tri_only == kTriUnitLower) return i == l ? 1.f : M.part[(size_t)i * M.n + l];
-        float v = 0.f;
-        for (int p = 0; p < M.nparts; ++p) v += M.part[(size_t)p * M.ld * M.ld + (size_t)i * M.ld + l];
-        return v;
+        return M.part[(size_t)i * M.ld + l];
     };
     if (warp == 0) {                                   // trace: a warp sum in a fixed order
         float tr = 0.f;
@@ -597,6 +595,7 @@ __global__ void __launch_bounds__(CWARPS * 32) chol_group_kernel(const __grid_co
     int attempt = 0;
     for (; attempt < 6; ++attempt) {
         __syncthreads();
+#pragma unroll 4
         for (int q = warp; q < nb * (nb + 1) / 2 * CB; q += CWARPS) {    // a block row a warp
             int i = 0, j = q / CB;                                       // j = i (i + 1) / 2 + block column
             while (j > i) { j -= i + 1; ++i; }

@@ -1095,7 +1095,7 @@ using PowN = Pow<1>;
 // Gram: tile = (matrix, chunk of kGramChunk rows).  D_h (128 x kpad) = X^T[h 128 .., rows] X over
 // the chunk's rows (A = X^T slices of 128 rows, B = X^T with all kpad rows; X^T is TF32, kpad x
 // rows).  The epilogue writes the chunk's partial Gram matrix out[chunk][l][l'] (kpad x kpad);
-// the consumer sums the chunks in order.
+// gram_sum_kernel adds the chunks in order into out[0].
 // ------------------------------------------------------------------------------------------
 struct Gram : NoData {
     static __device__ __forceinline__ int halves(const TcMat& M) { return (M.kpad + 127) / 128; }
@@ -1316,7 +1316,31 @@ int pow_splits(int kdim, int k, int* chunk) {
 
 cudaError_t launch_powt(TcGroup& g, cudaStream_t st) { return launch_pow<PowT>(g, st); }
 cudaError_t launch_pown(TcGroup& g, cudaStream_t st) { return launch_pow<PowN>(g, st); }
-cudaError_t launch_gram(TcGroup& g, cudaStream_t st) { return launch<Gram>(g, st); }
+
+namespace {
+// The row chunks' partial Gram matrices added in order into the first one: by all SMs, where the
+// one-CTA consumers waited out a load's latency per chunk and row (k = 128: 90 of a factor's 120 us).
+__global__ void __launch_bounds__(256) gram_sum_kernel(const __grid_constant__ TcGroup g) {
+    const TcMat& M = g.mat[blockIdx.y];
+    const int64_t n4 = (int64_t)M.kpad * M.kpad / 4;
+    float4* out = reinterpret_cast<float4*>(M.out);
+    for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < n4; e += (int64_t)gridDim.x * 256) {
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+        for (int c = 0; c < M.ntiles; ++c) {
+            const float4 x = out[c * n4 + e];
+            s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
+        }
+        out[e] = s;
+    }
+}
+}  // namespace
+cudaError_t launch_gram(TcGroup& g, cudaStream_t st) {
+    const cudaError_t e = launch<Gram>(g, st);
+    if (e != cudaSuccess || g.nmat <= 0) return e;
+    gram_sum_kernel<<<dim3(64, g.nmat), 256, 0, st>>>(g);
+    return cudaGetLastError();
+}
 cudaError_t launch_apply(TcGroup& g, cudaStream_t st) { return launch<Apply>(g, st); }
 
 int compose_bn() { return Compose::BN; }
