@@ -138,7 +138,7 @@ int refresh_tails(std::vector<glr_handle*>& hs) {
 // (k_power.cu): the same iteration as refresh_power (q power iterations, each half re-normalised by
 // CholeskyQR, then CholeskyQR2 and the Rayleigh-Ritz Gram), one launch per stage for all of
 // them on the first handle's side stream; the k x k tails run on each handle's own stream.
-int refresh_grouped(std::vector<glr_handle*>& hs) {
+int refresh_power_group(const std::vector<glr_handle*>& hs) {
     glr_handle* h0 = hs[0];
     cudaStream_t s0 = h0->rstream;
     for (glr_handle* h : hs) GLR_CK(h0, cudaStreamWaitEvent(s0, h->rfork, 0));
@@ -183,6 +183,23 @@ int refresh_grouped(std::vector<glr_handle*>& hs) {
         const int rc = refresh_tail(h, h->rstream);
         g_ws = nullptr;
         if (rc != GLR_OK) return rc;
+    }
+    return GLR_OK;
+}
+
+// The handles in groups of one buffer pitch (k <= 16 or k <= 32: the partials are laid out for it) and
+// at most kGroupMax matrices.
+int refresh_grouped(std::vector<glr_handle*>& hs) {
+    for (int wide = 0; wide < 2; ++wide) {
+        std::vector<glr_handle*> part;
+        for (size_t i = 0; i < hs.size(); ++i) {
+            if ((hs[i]->k > 16) == (wide != 0)) part.push_back(hs[i]);
+            if (!part.empty() && (part.size() == (size_t)kGroupMax || i + 1 == hs.size())) {
+                const int rc = refresh_power_group(part);
+                if (rc != GLR_OK) return rc;
+                part.clear();
+            }
+        }
     }
     return GLR_OK;
 }
