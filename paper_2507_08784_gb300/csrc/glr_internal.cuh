@@ -259,6 +259,20 @@ struct FinishMat {
 };
 struct FinishGroup { int nmat; FinishMat mat[64]; };
 cudaError_t finish_group(const FinishGroup& g, int stage, cudaStream_t st);
+// The end of truncated refreshes with k <= 32 whose orthonormal iterate and H = Q^T Mbar Mbar^T Q are
+// there, up to kGroupMax at once.  stage 0: the eigenproblem H (k x k, read only), eigenvalues to
+// evals (descending to evals_sorted), the sorted, sign-fixed eigenvectors to R; 1 (Q already holds Q R):
+// the column signs to sign and the Householder top block: W = L1 \ Utilde, T, s; 2: Q with its signs,
+// Y, Yt = Y T^T, and their copies YT, YtT (k x tp, zero-padded) and YF, YtF (fragment order, may
+// be null).
+struct TailMat {
+    int mp, k, tp;
+    const float* H; float* evals; float* evals_sorted; int* sweeps; float* R;
+    float* Q; float* sign; float* W; float* T; float* s;
+    float* Y; float* Yt; float* YT; float* YtT; float* YF; float* YtF;
+};
+struct TailGroup { int nmat; TailMat mat[kGroupMax]; };
+cudaError_t tail_group(const TailGroup& g, int stage, cudaStream_t st);
 // C = A B in fp32 (FFMA) for several independent products, one launch: A(i, p) = A[i sAi + p sAp],
 // B(p, j) = B[p sBp + j sBj], C(i, j) = C[i sCi + j sCj]; 64 x 64 output tiles.
 struct GemmMat {
@@ -445,6 +459,16 @@ cudaError_t stream_group_mma(const StreamGroup& g, const TmaMaps* maps, size_t s
 // src (rows x cols, row-major, leading dimension ld) in the tensor-core kernel's fragment order
 // (up8(rows) x up8(cols) floats, zero-padded); form 0 for Y, form 1 for Yt.
 cudaError_t pack_frag(float* dst, const float* src, int rows, int cols, int ld, int form, cudaStream_t st);
+// Element idx of that order: block (group of 8 rows G8, n-tile nt) holds 64 floats, lane L = 4g + t's pair
+// at 2L, 2L + 1, with rho(t) = (t % 2) + 4 (t / 2) and prow(g) = rho(g / 2) + 2 (g % 2).
+//   form 0 (B fragment of X^T Y):  src(8 G8 + rho(t), 8 nt + g), src(8 G8 + rho(t) + 2, 8 nt + g)
+//   form 1 (B fragment of W Y^T): src(8 G8 + prow(g), 8 nt + 2t), src(8 G8 + prow(g), 8 nt + 2t + 1)
+__device__ __forceinline__ void frag_coord(int idx, int KT, int form, int& row, int& col) {
+    const int blk = idx >> 6, L = (idx >> 1) & 31, e = idx & 1;
+    const int G8 = blk / KT, nt = blk % KT, g = L >> 2, t = L & 3;
+    if (form == 0) { row = 8 * G8 + (t & 1) + 4 * (t >> 1) + 2 * e; col = 8 * nt + g; }
+    else { row = 8 * G8 + ((g >> 1) & 1) + 4 * (g >> 2) + 2 * (g & 1); col = 8 * nt + 2 * t + e; }
+}
 // dst (cols x tp) = src^T for row-major src (rows x cols), entries a >= rows set to 0.
 cudaError_t transpose_pad(float* dst, int tp, const float* src, int rows, int cols, cudaStream_t st);
 

@@ -98,13 +98,6 @@ int refresh_finish(glr_handle* h, cudaStream_t st) {
     return wy_from_Q(h, st);
 }
 
-// The end of a truncated refresh with k <= 32, Q orthonormal and H = Q^T Mbar Mbar^T Q in Hk: the
-// k x k Jacobi in one CTA, then refresh_finish.
-int refresh_tail(glr_handle* h, cudaStream_t st) {
-    GLR_LAUNCH(h, 1, jacobi_eig(h->Hk, h->k, h->Vk, h->evals, h->dflags + 1, st));
-    return refresh_finish(h, st);
-}
-
 // The end of truncated refreshes whose Q is orthonormal and whose H = Q^T Mbar Mbar^T Q is in Hk,
 // each on its own side stream: the eigenproblems together, then each handle's finish.
 int refresh_tails(std::vector<glr_handle*>& hs) {
@@ -134,10 +127,25 @@ int refresh_tails(std::vector<glr_handle*>& hs) {
     return GLR_OK;
 }
 
+// One grouped fp32 product per handle (fill describes it), 64 per launch.
+template <class Fill>
+int fp32_products(const std::vector<glr_handle*>& hs, cudaStream_t st, Fill fill) {
+    for (size_t c0 = 0; c0 < hs.size(); c0 += 64) {
+        GemmGroup gg{};
+        for (size_t i = c0; i < hs.size() && i < c0 + 64; ++i) {
+            gg.mat[gg.nmat].ws = hs[i]->gemm_ws;
+            fill(hs[i], gg.mat[gg.nmat++]);
+        }
+        PhaseScope ps(hs[c0], GLR_PH_REFRESH, st);
+        GLR_LAUNCH(hs[c0], 1, gemm_group_f32(gg, st));
+    }
+    return GLR_OK;
+}
+
 // Truncated refreshes of several matrices through the grouped block power iteration
 // (k_power.cu): the same iteration as refresh_power (q power iterations, each half re-normalised by
 // CholeskyQR, then CholeskyQR2 and the Rayleigh-Ritz Gram), one launch per stage for all of
-// them on the first handle's side stream; the k x k tails run on each handle's own stream.
+// them on the first handle's side stream.
 int refresh_power_group(const std::vector<glr_handle*>& hs) {
     glr_handle* h0 = hs[0];
     cudaStream_t s0 = h0->rstream;
@@ -175,15 +183,32 @@ int refresh_power_group(const std::vector<glr_handle*>& hs) {
         GLR_LAUNCH(h0, 1, pow_stage(g, 0, 0, s0));                    // Rayleigh-Ritz: Z = Mbar^T Q
         GLR_LAUNCH(h0, 1, pow_stage(g, 5, 1, s0));                    // H = Z^T Z
     }
-    GLR_CK(h0, cudaEventRecord(h0->rpow, s0));
+    // Rayleigh-Ritz and the WY form: four launches for all of them
+    TailGroup tg{};
     for (glr_handle* h : hs) {
-        if (h != h0) GLR_CK(h, cudaStreamWaitEvent(h->rstream, h0->rpow, 0));
-        PhaseScope ps(h, GLR_PH_REFRESH, h->rstream);
-        g_ws = h->gemm_ws;
-        const int rc = refresh_tail(h, h->rstream);
-        g_ws = nullptr;
-        if (rc != GLR_OK) return rc;
+        TailMat& M = tg.mat[tg.nmat++];
+        M.mp = h->mp; M.k = h->k; M.tp = transposed_pitch(h->mp);
+        M.H = h->Hk; M.evals = h->evals; M.evals_sorted = h->evals_sorted; M.sweeps = h->dflags + 1; M.R = h->gram;
+        M.Q = h->Qn; M.sign = h->sort_ws; M.W = h->scratch; M.T = h->T; M.s = h->dsign;
+        M.Y = h->Y; M.Yt = h->Yt; M.YT = h->YT; M.YtT = h->YtT;
+        if (h->mma) { M.YF = h->YF; M.YtF = h->YtF; }
     }
+    for (int stage = 0; stage < 3; ++stage) {
+        if (stage == 1) {                                            // Qn = Q R
+            const int rc = fp32_products(hs, s0, [](glr_handle* h, GemmMat& G) {
+                G.M = h->mp; G.N = h->k; G.K = h->k;
+                G.A = h->Q; G.sAi = h->k; G.sAp = 1; G.B = h->gram; G.sBp = h->k; G.sBj = 1;
+                G.C = h->Qn; G.sCi = h->k; G.sCj = 1;
+            });
+            if (rc != GLR_OK) return rc;
+            for (glr_handle* h : hs) std::swap(h->Q, h->Qn);
+        }
+        PhaseScope ps(h0, GLR_PH_REFRESH, s0);
+        GLR_LAUNCH(h0, 1, tail_group(tg, stage, s0));
+    }
+    GLR_CK(h0, cudaEventRecord(h0->rpow, s0));
+    for (glr_handle* h : hs)
+        if (h != h0) GLR_CK(h, cudaStreamWaitEvent(h->rstream, h0->rpow, 0));
     return GLR_OK;
 }
 
@@ -292,21 +317,6 @@ int refresh_exact_grouped(std::vector<glr_handle*>& hs) {
             const int rc = sort_full_basis(h, h->rstream);
             if (rc != GLR_OK) return rc;
         }
-    }
-    return GLR_OK;
-}
-
-// One grouped fp32 product per handle (fill describes it), 64 per launch.
-template <class Fill>
-int fp32_products(std::vector<glr_handle*>& hs, cudaStream_t st, Fill fill) {
-    for (size_t c0 = 0; c0 < hs.size(); c0 += 64) {
-        GemmGroup gg{};
-        for (size_t i = c0; i < hs.size() && i < c0 + 64; ++i) {
-            gg.mat[gg.nmat].ws = hs[i]->gemm_ws;
-            fill(hs[i], gg.mat[gg.nmat++]);
-        }
-        PhaseScope ps(hs[c0], GLR_PH_REFRESH, st);
-        GLR_LAUNCH(hs[c0], 1, gemm_group_f32(gg, st));
     }
     return GLR_OK;
 }

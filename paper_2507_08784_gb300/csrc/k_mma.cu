@@ -701,20 +701,13 @@ __global__ void __launch_bounds__(T, 1) stream_tma_kernel(const __grid_constant_
                                                           const __grid_constant__ TmaMaps maps) {
     compose_strip<GT, NQ, true>(g, &maps);
 }
-// dst = src (rows x cols, row-major, ld) in fragment order, up8(rows) x up8(cols) floats:
-// block (group G8, n-tile nt) holds 64 floats, lane L = 4g + t's pair at 2L, 2L + 1.
-//   form 0 (B fragment of X^T Y):  src(8 G8 + rho(t), 8 nt + g), src(8 G8 + rho(t) + 2, 8 nt + g)
-//   form 1 (B fragment of W Y^T): src(8 G8 + prow(g), 8 nt + 2t), src(8 G8 + prow(g), 8 nt + 2t + 1)
-// with rho(t) = (t % 2) + 4 (t / 2) and prow(g) = rho(g / 2) + 2 (g % 2).
+// dst = src (rows x cols, row-major, ld) in fragment order (frag_coord), up8(rows) x up8(cols) floats.
 __global__ void pack_frag_kernel(float* dst, const float* src, int rows, int cols, int ld, int form) {
     const int KT = up8(cols) >> 3;
     const int total = up8(rows) * KT * 8;
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
-        const int blk = idx >> 6, L = (idx >> 1) & 31, e = idx & 1;
-        const int G8 = blk / KT, nt = blk % KT, g = L >> 2, t = L & 3;
         int row, col;
-        if (form == 0) { row = 8 * G8 + (t & 1) + 4 * (t >> 1) + 2 * e; col = 8 * nt + g; }
-        else { row = 8 * G8 + ((g >> 1) & 1) + 4 * (g >> 2) + 2 * (g & 1); col = 8 * nt + 2 * t + e; }
+        frag_coord(idx, KT, form, row, col);
         dst[idx] = row < rows && col < cols ? src[(int64_t)row * ld + col] : 0.f;
     }
 }

@@ -767,6 +767,310 @@ __global__ void __launch_bounds__(CWARPS * 32) hh_lu_group_kernel(const __grid_c
         M.Us[e] = i <= l ? w * M.s[l] : 0.f;
     }
 }
+
+// ---- the end of the k <= 32 refreshes (the fp32 conv layers), all matrices of a step in each launch ----
+// Bound by chains of quotients, roots and barriers at these sizes, so a matrix's small work sits in
+// one CTA or warp, and the four launches replace twelve a matrix on as many streams.  The operations
+// and their order are those of jacobi_kernel, hh_top_kernel, hh_rows_kernel and the products.
+
+// jacobi_kernel and sort_rank_kernel for n <= 32: a thread keeps one 2 x 2 block of H and one pair of V's
+// entries for all rounds, so their indices are formed once, and the round's pairs advance along the
+// circle by increments (eight matrices, k = 16: 43 us; 68 + 9 us for the two kernels).
+__host__ __device__ __forceinline__ int tail_threads(int n) { return (n * ((n + 1) / 2) + 31) / 32 * 32; }
+
+__global__ void __launch_bounds__(512) tail_ritz_kernel(const __grid_constant__ TailGroup g) {
+    constexpr int P = 33;
+    __shared__ float H[32 * P], V[32 * P];
+    __shared__ float4 rot[16];                             // c, s, then p and q as row offsets
+    __shared__ float red_off[16], red_tot[16], ev[32];
+    __shared__ int done;
+    const TailMat& M = g.mat[blockIdx.x];
+    const int n = M.k, half = (n + 1) / 2, nm1 = 2 * half - 1, nth = tail_threads(n), max_sweeps = 40;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const float tol = 4.f * 5.96e-8f * sqrtf(static_cast<float>(n)) + 1e-7f;
+    // this thread's entries of the norms (n^2 <= 2 nth), its block of H and its entries of V
+    int he[2];
+    bool hd[2];
+    for (int i = 0; i < 2; ++i) {
+        const int e = tid + i * nth, r = e / n, c = e % n;
+        he[i] = tid < nth && e < n * n ? r * P + c : -1;
+        hd[i] = r == c;
+        if (he[i] >= 0) {
+            H[he[i]] = M.H[e];
+            V[he[i]] = hd[i] ? 1.f : 0.f;
+        }
+    }
+    const int bi = tid / half, bj = tid % half;
+    int xp = tid % nm1, xq = (nm1 - tid % nm1) % nm1;      // the circle's places of pair tid < half
+    const int xp0 = xp, xq0 = xq;
+    __syncthreads();
+    int sweep = 0;
+    for (; sweep < max_sweeps; ++sweep) {
+        float off = 0.f, tot = 0.f;
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            if (he[i] >= 0) {
+                const float h = H[he[i]];
+                tot += h * h;
+                if (!hd[i]) off += h * h;
+            }
+        for (int o = 16; o > 0; o >>= 1) {
+            off += __shfl_xor_sync(0xffffffffu, off, o);
+            tot += __shfl_xor_sync(0xffffffffu, tot, o);
+        }
+        if (lane == 0) { red_off[warp] = off; red_tot[warp] = tot; }
+        __syncthreads();
+        if (tid == 0) {
+            float o2 = 0.f, t2 = 0.f;
+            for (int w = 0; w < nth / 32; ++w) { o2 += red_off[w]; t2 += red_tot[w]; }
+            done = (o2 <= tol * tol * t2) ? 1 : 0;
+        }
+        __syncthreads();
+        if (done) break;
+        xp = xp0; xq = xq0;
+        for (int rd = 0; rd < nm1; ++rd) {
+            if (tid < half) {
+                int p = (tid == 0) ? 0 : 1 + xp;
+                int q = 1 + xq;
+                if (p > q) { const int tmp = p; p = q; q = tmp; }
+                float c = 1.f, s = 0.f;
+                if (q < n) {
+                    const float hpq = H[p * P + q];
+                    const float hpp = H[p * P + p], hqq = H[q * P + q];
+                    if (fabsf(hpq) > 1e-30f && fabsf(hpq) > 1e-9f * sqrtf(fabsf(hpp * hqq))) {
+                        const float theta = (hqq - hpp) / (2.f * hpq);
+                        float t;
+                        if (fabsf(theta) > 1e15f) t = 0.5f / theta;
+                        else t = copysignf(1.f, theta) / (fabsf(theta) + sqrtf(theta * theta + 1.f));
+                        c = 1.f / sqrtf(t * t + 1.f);
+                        s = t * c;
+                    }
+                }
+                rot[tid] = make_float4(c, s, __int_as_float(p), __int_as_float(q));
+                xp = xp + 1 == nm1 ? 0 : xp + 1;
+                xq = xq + 1 == nm1 ? 0 : xq + 1;
+            }
+            __syncthreads();
+            if (tid < n * half) {
+                const float4 rj = rot[bj];
+                const float cj = rj.x, sj = rj.y;
+                const int pj = __float_as_int(rj.z), qj = __float_as_int(rj.w);
+                if (tid < half * half) {
+                    const float4 ri = rot[bi];
+                    const float ci = ri.x, si = ri.y;
+                    const int pi = __float_as_int(ri.z), qi = __float_as_int(ri.w);
+                    if (si != 0.f || sj != 0.f) {
+                        const bool vqi = qi < n, vqj = qj < n;
+                        float h00 = H[pi * P + pj];
+                        float h01 = vqj ? H[pi * P + qj] : 0.f;
+                        float h10 = vqi ? H[qi * P + pj] : 0.f;
+                        float h11 = (vqi && vqj) ? H[qi * P + qj] : 0.f;
+                        const float a00 = ci * h00 - si * h10, a01 = ci * h01 - si * h11;
+                        const float a10 = si * h00 + ci * h10, a11 = si * h01 + ci * h11;
+                        float n00 = cj * a00 - sj * a01, n01 = sj * a00 + cj * a01;
+                        float n10 = cj * a10 - sj * a11, n11 = sj * a10 + cj * a11;
+                        if (bi == bj && si != 0.f) { n01 = 0.f; n10 = 0.f; }
+                        H[pi * P + pj] = n00;
+                        if (vqj) H[pi * P + qj] = n01;
+                        if (vqi) H[qi * P + pj] = n10;
+                        if (vqi && vqj) H[qi * P + qj] = n11;
+                    }
+                }
+                if (sj != 0.f) {                           // row bi of V
+                    const float vp = V[bi * P + pj], vq = V[bi * P + qj];
+                    V[bi * P + pj] = cj * vp - sj * vq;
+                    V[bi * P + qj] = sj * vp + cj * vq;
+                }
+            }
+            __syncthreads();
+        }
+    }
+    if (tid < n) {
+        ev[tid] = H[tid * P + tid];
+        M.evals[tid] = ev[tid];
+    }
+    if (tid == 0 && M.sweeps) *M.sweeps = sweep;
+    __syncthreads();
+    // sorted by descending value (ties by index), unit columns, largest entry positive: a warp a column
+    for (int col = warp; col < n; col += blockDim.x >> 5) {
+        const uint32_t mine = float_order(ev[col]), other = lane < n ? float_order(ev[lane]) : 0u;
+        const int rank = __popc(__ballot_sync(0xffffffffu, lane < n && (other > mine || (other == mine && lane < col))));
+        const float v = lane < n ? V[lane * P + col] : 0.f;
+        float ss = v * v, best = lane < n && fabsf(v) >= 0.f ? fabsf(v) : -1.f, val = best < 0.f ? 0.f : v;
+        int idx = best < 0.f ? 0x7fffffff : lane;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            ss += __shfl_xor_sync(0xffffffffu, ss, o);
+            const float ob = __shfl_xor_sync(0xffffffffu, best, o), ov = __shfl_xor_sync(0xffffffffu, val, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
+            if (ob > best || (ob == best && oi < idx)) { best = ob; val = ov; idx = oi; }
+        }
+        const float scale = (val < 0.f ? -1.f : 1.f) / sqrtf(ss);
+        if (lane < n) M.R[lane * n + rank] = scale * v;
+        if (lane == 0 && M.evals_sorted) M.evals_sorted[rank] = ev[col];
+    }
+}
+
+// The sign of each column of Q (its largest-|entry| positive, the first row on ties) by the whole CTA, then
+// the top block of the Householder reconstruction by one warp, a row a lane in registers that move
+// down by one a column: the modified LU of hh_top_kernel and T by substitution along its columns
+// (m' = 512, k = 16: 11 us; fix_signs and hh_top_kernel 13 + 17 us).
+template <int KM>
+__global__ void __launch_bounds__(1024) tail_top_kernel(const __grid_constant__ TailGroup g) {
+    constexpr int RG = 1024 / KM;
+    __shared__ float sbest[RG][KM + 1], sval[RG][KM + 1];
+    __shared__ int sidx[RG][KM + 1];
+    __shared__ float sg[32], Ss[32];
+    __shared__ float Ws[2 * KM][KM + 1];                   // rows past k: read for values nobody uses
+    const TailMat& M = g.mat[blockIdx.x];
+    const int k = M.k, mp = M.mp, tid = threadIdx.x, lane = tid & 31;
+    {
+        const int col = tid % KM, rg = tid / KM;
+        float best = -1.f, val = 0.f;
+        int idx = 0x7fffffff;
+        if (col < k)
+#pragma unroll 8
+            for (int a = rg; a < mp; a += RG) {
+                const float v = M.Q[(size_t)a * k + col], m = fabsf(v);
+                if (m > best) { best = m; val = v; idx = a; }
+            }
+        sbest[rg][col] = best; sval[rg][col] = val; sidx[rg][col] = idx;
+    }
+    for (int e = tid; e < 2 * KM * (KM + 1); e += 1024) (&Ws[0][0])[e] = 0.f;
+    __syncthreads();
+    for (int col = tid >> 5; col < k; col += 32) {         // a warp a column
+        float best = -1.f, val = 0.f;
+        int idx = 0x7fffffff;
+#pragma unroll
+        for (int q = lane; q < RG; q += 32)
+            if (sbest[q][col] > best || (sbest[q][col] == best && sidx[q][col] < idx)) {
+                best = sbest[q][col]; val = sval[q][col]; idx = sidx[q][col];
+            }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float ob = __shfl_xor_sync(0xffffffffu, best, o), ov = __shfl_xor_sync(0xffffffffu, val, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
+            if (ob > best || (ob == best && oi < idx)) { best = ob; val = ov; idx = oi; }
+        }
+        if (lane == 0) { sg[col] = val < 0.f ? -1.f : 1.f; M.sign[col] = sg[col]; }
+    }
+    __syncthreads();
+    if (tid >= 32) return;
+    float a[KM];
+#pragma unroll
+    for (int c = 0; c < KM; ++c) {
+        const float q = lane < k && c < k ? M.Q[(size_t)lane * k + c] : 0.f;
+        a[c] = c < k && sg[c] < 0.f ? q : -q;              // -Q with the signs
+    }
+#pragma unroll 1
+    for (int j = 0; j < k; ++j) {
+        const float wjj = __shfl_sync(0xffffffffu, a[0], j), sj = -wjj >= 0.f ? -1.f : 1.f, piv = wjj + sj;
+        const float v = lane > j ? a[0] / piv : lane == j ? piv : a[0];
+#pragma unroll
+        for (int q = 1; q < KM; ++q) {
+            const float u = __shfl_sync(0xffffffffu, a[q], j);
+            a[q - 1] = lane > j ? fmaf(-v, u, a[q]) : a[q];
+        }
+        a[KM - 1] = 0.f;
+        if (lane < KM) Ws[lane][j] = v;
+        if (lane == 0) Ss[j] = sj;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int l = 0; l < KM; ++l) a[l] = lane < KM && l < k ? Ws[lane][l] * Ss[l] : 0.f;
+    float* Ti = M.T + (size_t)lane * k;
+#pragma unroll 1
+    for (int c = 0; c < k; ++c) {                          // T[i][l] -= T[i][c] Y1[l][c] for l > c
+        const bool in = c >= lane;
+        const float x = in ? a[0] : 0.f;
+#pragma unroll
+        for (int q = 1; q < KM; ++q) a[q - 1] = in ? fmaf(-x, Ws[c + q][c], a[q]) : a[q];
+        if (lane < k) Ti[c] = x;
+    }
+    for (int e = lane; e < k * k; e += 32) M.W[e] = Ws[e / k][e % k];
+    if (lane < k) M.s[lane] = Ss[lane];
+}
+
+// A CTA per 32 rows, a warp four rows side by side, lane = column: the signs, Y (rows >= k by
+// substitution against Utilde, the others from L1), Yt = Y T^T, and the copies of both (17 us for eight
+// matrices up to m' = 512; six kernels a matrix, 29 us together).
+__global__ void __launch_bounds__(256) tail_rows_kernel(const __grid_constant__ TailGroup g) {
+    __shared__ float Ws[32][33], Ts[32][33], ys[2][32][33];
+    const TailMat& M = g.mat[blockIdx.y];
+    const int k = M.k, mp = M.mp, tp = M.tp, a0 = blockIdx.x * 32;
+    if (a0 >= tp) return;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int e = tid; e < k * k; e += 256) {
+        Ws[e / k][e % k] = M.W[e];
+        Ts[e / k][e % k] = M.T[e];
+    }
+    const float sg = lane < k ? M.sign[lane] : 1.f;
+    float q[4], y[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int a = a0 + 4 * warp + i;
+        q[i] = 0.f; y[i] = 0.f;
+        if (a < mp && lane < k) {
+            q[i] = M.Q[(size_t)a * k + lane];
+            if (sg < 0.f) M.Q[(size_t)a * k + lane] = q[i] = -q[i];
+        }
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int l = 0; l < k; ++l) {
+        const float w = lane < l ? Ws[lane][l] : 0.f, d = Ws[l][l];
+        float acc[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[i] = lane < l ? fmaf(y[i], w, 0.f) : 0.f;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float val = (-__shfl_sync(0xffffffffu, q[i], l) - acc[i]) / d;
+            if (lane == l) y[i] = val;
+        }
+    }
+    float yt[4] = {};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int a = a0 + 4 * warp + i;
+        if (a < k) y[i] = lane < a ? Ws[a][lane] : lane == a ? 1.f : 0.f;
+        if (a >= mp || lane >= k) y[i] = 0.f;
+    }
+#pragma unroll 4
+    for (int c = 0; c < k; ++c) {
+        const float t = lane < k ? Ts[lane][c] : 0.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) yt[i] = fmaf(__shfl_sync(0xffffffffu, y[i], c), t, yt[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        ys[0][4 * warp + i][lane] = y[i];
+        ys[1][4 * warp + i][lane] = lane < k ? yt[i] : 0.f;
+    }
+    __syncthreads();
+    const int rows = mp - a0 < 32 ? mp - a0 : 32;          // may be <= 0: padding only
+    for (int e = tid; e < rows * k; e += 256) {
+        M.Y[(size_t)a0 * k + e] = ys[0][e / k][e % k];
+        M.Yt[(size_t)a0 * k + e] = ys[1][e / k][e % k];
+    }
+    for (int c = warp; c < k; c += 8)
+        if (a0 + lane < tp) {
+            M.YT[(size_t)c * tp + a0 + lane] = ys[0][lane][c];
+            M.YtT[(size_t)c * tp + a0 + lane] = ys[1][lane][c];
+        }
+    if (!M.YF) return;
+    const int KT = (k + 7) / 8, up = (mp + 7) & ~7, frows = up - a0 < 32 ? up - a0 : 32;
+    for (int e = tid; e < frows * KT * 8; e += 256) {
+        int r, c;
+        frag_coord(e, KT, 0, r, c);
+        M.YF[(size_t)a0 * KT * 8 + e] = ys[0][r][c];
+        frag_coord(e, KT, 1, r, c);
+        M.YtF[(size_t)a0 * KT * 8 + e] = ys[1][r][c];
+    }
+}
 }  // namespace
 
 cudaError_t finish_group(const FinishGroup& g, int stage, cudaStream_t st) {
@@ -783,6 +1087,21 @@ cudaError_t finish_group(const FinishGroup& g, int stage, cudaStream_t st) {
         if (ea != cudaSuccess) return ea;
         hh_lu_group_kernel<<<g.nmat, CWARPS * 32, kHhSmem, st>>>(g);
     }
+    return cudaGetLastError();
+}
+
+cudaError_t tail_group(const TailGroup& g, int stage, cudaStream_t st) {
+    if (g.nmat <= 0) return cudaSuccess;
+    int kmax = 0, tp = 0;
+    for (int i = 0; i < g.nmat; ++i) {
+        if (g.mat[i].k < 1 || g.mat[i].k > 32) return cudaErrorInvalidValue;
+        kmax = g.mat[i].k > kmax ? g.mat[i].k : kmax;
+        tp = g.mat[i].tp > tp ? g.mat[i].tp : tp;
+    }
+    if (stage == 0) tail_ritz_kernel<<<g.nmat, tail_threads(kmax), 0, st>>>(g);
+    else if (stage == 2) tail_rows_kernel<<<dim3((tp + 31) / 32, g.nmat), 256, 0, st>>>(g);
+    else if (kmax <= 16) tail_top_kernel<16><<<g.nmat, 1024, 0, st>>>(g);
+    else tail_top_kernel<32><<<g.nmat, 1024, 0, st>>>(g);
     return cudaGetLastError();
 }
 
