@@ -6,55 +6,91 @@
 // where S (k x k) is the inverse Cholesky factor that orthonormalises the previous iterate
 // (CholeskyQR, Yamamoto et al. 2015), applied to the small output instead of the tall input:
 // Mbar^T (Q S) = (Mbar^T Q) S.  The Gram matrices are summed from per-tile partials in a fixed
-// order and factored in fp64 by one warp per matrix (pow_chol_kernel).  The final CholeskyQR2
+// order in fp64 and factored by one CTA per matrix (pow_chol_kernel).  The final CholeskyQR2
 // uses pow_apply_kernel; the Rayleigh-Ritz Gram H = Z^T Z comes out of pow_t_kernel the same way.
+#include <cooperative_groups.h>
+
 #include "glr_internal.cuh"
 
 namespace glr {
 
 namespace {
 
-constexpr int TP = 256;                // threads per CTA
+constexpr int TP = 256;                // threads per CTA (pow_r_kernel, pow_apply_kernel)
+constexpr int TM = 128;                // threads per CTA of the products
 constexpr int PC = 64;                 // columns of Mbar per tile / split-K chunk, rows per row tile
 constexpr int PR = 32;                 // rows of Mbar per staged block (pow_t_kernel)
+constexpr int PS = 6;                  // staged blocks in flight (pow_t_kernel)
 constexpr int NCH = 512;               // columns per split-K chunk (pow_n_kernel)
+constexpr int NR = 32;                 // rows per CTA (pow_n_kernel)
+constexpr int NS = 4;                  // its staged 32 x 64 blocks in flight
+constexpr int NP = PC + 4;             // their row pitch: 16-byte rows, no bank conflicts down a column of float4
 
-// Gram partial of the 64 x KM block Zs (rows < nrows valid) into gout (KM x KM, row-major).
-template <int KM>
+// 16 or 4 bytes into shared memory asynchronously, zeros where !in (src is not read then).
+__device__ __forceinline__ void cp16(void* dst, const float* src, bool in) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                     static_cast<uint32_t>(__cvta_generic_to_shared(dst))), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp4(void* dst, const float* src, bool in) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                     static_cast<uint32_t>(__cvta_generic_to_shared(dst))), "l"(src), "r"(in ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// Gram partial of the 64 x KM block Zs (rows < nrows valid) into gout (KM x KM, row-major), a 2 x 2 block of
+// entries at a time.
+template <int KM, int NT>
 __device__ __forceinline__ void gram_partial(const float* Zs, int nrows, float* gout) {
-    for (int o = threadIdx.x; o < KM * KM; o += TP) {
-        const int a = o / KM, b = o % KM;
-        float s = 0.f;
-        for (int c = 0; c < nrows; ++c) s = fmaf(Zs[c * KM + a], Zs[c * KM + b], s);
-        gout[o] = s;
+    constexpr int KH = KM / 2;
+    for (int o = threadIdx.x; o < KH * KH; o += NT) {
+        const int a = 2 * (o / KH), b = 2 * (o % KH);
+        float s00 = 0.f, s01 = 0.f, s10 = 0.f, s11 = 0.f;
+#pragma unroll 8
+        for (int c = 0; c < nrows; ++c) {
+            const float2 x = *reinterpret_cast<const float2*>(Zs + c * KM + a);
+            const float2 y = *reinterpret_cast<const float2*>(Zs + c * KM + b);
+            s00 = fmaf(x.x, y.x, s00); s01 = fmaf(x.x, y.y, s01);
+            s10 = fmaf(x.y, y.x, s10); s11 = fmaf(x.y, y.y, s11);
+        }
+        *reinterpret_cast<float2*>(gout + a * KM + b) = make_float2(s00, s01);
+        *reinterpret_cast<float2*>(gout + (a + 1) * KM + b) = make_float2(s10, s11);
     }
 }
 
 // out (64 x KM block in smem, rows < nrows) <- in S (KM x KM in smem), into out (may alias
-// nothing).  Thread (row = tid % 64, quarter) computes KM / 4 entries of its row.
-template <int KM>
+// nothing).  A thread computes KM / 4 entries of a row.
+template <int KM, int NT>
 __device__ __forceinline__ void apply_S(const float* in, const float* S, float* out) {
     constexpr int KPT = KM / 4;
-    const int row = threadIdx.x & 63, kq = threadIdx.x >> 6;
-    float acc[KPT];
+    const int row = threadIdx.x & 63;
+    for (int kq = threadIdx.x >> 6; kq < 4; kq += NT / 64) {
+        float acc[KPT];
 #pragma unroll
-    for (int e = 0; e < KPT; ++e) acc[e] = 0.f;
-    for (int l = 0; l < KM; ++l) {
-        const float v = in[row * KM + l];
+        for (int e = 0; e < KPT; ++e) acc[e] = 0.f;
+#pragma unroll 8
+        for (int l = 0; l < KM; ++l) {
+            const float v = in[row * KM + l];
 #pragma unroll
-        for (int e = 0; e < KPT; ++e) acc[e] = fmaf(v, S[l * KM + kq * KPT + e], acc[e]);
+            for (int e = 0; e < KPT; ++e) acc[e] = fmaf(v, S[l * KM + kq * KPT + e], acc[e]);
+        }
+#pragma unroll
+        for (int e = 0; e < KPT; ++e) out[row * KM + kq * KPT + e] = acc[e];
     }
-#pragma unroll
-    for (int e = 0; e < KPT; ++e) out[row * KM + kq * KPT + e] = acc[e];
 }
 
+template <int KM> constexpr size_t kPowTSmem = sizeof(float) * PS * (PR * PC + PR * KM);
+template <int KM> constexpr size_t kPowNSmem = sizeof(float) * NS * (NR * NP + PC * KM);
+
 // Z[c][:] = (sum_a Mbar[a][c] Q[a][:]) (S if apply_s), for a tile of 64 columns; Gram partial of
-// the tile's rows of Z into G[tile].
+// the tile's rows of Z into G[tile].  Bound by what shared memory can return to registers (6 floats a
+// thread for 8 products) and its latency: six blocks of 32 rows in flight by cp.async, a thread two
+// columns by KM / 4, a few rows' reads issued together (conv stack, k = 16: 23.4 -> 18.5 us a pass;
+// four columns a thread on half the warps 20.5).
 template <int KM>
-__global__ void __launch_bounds__(TP) pow_t_kernel(const __grid_constant__ PowGroup g, int apply_s) {
-    constexpr int KPT = KM / 4;
-    __shared__ __align__(16) float As[PR][PC];
-    __shared__ __align__(16) float Xs[PR * KM];
+__global__ void __launch_bounds__(TM) pow_t_kernel(const __grid_constant__ PowGroup g, int apply_s) {
+    constexpr int KPT = KM / 4, RB = KM == 16 ? 8 : 4;
+    extern __shared__ __align__(16) float stage[];             // PS blocks of PR x PC of Mbar, then of PR x KM of Q
     __shared__ __align__(16) float Zs[PC * KM];
     __shared__ __align__(16) float Z2[PC * KM];
     __shared__ __align__(16) float Ss[KM * KM];
@@ -64,142 +100,180 @@ __global__ void __launch_bounds__(TP) pow_t_kernel(const __grid_constant__ PowGr
     if (!M.active) return;
     const int tile = blockIdx.x - M.t0, c0 = tile * PC;
     const int mp = M.mp, np = M.np, k = M.k;
-    const int tid = threadIdx.x, cl = tid & 63, kq = tid >> 6;
-    float acc[KPT];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int cl = 2 * ((lane & 15) + 16 * (warp & 1)), kq = (lane >> 4) + 2 * (warp >> 1);
+    float* As = stage;
+    float* Xs = stage + PS * PR * PC;
+    // this thread's copies of a block: rows tid / 16 + 8 l of Mbar, four columns each; Q's rows are one
+    // contiguous piece when k = KM
+    const int fr = tid >> 4, fc = 4 * (tid & 15);
+    const bool fin = c0 + fc < np;                             // n' % 4 == 0
+    const float* fsrc = fin ? M.Mbar + (int64_t)fr * np + c0 + fc : M.Mbar;
+    auto fetch = [&](int blk) {                                // block blk of 32 rows
+        const int a0 = blk * PR, b = blk % PS;
+        if (a0 < mp) {
+            const float* src = fin ? fsrc + (int64_t)a0 * np : fsrc;
+            float* dst = As + b * PR * PC + fr * PC + fc;
 #pragma unroll
-    for (int e = 0; e < KPT; ++e) acc[e] = 0.f;
-    // each thread stages two float4 of every 32 x 64 block of Mbar; the next block's loads are
-    // issued before the current block is used
-    constexpr int LPT = PR * PC / 4 / TP;                      // = 2 float4 of Mbar
-    constexpr int XPT = PR * KM / TP;                          // = 2 or 4 entries of Q
-    float4 nxt[2][LPT];                                        // two blocks in flight
-    float xn[2][XPT];
-    auto fetch = [&](int a0, int bufi) {
+            for (int l = 0; l < PR / 8; ++l) {
+                const bool in = fin && a0 + fr + 8 * l < mp;
+                cp16(dst + 8 * l * PC, in ? src + (int64_t)8 * l * np : M.Mbar, in);
+            }
+            float* xd = Xs + b * PR * KM;
+            if (k == KM) {
 #pragma unroll
-        for (int l = 0; l < LPT; ++l) {
-            const int o = tid + l * TP, rr = o / (PC / 4), cc = 4 * (o % (PC / 4));
-            const int a = a0 + rr, c = c0 + cc;
-            nxt[bufi][l] = a < mp && c < np ? *reinterpret_cast<const float4*>(M.Mbar + (int64_t)a * np + c)   // n' % 4 == 0
-                                            : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int l = 0; l < PR * KM / 4 / TM; ++l) {
+                    const int o = 4 * (tid + l * TM);
+                    const bool in = a0 + o / KM < mp;
+                    cp16(xd + o, in ? M.Q + (int64_t)a0 * KM + o : M.Q, in);
+                }
+            } else {
+#pragma unroll
+                for (int l = 0; l < PR * KM / TM; ++l) {
+                    const int o = tid + l * TM, rr = o / KM, q = o % KM, a = a0 + rr;
+                    const bool in = a < mp && q < k;
+                    cp4(xd + o, in ? M.Q + (int64_t)a * k + q : M.Q, in);
+                }
+            }
         }
-#pragma unroll
-        for (int l = 0; l < XPT; ++l) {
-            const int o = tid + l * TP, rr = o / KM, q = o % KM, a = a0 + rr;
-            xn[bufi][l] = a < mp && q < k ? M.Q[(int64_t)a * k + q] : 0.f;
-        }
+        cp_commit();
     };
-    fetch(0, 0);
-    if (PR < mp) fetch(PR, 1);
-    for (int a0 = 0, bi = 0; a0 < mp; a0 += PR, bi ^= 1) {
-        if (bi == 0) {
+    float acc[2][KPT] = {};
+    const int nblk = (mp + PR - 1) / PR;
+    for (int i = 0; i < PS - 1; ++i) fetch(i);
+    if (apply_s)
+        for (int o = tid; o < KM * KM; o += TM) {
+            const int a = o / KM, b = o % KM;
+            Ss[o] = a < k && b < k ? M.S[a * k + b] : (a == b ? 1.f : 0.f);
+        }
+    for (int blk = 0; blk < nblk; ++blk) {
+        cp_wait<PS - 2>();                                     // this thread's copies of the block, then everyone's
+        __syncthreads();
+        fetch(blk + PS - 1);                                   // over the block read before the barrier
+        const float* A = As + (blk % PS) * PR * PC + cl;
+        const float* X = Xs + (blk % PS) * PR * KM + kq * KPT;
+#pragma unroll 2
+        for (int r0 = 0; r0 < PR; r0 += RB) {                  // RB rows' reads issued together
+            float2 m[RB];
+            float4 x[RB][KPT / 4];
 #pragma unroll
-            for (int l = 0; l < LPT; ++l) {
-                const int o = tid + l * TP, rr = o / (PC / 4), cc = 4 * (o % (PC / 4));
-                *reinterpret_cast<float4*>(&As[rr][cc]) = nxt[0][l];
+            for (int r = 0; r < RB; ++r) {
+                m[r] = *reinterpret_cast<const float2*>(A + (r0 + r) * PC);
+#pragma unroll
+                for (int e = 0; e < KPT; e += 4) x[r][e / 4] = *reinterpret_cast<const float4*>(X + (r0 + r) * KM + e);
             }
 #pragma unroll
-            for (int l = 0; l < XPT; ++l) Xs[tid + l * TP] = xn[0][l];
-        } else {
+            for (int r = 0; r < RB; ++r)
 #pragma unroll
-            for (int l = 0; l < LPT; ++l) {
-                const int o = tid + l * TP, rr = o / (PC / 4), cc = 4 * (o % (PC / 4));
-                *reinterpret_cast<float4*>(&As[rr][cc]) = nxt[1][l];
-            }
+                for (int e = 0; e < KPT; e += 4) {
+                    const float xv[4] = {x[r][e / 4].x, x[r][e / 4].y, x[r][e / 4].z, x[r][e / 4].w};
 #pragma unroll
-            for (int l = 0; l < XPT; ++l) Xs[tid + l * TP] = xn[1][l];
+                    for (int j = 0; j < 4; ++j) {
+                        acc[0][e + j] = fmaf(m[r].x, xv[j], acc[0][e + j]);
+                        acc[1][e + j] = fmaf(m[r].y, xv[j], acc[1][e + j]);
+                    }
+                }
         }
-        __syncthreads();
-        if (a0 + 2 * PR < mp) {
-            if (bi == 0) fetch(a0 + 2 * PR, 0);
-            else fetch(a0 + 2 * PR, 1);
-        }
-#pragma unroll 8
-        for (int rr = 0; rr < PR; ++rr) {
-            const float m = As[rr][cl];
-#pragma unroll
-            for (int e = 0; e < KPT; ++e) acc[e] = fmaf(m, Xs[rr * KM + kq * KPT + e], acc[e]);
-        }
-        __syncthreads();
     }
 #pragma unroll
-    for (int e = 0; e < KPT; ++e) Zs[cl * KM + kq * KPT + e] = acc[e];
-    for (int o = tid; o < KM * KM; o += TP) {
-        const int a = o / KM, b = o % KM;
-        Ss[o] = a < k && b < k ? M.S[a * k + b] : (a == b ? 1.f : 0.f);
-    }
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int e = 0; e < KPT; ++e) Zs[(cl + j) * KM + kq * KPT + e] = acc[j][e];
     __syncthreads();
     const float* Zo = Zs;
     if (apply_s) {
-        apply_S<KM>(Zs, Ss, Z2);
+        apply_S<KM, TM>(Zs, Ss, Z2);
         Zo = Z2;
+        __syncthreads();
     }
-    __syncthreads();
     const int nrows = np - c0 < PC ? np - c0 : PC;
-    for (int o = tid; o < nrows * KM; o += TP) {
+    for (int o = tid; o < nrows * KM; o += TM) {
         const int c = o / KM, q = o % KM;
         if (q < k) M.Z[(int64_t)(c0 + c) * k + q] = Zo[o];
     }
-    gram_partial<KM>(Zo, nrows, M.G + (int64_t)tile * KM * KM);
+    gram_partial<KM, TM>(Zo, nrows, M.G + (int64_t)tile * KM * KM);
 }
 
 // part[chunk][q][a] = sum over the chunk's NCH columns c of Mbar[a][c] Z[c][q], for one tile of
-// 64 rows a: CTA (row tile, chunk), the chunk walked in 64-column blocks.
+// 32 rows a: CTA (row tile, chunk), the chunk walked in 64-column blocks, four in flight; a thread holds
+// one row by KM / 4 (conv stack: 20.4 -> 16.4 us; 64-row tiles, four rows a thread 20.5).
 template <int KM>
-__global__ void __launch_bounds__(TP) pow_n_kernel(const __grid_constant__ PowGroup g) {
+__global__ void __launch_bounds__(TM) pow_n_kernel(const __grid_constant__ PowGroup g) {
     constexpr int KPT = KM / 4;
-    __shared__ __align__(16) float As[PC][PC + 1];            // 64 rows x 64 columns
-    __shared__ __align__(16) float Ys[PC * KM];
+    extern __shared__ __align__(16) float stage[];             // NS blocks of NR x NP of Mbar, then of PC x KM of Z
     int mi = 0;
-    while (mi + 1 < g.nmat && blockIdx.x >= static_cast<unsigned>(g.mat[mi + 1].n0)) ++mi;
+    const int bid = blockIdx.x / (PC / NR);                    // the group counts tiles of 64 rows
+    while (mi + 1 < g.nmat && bid >= g.mat[mi + 1].n0) ++mi;
     const PowMat& M = g.mat[mi];
-    if (!M.active) return;
     const int nrt = (M.mp + PC - 1) / PC;
-    const int chunk = (blockIdx.x - M.n0) / nrt, rt = (blockIdx.x - M.n0) % nrt;
-    const int a0 = rt * PC, cbeg = chunk * NCH;
+    const int chunk = (bid - M.n0) / nrt, rt = (bid - M.n0) % nrt;
+    const int a0 = rt * PC + NR * (blockIdx.x % (PC / NR)), cbeg = chunk * NCH;
     const int mp = M.mp, np = M.np, k = M.k;
+    if (!M.active || a0 >= mp) return;
     const int cend = cbeg + NCH < np ? cbeg + NCH : np;
-    const int tid = threadIdx.x, al = tid & 63, kq = tid >> 6;
-    constexpr int LPT = PC * PC / 4 / TP;                      // = 4 float4 of each 64 x 64 block
-    constexpr int YPT = PC * KM / TP;                          // = 4 or 8 entries of Z
-    float4 nxt[LPT];
-    float yn[YPT];
-    auto fetch = [&](int c0) {
+    const int tid = threadIdx.x, lane = tid & 31, kq = tid >> 5;
+    float* As = stage;
+    float* Ys = stage + NS * NR * NP;
+    const int fr = tid >> 4, fc = 4 * (tid & 15);
+    const float* fsrc = M.Mbar + (int64_t)(a0 + fr) * np + cbeg + fc;
+    auto fetch = [&](int blk) {
+        const int c0 = cbeg + blk * PC, b = blk % NS;
+        if (c0 < cend) {
+            const bool fin = c0 + fc < cend;
+            float* dst = As + b * NR * NP + fr * NP + fc;
 #pragma unroll
-        for (int l = 0; l < LPT; ++l) {
-            const int o = tid + l * TP, rr = o / (PC / 4), cc = 4 * (o % (PC / 4));
-            const int a = a0 + rr, c = c0 + cc;
-            nxt[l] = a < mp && c < cend ? *reinterpret_cast<const float4*>(M.Mbar + (int64_t)a * np + c)
-                                        : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+            for (int l = 0; l < NR / 8; ++l) {
+                const bool in = fin && a0 + fr + 8 * l < mp;
+                cp16(dst + 8 * l * NP, in ? fsrc + (int64_t)8 * l * np + blk * PC : M.Mbar, in);
+            }
+            float* yd = Ys + b * PC * KM;
+            if (k == KM) {
 #pragma unroll
-        for (int l = 0; l < YPT; ++l) {
-            const int o = tid + l * TP, cc = o / KM, q = o % KM, c = c0 + cc;
-            yn[l] = c < cend && q < k ? M.Z[(int64_t)c * k + q] : 0.f;
+                for (int l = 0; l < PC * KM / 4 / TM; ++l) {
+                    const int o = 4 * (tid + l * TM);
+                    const bool in = c0 + o / KM < cend;
+                    cp16(yd + o, in ? M.Z + (int64_t)c0 * KM + o : M.Z, in);
+                }
+            } else {
+#pragma unroll
+                for (int l = 0; l < PC * KM / TM; ++l) {
+                    const int o = tid + l * TM, cc = o / KM, q = o % KM, c = c0 + cc;
+                    const bool in = c < cend && q < k;
+                    cp4(yd + o, in ? M.Z + (int64_t)c * k + q : M.Z, in);
+                }
+            }
         }
+        cp_commit();
     };
-    float acc[KPT];
-#pragma unroll
-    for (int e = 0; e < KPT; ++e) acc[e] = 0.f;
-    fetch(cbeg);
-    for (int c0 = cbeg; c0 < cend; c0 += PC) {
+    float acc[KPT] = {};
+    const int nblk = (cend - cbeg + PC - 1) / PC;
+    for (int i = 0; i < NS - 1; ++i) fetch(i);
+    for (int blk = 0; blk < nblk; ++blk) {
+        cp_wait<NS - 2>();
         __syncthreads();
+        fetch(blk + NS - 1);
+        const float* A = As + (blk % NS) * NR * NP + lane * NP;
+        const float* Y = Ys + (blk % NS) * PC * KM + kq * KPT;
+#pragma unroll 2
+        for (int cc = 0; cc < PC; cc += 8) {                   // eight columns' reads issued together
+            const float4 p = *reinterpret_cast<const float4*>(A + cc), q = *reinterpret_cast<const float4*>(A + cc + 4);
+            const float m[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+            float4 y[8][KPT / 4];
 #pragma unroll
-        for (int l = 0; l < LPT; ++l) {
-            const int o = tid + l * TP, rr = o / (PC / 4), cc = 4 * (o % (PC / 4));
-            As[rr][cc] = nxt[l].x; As[rr][cc + 1] = nxt[l].y; As[rr][cc + 2] = nxt[l].z; As[rr][cc + 3] = nxt[l].w;
-        }
+            for (int j = 0; j < 8; ++j)
 #pragma unroll
-        for (int l = 0; l < YPT; ++l) Ys[tid + l * TP] = yn[l];
-        __syncthreads();
-        if (c0 + PC < cend) fetch(c0 + PC);
-#pragma unroll 8
-        for (int cc = 0; cc < PC; ++cc) {
-            const float m = As[al][cc];
+                for (int e = 0; e < KPT; e += 4) y[j][e / 4] = *reinterpret_cast<const float4*>(Y + (cc + j) * KM + e);
 #pragma unroll
-            for (int e = 0; e < KPT; ++e) acc[e] = fmaf(m, Ys[cc * KM + kq * KPT + e], acc[e]);
+            for (int j = 0; j < 8; ++j)
+#pragma unroll
+                for (int e = 0; e < KPT; e += 4) {
+                    const float4 v = y[j][e / 4];
+                    acc[e] = fmaf(m[j], v.x, acc[e]); acc[e + 1] = fmaf(m[j], v.y, acc[e + 1]);
+                    acc[e + 2] = fmaf(m[j], v.z, acc[e + 2]); acc[e + 3] = fmaf(m[j], v.w, acc[e + 3]);
+                }
         }
     }
-    const int a = a0 + al;
+    const int a = a0 + lane;
     float* part = M.part + (int64_t)chunk * KM * mp;
     if (a < mp)
 #pragma unroll
@@ -225,7 +299,7 @@ __global__ void __launch_bounds__(TP) pow_r_kernel(const __grid_constant__ PowGr
 #pragma unroll
     for (int e = 0; e < KPT; ++e) acc[e] = 0.f;
     if (a < mp)
-#pragma unroll 4
+#pragma unroll 8
         for (int ch = 0; ch < nch; ++ch) {                      // fixed order over the chunks
             const float* p = M.part + (int64_t)ch * KM * mp + a;
 #pragma unroll
@@ -238,14 +312,14 @@ __global__ void __launch_bounds__(TP) pow_r_kernel(const __grid_constant__ PowGr
         Ss[o] = r < k && c < k ? M.S[r * k + c] : (r == c ? 1.f : 0.f);
     }
     __syncthreads();
-    apply_S<KM>(Qs, Ss, Q2);
+    apply_S<KM, TP>(Qs, Ss, Q2);
     __syncthreads();
     const int nrows = mp - a0 < PC ? mp - a0 : PC;
     for (int o = tid; o < nrows * KM; o += TP) {
         const int r = o / KM, q = o % KM;
         if (q < k) M.Q[(int64_t)(a0 + r) * k + q] = Q2[o];
     }
-    gram_partial<KM>(Q2, nrows, M.G + (int64_t)tile * KM * KM);
+    gram_partial<KM, TP>(Q2, nrows, M.G + (int64_t)tile * KM * KM);
 }
 
 // Q[a][:] <- Q[a][:] S for a tile of 64 rows (rows are independent: in place); Gram partial
@@ -271,113 +345,159 @@ __global__ void __launch_bounds__(TP) pow_apply_kernel(const __grid_constant__ P
         Ss[o] = r < k && c < k ? M.S[r * k + c] : (r == c ? 1.f : 0.f);
     }
     __syncthreads();
-    apply_S<KM>(Qs, Ss, Q2);
+    apply_S<KM, TP>(Qs, Ss, Q2);
     __syncthreads();
     for (int o = tid; o < nrows * KM; o += TP) {
         const int r = o / KM, q = o % KM;
         if (q < k) M.Q[(int64_t)(a0 + r) * k + q] = Q2[o];
     }
-    if (gram) gram_partial<KM>(Q2, nrows, M.G + (int64_t)tile * KM * KM);
+    if (gram) gram_partial<KM, TP>(Q2, nrows, M.G + (int64_t)tile * KM * KM);
 }
 
-// One warp per matrix: Gm = sum over the ntile partials (fp64 accumulation, tile order).
+// Gm = sum over the ntile partials (fp64 accumulation, tile order), then by one CTA
 // mode 0: Gm = L L^T (fp32 Cholesky, retried with a growing diagonal shift on breakdown) and
 // S = L^{-T}, so X S has orthonormal columns when Gm = X^T X; mode 1: the sum itself into H (the
-// Rayleigh-Ritz Gram).
-constexpr int TCH = 1024;              // threads of pow_chol_kernel
+// Rayleigh-Ritz Gram).  The fp64 additions and conversions of 72 partials took one SM most of 17 us, so a
+// cluster of eight CTAs shares a matrix's lower triangle; the first one factors, a column bound by its
+// root, quotient and barrier (17 -> 10 us).
+constexpr int TCH = 256, CCH = 8;      // threads and CTAs per matrix of pow_chol_kernel
+
+// num / den; a zero numerator (most of the identity's) does not take the division's slow path.
+__device__ __forceinline__ float quotient(float num, float den) {
+    const float q = (num == 0.f ? 1.f : num) / den;
+    return num == 0.f ? num : q;
+}
 
 template <int KM>
-__global__ void __launch_bounds__(TCH) pow_chol_kernel(const __grid_constant__ PowGroup g, int use_t_tiles, int mode) {
+__global__ void __cluster_dims__(CCH, 1, 1) __launch_bounds__(TCH)
+    pow_chol_kernel(const __grid_constant__ PowGroup g, int use_t_tiles, int mode) {
     __shared__ float Gs[KM][KM + 1];
-    __shared__ float Ls[2 * KM][KM + 1];                       // rows past k: read for values nobody uses
-    __shared__ float Xi[KM][KM + 1];                           // L^{-1}, column c by lane c
-    __shared__ double Gq[4][KM * KM];
-    const PowMat& M = g.mat[blockIdx.x];
+    __shared__ float colj[2][KM], rowj[2][KM];
+    const PowMat& M = g.mat[blockIdx.x / CCH];
     if (!M.active) return;
-    const int k = M.k, lane = threadIdx.x;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int k = M.k, tid = threadIdx.x, lane = tid & 31, rank = blockIdx.x % CCH;
     const int nt = use_t_tiles ? M.nt : M.nr;
-    // entry o of the sum over the nt partials: four threads take the tiles t = j (mod 4), each
-    // with two accumulators, and the four slices are added in order
-    for (int w = threadIdx.x; w < 4 * k * k; w += TCH) {
-        const int o = w >> 2, j = w & 3, a = o / k, b = o % k;
-        const float* p = M.G + a * KM + b;
+    cl.sync();                                                 // the first CTA's shared memory is there
+    float* G0 = cl.map_shared_rank(&Gs[0][0], 0);
+    // entry o = a (a + 1) / 2 + b of the sum over the nt partials (the other triangle is the same bits): four
+    // threads take the tiles t = j (mod 4), each with two accumulators, and the four slices are
+    // added in order
+    const int tri = k * (k + 1) / 2;
+    for (int w0 = 0; w0 < 4 * tri; w0 += CCH * TCH) {          // a warp's eight entries to each CTA in turn
+        const int w = w0 + ((tid >> 5) * CCH + rank) * 32 + (tid & 31), o = w >> 2, j = w & 3;
+        int a = 0;
+        while ((a + 1) * (a + 2) / 2 <= o) ++a;
+        const int b = o - a * (a + 1) / 2;
         double s0 = 0.0, s1 = 0.0;
-        int t = j;
+        if (o < tri) {
+            const float* p = M.G + a * KM + b;
+            int t = j;
 #pragma unroll 4
-        for (; t + 4 < nt; t += 8) {
-            s0 += static_cast<double>(p[(int64_t)t * KM * KM]);
-            s1 += static_cast<double>(p[(int64_t)(t + 4) * KM * KM]);
+            for (; t + 4 < nt; t += 8) {
+                s0 += static_cast<double>(p[(int64_t)t * KM * KM]);
+                s1 += static_cast<double>(p[(int64_t)(t + 4) * KM * KM]);
+            }
+            if (t < nt) s0 += static_cast<double>(p[(int64_t)t * KM * KM]);
         }
-        if (t < nt) s0 += static_cast<double>(p[(int64_t)t * KM * KM]);
-        Gq[j][o] = s0 + s1;
+        double s = s0 + s1;
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        if (o < tri && j == 0) {
+            const float v = static_cast<float>(s);
+            G0[a * (KM + 1) + b] = v;
+            G0[b * (KM + 1) + a] = v;
+        }
     }
-    __syncthreads();
-    for (int o = threadIdx.x; o < k * k; o += TCH)
-        Gs[o / k][o % k] = static_cast<float>((Gq[0][o] + Gq[1][o]) + (Gq[2][o] + Gq[3][o]));
-    __syncthreads();
-    if (threadIdx.x >= 32) return;                             // one warp factors
+    cl.sync();
+    if (rank != 0) return;
     if (mode == 1) {
-        for (int o = lane; o < k * k; o += 32) M.H[o] = Gs[o / k][o % k];
+        for (int o = tid; o < k * k; o += TCH) M.H[o] = Gs[o / k][o % k];
         return;
     }
     float tr = 0.f;
     for (int i = 0; i < k; ++i) tr += Gs[i][i];
-    if (lane == 0 && M.flag && (!(tr > 0.f) || !isfinite(tr))) atomicAdd(M.flag + 6, 1);   // degenerate block
+    if (tid == 0 && M.flag && (!(tr > 0.f) || !isfinite(tr))) atomicAdd(M.flag + 6, 1);   // degenerate block
+    // right-looking factor and, in the same steps, the substitution for L^{-1} along L's columns: a thread
+    // holds entries (i, c) of both; a step needs column j of the one and row j of the other
+    constexpr int E = KM * KM / TCH;
+    const int c = tid % KM, i0 = tid / KM;
     float shift = 0.f;
     for (int attempt = 0; attempt < 6; ++attempt) {
-        // right-looking factor with lane = row: the row's entries in registers, moved down by one a column,
-        // so that every column runs the same few instructions; a row past k stays zero
-        float a[KM];
+        float a[E], r[E], x[E];
 #pragma unroll
-        for (int c = 0; c < KM; ++c) a[c] = lane < k && c < k ? Gs[lane < KM ? lane : 0][c] + (lane == c ? shift : 0.f) : 0.f;
+        for (int m = 0; m < E; ++m) {
+            const int i = i0 + m * (TCH / KM);
+            a[m] = i < k && c < k ? Gs[i][c] + (i == c ? shift : 0.f) : 0.f;
+            r[m] = i == c ? 1.f : 0.f;
+            x[m] = 0.f;
+            if (c == 0) colj[0][i] = a[m];
+            if (i == 0) rowj[0][c] = r[m];
+        }
+        __syncthreads();
         bool ok = true;
-#pragma unroll 1
-        for (int j = 0; j < k && ok; ++j) {
-            const float d = __shfl_sync(0xffffffffu, a[0], j);
-            ok = d > 0.f;                                      // same value in every lane
-            const float ljj = sqrtf(d);
-            const float v = lane == j ? ljj : lane > j ? a[0] / ljj : 0.f;
+        for (int j = 0; j < k; ++j) {
+            const float* cj = colj[j & 1];
+            const float d = cj[j];
+            ok = d > 0.f;                                      // the same value in every thread
+            if (!ok) break;
+            // every warp forms L's column and the inverse's row: a quotient a lane (two for KM = 32)
+            const float ljj = sqrtf(d), *rj = rowj[j & 1];
+            const float q0 = quotient(KM == 32 || lane < KM ? cj[lane] : rj[lane % KM], ljj);
+            const float q1 = KM == 32 ? quotient(rj[lane], ljj) : q0;
+            const float qc = __shfl_sync(0xffffffffu, q0, c), xj = __shfl_sync(0xffffffffu, q1, KM == 32 ? c : KM + c);
+            const float vc = c > j ? qc : 0.f;
 #pragma unroll
-            for (int q = 1; q < KM; ++q) a[q - 1] = fmaf(-v, __shfl_sync(0xffffffffu, v, (j + q) & 31), a[q]);
-            a[KM - 1] = 0.f;
-            if (lane < KM) Ls[lane][j] = v;
+            for (int m = 0; m < E; ++m) {
+                const int i = i0 + m * (TCH / KM);
+                const float vi = __shfl_sync(0xffffffffu, q0, i);
+                if (i == j) x[m] = xj;
+                if (i > j) {
+                    a[m] = fmaf(-vi, vc, a[m]);
+                    r[m] = fmaf(-xj, vi, r[m]);
+                }
+                if (c == j + 1) colj[(j + 1) & 1][i] = a[m];
+                if (i == j + 1) rowj[(j + 1) & 1][c] = r[m];
+            }
+            __syncthreads();
         }
         if (ok) {
-            __syncwarp();
-            // column c = lane of L^{-1}, by substitution along the columns of L (the same sums, row by row)
-            if (lane < KM) {
 #pragma unroll
-                for (int i = 0; i < KM; ++i) a[i] = i == lane ? 1.f : 0.f;
-#pragma unroll 1
-                for (int l = 0; l < k; ++l) {
-                    const float x = a[0] / Ls[l][l];
-#pragma unroll
-                    for (int q = 1; q < KM; ++q) a[q - 1] = fmaf(-x, Ls[l + q][l], a[q]);
-                    Xi[l][lane] = x;
-                }
+            for (int m = 0; m < E; ++m) {
+                const int i = i0 + m * (TCH / KM);
+                if (i < k && c < k) M.S[c * k + i] = x[m];     // S = L^{-T}
             }
-            __syncwarp();
-            for (int o = lane; o < k * k; o += 32) M.S[o] = Xi[o % k][o / k];   // S = L^{-T}
-            if (attempt > 0 && lane == 0 && M.flag) atomicAdd(M.flag, 1);
+            if (attempt > 0 && tid == 0 && M.flag) atomicAdd(M.flag, 1);
             return;
         }
         shift = (shift == 0.f ? 1e-7f : shift * 100.f) * (tr > 0.f ? tr / k : 1.f);
-        __syncwarp();
+        __syncthreads();
     }
     // no factorisation: leave S as identity and count it
-    for (int o = lane; o < k * k; o += 32) M.S[o] = o / k == o % k ? 1.f : 0.f;
-    if (lane == 0 && M.flag) { atomicAdd(M.flag, 1000); atomicAdd(M.flag + 6, 1); }
+    for (int o = tid; o < k * k; o += TCH) M.S[o] = o / k == o % k ? 1.f : 0.f;
+    if (tid == 0 && M.flag) { atomicAdd(M.flag, 1000); atomicAdd(M.flag + 6, 1); }
 }
 
 template <int KM>
 cudaError_t pow_launch(const PowGroup& g, int stage, int arg, cudaStream_t st) {
     switch (stage) {
-        case 0: pow_t_kernel<KM><<<g.tot_t, TP, 0, st>>>(g, arg); break;
-        case 1: pow_n_kernel<KM><<<g.tot_n, TP, 0, st>>>(g); break;
+        case 0: {
+            const cudaError_t e = cudaFuncSetAttribute(pow_t_kernel<KM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPowTSmem<KM>);
+            if (e != cudaSuccess) return e;
+            pow_t_kernel<KM><<<g.tot_t, TM, kPowTSmem<KM>, st>>>(g, arg);
+            break;
+        }
+        case 1: {
+            const cudaError_t e = cudaFuncSetAttribute(pow_n_kernel<KM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPowNSmem<KM>);
+            if (e != cudaSuccess) return e;
+            pow_n_kernel<KM><<<g.tot_n * (PC / NR), TM, kPowNSmem<KM>, st>>>(g);
+            break;
+        }
         case 2: pow_r_kernel<KM><<<g.tot_r, TP, 0, st>>>(g); break;
         case 3: pow_apply_kernel<KM><<<g.tot_r, TP, 0, st>>>(g, arg); break;
-        case 4: pow_chol_kernel<KM><<<g.nmat, TCH, 0, st>>>(g, arg, 0); break;
-        case 5: pow_chol_kernel<KM><<<g.nmat, TCH, 0, st>>>(g, arg, 1); break;
+        case 4: pow_chol_kernel<KM><<<g.nmat * CCH, TCH, 0, st>>>(g, arg, 0); break;
+        case 5: pow_chol_kernel<KM><<<g.nmat * CCH, TCH, 0, st>>>(g, arg, 1); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
