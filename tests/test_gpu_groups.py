@@ -47,3 +47,20 @@ def test_refreshes_of_mixed_widths_and_more_than_a_launch():
     ks = (8, 16, 20, 32)
     mats = [(40 + 8 * (j % 5), 96 + 4 * (j % 7), 4, ks[j % 4]) for j in range(36)]
     _group_equals_single(mats, tau=2, optimizer="msgd", lr=0.05, beta1=0.9)
+
+
+@pytest.mark.parametrize("opt", ["msgd", "adam"])
+def test_ragged_sizes_grouped(opt):
+    """The unfused steps of several matrices share their launches: sizes on both sides of the 64 x 64 tiles
+    and of the products' K slices, rows of odd length, both orientations, the full basis beside
+    truncated ones."""
+    mats = [(20, 31, 3, 8), (63, 65, 5, 12), (64, 129, 4, 16), (129, 63, 7, 24), (333, 777, 9, 24),
+            (777, 333, 6, 33), (65, 257, 5, 0), (129, 65, 3, 0)]
+    _group_equals_single(mats, tau=2, optimizer=opt, lr=0.01, beta1=0.9)
+
+
+def test_tcgen05_sizes_grouped():
+    """m' = 136 and 200 end in a 128-row tile whose lower half holds no row, k = 20 to 132 take the
+    small and the blocked eigenproblem beside each other."""
+    mats = [(136, 264, 16, 20), (264, 136, 16, 64), (200, 328, 32, 68), (192, 136, 20, 128), (256, 520, 16, 132)]
+    _group_equals_single(mats, dtype="bf16", tau=2, optimizer="adam", lr=0.01, beta1=0.9, beta2=0.99)
