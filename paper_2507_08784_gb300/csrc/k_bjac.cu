@@ -31,6 +31,7 @@ namespace {
 // Per matrix, per CTA: the squared diagonal and off-diagonal sums of H (part[2 (mat G + cta)]), from its
 // 128 x 128 blocks on and below the diagonal.
 __global__ void __launch_bounds__(256) bjac_norms_kernel(const __grid_constant__ BjacGroup g, float* part) {
+    chain_begin();
     const BjacMat& M = g.mat[blockIdx.y];
     const int n = M.n;
     float d = 0.f, o = 0.f;
@@ -68,6 +69,7 @@ __global__ void __launch_bounds__(256) bjac_norms_kernel(const __grid_constant__
 // of W's rows (WR = 2): the same bits.
 template <int WR>
 __global__ void __launch_bounds__(pair::PTHREADS, 1) bjac_pair_kernel(const __grid_constant__ BjacGroup g, int full) {
+    chain_begin();
     using namespace pair;
     constexpr int PARTS = 8 / WR, ROWS = 16 * WR;
     extern __shared__ __align__(16) float psm[];
@@ -131,14 +133,14 @@ cudaError_t bjac_pairs(BjacGroup& g, int full, cudaStream_t st) {
     e = parts ? cudaFuncSetAttribute(bjac_pair_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair::kSmem)
               : cudaFuncSetAttribute(bjac_pair_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair::kSmem);
     if (e != cudaSuccess) return e;
-    if (parts) bjac_pair_kernel<2><<<4 * tiles, pair::PTHREADS, pair::kSmem, st>>>(g, full);
-    else bjac_pair_kernel<8><<<tiles, pair::PTHREADS, pair::kSmem, st>>>(g, full);
+    if (parts) launch_chain(bjac_pair_kernel<2>, 4 * tiles, pair::PTHREADS, pair::kSmem, st, g, full);
+    else launch_chain(bjac_pair_kernel<8>, tiles, pair::PTHREADS, pair::kSmem, st, g, full);
     return cudaGetLastError();
 }
 
 cudaError_t bjac_norms(const BjacGroup& g, float* part, cudaStream_t st) {
     if (g.nmat <= 0) return cudaSuccess;
-    bjac_norms_kernel<<<dim3(kBjacNormCtas, g.nmat), 256, 0, st>>>(g, part);
+    launch_chain(bjac_norms_kernel, dim3(kBjacNormCtas, g.nmat), 256, 0, st, g, part);
     return cudaGetLastError();
 }
 

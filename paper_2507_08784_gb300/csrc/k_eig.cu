@@ -71,6 +71,7 @@ __device__ __forceinline__ void small_product(const float* A, const float* B, in
 
 template <int LIM>
 __global__ void __launch_bounds__(8 * LIM, 1) eig_small_kernel(const __grid_constant__ EigGroup g) {
+    chain_begin();
     constexpr int R = 2 * LIM, NT = 8 * LIM;
     extern __shared__ __align__(16) float esm[];
     float* S = esm;
@@ -567,7 +568,7 @@ cudaError_t launch_small(const EigGroup& g, cudaStream_t st) {
     const cudaError_t e = cudaFuncSetAttribute(eig_small_kernel<LIM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)small_smem<LIM>());
     if (e != cudaSuccess) return e;
-    eig_small_kernel<LIM><<<g.nmat, 8 * LIM, small_smem<LIM>(), st>>>(g);
+    launch_chain(eig_small_kernel<LIM>, g.nmat, 8 * LIM, small_smem<LIM>(), st, g);
     return cudaGetLastError();
 }
 

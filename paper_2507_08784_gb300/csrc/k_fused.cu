@@ -189,6 +189,7 @@ __device__ __forceinline__ StreamSmem carve_stream(unsigned char* smem, int mp, 
 // ------------------------------------------------------------------------------------------
 template <int BN, typename GT>
 __global__ void __launch_bounds__(NT, 1) stream_kernel(const __grid_constant__ StreamGroup g) {
+    chain_begin();
     extern __shared__ __align__(16) unsigned char smem[];
     int mi = 0;
     while (mi + 1 < g.nmat && blockIdx.x >= static_cast<unsigned>(g.mat[mi + 1].strip0)) ++mi;
@@ -327,6 +328,7 @@ __global__ void __launch_bounds__(NT, 1) stream_kernel(const __grid_constant__ S
 // ------------------------------------------------------------------------------------------
 template <int BN>
 __global__ void __launch_bounds__(NTU) update_kernel_fused(const __grid_constant__ UpdateGroup g) {
+    chain_begin();
     extern __shared__ __align__(16) unsigned char smem[];
     int mi = 0;
     while (mi + 1 < g.nmat && blockIdx.x >= static_cast<unsigned>(g.mat[mi + 1].strip0)) ++mi;
@@ -462,7 +464,7 @@ static cudaError_t launch_stream(const StreamGroup& g, size_t smem, cudaStream_t
                                              227 * 1024);
         if (ea != cudaSuccess) return ea;
     }
-    stream_kernel<BN, GT><<<g.total_strips, NT, smem, st>>>(g);
+    launch_chain(stream_kernel<BN, GT>, g.total_strips, NT, smem, st, g);
     return cudaGetLastError();
 }
 
@@ -485,7 +487,7 @@ static cudaError_t launch_update(const UpdateGroup& g, size_t smem, cudaStream_t
                                              227 * 1024);
         if (ea != cudaSuccess) return ea;
     }
-    update_kernel_fused<BN><<<g.total_strips, NTU, smem, st>>>(g);
+    launch_chain(update_kernel_fused<BN>, g.total_strips, NTU, smem, st, g);
     return cudaGetLastError();
 }
 

@@ -694,11 +694,13 @@ __device__ __forceinline__ void compose_strip(const StreamGroup& g, const TmaMap
 
 template <typename GT, int NQ>
 __global__ void __launch_bounds__(T, 1) stream_mma_kernel(const __grid_constant__ StreamGroup g) {
+    chain_begin();
     compose_strip<GT, NQ, false>(g, nullptr);
 }
 template <typename GT, int NQ>
 __global__ void __launch_bounds__(T, 1) stream_tma_kernel(const __grid_constant__ StreamGroup g,
                                                           const __grid_constant__ TmaMaps maps) {
+    chain_begin();
     compose_strip<GT, NQ, true>(g, &maps);
 }
 // dst = src (rows x cols, row-major, ld) in fragment order (frag_coord), up8(rows) x up8(cols) floats.
@@ -750,7 +752,7 @@ static cudaError_t launch_mma(const StreamGroup& g, size_t smem, cudaStream_t st
                                              227 * 1024);
         if (ea != cudaSuccess) return ea;
     }
-    stream_mma_kernel<GT, NQ><<<g.total_strips, T, smem, st>>>(g);
+    launch_chain(stream_mma_kernel<GT, NQ>, g.total_strips, T, smem, st, g);
     return cudaGetLastError();
 }
 template <typename GT, int NQ>
@@ -760,7 +762,7 @@ static cudaError_t launch_tma(const StreamGroup& g, const TmaMaps& maps, size_t 
                                              227 * 1024);
         if (ea != cudaSuccess) return ea;
     }
-    stream_tma_kernel<GT, NQ><<<g.total_strips, T, smem, st>>>(g, maps);
+    launch_chain(stream_tma_kernel<GT, NQ>, g.total_strips, T, smem, st, g, maps);
     return cudaGetLastError();
 }
 

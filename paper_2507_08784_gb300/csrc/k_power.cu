@@ -89,6 +89,7 @@ template <int KM> constexpr size_t kPowNSmem = sizeof(float) * NS * (NR * NP + P
 // four columns a thread on half the warps 20.5).
 template <int KM>
 __global__ void __launch_bounds__(TM) pow_t_kernel(const __grid_constant__ PowGroup g, int apply_s) {
+    chain_begin();
     constexpr int KPT = KM / 4, RB = KM == 16 ? 8 : 4;
     extern __shared__ __align__(16) float stage[];             // PS blocks of PR x PC of Mbar, then of PR x KM of Q
     __shared__ __align__(16) float Zs[PC * KM];
@@ -199,6 +200,7 @@ __global__ void __launch_bounds__(TM) pow_t_kernel(const __grid_constant__ PowGr
 // one row by KM / 4 (conv stack: 20.4 -> 16.4 us; 64-row tiles, four rows a thread 20.5).
 template <int KM>
 __global__ void __launch_bounds__(TM) pow_n_kernel(const __grid_constant__ PowGroup g) {
+    chain_begin();
     constexpr int KPT = KM / 4;
     extern __shared__ __align__(16) float stage[];             // NS blocks of NR x NP of Mbar, then of PC x KM of Z
     int mi = 0;
@@ -283,6 +285,7 @@ __global__ void __launch_bounds__(TM) pow_n_kernel(const __grid_constant__ PowGr
 // Q[a][:] = (sum over chunks of part[chunk][:][a]) S for a tile of 64 rows; Gram partial into G.
 template <int KM>
 __global__ void __launch_bounds__(TP) pow_r_kernel(const __grid_constant__ PowGroup g) {
+    chain_begin();
     constexpr int KPT = KM / 4;
     __shared__ __align__(16) float Qs[PC * KM];
     __shared__ __align__(16) float Q2[PC * KM];
@@ -326,6 +329,7 @@ __global__ void __launch_bounds__(TP) pow_r_kernel(const __grid_constant__ PowGr
 // into G when gram.
 template <int KM>
 __global__ void __launch_bounds__(TP) pow_apply_kernel(const __grid_constant__ PowGroup g, int gram) {
+    chain_begin();
     __shared__ __align__(16) float Qs[PC * KM];
     __shared__ __align__(16) float Q2[PC * KM];
     __shared__ __align__(16) float Ss[KM * KM];
@@ -371,6 +375,7 @@ __device__ __forceinline__ float quotient(float num, float den) {
 template <int KM>
 __global__ void __cluster_dims__(CCH, 1, 1) __launch_bounds__(TCH)
     pow_chol_kernel(const __grid_constant__ PowGroup g, int use_t_tiles, int mode) {
+    chain_begin();
     __shared__ float Gs[KM][KM + 1];
     __shared__ float colj[2][KM], rowj[2][KM];
     const PowMat& M = g.mat[blockIdx.x / CCH];
@@ -485,19 +490,19 @@ cudaError_t pow_launch(const PowGroup& g, int stage, int arg, cudaStream_t st) {
         case 0: {
             const cudaError_t e = cudaFuncSetAttribute(pow_t_kernel<KM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPowTSmem<KM>);
             if (e != cudaSuccess) return e;
-            pow_t_kernel<KM><<<g.tot_t, TM, kPowTSmem<KM>, st>>>(g, arg);
+            launch_chain(pow_t_kernel<KM>, g.tot_t, TM, kPowTSmem<KM>, st, g, arg);
             break;
         }
         case 1: {
             const cudaError_t e = cudaFuncSetAttribute(pow_n_kernel<KM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPowNSmem<KM>);
             if (e != cudaSuccess) return e;
-            pow_n_kernel<KM><<<g.tot_n * (PC / NR), TM, kPowNSmem<KM>, st>>>(g);
+            launch_chain(pow_n_kernel<KM>, g.tot_n * (PC / NR), TM, kPowNSmem<KM>, st, g);
             break;
         }
-        case 2: pow_r_kernel<KM><<<g.tot_r, TP, 0, st>>>(g); break;
-        case 3: pow_apply_kernel<KM><<<g.tot_r, TP, 0, st>>>(g, arg); break;
-        case 4: pow_chol_kernel<KM><<<g.nmat * CCH, TCH, 0, st>>>(g, arg, 0); break;
-        case 5: pow_chol_kernel<KM><<<g.nmat * CCH, TCH, 0, st>>>(g, arg, 1); break;
+        case 2: launch_chain(pow_r_kernel<KM>, g.tot_r, TP, 0, st, g); break;
+        case 3: launch_chain(pow_apply_kernel<KM>, g.tot_r, TP, 0, st, g, arg); break;
+        case 4: launch_chain(pow_chol_kernel<KM>, g.nmat * CCH, TCH, 0, st, g, arg, 0); break;
+        case 5: launch_chain(pow_chol_kernel<KM>, g.nmat * CCH, TCH, 0, st, g, arg, 1); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

@@ -160,6 +160,7 @@ __device__ __forceinline__ void column_stats(const float* A, int rows, int64_t l
 // norm: thousands of plane rotations let the norms drift by a few ulp each) there, then a CTA per
 // row gathers the row.  One CTA sorting and moving everything took 10.3 ms for n = 2048.
 __global__ void __launch_bounds__(1024) sort_rank_kernel(const __grid_constant__ SortGroup g) {
+    chain_begin();
     const SortMat& M = g.mat[blockIdx.y];
     const int n = M.n, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     if ((int)blockIdx.x * 32 >= n) return;
@@ -188,6 +189,7 @@ __global__ void __launch_bounds__(1024) sort_rank_kernel(const __grid_constant__
     if (col < n && ty < n) M.Out[(size_t)ty * n + col] = M.scale[col] * M.V[(size_t)ty * n + M.order[col]];
 }
 __global__ void __launch_bounds__(256) sort_gather_kernel(const __grid_constant__ SortGroup g) {
+    chain_begin();
     extern __shared__ float srow[];
     const SortMat& M = g.mat[blockIdx.y];
     const int n = M.n;
@@ -202,6 +204,7 @@ __global__ void __launch_bounds__(256) sort_gather_kernel(const __grid_constant_
 
 // The largest-magnitude entry of each column of Q (m' x k) positive; a CTA per 32 columns.
 __global__ void __launch_bounds__(1024) fix_signs_group_kernel(const __grid_constant__ FinishGroup g) {
+    chain_begin();
     const FinishMat& M = g.mat[blockIdx.y];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, col = blockIdx.x * 32 + tx;
     if ((int)blockIdx.x * 32 >= M.k) return;
@@ -390,9 +393,9 @@ cudaError_t sort_group(const SortGroup& g, cudaStream_t st) {
     if (g.nmat <= 0) return cudaSuccess;
     int n = 0;
     for (int i = 0; i < g.nmat; ++i) n = g.mat[i].n > n ? g.mat[i].n : n;
-    sort_rank_kernel<<<dim3((n + 31) / 32, g.nmat), 1024, 0, st>>>(g);
+    launch_chain(sort_rank_kernel, dim3((n + 31) / 32, g.nmat), 1024, 0, st, g);
     if (n <= 32) return cudaGetLastError();
-    sort_gather_kernel<<<dim3(n < 1024 ? n : 1024, g.nmat), 256, sizeof(float) * n, st>>>(g);
+    launch_chain(sort_gather_kernel, dim3(n < 1024 ? n : 1024, g.nmat), 256, sizeof(float) * n, st, g);
     return cudaGetLastError();
 }
 
@@ -572,6 +575,7 @@ __device__ __forceinline__ bool chol_diag(float* D, float thresh, int lane) {
 }
 
 __global__ void __launch_bounds__(CWARPS * 32) chol_group_kernel(const __grid_constant__ CholGroup g) {
+    chain_begin();
     extern __shared__ __align__(16) float csm[];
     const CholMat& M = g.mat[blockIdx.x];
     const int n = M.n, nb = (n + CB - 1) / CB, t = threadIdx.x, warp = t >> 5, lane = t & 31;
@@ -694,6 +698,7 @@ __global__ void __launch_bounds__(CWARPS * 32) chol_group_kernel(const __grid_co
 constexpr size_t kHhSmem = sizeof(float) * CBLK * (2 * kCholMaxBlocks);
 
 __global__ void __launch_bounds__(CWARPS * 32) hh_lu_group_kernel(const __grid_constant__ FinishGroup g) {
+    chain_begin();
     extern __shared__ __align__(16) float hsm[];
     const FinishMat& M = g.mat[blockIdx.x];
     const int k = M.k, nb = (k + CB - 1) / CB, t = threadIdx.x, warp = t >> 5, lane = t & 31;
@@ -779,6 +784,7 @@ __global__ void __launch_bounds__(CWARPS * 32) hh_lu_group_kernel(const __grid_c
 __host__ __device__ __forceinline__ int tail_threads(int n) { return (n * ((n + 1) / 2) + 31) / 32 * 32; }
 
 __global__ void __launch_bounds__(512) tail_ritz_kernel(const __grid_constant__ TailGroup g) {
+    chain_begin();
     constexpr int P = 33;
     __shared__ float H[32 * P], V[32 * P];
     __shared__ float4 rot[16];                             // c, s, then p and q as row offsets
@@ -917,6 +923,7 @@ __global__ void __launch_bounds__(512) tail_ritz_kernel(const __grid_constant__ 
 // (m' = 512, k = 16: 11 us; fix_signs and hh_top_kernel 13 + 17 us).
 template <int KM>
 __global__ void __launch_bounds__(1024) tail_top_kernel(const __grid_constant__ TailGroup g) {
+    chain_begin();
     constexpr int RG = 1024 / KM;
     __shared__ float sbest[RG][KM + 1], sval[RG][KM + 1];
     __shared__ int sidx[RG][KM + 1];
@@ -995,6 +1002,7 @@ __global__ void __launch_bounds__(1024) tail_top_kernel(const __grid_constant__ 
 // substitution against Utilde, the others from L1), Yt = Y T^T, and the copies of both (17 us for eight
 // matrices up to m' = 512; six kernels a matrix, 29 us together).
 __global__ void __launch_bounds__(256) tail_rows_kernel(const __grid_constant__ TailGroup g) {
+    chain_begin();
     __shared__ float Ws[32][33], Ts[32][33], ys[2][32][33];
     const TailMat& M = g.mat[blockIdx.y];
     const int k = M.k, mp = M.mp, tp = M.tp, a0 = blockIdx.x * 32;
@@ -1081,11 +1089,11 @@ cudaError_t finish_group(const FinishGroup& g, int stage, cudaStream_t st) {
         if (stage == 2 && (g.mat[i].k > CB * kCholMaxBlocks || g.mat[i].k % 4)) return cudaErrorInvalidValue;
     }
     if (stage == 1) {                                   // column signs of Q
-        fix_signs_group_kernel<<<dim3((kmax + 31) / 32, g.nmat), 1024, 0, st>>>(g);
+        launch_chain(fix_signs_group_kernel, dim3((kmax + 31) / 32, g.nmat), 1024, 0, st, g);
     } else {                                            // Householder top block
         const cudaError_t ea = cudaFuncSetAttribute(hh_lu_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHhSmem);
         if (ea != cudaSuccess) return ea;
-        hh_lu_group_kernel<<<g.nmat, CWARPS * 32, kHhSmem, st>>>(g);
+        launch_chain(hh_lu_group_kernel, g.nmat, CWARPS * 32, kHhSmem, st, g);
     }
     return cudaGetLastError();
 }
@@ -1098,10 +1106,10 @@ cudaError_t tail_group(const TailGroup& g, int stage, cudaStream_t st) {
         kmax = g.mat[i].k > kmax ? g.mat[i].k : kmax;
         tp = g.mat[i].tp > tp ? g.mat[i].tp : tp;
     }
-    if (stage == 0) tail_ritz_kernel<<<g.nmat, tail_threads(kmax), 0, st>>>(g);
-    else if (stage == 2) tail_rows_kernel<<<dim3((tp + 31) / 32, g.nmat), 256, 0, st>>>(g);
-    else if (kmax <= 16) tail_top_kernel<16><<<g.nmat, 1024, 0, st>>>(g);
-    else tail_top_kernel<32><<<g.nmat, 1024, 0, st>>>(g);
+    if (stage == 0) launch_chain(tail_ritz_kernel, g.nmat, tail_threads(kmax), 0, st, g);
+    else if (stage == 2) launch_chain(tail_rows_kernel, dim3((tp + 31) / 32, g.nmat), 256, 0, st, g);
+    else if (kmax <= 16) launch_chain(tail_top_kernel<16>, g.nmat, 1024, 0, st, g);
+    else launch_chain(tail_top_kernel<32>, g.nmat, 1024, 0, st, g);
     return cudaGetLastError();
 }
 
@@ -1119,7 +1127,7 @@ cudaError_t chol_group(const CholGroup& g, cudaStream_t st) {
                                                    (int)kCholSmem);
         if (ea != cudaSuccess) return ea;
     }
-    chol_group_kernel<<<g.nmat, CWARPS * 32, smem, st>>>(g);
+    launch_chain(chol_group_kernel, g.nmat, CWARPS * 32, smem, st, g);
     return cudaGetLastError();
 }
 

@@ -12,6 +12,7 @@ constexpr int LK = 16;
 // C(j, b) = sum_p A(j, p) B(p, b) for a 64 x 64 tile; then for each row j the partial
 // sum over the tile's columns of C'(j, b) v_j[b], with C' = C (dense) or Mbar - C (wy).
 __global__ void __launch_bounds__(256) lambda_kernel(const __grid_constant__ LambdaGroup lg) {
+    chain_begin();
     int mi = 0;
     while (mi + 1 < lg.nmat && lg.tile0[mi + 1] <= (int)blockIdx.x) ++mi;
     const LambdaArgs& a = lg.mat[mi];
@@ -101,6 +102,7 @@ __device__ __forceinline__ void lm_mma(float (&d)[4], uint32_t a0, uint32_t a1, 
 }
 
 __global__ void __launch_bounds__(128) lambda_mma_kernel(const __grid_constant__ LambdaGroup lg) {
+    chain_begin();
     int mi = 0;
     while (mi + 1 < lg.nmat && lg.tile0[mi + 1] <= (int)blockIdx.x) ++mi;
     const LambdaArgs& a = lg.mat[mi];
@@ -216,7 +218,7 @@ cudaError_t lambda_partials(const LambdaGroup& all, cudaStream_t st) {
                 tiles += a.ntiles * ((a.mp + LT - 1) / LT);
             }
         if (!tiles) continue;
-        if (mode == 0) lambda_mma_kernel<<<tiles, 128, 0, st>>>(g);   // dense U: a dense contraction
+        if (mode == 0) launch_chain(lambda_mma_kernel, tiles, 128, 0, st, g);   // dense U: a dense contraction
         else lambda_kernel<<<tiles, 256, 0, st>>>(g);
     }
     return cudaGetLastError();
@@ -394,6 +396,7 @@ __device__ __forceinline__ void select_top_r_block(const SelectMat& M, unsigned 
 }
 
 __global__ void __launch_bounds__(1024) select_group_kernel(const __grid_constant__ SelectGroup g) {
+    chain_begin();
     extern __shared__ unsigned long long keys[];
     const SelectMat& M = g.mat[blockIdx.x];
     if (M.do_select) select_top_r_block(M, keys);           // otherwise J was supplied
@@ -411,6 +414,7 @@ __global__ void __launch_bounds__(1024) select_group_kernel(const __grid_constan
 // Output o of the group: matrix i owns [out0, out0 + m' r) for P (row-major m' x r) and, when
 // rbar is set, the next r n' for Rbar.
 __global__ void __launch_bounds__(256) pr_kernel(const __grid_constant__ SelectGroup g) {
+    chain_begin();
     const int64_t o = (int64_t)blockIdx.x * 256 + threadIdx.x;
     int mi = 0;
     while (mi + 1 < g.nmat && o >= g.mat[mi + 1].out0) ++mi;
@@ -455,6 +459,7 @@ __global__ void __launch_bounds__(256) pr_kernel(const __grid_constant__ SelectG
 // lambda-bar_j = d_j * sum_t part[t][j]: block (x, matrix) covers 32 consecutive j (lanes)
 // with its 32 warps taking every 32nd tile; the warp sums are added in warp order.
 __global__ void __launch_bounds__(1024) lambda_reduce_kernel(const __grid_constant__ SelectGroup g) {
+    chain_begin();
     const SelectMat& M = g.mat[blockIdx.y];
     if (!M.do_select) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -480,7 +485,7 @@ cudaError_t select_group(const SelectGroup& g, cudaStream_t st, int stages) {
     for (int i = 0; i < g.nmat; ++i) maxmp = g.mat[i].mp > maxmp ? g.mat[i].mp : maxmp;
     cudaError_t e = cudaSuccess;
     if (stages & 1) {
-        lambda_reduce_kernel<<<dim3((maxmp + 31) / 32, g.nmat), 1024, 0, st>>>(g);
+        launch_chain(lambda_reduce_kernel, dim3((maxmp + 31) / 32, g.nmat), 1024, 0, st, g);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (!(stages & 2)) return cudaSuccess;
@@ -490,21 +495,23 @@ cudaError_t select_group(const SelectGroup& g, cudaStream_t st, int stages) {
         const cudaError_t ea = cudaFuncSetAttribute(select_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (ea != cudaSuccess) return ea;
     }
-    select_group_kernel<<<g.nmat, 1024, sizeof(unsigned long long) * npow2, st>>>(g);
+    launch_chain(select_group_kernel, g.nmat, 1024, sizeof(unsigned long long) * npow2, st, g);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (g.total_out <= 0) return cudaSuccess;              // every P formed by the caller
-    pr_kernel<<<(unsigned)((g.total_out + 255) / 256), 256, 0, st>>>(g);
+    launch_chain(pr_kernel, (unsigned)((g.total_out + 255) / 256), 256, 0, st, g);
     return cudaGetLastError();
 }
 
 namespace {
 __global__ void wy_gather_kernel(const float* Yt, const int32_t* J, int r, int k, float* YtJ) {
+    chain_begin();
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= r * k) return;
     const int q = e / k, c = e % k;
     YtJ[e] = Yt[(int64_t)J[q] * k + c];
 }
 __global__ void wy_fix_kernel(float* P, const int32_t* J, const float* dsign, int mp, int r, int k) {
+    chain_begin();
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)mp * r) return;
     const int a = static_cast<int>(e / r), q = static_cast<int>(e % r);
@@ -516,13 +523,13 @@ __global__ void wy_fix_kernel(float* P, const int32_t* J, const float* dsign, in
 }  // namespace
 
 cudaError_t wy_columns_gather(const float* Yt, const int32_t* J, int r, int k, float* YtJ, cudaStream_t st) {
-    wy_gather_kernel<<<(r * k + 255) / 256, 256, 0, st>>>(Yt, J, r, k, YtJ);
+    launch_chain(wy_gather_kernel, (r * k + 255) / 256, 256, 0, st, Yt, J, r, k, YtJ);
     return cudaGetLastError();
 }
 
 cudaError_t wy_columns_fix(float* P, const int32_t* J, const float* dsign, int mp, int r, int k, cudaStream_t st) {
     const int64_t n = (int64_t)mp * r;
-    wy_fix_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(P, J, dsign, mp, r, k);
+    launch_chain(wy_fix_kernel, (unsigned)((n + 255) / 256), 256, 0, st, P, J, dsign, mp, r, k);
     return cudaGetLastError();
 }
 

@@ -75,6 +75,7 @@ __device__ __forceinline__ void gemm_tile(const GemmTile& g, int i0, int j0, int
 }
 
 __global__ void __launch_bounds__(256) gemm_f32_kernel(GemmDesc d, int kchunk) {
+    chain_begin();
     const bool split = kchunk > 0;                  // blockIdx.z = K slice (batch == 1)
     const int z = split ? 0 : blockIdx.z;
     float* C = d.C + z * d.sCz;
@@ -106,6 +107,7 @@ __global__ void __launch_bounds__(256) gemm_f32_kernel(GemmDesc d, int kchunk) {
 
 // C = alpha * sum_z ws[z] + beta * C, slices added in order.
 __global__ void gemm_splitk_reduce(GemmDesc d, int splits) {
+    chain_begin();
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)d.M * d.N) return;
     const int i = static_cast<int>(e / d.N), j = static_cast<int>(e % d.N);
@@ -135,7 +137,7 @@ cudaError_t gemm_f32(const GemmDesc& d, cudaStream_t st) {
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         const int64_t total = (int64_t)d.M * d.N;
-        gemm_splitk_reduce<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(d, splits);
+        launch_chain(gemm_splitk_reduce, (unsigned)((total + 255) / 256), 256, 0, st, d, splits);
         return cudaGetLastError();
     }
     dim3 grid((d.N + GB_N - 1) / GB_N, (d.M + GB_M - 1) / GB_M, d.batch);
@@ -153,6 +155,7 @@ namespace {
 constexpr int CT = 32;
 
 __global__ void __launch_bounds__(256) compose_kernel(const __grid_constant__ ComposeGroup g) {
+    chain_begin();
     int mi = 0;
     while (mi + 1 < g.nmat && g.tile0[mi + 1] <= (int)blockIdx.x) ++mi;
     const ComposeArgs& a = g.mat[mi];
@@ -255,6 +258,7 @@ cudaError_t compose(ComposeGroup& g, cudaStream_t st) {
 // ------------------------------------------------------------------------------------------
 namespace {
 __global__ void __launch_bounds__(256) update_kernel(const __grid_constant__ UpdateTileGroup grp) {
+    chain_begin();
     int mi = 0;
     while (mi + 1 < grp.nmat && grp.tile0[mi + 1] <= (int)blockIdx.x) ++mi;
     const UpdateArgs& a = grp.mat[mi];
@@ -371,6 +375,7 @@ __host__ __device__ __forceinline__ int gemm_chunk(const GemmMat& M) {
 }
 
 __global__ void __launch_bounds__(256) gemm_group_kernel(const __grid_constant__ GemmGroup g) {
+    chain_begin();
     const int tile = blockIdx.x;
     int lo = 0, hi = g.nmat - 1;
     while (lo < hi) {
@@ -400,6 +405,7 @@ __global__ void __launch_bounds__(256) gemm_group_kernel(const __grid_constant__
 
 // C = alpha times the sum of the K slices, added in order.
 __global__ void __launch_bounds__(256) gemm_group_reduce(const __grid_constant__ GemmGroup g) {
+    chain_begin();
     const GemmMat& M = g.mat[blockIdx.y];
     if (M.splits <= 1) return;
     const float alpha = M.alpha != 0.f ? M.alpha : 1.f;
@@ -434,7 +440,7 @@ cudaError_t gemm_group_f32(GemmGroup& g, cudaStream_t st) {
     }
     if (g.total_tiles <= 0) return cudaSuccess;
     gemm_group_kernel<<<g.total_tiles, 256, 0, st>>>(g);
-    if (reduce) gemm_group_reduce<<<dim3(64, g.nmat), 256, 0, st>>>(g);
+    if (reduce) launch_chain(gemm_group_reduce, dim3(64, g.nmat), 256, 0, st, g);
     return cudaGetLastError();
 }
 

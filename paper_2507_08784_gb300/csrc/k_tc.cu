@@ -232,6 +232,7 @@ struct NoStore { __device__ bool operator()(uint32_t) const { return false; } };
 // Ops without epilogue data.
 struct NoData {
     static constexpr int kEpi = 8;
+    static constexpr bool kChained = true;            // launched by launch_chain
     static constexpr int kHalves = 1;                 // 2: a data stage is 64 rows of the tile, even ones the upper
     static __device__ __forceinline__ int ndata(const TcGroup&, const Tile&) { return 0; }
     static __device__ __forceinline__ uint32_t data_tx(const TcGroup&, const Tile&, int) { return 0; }
@@ -240,6 +241,7 @@ struct NoData {
 
 template <class Op>
 __global__ void __launch_bounds__(threads_of<Op>(), 1) tc_kernel(const __grid_constant__ TcGroup g) {
+    chain_begin();
     constexpr int kEpiWarps = Op::kEpi;
     constexpr int kProdWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1, kDataWarp = kEpiWarps + 2;
     extern __shared__ uint8_t dyn_smem[];
@@ -387,6 +389,7 @@ __device__ __forceinline__ void mma_slice(uint32_t d, uint32_t a, uint32_t b, in
 // m' x n' x N), B = P_prev^T (rpad x m').
 // ------------------------------------------------------------------------------------------
 struct PrevProj : NoData {
+    static constexpr bool kChained = false;
     static __device__ __forceinline__ int nk(const TcGroup& g, const Tile& t) { return (g.mat[t.mat].mp + 31) / 32; }
     static __device__ __forceinline__ void decode(const TcMat& M, int lt, int& ct, int& i0, int& ni) {
         ct = lt / M.ng;
@@ -447,6 +450,7 @@ struct PrevProj : NoData {
 // flight while the other is worked on.
 // ------------------------------------------------------------------------------------------
 struct Compose {
+    static constexpr bool kChained = false;
     static constexpr int kEpi = 16;
     static constexpr int BN = 64;
     static constexpr int kHalves = 2;
@@ -562,6 +566,7 @@ struct Compose {
 // K = m'; the epilogue writes W^T[c][q] (rounded to TF32).  A = Mbar^T (n' x m'), B = Y^T (kpad x m').
 // ------------------------------------------------------------------------------------------
 struct WBar : NoData {
+    static constexpr bool kChained = false;
     static __device__ __forceinline__ int nk(const TcGroup& g, const Tile& t) { return (g.mat[t.mat].mp + 31) / 32; }
     static __device__ __forceinline__ uint32_t tx_bytes(const TcGroup& g, const Tile& t, int) {
         return 2u * 16384u + (uint32_t)g.mat[t.mat].kpad * 128u;
@@ -603,6 +608,7 @@ struct WBar : NoData {
 // the Mbar^T tile (128 columns x 128 rows fp32, 64 KiB).
 // ------------------------------------------------------------------------------------------
 struct Lambda {
+    static constexpr bool kChained = false;
     static constexpr int kEpi = 16;
     static constexpr int kHalves = 1;
     static __device__ __forceinline__ int nk(const TcGroup& g, const Tile& t) { return g.mat[t.mat].kpad / 32; }
@@ -664,6 +670,7 @@ struct Lambda {
 // the scores).  A = U^T (m' x m', TF32), B = Mbar^T (n' x m') in two 128-row boxes.
 // ------------------------------------------------------------------------------------------
 struct LambdaU : NoData {
+    static constexpr bool kChained = false;
     static constexpr int kEpi = 16;
     static __device__ __forceinline__ int nk(const TcGroup& g, const Tile& t) { return (g.mat[t.mat].mp + 31) / 32; }
     static __device__ __forceinline__ uint32_t tx_bytes(const TcGroup&, const Tile&, int) { return 3u * 16384u; }
@@ -801,6 +808,7 @@ struct BjacMul : NoData {
 // (r x k, rows past r read as zeros).
 // ------------------------------------------------------------------------------------------
 struct PBuild : NoData {
+    static constexpr bool kChained = false;
     static __device__ __forceinline__ int nk(const TcGroup& g, const Tile& t) { return g.mat[t.mat].kpad / 32; }
     static __device__ __forceinline__ uint32_t tx_bytes(const TcGroup& g, const Tile& t, int) {
         return 16384u + (uint32_t)g.mat[t.mat].rpad * 128u;
@@ -844,6 +852,7 @@ struct PBuild : NoData {
 // the 32 gathered Mbar(J_q, b) are loaded before any store so that they are all in flight.
 // ------------------------------------------------------------------------------------------
 struct RBar : NoData {
+    static constexpr bool kChained = false;
     static constexpr int kEpi = 16;
     static __device__ __forceinline__ int nk(const TcGroup& g, const Tile& t) { return g.mat[t.mat].kpad / 32; }
     static __device__ __forceinline__ uint32_t tx_bytes(const TcGroup&, const Tile&, int) { return 2u * 16384u; }
@@ -888,6 +897,7 @@ struct RBar : NoData {
 // bytes), plus Mbar^T's tile when uncompressed; X, Mo, Vo are stored back from the stage.
 // ------------------------------------------------------------------------------------------
 struct Update {
+    static constexpr bool kChained = false;
     static constexpr int kEpi = 16;
     static constexpr int kHalves = 1;
     static __device__ __forceinline__ int nk(const TcGroup& g, const Tile& t) {
@@ -1258,7 +1268,8 @@ cudaError_t launch(TcGroup& g, cudaStream_t st) {
     cudaError_t e = cudaFuncSetAttribute(tc_kernel<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int grid = std::min(g.total_tiles, g_sms);
-    tc_kernel<Op><<<grid, threads_of<Op>(), smem, st>>>(g);
+    if constexpr (Op::kChained) launch_chain(tc_kernel<Op>, grid, threads_of<Op>(), smem, st, g);
+    else tc_kernel<Op><<<grid, threads_of<Op>(), smem, st>>>(g);
     return cudaGetLastError();
 }
 
@@ -1276,6 +1287,7 @@ cudaError_t launch_update(TcGroup& g, cudaStream_t st) { return launch<Update>(g
 namespace {
 // The K slices of Pow added in order: out (rows x k, fp32) and outT (kpad x rows, TF32).
 __global__ void __launch_bounds__(256) pow_reduce_kernel(const __grid_constant__ TcGroup g) {
+    chain_begin();
     __shared__ float tile[32][33];
     const TcMat& M = g.mat[blockIdx.y];
     const int r0 = blockIdx.x * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -1303,7 +1315,7 @@ cudaError_t launch_pow(TcGroup& g, cudaStream_t st) {
     for (int i = 0; i < g.nmat; ++i)
         if (g.mat[i].splits > 1) rows = std::max(rows, g.mat[i].rows);
     if (e != cudaSuccess || !rows) return e;
-    pow_reduce_kernel<<<dim3((rows + 31) / 32, g.nmat), 256, 0, st>>>(g);
+    launch_chain(pow_reduce_kernel, dim3((rows + 31) / 32, g.nmat), 256, 0, st, g);
     return cudaGetLastError();
 }
 }  // namespace
@@ -1321,6 +1333,7 @@ namespace {
 // The row chunks' partial Gram matrices added in order into the first one: by all SMs, where the
 // one-CTA consumers waited out a load's latency per chunk and row (k = 128: 90 of a factor's 120 us).
 __global__ void __launch_bounds__(256) gram_sum_kernel(const __grid_constant__ TcGroup g) {
+    chain_begin();
     const TcMat& M = g.mat[blockIdx.y];
     const int64_t n4 = (int64_t)M.kpad * M.kpad / 4;
     float4* out = reinterpret_cast<float4*>(M.out);
@@ -1338,7 +1351,7 @@ __global__ void __launch_bounds__(256) gram_sum_kernel(const __grid_constant__ T
 cudaError_t launch_gram(TcGroup& g, cudaStream_t st) {
     const cudaError_t e = launch<Gram>(g, st);
     if (e != cudaSuccess || g.nmat <= 0) return e;
-    gram_sum_kernel<<<dim3(64, g.nmat), 256, 0, st>>>(g);
+    launch_chain(gram_sum_kernel, dim3(64, g.nmat), 256, 0, st, g);
     return cudaGetLastError();
 }
 cudaError_t launch_apply(TcGroup& g, cudaStream_t st) { return launch<Apply>(g, st); }
@@ -1352,6 +1365,7 @@ namespace {
 // P = U[:, J] (m' x r, row-major) and P^T (r x m'), rounded to TF32: the projector of a full basis.
 __global__ void gather_p_kernel(const float* __restrict__ U, int mp, const int32_t* __restrict__ J, int r,
                                 float* __restrict__ P, float* __restrict__ PT) {
+    chain_begin();
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)mp * r) return;
     const int q = (int)(e / mp), a = (int)(e % mp);
@@ -1361,6 +1375,7 @@ __global__ void gather_p_kernel(const float* __restrict__ U, int mp, const int32
 }
 
 __global__ void transpose_round_kernel(float* dst, int ldd, const float* src, int rows, int cols, int lds) {
+    chain_begin();
     __shared__ float tile[32][33];
     const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
     for (int y = threadIdx.y; y < 32; y += 8) {
@@ -1408,6 +1423,7 @@ __global__ void expire_kernel(int* err, int polls) {
 namespace {
 // lo = x - (x truncated to TF32): what a TF32 product of x leaves out
 __global__ void split_lo_kernel(const float4* src, float4* lo, int64_t n4) {
+    chain_begin();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
         const float4 v = src[i];
         auto l = [](float x) { return x - __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); };
@@ -1418,7 +1434,7 @@ __global__ void split_lo_kernel(const float4* src, float4* lo, int64_t n4) {
 
 cudaError_t split_lo(const float* src, float* lo, int64_t n, cudaStream_t st) {
     if (n % 4) return cudaErrorInvalidValue;
-    split_lo_kernel<<<(unsigned)std::min<int64_t>((n / 4 + 255) / 256, 8 * 152), 256, 0, st>>>(
+    launch_chain(split_lo_kernel, (unsigned)std::min<int64_t>((n / 4 + 255) / 256, 8 * 152), 256, 0, st, 
         reinterpret_cast<const float4*>(src), reinterpret_cast<float4*>(lo), n / 4);
     return cudaGetLastError();
 }
@@ -1430,13 +1446,13 @@ cudaError_t expire_wait(int* err, int polls, cudaStream_t st) {
 
 cudaError_t gather_p(const float* U, int mp, const int32_t* J, int r, float* P, float* PT, cudaStream_t st) {
     const int64_t n = (int64_t)mp * r;
-    gather_p_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(U, mp, J, r, P, PT);
+    launch_chain(gather_p_kernel, (unsigned)((n + 255) / 256), 256, 0, st, U, mp, J, r, P, PT);
     return cudaGetLastError();
 }
 
 cudaError_t transpose_round(float* dst, int ldd, const float* src, int rows, int cols, int lds, cudaStream_t st) {
     dim3 grid((cols + 31) / 32, (rows + 31) / 32), block(32, 8);
-    transpose_round_kernel<<<grid, block, 0, st>>>(dst, ldd, src, rows, cols, lds);
+    launch_chain(transpose_round_kernel, grid, block, 0, st, dst, ldd, src, rows, cols, lds);
     return cudaGetLastError();
 }
 cudaError_t round_tf32(float* p, int64_t n, cudaStream_t st) {

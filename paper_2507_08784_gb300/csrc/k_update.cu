@@ -90,6 +90,7 @@ __device__ __forceinline__ void optimizer_cols(const UpdStreamGroup& g, const Up
 // transposed); each thread issues the loads of four rows (or columns) before using them.
 template <int RM, bool ADAM, bool TRANS>
 __global__ void __launch_bounds__(TU, TRANS ? 1 : 3) update_stream_kernel(const __grid_constant__ UpdStreamGroup g) {
+    chain_begin();
     __shared__ __align__(16) float Rs[RM * TC];             // Rbar[q][c0 + cc]
     int mi = 0;
     while (mi + 1 < g.nmat && blockIdx.x >= static_cast<unsigned>(g.mat[mi + 1].tile0)) ++mi;
@@ -176,8 +177,8 @@ __global__ void __launch_bounds__(TU, TRANS ? 1 : 3) update_stream_kernel(const 
 
 template <int RM, bool TRANS>
 cudaError_t launch_update_stream(const UpdStreamGroup& g, cudaStream_t st) {
-    if (g.optimizer == GLR_ADAM) update_stream_kernel<RM, true, TRANS><<<g.total_tiles, TU, 0, st>>>(g);
-    else update_stream_kernel<RM, false, TRANS><<<g.total_tiles, TU, 0, st>>>(g);
+    if (g.optimizer == GLR_ADAM) launch_chain(update_stream_kernel<RM, true, TRANS>, g.total_tiles, TU, 0, st, g);
+    else launch_chain(update_stream_kernel<RM, false, TRANS>, g.total_tiles, TU, 0, st, g);
     return cudaGetLastError();
 }
 
