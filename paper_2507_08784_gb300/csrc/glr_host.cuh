@@ -30,6 +30,7 @@ struct glr_handle {
     int tma = 0;                          // ... with its ring filled by tile copies
     CUtensorMap Bmap{};                   // tile-copy descriptor of B (n' x m' x N)
     struct GMap { const void* ptr; CUtensorMap map; };
+    std::vector<std::vector<CUtensorMap>> captured_maps;   // tile-copy descriptors that recorded steps copy at replay
     std::vector<GMap> gmaps;              // per node: the descriptors of its last two gradient buffers
     float *Mo = nullptr, *Vo = nullptr;
     float *U = nullptr, *Hbuf = nullptr, *Vbuf = nullptr, *evals = nullptr, *evals_sorted = nullptr;

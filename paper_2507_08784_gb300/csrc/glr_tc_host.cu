@@ -162,19 +162,40 @@ int tcl_maps(glr_handle* h) {
     }
     if (!ok) return fail(h, GLR_ECUDA, "could not describe the operands for tile copies%s");
     CUtensorMap* d = nullptr;
-    int rc = alloc(h, &d, maps.size() + 2 * (size_t)h->N + 2);
+    int rc = alloc(h, &d, maps.size() + 3 * (size_t)h->N + 3);
     if (rc != GLR_OK) return rc;
     GLR_CK(h, cudaMemcpy(d, maps.data(), sizeof(CUtensorMap) * maps.size(), cudaMemcpyHostToDevice));
     h->dmaps = d;
     return GLR_OK;
 }
 
+namespace {
+bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &s) == cudaSuccess) return s == cudaStreamCaptureStatusActive;
+    cudaGetLastError();                            // the legacy stream beside a capture: not this step's
+    return false;
+}
+
+// Maps copied to the device in stream order.  A copy recorded into a graph reads its source at every
+// replay, long after this call: the handle keeps it.
+cudaError_t put_maps(glr_handle* h, CUtensorMap* dst, const CUtensorMap* maps, int n, bool cap, cudaStream_t st) {
+    if (cap) {
+        h->captured_maps.emplace_back(maps, maps + n);
+        maps = h->captured_maps.back().data();
+    }
+    return cudaMemcpyAsync(dst, maps, sizeof(CUtensorMap) * n, cudaMemcpyHostToDevice, st);
+}
+}  // namespace
+
 // The maps of this step's N gradients (bf16 tiles of 64 rows x 64 columns, read in the caller's
 // layout): one of two slots, re-encoded and copied to the device (stream-ordered) only when the
-// set of pointers differs from both.
+// set of pointers differs from both; a step recorded into a graph always copies its own, to a third slot
+// that no other step reads, so that a replay finds them whatever ran in between.
 const CUtensorMap* tcl_grad_maps(glr_handle* h, const void* const* G, cudaStream_t st, int* rc) {
     *rc = GLR_OK;
-    for (int q = 0; q < 2; ++q) {
+    const bool cap = capturing(st);
+    for (int q = 0; q < 2 && !cap; ++q) {
         bool same = true;
         for (int i = 0; i < h->N && same; ++i) same = h->tc_gptr[q][i] == G[i];
         if (same) { h->tc_glast = q; return h->dmaps + kNumTcMaps + q * h->N; }
@@ -198,9 +219,10 @@ const CUtensorMap* tcl_grad_maps(glr_handle* h, const void* const* G, cudaStream
             return nullptr;
         }
     }
-    CUtensorMap* dst = h->dmaps + kNumTcMaps + q * h->N;
-    const cudaError_t e = cudaMemcpyAsync(dst, maps.data(), sizeof(CUtensorMap) * h->N, cudaMemcpyHostToDevice, st);
+    CUtensorMap* dst = h->dmaps + kNumTcMaps + (cap ? 2 * h->N + 2 : q * h->N);
+    const cudaError_t e = put_maps(h, dst, maps.data(), h->N, cap, st);
     if (e != cudaSuccess) { *rc = fail_cuda(h, e, __FILE__, __LINE__); return nullptr; }
+    if (cap) return dst;
     for (int i = 0; i < h->N; ++i) h->tc_gptr[q][i] = G[i];
     h->tc_glast = q;
     return dst;
@@ -210,7 +232,8 @@ const CUtensorMap* tcl_grad_maps(glr_handle* h, const void* const* G, cudaStream
 const CUtensorMap* tcl_x_map(glr_handle* h, const float* X, cudaStream_t st, int* rc) {
     *rc = GLR_OK;
     CUtensorMap* slots = h->dmaps + kNumTcMaps + 2 * h->N;
-    for (int q = 0; q < 2; ++q)
+    const bool cap = capturing(st);
+    for (int q = 0; q < 2 && !cap; ++q)
         if (h->tc_xptr[q] == X) { h->tc_xlast = q; return slots + q; }
     const int q = h->tc_xlast ^ 1;
     const uint64_t mp = h->mp, np = h->np;
@@ -226,8 +249,10 @@ const CUtensorMap* tcl_x_map(glr_handle* h, const float* X, cudaStream_t st, int
         ok = encode_map(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, X, 2, d, s, b, CU_TENSOR_MAP_SWIZZLE_128B);
     }
     if (!ok) { *rc = fail(h, GLR_ECUDA, "could not describe X for tile copies%s"); return nullptr; }
-    const cudaError_t e = cudaMemcpyAsync(slots + q, &map, sizeof(CUtensorMap), cudaMemcpyHostToDevice, st);
+    CUtensorMap* dst = cap ? slots + 2 + h->N : slots + q;
+    const cudaError_t e = put_maps(h, dst, &map, 1, cap, st);
     if (e != cudaSuccess) { *rc = fail_cuda(h, e, __FILE__, __LINE__); return nullptr; }
+    if (cap) return dst;
     h->tc_xptr[q] = X;
     h->tc_xlast = q;
     return slots + q;

@@ -64,3 +64,37 @@ def test_tcgen05_sizes_grouped():
     small and the blocked eigenproblem beside each other."""
     mats = [(136, 264, 16, 20), (264, 136, 16, 64), (200, 328, 32, 68), (192, 136, 20, 128), (256, 520, 16, 132)]
     _group_equals_single(mats, dtype="bf16", tau=2, optimizer="adam", lr=0.01, beta1=0.9, beta2=0.99)
+
+
+@pytest.mark.parametrize("m,n,r,k,dtype,opt", [(64, 576, 8, 16, "f32", "msgd"), (65, 131, 4, 12, "f32", "adam"),
+                                               (64, 128, 4, 0, "f32", "msgd"), (256, 704, 32, 64, "bf16", "adam")])
+@pytest.mark.parametrize("t", [2, 3])
+def test_step_recorded_into_a_graph(m, n, r, k, dtype, opt, t):
+    """A step (t = 2: a refresh, 3: compressed) recorded on a capturing stream with new gradient buffers,
+    replayed, and followed by an ordinary step: the same bits as ordinary steps throughout.  The
+    tile-copy descriptors of the recorded step's gradients have to outlive the call that recorded
+    them."""
+    import torch
+    import paper_2507_08784_gb300 as glr
+    N = 4
+    tdt = torch.float32 if dtype == "f32" else torch.bfloat16
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    kw = dict(tau=2, optimizer=opt, lr=0.01, beta1=0.9, beta2=0.99, basis_rank=k, seed=4, grad_dtype=dtype)
+    a, b = glr.GreedyLore(m, n, r, N, **kw), glr.GreedyLore(m, n, r, N, **kw)
+    Xa, Xb = torch.zeros(m, n, device="cuda"), torch.zeros(m, n, device="cuda")
+    G = [[torch.randn(m, n, device="cuda", generator=gen).to(tdt) for _ in range(N)] for _ in range(t + 2)]
+    for g in G:
+        a.step(g, Xa)
+    for g in G[:t]:
+        b.step(g, Xb)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        b.step(G[t], Xb)
+    graph.replay()
+    torch.cuda.synchronize()
+    b.step(G[t + 1], Xb)
+    torch.cuda.synchronize()
+    assert torch.equal(Xa, Xb)
+    a.close()
+    b.close()
