@@ -17,8 +17,9 @@
 //      H is symmetric: after the first round only its 128 x 128 blocks on and below the diagonal
 //      hold values;
 // and a sweep ends with the off-diagonal norm, checked on the host against tol^2 of the total.
-// V starts as the identity, so its columns follow H's storage order; at the end diag(H) and V
-// orthogonalised once more in fp32 and sorted by descending eigenvalue with the sign rule of the small solvers (sort_group).
+// V starts as the identity, so its columns follow H's storage order; at the end V is orthogonalised
+// once more in fp32, and diag(H) and V are sorted by descending eigenvalue with the sign rule of the
+// small solvers (sort_group).
 //
 // Every product keeps its output's TF32 low part beside it (H_lo, T^T_lo, V_lo; J_lo from the
 // pair sweep), so each operand enters the MMAs as hi + lo.

@@ -1,6 +1,6 @@
 // Full-basis refresh (Eq. SVD-P1, the paper-exact basis): the eigen-decomposition of the m' x m'
 // Gram matrices H = Mbar Mbar^T of every refreshing matrix by parallel cyclic two-sided Jacobi,
-// all matrices in one cooperative launch.  A round applies n/2 disjoint plane rotations chosen by
+// above m' = 512 all matrices in one cooperative launch.  A round applies n/2 disjoint plane rotations chosen by
 // the circle (round-robin) ordering — each angle from its own 2 x 2 diagonal block (Golub & Van
 // Loan, sym.schur2) — then H <- J^T H J block-wise (each 2 x 2 block of H depends only on the
 // rotations of its row and column pairs) and V <- V J.  The updates of a round are spread over
@@ -15,12 +15,13 @@
 // line survives a barrier.
 //
 // For n <= 512 a matrix fits the shared memory of one thread-block cluster and is solved there
-// (jacobi_cluster_kernel): the row pairs of H are spread over up to 16 CTAs, a round's rotations go to
-// all of them over distributed shared memory; two hardware cluster barriers a round.  The rotations, their order and every product and sum are
-// those of the grid-wide kernel, so the results are the same bits.  A round takes 3.2 us at n = 512
-// (bound by instruction issue) and 2 us below n = 128 (the rotation's chain of quotients and roots,
-// two cluster barriers); the grid-wide kernel pays 6 us at n = 512 alone and 14 us for the eight
-// matrices of a conv stack, its barrier in global memory and the L2 round trips.
+// (jacobi_cluster_kernel): the row pairs of H are spread over up to 16 CTAs, a round's rotations go
+// to all of them over distributed shared memory; two hardware cluster barriers a round.  The
+// rotations, their order and every product and sum are those of the grid-wide kernel, so the results
+// are the same bits.  A round takes 3.2 us at n = 512 (bound by instruction issue) and 2 us below
+// n = 128 (the rotation's chain of quotients and roots, two cluster barriers); the grid-wide kernel
+// pays 6 us at n = 512 alone and 14 us for the eight matrices of a conv stack, its barrier in global
+// memory and the L2 round trips.
 #include <cooperative_groups.h>
 
 #include "glr_internal.cuh"

@@ -132,11 +132,17 @@ __device__ __forceinline__ void column_stats(const float* A, int rows, int64_t l
     float best = -1.f, val = 0.f, sum = 0.f;
     int idx = 0x7fffffff;
     if (in)
-#pragma unroll 8
-        for (int a = ty; a < rows; a += 32) {
-            const float v = A[a * ld + col], m = fabsf(v);
-            sum = fmaf(v, v, sum);
-            if (m > best) { best = m; val = v; idx = a; }
+        for (int a0 = ty; a0 < rows; a0 += 32 * 8) {       // eight rows' reads in flight
+            float v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = a0 + 32 * i < rows ? A[(a0 + 32 * i) * ld + col] : 0.f;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float m = fabsf(v[i]);
+                if (a0 + 32 * i >= rows) break;
+                sum = fmaf(v[i], v[i], sum);
+                if (m > best) { best = m; val = v[i]; idx = a0 + 32 * i; }
+            }
         }
     __syncthreads();
     sbest[ty][tx] = best; sval[ty][tx] = val; ssum[ty][tx] = sum; sidx[ty][tx] = idx;
@@ -214,7 +220,14 @@ __global__ void __launch_bounds__(1024) fix_signs_group_kernel(const __grid_cons
     if (ty == 0) sg[tx] = sign;
     __syncthreads();
     if (col < M.k && sg[tx] < 0.f)
-        for (int a = ty; a < M.mp; a += 32) M.Q[(size_t)a * M.k + col] = -M.Q[(size_t)a * M.k + col];
+        for (int a0 = ty; a0 < M.mp; a0 += 32 * 8) {       // eight rows' reads in flight
+            float v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = a0 + 32 * i < M.mp ? M.Q[(size_t)(a0 + 32 * i) * M.k + col] : 0.f;
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (a0 + 32 * i < M.mp) M.Q[(size_t)(a0 + 32 * i) * M.k + col] = -v[i];
+        }
 }
 
 // Right-looking Cholesky (one CTA) with a diagonal shift retry on breakdown.
@@ -489,11 +502,12 @@ __global__ void __launch_bounds__(1024) chol_inverse_kernel(const float* G, int 
 // One CTA of 16 warps a matrix, the lower triangle as 32 x 32 blocks in shared memory (block (i, j) at
 // i (i + 1) / 2 + j, pitch 36: rows 16-byte aligned, the products' reads free of bank conflicts),
 // padded to whole blocks with the identity.  A panel: one warp factors the diagonal block with a row
-// a lane, a warp per block below solves against it by substitution, then the trailing blocks are
-// 32 x 32 x 32 products, a warp each.  The inverse goes block column by block column from the last,
-// in place: T_i = sum_{j < k <= i} X_ik L_kj, X_ij = -T_i X_jj.  Bound by the diagonal blocks' chain of
-// square roots, quotients and shuffles and by shared-memory reads; factoring and inverting column by
-// column, four barriers each, took 0.80 ms for n = 256 and 0.22 ms for n = 128.
+// a lane and hands each column on; in the same steps a warp inverts that block and a warp per block
+// below solves against it by substitution; then the trailing blocks are 32 x 32 x 32 products, a
+// warp each.  The inverse goes block column by block column from the last, in place:
+// T_i = sum_{j < k <= i} X_ik L_kj, X_ij = -T_i X_jj.  Bound by the diagonal blocks' chain of square
+// roots, quotients and shuffles (n = 256: 0.20 ms, n = 128: 66 us; factoring and inverting column by
+// column, four barriers each, took 0.80 and 0.22 ms).
 constexpr int CB = 32, CP = 36, CBLK = CB * CP, CWARPS = 16;
 constexpr int kCholMaxBlocks = 8;
 // a block more than the triangle and T: the eliminations' dead reads
@@ -555,25 +569,6 @@ __device__ __forceinline__ void eliminate(float (&a)[CB], const float* D, int dq
     }
 }
 
-// A diagonal block's Cholesky factor in place (upper part zeroed), one warp, lane = row; false when a
-// pivot is not above thresh.
-__device__ __forceinline__ bool chol_diag(float* D, float thresh, int lane) {
-    float a[CB];
-    load_row(a, D + lane * CP);
-    bool ok = true;
-#pragma unroll 1
-    for (int c = 0; c < CB; ++c) {
-        const float d = __shfl_sync(0xffffffffu, a[0], c);
-        ok = ok && d > thresh;
-        const float l = sqrtf(d), v = lane == c ? l : lane > c ? a[0] / l : 0.f;
-#pragma unroll
-        for (int q = 1; q < CB; ++q) a[q - 1] = fmaf(-v, __shfl_sync(0xffffffffu, v, (c + q) & 31), a[q]);
-        a[CB - 1] = 0.f;
-        D[lane * CP + c] = v;
-    }
-    return ok;
-}
-
 __global__ void __launch_bounds__(CWARPS * 32) chol_group_kernel(const __grid_constant__ CholGroup g) {
     chain_begin();
     extern __shared__ __align__(16) float csm[];
@@ -583,6 +578,8 @@ __global__ void __launch_bounds__(CWARPS * 32) chol_group_kernel(const __grid_co
     float* T = L + (size_t)(nb * (nb + 1) / 2) * CBLK;
     __shared__ int fail;
     __shared__ float shift, trace;
+    __shared__ float colb[2][2 * CB];                  // column c of L_pp; past it zeros, read for dead values
+    if (t < 2 * CB) colb[t / CB][CB + t % CB] = 0.f;
     auto entry = [&](int i, int l) {
         if (M.tri_only == kTriUpper) return M.part[(size_t)l * M.n + i];           // L = U^T
         if (M.tri_only == kTriUnitLower) return i == l ? 1.f : M.part[(size_t)i * M.n + l];
@@ -616,16 +613,46 @@ __global__ void __launch_bounds__(CWARPS * 32) chol_group_kernel(const __grid_co
         if (M.tri_only) break;
         const float thresh = 1e-12f * fmaxf(trace / n, 1e-30f);
         for (int p = 0; p < nb; ++p) {
-            if (warp == 0 && !chol_diag(cblk(L, p, p), thresh, lane) && lane == 0) fail = 1;
+            // L_pp by warp 0 (lane = row), a column a step; the others take each column as it comes: warp 1
+            // to X_pp = L_pp^{-1} (lane = column, over L_pp, which nothing else reads), a warp per block
+            // below to L_ip = A_ip L_pp^{-T} (lane = row)
+            const int i = p + warp - 1;
+            const bool on = warp < 2 || i < nb;
+            float* A = warp < 2 ? cblk(L, p, p) + (warp ? lane : lane * CP) : on ? cblk(L, i, p) + lane * CP : nullptr;
+            const int os = warp == 1 ? CP : 1;
+            float a[CB];
+            if (warp != 1 && on) load_row(a, A);
+            else
+#pragma unroll
+                for (int q = 0; q < CB; ++q) a[q] = lane == q ? 1.f : 0.f;
+            bool ok = true;
+#pragma unroll 1
+            for (int c = 0; c < CB; ++c) {
+                float* cb = colb[c & 1];
+                float v = 0.f;
+                if (warp == 0) {
+                    const float d = __shfl_sync(0xffffffffu, a[0], c);
+                    ok = ok && d > thresh;
+                    const float l = sqrtf(d);
+                    v = lane == c ? l : lane > c ? a[0] / l : 0.f;
+                    cb[lane] = v;
+                }
+                __syncthreads();
+                if (warp == 0) {
+#pragma unroll
+                    for (int q = 1; q < CB; ++q) a[q - 1] = fmaf(-v, __shfl_sync(0xffffffffu, v, (c + q) & 31), a[q]);
+                    a[CB - 1] = 0.f;
+                } else if (on) {
+                    const float x = a[0] / cb[c];
+#pragma unroll
+                    for (int q = 1; q < CB; ++q) a[q - 1] = fmaf(-x, cb[c + q], a[q]);
+                    a[CB - 1] = 0.f;
+                    A[c * os] = x;
+                }
+            }
+            if (warp == 0 && lane == 0 && !ok) fail = 1;
             __syncthreads();
             if (fail) break;                           // uniform: read after the barrier, written before it
-            for (int i = p + 1 + warp; i < nb; i += CWARPS) {            // L_ip = A_ip L_pp^{-T}, lane = row
-                float a[CB];
-                float* A = cblk(L, i, p) + lane * CP;
-                load_row(a, A);
-                eliminate<true>(a, cblk(L, p, p), CP, A, 1);
-            }
-            __syncthreads();
             const int m = nb - p - 1;
             for (int q = warp; q < m * (m + 1) / 2; q += CWARPS) {       // A_ij -= L_ip L_jp^T
                 int i = 0, j = q;
@@ -652,7 +679,7 @@ __global__ void __launch_bounds__(CWARPS * 32) chol_group_kernel(const __grid_co
         // non-finite block): the refresh cannot orthonormalise it (flag + 6 counts these)
         if (attempt == 6 || !(trace > 0.f) || !isfinite(trace)) atomicAdd(M.flag + 6, 1);
     }
-    for (int j = warp; j < nb; j += CWARPS) {          // X_jj in place, lane = column
+    for (int j = warp; j < nb && M.tri_only; j += CWARPS) {              // X_jj in place, lane = column
         float a[CB];
 #pragma unroll
         for (int i = 0; i < CB; ++i) a[i] = lane == i ? 1.f : 0.f;
