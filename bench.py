@@ -474,7 +474,7 @@ def bench_paper_exact(torch, glr, K, Wm, ctx, hbm_peak):
                       "refresh_ms_per_matrix": ref / len(xc.shapes) if ref else None,
                       "jacobi_sweeps": xr["sweeps"],
                       "method": "H = Mbar Mbar^T (FFMA), blocked two-sided Jacobi: 128-index pair blocks "
-                                "solved by one scalar-Jacobi sweep each, block rotations as FFMA products"}
+                                "solved by one scalar-Jacobi sweep each, block rotations as split-TF32 tcgen05 products"}
     del xs
     torch.cuda.empty_cache()
     return out
