@@ -13,9 +13,12 @@ namespace glr {
 namespace {
 constexpr int GB_M = 64, GB_N = 64, GB_K = 16;
 
-// 64 x 64 tile (i0, j0) of A B over [kbeg, kend): the next slab's elements are on their way to
+// 64 x 64 tile (i0, j0) of A B over [kbeg, kend): the next two slabs' elements are on their way to
 // registers while the current one is multiplied (one barrier a slab); every output is one fma chain
-// over k ascending.  Without the prefetch a slab of 16 waited out the whole load latency (3.4 us).
+// over k ascending.  Without prefetch a slab of 16 waited out the whole load latency (3.4 us), with one
+// slab ahead still half of it where a product has fewer tiles than SMs, and the warps past a thin
+// product's rows took their share of the shared-memory reads (four 333 x 777 layers, r = 5: a step
+// 141 -> 111 us with two slabs ahead and those warps idle).
 struct GemmTile {
     const float* A; int64_t sAi, sAp;
     const float* B; int64_t sBp, sBj;
@@ -34,9 +37,10 @@ __device__ __forceinline__ void gemm_tile(const GemmTile& g, int i0, int j0, int
     const int aii = ai ? tid & 63 : tid / GB_K, app = ai ? tid >> 6 : tid % GB_K;
     const int bjj = bj ? tid & 63 : tid / GB_K, bpp = bj ? tid >> 6 : tid % GB_K;
     constexpr int NL = GB_K / 4, IS = 256 / GB_K;           // elements a thread; index step along i or j
-    float ra[NL], rb[NL];
+    float ra[2][NL], rb[2][NL];                             // two slabs on their way
     f32x2 c[4][2] = {};
-    auto load = [&](int p0) {
+    const bool rows = i0 + (tid >> 5) * 8 < g.M;            // a warp whose eight rows are past M only stages
+    auto load = [&](int p0, float (&ra)[NL], float (&rb)[NL]) {
 #pragma unroll
         for (int u = 0; u < NL; ++u) {
             const int ii = ai ? aii : aii + IS * u, pa = p0 + (ai ? app + 4 * u : app);
@@ -45,26 +49,32 @@ __device__ __forceinline__ void gemm_tile(const GemmTile& g, int i0, int j0, int
             rb[u] = j0 + jj < g.N && pb < kend ? g.B[(int64_t)pb * g.sBp + (int64_t)(j0 + jj) * g.sBj] : 0.f;
         }
     };
-    if (kbeg < kend) load(kbeg);
-    int s = 0;
-    for (int p0 = kbeg; p0 < kend; p0 += GB_K, s ^= 1) {
+    if (kbeg < kend) load(kbeg, ra[0], rb[0]);
+    if (kbeg + GB_K < kend) load(kbeg + GB_K, ra[1], rb[1]);
+    for (int p0 = kbeg; p0 < kend; p0 += 2 * GB_K) {
 #pragma unroll
-        for (int u = 0; u < NL; ++u) {
-            As[s][ai ? app + 4 * u : app][ai ? aii : aii + IS * u] = ra[u];
-            Bs[s][bj ? bpp + 4 * u : bpp][bj ? bjj : bjj + IS * u] = rb[u];
-        }
-        __syncthreads();                                    // the other buffer is read up to here
-        if (p0 + GB_K < kend) load(p0 + GB_K);
+        for (int s = 0; s < 2; ++s) {
+            const int ps = p0 + s * GB_K;
+            if (ps >= kend) break;
 #pragma unroll
-        for (int p = 0; p < GB_K; ++p) {
-            const float4 a = *reinterpret_cast<const float4*>(&As[s][p][ty * 4]);
-            const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(&Bs[s][p][tx * 4]);
-            const float av[4] = {a.x, a.y, a.z, a.w};
+            for (int u = 0; u < NL; ++u) {
+                As[s][ai ? app + 4 * u : app][ai ? aii : aii + IS * u] = ra[s][u];
+                Bs[s][bj ? bpp + 4 * u : bpp][bj ? bjj : bjj + IS * u] = rb[s][u];
+            }
+            __syncthreads();                                // the other buffer is read up to here
+            if (ps + 2 * GB_K < kend) load(ps + 2 * GB_K, ra[s], rb[s]);
+            if (!rows) continue;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const f32x2 aa = pack2(av[u], av[u]);
-                asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c[u][0]) : "l"(aa), "l"(b.x));
-                asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c[u][1]) : "l"(aa), "l"(b.y));
+            for (int p = 0; p < GB_K; ++p) {
+                const float4 a = *reinterpret_cast<const float4*>(&As[s][p][ty * 4]);
+                const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(&Bs[s][p][tx * 4]);
+                const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const f32x2 aa = pack2(av[u], av[u]);
+                    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c[u][0]) : "l"(aa), "l"(b.x));
+                    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c[u][1]) : "l"(aa), "l"(b.y));
+                }
             }
         }
     }
