@@ -79,7 +79,8 @@ __device__ __forceinline__ float4 gauss4_fast(uint64_t seed, uint32_t t, uint32_
 // be launched so without it.  One iteration of the k = 16 power iteration (five launches):
 // 65.6 -> 49.8 us.  Launched ordinarily: kernels whose many equal CTAs would crowd onto the SMs that
 // free first (the unfused compose, update and products: ragged layers 162 us a step chained, 141
-// so, before the products read two slabs ahead), and the tcgen05 step's streaming ops (d = 4096 layers 7.57 ms chained, 7.46 so).
+// so, before the products read two slabs ahead), and the tcgen05 step's streaming ops (d = 4096
+// layers 7.57 ms chained, 7.46 so).
 template <class... P, class... A>
 inline cudaError_t launch_chain(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
     cudaLaunchAttribute attr{};

@@ -1285,37 +1285,40 @@ cudaError_t launch_pbuild(TcGroup& g, cudaStream_t st) { return launch<PBuild>(g
 cudaError_t launch_rbar(TcGroup& g, cudaStream_t st) { return launch<RBar>(g, st); }
 cudaError_t launch_update(TcGroup& g, cudaStream_t st) { return launch<Update>(g, st); }
 namespace {
-// The K slices of Pow added in order: out (rows x k, fp32) and outT (kpad x rows, TF32).
+// The K slices of Pow added in order: out (rows x k, fp32) and outT (kpad x rows, TF32).  A CTA a 32 x 32
+// block, a thread four rows with the slices' reads of all of them in flight (all columns a CTA, row by
+// row and slice by slice, took 24 us for 11008 x 128).
 __global__ void __launch_bounds__(256) pow_reduce_kernel(const __grid_constant__ TcGroup g) {
     chain_begin();
     __shared__ float tile[32][33];
     const TcMat& M = g.mat[blockIdx.y];
-    const int r0 = blockIdx.x * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    if (M.splits <= 1 || r0 >= M.rows) return;
-    for (int q0 = 0; q0 < M.kpad; q0 += 32) {
-        __syncthreads();
-        for (int y = ty; y < 32; y += 8) {
-            float v = 0.f;
-            if (r0 + y < M.rows) {
-                const float* p = M.pws + (int64_t)(r0 + y) * M.kpad + q0 + tx;
-                for (int z = 0; z < M.splits; ++z) v += p[(int64_t)z * M.rows * M.kpad];
-                if (q0 + tx < M.k) M.out[(int64_t)(r0 + y) * M.ld_out + q0 + tx] = v;
-            }
-            tile[y][tx] = v;
-        }
-        __syncthreads();
-        for (int y = ty; y < 32; y += 8)
-            if (r0 + tx < M.rows) M.outT[(int64_t)(q0 + y) * M.rows + r0 + tx] = rna_tf32(tile[tx][y]);
+    const int r0 = blockIdx.x * 32, q0 = blockIdx.z * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    if (M.splits <= 1 || r0 >= M.rows || q0 >= M.kpad) return;
+    float v[4] = {};
+    const float* p = M.pws + (int64_t)(r0 + ty) * M.kpad + q0 + tx;
+#pragma unroll 4
+    for (int z = 0; z < M.splits; ++z)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (r0 + ty + 8 * i < M.rows) v[i] += p[((int64_t)z * M.rows + 8 * i) * M.kpad];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int y = ty + 8 * i;
+        if (r0 + y < M.rows && q0 + tx < M.k) M.out[(int64_t)(r0 + y) * M.ld_out + q0 + tx] = v[i];
+        tile[y][tx] = v[i];
     }
+    __syncthreads();
+    for (int y = ty; y < 32; y += 8)
+        if (r0 + tx < M.rows) M.outT[(int64_t)(q0 + y) * M.rows + r0 + tx] = rna_tf32(tile[tx][y]);
 }
 template <class Op>
 cudaError_t launch_pow(TcGroup& g, cudaStream_t st) {
     const cudaError_t e = launch<Op>(g, st);
-    int rows = 0;
+    int rows = 0, kpad = 0;
     for (int i = 0; i < g.nmat; ++i)
-        if (g.mat[i].splits > 1) rows = std::max(rows, g.mat[i].rows);
+        if (g.mat[i].splits > 1) { rows = std::max(rows, g.mat[i].rows); kpad = std::max(kpad, g.mat[i].kpad); }
     if (e != cudaSuccess || !rows) return e;
-    launch_chain(pow_reduce_kernel, dim3((rows + 31) / 32, g.nmat), 256, 0, st, g);
+    launch_chain(pow_reduce_kernel, dim3((rows + 31) / 32, g.nmat, (kpad + 31) / 32), 256, 0, st, g);
     return cudaGetLastError();
 }
 }  // namespace
@@ -1331,7 +1334,8 @@ cudaError_t launch_pown(TcGroup& g, cudaStream_t st) { return launch_pow<PowN>(g
 
 namespace {
 // The row chunks' partial Gram matrices added in order into the first one: by all SMs, where the
-// one-CTA consumers waited out a load's latency per chunk and row (k = 128: 90 of a factor's 120 us).
+// one-CTA consumers waited out a load's latency per chunk and row (factors of k = 256: 294 -> 205 us,
+// of k = 128: 94 -> 71, for 8 and 6 us here).
 __global__ void __launch_bounds__(256) gram_sum_kernel(const __grid_constant__ TcGroup g) {
     chain_begin();
     const TcMat& M = g.mat[blockIdx.y];
