@@ -632,7 +632,7 @@ __global__ void __launch_bounds__(CWARPS * 32) chol_group_kernel(const __grid_co
                 float v = 0.f;
                 if (warp == 0) {
                     const float d = __shfl_sync(0xffffffffu, a[0], c);
-                    ok = ok && d > thresh;
+                    ok = ok && (d > thresh || p * CB + c >= n);   // the padding's pivots are 1 at any scale
                     const float l = sqrtf(d);
                     v = lane == c ? l : lane > c ? a[0] / l : 0.f;
                     cb[lane] = v;

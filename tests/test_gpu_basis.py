@@ -94,6 +94,22 @@ def test_truncated_basis(m, n, r, k, dtype):
     assert np.all(np.diff(np.diag(D)) <= 2 * tol * D[0, 0])
 
 
+@pytest.mark.parametrize("m,n,r,k", [(136, 520, 16, 20), (200, 328, 16, 36), (256, 1288, 16, 132)])
+@pytest.mark.parametrize("scale", [1e-6, 1.0, 1e7])
+def test_truncated_basis_at_any_gradient_scale(m, n, r, k, scale):
+    """k no multiple of the factors' 32-column blocks: the padding must not be taken for pivots, whatever the
+    size of the real ones (their mean is 6e13 for gradients of loss-scaled size).  The subspace and the
+    bounds are those of test_truncated_basis, and the handle reports no failed factorisation."""
+    G = (_gapped(m, n, k, seed=m + n + k) * scale).astype(np.float32)
+    h = _refreshed(m, n, r, k, G, "bf16")                # its stats() raises on a numeric failure
+    A = h.selection()[4].double().cpu().numpy() / scale
+    U = h.basis().double().cpu().numpy()
+    h.close()
+    assert np.abs(U.T @ U - np.eye(U.shape[0])).max() <= 2e-5
+    Us = np.linalg.svd(A, full_matrices=False)[0][:, :k]
+    assert np.linalg.norm(U[:, :k] - Us @ (Us.T @ U[:, :k]), 2) <= 1e-4
+
+
 @pytest.mark.parametrize("m,n,r,k", [(33, 64, 1, 1), (65, 132, 3, 5), (130, 516, 8, 31), (512, 576, 8, 32), (64, 100, 4, 16)])
 def test_scores_use_the_refreshed_basis(m, n, r, k):
     """The step after a refresh reads the copies of Y and Yt that the refresh left (transposed and in fragment
