@@ -262,6 +262,13 @@ cudaError_t sort_group(const SortGroup& g, cudaStream_t st);
 // pivot is not positive the diagonal is shifted and the factorisation restarted (*flag =
 // number of restarts).  scratch: n*n floats.
 cudaError_t cholesky(float* A, int n, float* scratch, int* flag, cudaStream_t st);
+// The diagonal shift of a factorisation's next attempt after `attempt` (0, 1, ..) broke down: 1e-7, 1e-5, ..
+// times the mean diagonal, so that a Gram matrix and its multiples are retried alike.
+__device__ __forceinline__ float chol_shift(int attempt, float mean) {
+    float rel = 1e-7f;
+    for (int i = 0; i < attempt; ++i) rel *= 100.f;
+    return rel * mean;
+}
 // S = L^{-T} for L L^T = G (n x n SPD, n <= 256), one CTA with the factor in shared memory; the
 // same shifted retries as cholesky(), attempts counted in *flag.
 cudaError_t chol_inverse(const float* G, int n, float* S, int* flag, cudaStream_t st);

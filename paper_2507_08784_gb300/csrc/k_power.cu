@@ -476,7 +476,7 @@ __global__ void __cluster_dims__(CCH, 1, 1) __launch_bounds__(TCH)
             if (attempt > 0 && tid == 0 && M.flag) atomicAdd(M.flag, 1);
             return;
         }
-        shift = (shift == 0.f ? 1e-7f : shift * 100.f) * (tr > 0.f ? tr / k : 1.f);
+        shift = chol_shift(attempt, tr > 0.f ? tr / k : 1.f);
         __syncthreads();
     }
     // no factorisation: leave S as identity and count it

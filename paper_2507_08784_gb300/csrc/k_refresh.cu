@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(1024) cholesky_kernel(float* A, int n, float* 
         }
         __syncthreads();
         if (!fail) break;
-        if (tid == 0) shift = (attempt == 0 ? 1e-7f : shift * 100.f) * fmaxf(trace / n, 1e-30f);
+        if (tid == 0) shift = chol_shift(attempt, fmaxf(trace / n, 1e-30f));
         __syncthreads();
     }
     for (int e = tid; e < n * n; e += nth)
@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(1024) chol_inverse_kernel(const float* G, int 
         }
         __syncthreads();
         if (!fail) break;
-        if (tid == 0) shift = (attempt == 0 ? 1e-7f : shift * 100.f) * fmaxf(trace / n, 1e-30f);
+        if (tid == 0) shift = chol_shift(attempt, fmaxf(trace / n, 1e-30f));
         __syncthreads();
     }
     if (tid == 0 && flag) {
@@ -670,7 +670,7 @@ __global__ void __launch_bounds__(CWARPS * 32) chol_group_kernel(const __grid_co
         }
         if (!fail) break;
         __syncthreads();
-        if (t == 0) shift = (attempt == 0 ? 1e-7f : shift * 100.f) * fmaxf(trace / n, 1e-30f);
+        if (t == 0) shift = chol_shift(attempt, fmaxf(trace / n, 1e-30f));
     }
     __syncthreads();
     if (t == 0 && !M.tri_only && M.flag) {

@@ -110,6 +110,28 @@ def test_truncated_basis_at_any_gradient_scale(m, n, r, k, scale):
     assert np.linalg.norm(U[:, :k] - Us @ (Us.T @ U[:, :k]), 2) <= 1e-4
 
 
+@pytest.mark.parametrize("m,n,r,k,dtype", [(96, 256, 4, 16, "f32"), (130, 516, 4, 31, "f32"), (160, 320, 4, 40, "f32"),
+                                           (300, 640, 4, 264, "f32"), (136, 520, 16, 20, "bf16"), (256, 520, 16, 132, "bf16")])
+@pytest.mark.parametrize("scale", [2.0 ** -17, 1.0, 2.0 ** 17])
+def test_rank_deficient_refresh_at_any_gradient_scale(m, n, r, k, dtype, scale):
+    """Gradients of rank 4 < k: the Gram matrices are singular to rounding and every factor needs a diagonal
+    shift, which has to grow from attempt to attempt relative to the matrix.  No factorisation is
+    given up, and the leading four basis vectors span the gradient's column space at each scale: in fp32 to
+    rounding (about 3e-7 in a CPU model of the iteration; 1e-4 allowed, as above).  On the bf16 path the
+    Ritz vectors come from TF32 operands, 2^-12 each in H relative to its largest entry 1, against the
+    smallest leading Ritz value 1/4: 2^-11 / (1/4)."""
+    rng = np.random.default_rng(k)
+    U4 = np.linalg.qr(rng.standard_normal((m, 4)))[0]
+    V4 = np.linalg.qr(rng.standard_normal((n, 4)))[0]
+    G = ((U4 * np.linspace(1.0, 0.5, 4)) @ V4.T * scale).astype(np.float32)
+    h = _refreshed(m, n, r, k, G, dtype)                 # its stats() raises on a numeric failure
+    A = h.selection()[4].double().cpu().numpy()          # bf16: the rounded gradient, rank 4 and small noise
+    U = h.basis().double().cpu().numpy()[:, :4]
+    h.close()
+    U4 = np.linalg.svd(A, full_matrices=False)[0][:, :4]
+    assert np.linalg.norm(U4 - U @ (U.T @ U4), 2) <= (2.0 ** -9 if dtype == "bf16" else 1e-4)
+
+
 @pytest.mark.parametrize("m,n,r,k", [(33, 64, 1, 1), (65, 132, 3, 5), (130, 516, 8, 31), (512, 576, 8, 32), (64, 100, 4, 16)])
 def test_scores_use_the_refreshed_basis(m, n, r, k):
     """The step after a refresh reads the copies of Y and Yt that the refresh left (transposed and in fragment
