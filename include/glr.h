@@ -137,7 +137,8 @@ typedef struct glr_stats {
     int32_t path;                   /* kernel family that runs the step: GLR_PATH_*          */
     int32_t nonfinite;              /* warps of the compose pass that found a NaN or Inf in  *
                                      * the node-mean gradient since creation (0: all finite) */
-    int32_t numeric_failures;       /* refresh factorisations that could not be completed    */
+    int32_t numeric_failures;       /* refresh factorisations that could not be completed and *
+                                     * eigenproblems that did not converge                   */
     int32_t reserved;
 } glr_stats;
 
@@ -287,9 +288,9 @@ int glr_refresh(glr_handle* h);
  * bounded wait inside a kernel of this handle's launches has given up since creation (the
  * results of those steps are not valid), else GLR_ENUMERIC when a refresh met a Gram matrix it
  * could not factor (a rank-deficient or zero node mean, e.g. all-zero gradients: the basis of
- * that refresh is not orthonormal), else GLR_ENONFINITE when a compose pass found a NaN or Inf
- * in the node-mean gradient (a node sent a non-finite gradient, or the error state overflowed),
- * else GLR_OK.                                                                             */
+ * that refresh is not orthonormal) or an eigenproblem that did not converge within its sweeps,
+ * else GLR_ENONFINITE when a compose pass found a NaN or Inf in the node-mean gradient (a node
+ * sent a non-finite gradient, or the error state overflowed), else GLR_OK.                 */
 int glr_get_stats(const glr_handle* h, glr_stats* out);
 
 /* Message of the last failure on h (or of the last failed glr_create when h is NULL);

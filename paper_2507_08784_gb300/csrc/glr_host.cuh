@@ -41,7 +41,7 @@ struct glr_handle {
     int* dflags = nullptr;   // [0] Cholesky restarts, [1] Jacobi sweeps of the last refresh,
                              // [2] bounded device waits that gave up, [3] warps that found a NaN /
                              // Inf in Mbar, [4..5] the cooperative Jacobi's grid barrier, [6]
-                             // refresh factorisations that failed (GLR_ENUMERIC), [7] unused
+                             // refresh factorisations and eigenproblems that failed (GLR_ENUMERIC), [7] unused
     float* gemm_ws = nullptr;   // split-K partial tiles of the refresh GEMMs
     // Large plain products (>= 2^26 flops) go to cuBLAS: one library handle for the step stream
     // and one for the refresh stream (a handle's workspace must not serve two streams at once).

@@ -246,8 +246,8 @@ cudaError_t materialize_error(int mp, int np, int r, int e_zero, const float* B,
 
 // ---- refresh ------------------------------------------------------------------------------
 // Cyclic two-sided Jacobi on the symmetric n x n matrix H (overwritten), one CTA:
-// eigenvalues to evals, eigenvectors (columns) to V; the sweep count to *sweeps.
-cudaError_t jacobi_eig(float* H, int n, float* V, float* evals, int* sweeps, cudaStream_t st);
+// eigenvalues to evals, eigenvectors (columns) to V; the sweep count to *sweeps; *failed as JacobiMat's.
+cudaError_t jacobi_eig(float* H, int n, float* V, float* evals, int* sweeps, int* failed, cudaStream_t st);
 // Eigenpairs by descending eigenvalue, several problems at once: V (n x n row-major, column j for
 // evals[j]) -> Out (n x n) with unit columns, the largest-|entry| of each positive, and
 // evals_sorted (may be null).  Two launches; order and scale: n entries of scratch each.
@@ -297,7 +297,7 @@ cudaError_t finish_group(const FinishGroup& g, int stage, cudaStream_t st);
 // be null).
 struct TailMat {
     int mp, k, tp;
-    const float* H; float* evals; float* evals_sorted; int* sweeps; float* R;
+    const float* H; float* evals; float* evals_sorted; int* sweeps; int* failed; float* R;
     float* Q; float* sign; float* W; float* T; float* s;
     float* Y; float* Yt; float* YT; float* YtT; float* YF; float* YtF;
 };
@@ -327,6 +327,7 @@ struct JacobiMat {
     float* H; float* H2; float* V; float* evals;   // H2: a second n x n buffer (rounds alternate)
     int* sweeps;
     int soff;               // first float of this matrix's rotations in shared memory (see jacobi_rot_floats)
+    int* failed;            // counts a problem that ends at the sweep limit with a finite norm above the bound (may be null)
     float* log;             // jacobi_cluster: jacobi_log_floats(n, max_sweeps) floats, every round's rotations
 };
 constexpr int kJacobiSweeps = 40;
@@ -358,6 +359,7 @@ struct EigMat {
     int n; float tol;
     const float* H; int ld;
     float* V; float* evals; int* sweeps; float* ws;
+    int* failed;                          // counts a problem that ends at the sweep limit unconverged (may be null)
 };
 struct EigGroup {
     int nmat, max_sweeps, parts;            // parts: CTAs a pair, set by eig_group

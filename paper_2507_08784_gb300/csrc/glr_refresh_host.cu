@@ -59,14 +59,14 @@ int eig_solve(const std::vector<EigItem>& items, cudaStream_t s0, cudaStream_t s
         for (size_t c0 = 0; c0 < cls[big].size(); c0 += kGroupMax) {
             EigGroup g{};
             glr_handle* h0 = cls[big][c0]->h;
-            g.max_sweeps = 40;
+            g.max_sweeps = kJacobiSweeps;
             g.bar = h0->dflags + 4; g.err = h0->dflags + 2; g.part = h0->jpart;
             for (size_t i = c0; i < cls[big].size() && i < c0 + (size_t)kGroupMax; ++i) {
                 const EigItem& it = *cls[big][i];
                 EigMat& M = g.mat[g.nmat++];
                 M.n = it.n; M.tol = 4.f * 5.96e-8f * sqrtf(static_cast<float>(it.n)) + 1e-7f;
                 M.H = it.H; M.ld = it.ld; M.V = it.V; M.evals = it.h->evals;
-                M.sweeps = it.h->dflags + 1; M.ws = it.h->eig_ws;
+                M.sweeps = it.h->dflags + 1; M.ws = it.h->eig_ws; M.failed = it.h->dflags + 6;
             }
             if (big) GLR_LAUNCH(h0, 1, eig_group(g, s0 != s1 ? (int)cls[0].size() : 0, s0));
             else GLR_LAUNCH(h0, 1, eig_small_group(g, s1));
@@ -188,7 +188,8 @@ int refresh_power_group(const std::vector<glr_handle*>& hs) {
     for (glr_handle* h : hs) {
         TailMat& M = tg.mat[tg.nmat++];
         M.mp = h->mp; M.k = h->k; M.tp = transposed_pitch(h->mp);
-        M.H = h->Hk; M.evals = h->evals; M.evals_sorted = h->evals_sorted; M.sweeps = h->dflags + 1; M.R = h->gram;
+        M.H = h->Hk; M.evals = h->evals; M.evals_sorted = h->evals_sorted; M.sweeps = h->dflags + 1; M.failed = h->dflags + 6;
+        M.R = h->gram;
         M.Q = h->Qn; M.sign = h->sort_ws; M.W = h->scratch; M.T = h->T; M.s = h->dsign;
         M.Y = h->Y; M.Yt = h->Yt; M.YT = h->YT; M.YtT = h->YtT;
         if (h->mma) { M.YF = h->YF; M.YtF = h->YtF; }
@@ -242,7 +243,7 @@ JacobiMat jacobi_mat(glr_handle* h) {
     JacobiMat M{};
     M.n = h->mp; M.tol = 4.f * 5.96e-8f * sqrtf(static_cast<float>(h->mp)) + 1e-7f;
     M.H = h->Hbuf; M.H2 = h->jwork; M.V = h->Vbuf; M.evals = h->evals;
-    M.sweeps = h->dflags + 1; M.log = h->jlog;
+    M.sweeps = h->dflags + 1; M.failed = h->dflags + 6; M.log = h->jlog;
     return M;
 }
 
@@ -285,7 +286,7 @@ int refresh_exact_grouped(std::vector<glr_handle*>& hs) {
             const int mp = h->mp, np = h->np;
             GLR_GEMM(h, gd(mp, mp, np, h->Mbar, np, 1, h->Mbar, 1, np, h->Hbuf, mp, 1), h->rstream);
             if (!grid) {                                         // no cooperative launch: one CTA each
-                GLR_LAUNCH(h, 1, jacobi_eig(h->Hbuf, mp, h->Vbuf, h->evals, h->dflags + 1, h->rstream));
+                GLR_LAUNCH(h, 1, jacobi_eig(h->Hbuf, mp, h->Vbuf, h->evals, h->dflags + 1, h->dflags + 6, h->rstream));
                 const int rc = sort_full_basis(h, h->rstream);
                 if (rc != GLR_OK) return rc;
                 continue;

@@ -1,6 +1,7 @@
 // The k x k Rayleigh-Ritz problems of truncated refreshes, several at once (any symmetric n x n
 // eigenproblem up to n = 1024).  Two-sided Jacobi in fp32; a problem stops at the start of the first sweep whose
-// off-diagonal norm is within tol of the total.
+// off-diagonal norm is within tol of the total; one that is not (or not a number) after max_sweeps ends there
+// and is counted in *failed.
 //
 // n <= 128: one CTA a problem (eig_small_kernel), every sweep on the registers of k_pair.cuh: 127
 // rounds for n > 64, 63, 31 or 15 for the smaller problems (with a quarter of the warps each).
@@ -108,7 +109,9 @@ __global__ void __launch_bounds__(8 * LIM, 1) eig_small_kernel(const __grid_cons
         if (t == 0) {
             float o2 = 0.f, t2 = 0.f;
             for (int w = 0; w < NT / 32; ++w) { o2 += red[0][w]; t2 += red[1][w]; }
-            stop = (o2 <= M.tol * M.tol * t2 || sweep >= g.max_sweeps) ? 1 : 0;
+            const bool converged = o2 <= M.tol * M.tol * t2;
+            stop = (converged || sweep >= g.max_sweeps) ? 1 : 0;
+            if (stop && !converged && M.failed) atomicAdd(M.failed, 1);
         }
         __syncthreads();
         if (stop) break;
@@ -454,9 +457,11 @@ __global__ void __launch_bounds__(PTHREADS, 1) eig_group_kernel(const __grid_con
             }
             __syncwarp();
             if (lane == 0) {
-                if (o2 <= M.tol * M.tol * t2 || ssweep[mi] >= g.max_sweeps) {
+                const bool converged = o2 <= M.tol * M.tol * t2;
+                if (converged || ssweep[mi] >= g.max_sweeps) {
                     sstate[mi] = kCopy;
                     if (b == 0 && M.sweeps) *M.sweeps = ssweep[mi];
+                    if (b == 0 && !converged && M.failed) atomicAdd(M.failed, 1);
                 } else {
                     sstate[mi] = kPair;
                     sround[mi] = 0;

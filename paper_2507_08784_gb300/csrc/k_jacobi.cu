@@ -5,7 +5,9 @@
 // Loan, sym.schur2) — then H <- J^T H J block-wise (each 2 x 2 block of H depends only on the
 // rotations of its row and column pairs) and V <- V J.  The updates of a round are spread over
 // every CTA of the grid, rounds separated by grid-wide barriers; a matrix stops at the start of
-// the first sweep whose off-diagonal norm is within tol of the total.
+// the first sweep whose off-diagonal norm is within tol of the total.  One that is not after max_sweeps ends
+// there and is counted in *failed (a matrix with NaNs, which no sweep can help, is not: the compose
+// pass has counted those).
 //
 // The grid barrier is an arrival counter and a generation word in global memory; a waiting CTA
 // polls with short sleeps and gives up after about a second, counts the event in *err and
@@ -93,6 +95,7 @@ __global__ void __launch_bounds__(JT) jacobi_group_kernel(const __grid_constant_
             if (o2 <= M.tol * M.tol * t2 || ssweep[t] >= g.max_sweeps) {
                 sstate[t] = kDone;
                 if (b == 0 && M.sweeps) *M.sweeps = ssweep[t];
+                if (b == 0 && o2 > M.tol * M.tol * t2 && M.failed) atomicAdd(M.failed, 1);
             } else {
                 sstate[t] = kRound;
                 sround[t] = 0;
@@ -331,6 +334,7 @@ __global__ void __launch_bounds__(CT, 1) jacobi_cluster_kernel(const __grid_cons
             float o2 = 0.f, t2 = 0.f;
             for (int c = 0; c < C; ++c) { o2 += peer(part, c)[0]; t2 += peer(part, c)[1]; }
             stop = (o2 <= M.tol * M.tol * t2 || sweep >= max_sweeps) ? 1 : 0;
+            if (stop && b == 0 && o2 > M.tol * M.tol * t2 && M.failed) atomicAdd(M.failed, 1);
         }
         cluster_sync();                                 // part is read before anyone writes it again
         if (stop) break;

@@ -17,7 +17,7 @@ namespace {
 __device__ __forceinline__ int circle(int x, int nm1) { return 1 + ((x % nm1) + nm1) % nm1; }
 
 __global__ void __launch_bounds__(1024) jacobi_kernel(float* Hg, int n, float* Vg, float* evals,
-                                                      int* sweeps_out, int use_smem, int max_sweeps,
+                                                      int* sweeps_out, int* failed, int use_smem, int max_sweeps,
                                                       float tol) {
     extern __shared__ float sm[];
     const int npad = n + (n & 1), half = npad / 2, nm1 = npad - 1;
@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(1024) jacobi_kernel(float* Hg, int n, float* V
     for (int e = tid; e < n * n; e += nth) V[e] = (e / n == e % n) ? 1.f : 0.f;
     __syncthreads();
     int sweep = 0;
-    for (; sweep < max_sweeps; ++sweep) {
+    for (;; ++sweep) {
         float off = 0.f, tot = 0.f;
         for (int e = tid; e < n * n; e += nth) {
             const float h = H[e];
@@ -51,7 +51,8 @@ __global__ void __launch_bounds__(1024) jacobi_kernel(float* Hg, int n, float* V
         if (tid == 0) {
             float o2 = 0.f, t2 = 0.f;
             for (int w = 0; w < (nth + 31) / 32; ++w) { o2 += red_off[w]; t2 += red_tot[w]; }
-            done = (o2 <= tol * tol * t2) ? 1 : 0;
+            done = (o2 <= tol * tol * t2 || sweep >= max_sweeps) ? 1 : 0;
+            if (done && o2 > tol * tol * t2 && failed) atomicAdd(failed, 1);
         }
         __syncthreads();
         if (done) break;
@@ -384,7 +385,7 @@ __global__ void wy_basis_kernel(int mp, int k, const float* Y, const float* Yt, 
 
 }  // namespace
 
-cudaError_t jacobi_eig(float* H, int n, float* V, float* evals, int* sweeps, cudaStream_t st) {
+cudaError_t jacobi_eig(float* H, int n, float* V, float* evals, int* sweeps, int* failed, cudaStream_t st) {
     const int npad = n + (n & 1), half = npad / 2;
     const size_t pair_bytes = (size_t)half * 16;
     const size_t full = 2 * sizeof(float) * (size_t)n * n + pair_bytes;
@@ -398,7 +399,7 @@ cudaError_t jacobi_eig(float* H, int n, float* V, float* evals, int* sweeps, cud
     // one thread per 2 x 2 block update of a round, rounded to whole warps (at most 1024)
     const int work = n * half > half * half ? n * half : half * half;
     const int nth = work >= 1024 ? 1024 : ((work + 31) / 32) * 32;
-    jacobi_kernel<<<1, nth, smem, st>>>(H, n, V, evals, sweeps, use_smem, 40, tol);
+    jacobi_kernel<<<1, nth, smem, st>>>(H, n, V, evals, sweeps, failed, use_smem, kJacobiSweeps, tol);
     return cudaGetLastError();
 }
 
@@ -818,7 +819,7 @@ __global__ void __launch_bounds__(512) tail_ritz_kernel(const __grid_constant__ 
     __shared__ float red_off[16], red_tot[16], ev[32];
     __shared__ int done;
     const TailMat& M = g.mat[blockIdx.x];
-    const int n = M.k, half = (n + 1) / 2, nm1 = 2 * half - 1, nth = tail_threads(n), max_sweeps = 40;
+    const int n = M.k, half = (n + 1) / 2, nm1 = 2 * half - 1, nth = tail_threads(n);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const float tol = 4.f * 5.96e-8f * sqrtf(static_cast<float>(n)) + 1e-7f;
     // this thread's entries of the norms (n^2 <= 2 nth), its block of H and its entries of V
@@ -838,7 +839,7 @@ __global__ void __launch_bounds__(512) tail_ritz_kernel(const __grid_constant__ 
     const int xp0 = xp, xq0 = xq;
     __syncthreads();
     int sweep = 0;
-    for (; sweep < max_sweeps; ++sweep) {
+    for (;; ++sweep) {
         float off = 0.f, tot = 0.f;
 #pragma unroll
         for (int i = 0; i < 2; ++i)
@@ -856,7 +857,9 @@ __global__ void __launch_bounds__(512) tail_ritz_kernel(const __grid_constant__ 
         if (tid == 0) {
             float o2 = 0.f, t2 = 0.f;
             for (int w = 0; w < nth / 32; ++w) { o2 += red_off[w]; t2 += red_tot[w]; }
-            done = (o2 <= tol * tol * t2) ? 1 : 0;
+            const bool converged = o2 <= tol * tol * t2;
+            done = (converged || sweep >= kJacobiSweeps) ? 1 : 0;
+            if (done && !converged && M.failed) atomicAdd(M.failed, 1);
         }
         __syncthreads();
         if (done) break;

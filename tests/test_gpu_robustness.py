@@ -160,3 +160,21 @@ def test_noalloc_binding_checks_the_caller_buffers():
         glr.glr_select_noalloc(U, Mb, 1, 1, r, lam, J.long())               # J not int32
     with pytest.raises(ValueError):
         glr.glr_select_noalloc(U, Mb, 1, 1, r, lam, J[: r - 1])             # J too small
+
+
+def test_unconverged_eigenproblems_are_counted(tmp_path):
+    """Every eigen-solver of the refresh counts a problem that ends at its sweep limit
+    (tests/solver_limit_check.cu, run against the built library)."""
+    import os
+    import shutil
+    import subprocess
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    pkg = os.path.join(root, "paper_2507_08784_gb300")
+    exe = str(tmp_path / "check")
+    subprocess.run([shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc", "-std=c++17", "-O1", "--expt-relaxed-constexpr",
+                    "-gencode", "arch=compute_103a,code=sm_103a", "-I", os.path.join(root, "include"), "-I",
+                    os.path.join(pkg, "csrc"), os.path.join(root, "tests", "solver_limit_check.cu"), "-o", exe, "-L",
+                    os.path.join(pkg, "lib"), "-lglr", "-Xlinker", "-rpath", "-Xlinker", os.path.join(pkg, "lib")],
+                   check=True)
+    out = subprocess.run([exe], capture_output=True, text=True, timeout=120)
+    assert out.returncode == 0 and out.stdout.strip() == "ok", out.stdout
