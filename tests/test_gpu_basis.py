@@ -152,13 +152,42 @@ def test_scores_use_the_refreshed_basis(m, n, r, k):
     h.close()
 
 
+@pytest.mark.parametrize("mp,r,k", [(33, 33, 0), (40, 33, 0), (1024, 33, 0), (1024, 512, 0), (1025, 1, 8), (1025, 32, 32),
+                                    (1536, 512, 512), (4096, 128, 128), (4096, 512, 512)])
+@pytest.mark.parametrize("kind", ["distinct", "half zero", "all equal"])
+def test_step_selection_is_a_stable_top_r(mp, r, k, kind):
+    """A step's J is the r largest lambda-bar^2, the lower index first on ties, for the sizes of the radix
+    search (m' > 1024 or r > 32; from one to four scores a thread): under an identity basis a zero row of
+    the gradients scores exactly 0, so J has to reach into ties ("half zero") or consists of them.
+    Exact: J is compared with a stable sort of the scores that the step used."""
+    import torch
+    import paper_2507_08784_gb300 as glr
+    n = mp + 8
+    gen = torch.Generator(device="cuda").manual_seed(mp + r)
+    h = glr.GreedyLore(mp, n, r, 1, tau=100, optimizer="msgd", lr=0.01, beta1=0.9, seed=5, basis_rank=k, grad_dtype="f32")
+    X = torch.zeros(mp, n, device="cuda")
+    h.step([torch.randn(mp, n, device="cuda", generator=gen)], X)        # the refresh; leaves no error behind
+    h.set_basis(torch.eye(mp, device="cuda")[:, :k or mp].contiguous())
+    G = torch.randn(mp, n, device="cuda", generator=gen)
+    if kind == "half zero":
+        G[torch.randperm(mp, device="cuda", generator=gen)[:mp - max(1, r // 2)]] = 0.0
+    if kind == "all equal":
+        G.zero_()
+    h.step([G], X)
+    J, _, _, lam, _ = h.selection()
+    h.close()
+    s = (lam * lam).cpu().numpy()
+    assert np.count_nonzero(s) == {"distinct": mp, "half zero": max(1, r // 2), "all equal": 0}[kind]
+    assert np.array_equal(J, np.sort(np.argsort(-s, kind="stable")[:r]))
+
+
 @pytest.mark.parametrize("mp,r", [(33, 33), (40, 33), (1024, 33), (1024, 1024), (1025, 1), (1025, 32), (4096, 128),
                                   (4096, 4096), (16384, 300)])
 @pytest.mark.parametrize("kind", ["distinct", "half zero", "all equal"])
 def test_selection_is_a_stable_top_r(mp, r, kind):
-    """J = the r largest lambda^2, the lower index first on ties, for the sizes of the radix search (m' > 1024
-    or r > 32): distinct scores, scores tied at 0 that J has to reach into, and all tied.  Exact: J is
-    compared with a stable sort of the scores that the kernel returns."""
+    """J of the allocation-free entry point (its sort of all keys, at any m' and r) = the r largest lambda^2,
+    the lower index first on ties: distinct scores, scores tied at 0 that J has to reach into, and all
+    tied.  Exact: J is compared with a stable sort of the scores that the kernel returns."""
     import torch
     import paper_2507_08784_gb300 as glr
     gen = torch.Generator(device="cuda").manual_seed(mp + r)
