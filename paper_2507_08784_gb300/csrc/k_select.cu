@@ -1,6 +1,8 @@
 // Approx-Top-r (Algorithm 2) on the device: the bilinear forms lambda_j = u_j^T Mbar v_j with
 // v_j generated in the GEMM epilogue (never stored), the fixed-order reduction, the arg-top-r
 // of lambda-bar^2 (Eq. semi-lazy-svd-3) and the gather of P = U[:, J].
+#include <algorithm>
+
 #include "glr_internal.cuh"
 
 namespace glr {
@@ -288,18 +290,25 @@ __device__ __forceinline__ unsigned long long shfl_xor_u64(unsigned long long v,
     return (static_cast<unsigned long long>(hi) << 32) | lo;
 }
 
-// Keys (lambda-bar_j^2 bits, ~j): distinct, larger score first and the lower index on ties.
+// Few scores and winners: sorted by warps; else the radix search.
+__host__ __device__ __forceinline__ bool select_by_warps(int mp, int r) { return mp <= 1024 && r <= 32; }
+// Shared memory of one: the warps' candidates, or every score (m' <= 46340: 181 KiB).
+size_t select_smem(int mp, int r) {
+    return select_by_warps(mp, r) ? sizeof(unsigned long long) * ((mp + 31) / 32) * r : sizeof(uint32_t) * mp;
+}
+
 __device__ __forceinline__ void select_top_r_block(const SelectMat& M, unsigned long long* keys) {
     const int tid = threadIdx.x, mp = M.mp, r = M.r, nth = blockDim.x;
-    auto key_of = [&](int j) -> unsigned long long {
-        return j < mp ? (static_cast<unsigned long long>(__float_as_uint(M.lam[j] * M.lam[j])) << 32) |
-                            static_cast<unsigned long long>(0xFFFFFFFFu - static_cast<uint32_t>(j))
-                      : 0ull;
-    };
-    auto index_of = [](unsigned long long key) { return static_cast<int32_t>(0xFFFFFFFFu - static_cast<uint32_t>(key)); };
-    if (mp <= 1024 && r <= 32) {
-        // each warp sorts its 32 keys (j = 32 w + lane) descending with a bitonic network and
-        // keeps its r largest: the top r of all keys are among these candidates
+    if (select_by_warps(mp, r)) {
+        // keys (lambda-bar_j^2 bits, ~j): distinct, larger score first and the lower index on ties; each warp
+        // sorts its 32 (j = 32 w + lane) descending with a bitonic network and keeps its r largest:
+        // the top r of all keys are among these candidates
+        auto key_of = [&](int j) -> unsigned long long {
+            return j < mp ? (static_cast<unsigned long long>(__float_as_uint(M.lam[j] * M.lam[j])) << 32) |
+                                static_cast<unsigned long long>(0xFFFFFFFFu - static_cast<uint32_t>(j))
+                          : 0ull;
+        };
+        auto index_of = [](unsigned long long key) { return static_cast<int32_t>(0xFFFFFFFFu - static_cast<uint32_t>(key)); };
         const int lane = tid & 31, w = tid >> 5, nw = (mp + 31) >> 5;
         unsigned long long key = key_of(tid);
 #pragma unroll
@@ -489,13 +498,13 @@ cudaError_t select_group(const SelectGroup& g, cudaStream_t st, int stages) {
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (!(stages & 2)) return cudaSuccess;
-    int npow2 = 1;
-    while (npow2 < maxmp) npow2 <<= 1;
+    size_t smem = 0;
+    for (int i = 0; i < g.nmat; ++i) smem = std::max(smem, select_smem(g.mat[i].mp, g.mat[i].r));
     {   // per device: set on every call (cheap next to the launch)
         const cudaError_t ea = cudaFuncSetAttribute(select_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (ea != cudaSuccess) return ea;
     }
-    launch_chain(select_group_kernel, g.nmat, 1024, sizeof(unsigned long long) * npow2, st, g);
+    launch_chain(select_group_kernel, g.nmat, 1024, smem, st, g);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (g.total_out <= 0) return cudaSuccess;              // every P formed by the caller
     launch_chain(pr_kernel, (unsigned)((g.total_out + 255) / 256), 256, 0, st, g);

@@ -153,11 +153,11 @@ def test_scores_use_the_refreshed_basis(m, n, r, k):
 
 
 @pytest.mark.parametrize("mp,r,k", [(33, 33, 0), (40, 33, 0), (1024, 33, 0), (1024, 512, 0), (1025, 1, 8), (1025, 32, 32),
-                                    (1536, 512, 512), (4096, 128, 128), (4096, 512, 512)])
+                                    (1536, 512, 512), (4096, 128, 128), (4096, 512, 512), (16392, 8, 16)])
 @pytest.mark.parametrize("kind", ["distinct", "half zero", "all equal"])
 def test_step_selection_is_a_stable_top_r(mp, r, k, kind):
     """A step's J is the r largest lambda-bar^2, the lower index first on ties, for the sizes of the radix
-    search (m' > 1024 or r > 32; from one to four scores a thread): under an identity basis a zero row of
+    search (m' > 1024 or r > 32; from one score a thread to 17, m' above 16384 among them): under an identity basis a zero row of
     the gradients scores exactly 0, so J has to reach into ties ("half zero") or consists of them.
     Exact: J is compared with a stable sort of the scores that the step used."""
     import torch
