@@ -318,6 +318,8 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 }  // namespace
 
+thread_local int glr::more_launches = 0;
+
 void glr::set_global_error(const char* msg) { g_create_err = msg ? msg : ""; }
 
 extern "C" {
@@ -1015,7 +1017,7 @@ int select_P_grouped(std::vector<StepPlan>& plans, cudaStream_t st, int stages =
     auto flush = [&]() -> int {
         if (g.nmat == 0) return GLR_OK;
         PhaseScope ps(h0, GLR_PH_SELECT, st);
-        GLR_LAUNCH(h0, (stages & 1) + 2 * ((stages >> 1) & 1), select_group(g, st, stages));
+        GLR_LAUNCH(h0, 1, select_group(g, st, stages));
         g = SelectGroup{};
         h0 = nullptr;
         return GLR_OK;

@@ -145,11 +145,14 @@ int fail_cuda(glr_handle* h, cudaError_t e, const char* file, int line);
         if (e__ != cudaSuccess) return ::glr::host::fail_cuda((h), e__, __FILE__, __LINE__);     \
     } while (0)
 
-// Count kernels launched by a launcher call and check its status.
+// Count kernels launched by a launcher call (nk, and what the launcher says it did beyond them) and
+// check its status.
 #define GLR_LAUNCH(h, nk, expr)                                                                \
     do {                                                                                       \
-        (h)->launches += (nk);                                                                 \
-        GLR_CK(h, expr);                                                                       \
+        ::glr::more_launches = 0;                                                              \
+        const cudaError_t launch_e__ = (expr);                                                 \
+        (h)->launches += (nk) + ::glr::more_launches;                                          \
+        GLR_CK(h, launch_e__);                                                                 \
     } while (0)
 
 cudaEvent_t take_event(glr_handle* h);

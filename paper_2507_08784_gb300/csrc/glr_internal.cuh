@@ -94,6 +94,9 @@ inline cudaError_t launch_chain(void (*kernel)(P...), dim3 grid, dim3 block, siz
 __device__ __forceinline__ void chain_begin() {
     asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
 }
+// A launcher is one kernel to its caller's count; one that launches more (or, given nothing to do, none)
+// says so here: the kernels beyond the first of the call in progress.
+extern thread_local int more_launches;
 constexpr int kGroupMax = 32;          // matrices per grouped launch
 
 // Streaming (evict-first) global stores of the error buffers.  Unlike the library's cache-hint
@@ -250,7 +253,7 @@ cudaError_t materialize_error(int mp, int np, int r, int e_zero, const float* B,
 cudaError_t jacobi_eig(float* H, int n, float* V, float* evals, int* sweeps, int* failed, cudaStream_t st);
 // Eigenpairs by descending eigenvalue, several problems at once: V (n x n row-major, column j for
 // evals[j]) -> Out (n x n) with unit columns, the largest-|entry| of each positive, and
-// evals_sorted (may be null).  Two launches; order and scale: n entries of scratch each.
+// evals_sorted (may be null).  Two launches (one if all n <= 32); order and scale: n entries of scratch each.
 struct SortMat {
     int n;
     const float* evals; const float* V; float* Out; float* evals_sorted;

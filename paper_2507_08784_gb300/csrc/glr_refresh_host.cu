@@ -27,7 +27,7 @@ int cholqr(glr_handle* h, float*& A, float*& tmp, int rows, cudaStream_t st) {
 
 int wy_from_Q(glr_handle* h, cudaStream_t st) {
     const int mp = h->mp, k = h->k;
-    GLR_LAUNCH(h, 2, householder_reconstruct(h->Q, mp, k, h->Y, h->T, h->dsign, h->scratch, st));
+    GLR_LAUNCH(h, 1, householder_reconstruct(h->Q, mp, k, h->Y, h->T, h->dsign, h->scratch, st));
     // Yt = Y T^T
     GLR_GEMM(h, gd(mp, k, k, h->Y, k, 1, h->T, 1, k, h->Yt, k, 1), st);
     // transposed copies (k x tp, zero-padded) for the fused compose kernel's lambda epilogue
@@ -88,7 +88,7 @@ int refresh_finish(glr_handle* h, cudaStream_t st) {
     const int mp = h->mp, k = h->k;
     SortGroup sg{};
     sg.mat[sg.nmat++] = sort_mat(h, k, h->Vk, h->gram);
-    GLR_LAUNCH(h, 2, sort_group(sg, st));
+    GLR_LAUNCH(h, 1, sort_group(sg, st));
     GLR_GEMM(h, gd(mp, k, k, h->Q, k, 1, h->gram, k, 1, h->Qn, k, 1), st);
     FinishGroup fg{};
     FinishMat& F = fg.mat[fg.nmat++];
@@ -234,7 +234,7 @@ int refresh_grouped(std::vector<glr_handle*>& hs) {
 int sort_full_basis(glr_handle* h, cudaStream_t st) {
     SortGroup sg{};
     sg.mat[sg.nmat++] = sort_mat(h, h->mp, h->Vbuf, h->U);
-    GLR_LAUNCH(h, 2, sort_group(sg, st));
+    GLR_LAUNCH(h, 1, sort_group(sg, st));
     return GLR_OK;
 }
 
@@ -259,7 +259,7 @@ int refresh_exact_grouped(std::vector<glr_handle*>& hs) {
         PhaseScope ps(h, GLR_PH_REFRESH, h->rstream);
         const int mp = h->mp, np = h->np;
         GLR_GEMM(h, gd(mp, mp, np, h->Mbar, np, 1, h->Mbar, 1, np, h->Hbuf, mp, 1), h->rstream);
-        GLR_LAUNCH(h, mp > 256 ? 2 : 1, jacobi_cluster(jacobi_mat(h), kJacobiSweeps, h->rstream));
+        GLR_LAUNCH(h, 1, jacobi_cluster(jacobi_mat(h), kJacobiSweeps, h->rstream));
         const int rc = sort_full_basis(h, h->rstream);
         if (rc != GLR_OK) return rc;
     }
@@ -508,7 +508,7 @@ int refresh_exact_blocked(std::vector<glr_handle*>& hs) {
         const int n = h->mp;
         SortGroup sg{};
         sg.mat[sg.nmat++] = sort_mat(h, n, h->bj_vpar ? h->Vbuf : h->Vbuf2, h->U);
-        GLR_LAUNCH(h, 2, sort_group(sg, s0));
+        GLR_LAUNCH(h, 1, sort_group(sg, s0));
         GLR_LAUNCH(h, 1, tc::transpose_round(h->UT, n, h->U, n, n, n, s0));
     }
     GLR_CK(h0, cudaEventRecord(h0->rpow, s0));
@@ -748,7 +748,7 @@ int refresh_tcl_grouped(std::vector<glr_handle*>& hs) {
         SortGroup sg{};
         for (size_t i = c0; i < hs.size() && i < c0 + 64; ++i) sg.mat[sg.nmat++] = sort_mat(hs[i], hs[i]->k, hs[i]->Vk, hs[i]->gram);
         PhaseScope ps(hs[c0], GLR_PH_REFRESH, s0);
-        GLR_LAUNCH(hs[c0], 2, sort_group(sg, s0));
+        GLR_LAUNCH(hs[c0], 1, sort_group(sg, s0));
     }
     if ((rc = fp32_products(hs, s0, [](glr_handle* h, GemmMat& G) {          // Qn = Q W
              G.M = h->mp; G.N = h->k; G.K = h->k;

@@ -587,6 +587,7 @@ size_t eig_ws_floats(int n) {
 
 // By size class (16, 32, 64, 128), so that a problem's rounds do not depend on the group.
 cudaError_t eig_small_group(const EigGroup& g, cudaStream_t st) {
+    --more_launches;
     for (int lim = 8; lim <= 64; lim *= 2) {
         EigGroup c = g;
         c.nmat = 0;
@@ -596,6 +597,7 @@ cudaError_t eig_small_group(const EigGroup& g, cudaStream_t st) {
             if (n <= 2 * lim && (lim == 8 || n > lim)) c.mat[c.nmat++] = g.mat[i];
         }
         if (c.nmat == 0) continue;
+        ++more_launches;
         const cudaError_t e = lim == 8 ? launch_small<8>(c, st) : lim == 16 ? launch_small<16>(c, st)
                               : lim == 32 ? launch_small<32>(c, st) : launch_small<64>(c, st);
         if (e != cudaSuccess) return e;

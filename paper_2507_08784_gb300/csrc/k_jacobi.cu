@@ -549,6 +549,7 @@ cudaError_t jacobi_cluster(const JacobiMat& M, int max_sweeps, cudaStream_t st) 
     const cudaLaunchConfig_t cfg = cluster_config(M.n, &attr, st);
     const cudaError_t le = cudaLaunchKernelEx(&cfg, cluster_kernel(M.n), M, max_sweeps);
     if (le != cudaSuccess || M.n <= 256) return le;
+    ++more_launches;
     if (M.n & 1) jacobi_rows_kernel<8, true><<<(M.n + 3) / 4, 128, sizeof(float) * 4 * M.n, st>>>(M);
     else jacobi_rows_kernel<8, false><<<(M.n + 3) / 4, 128, sizeof(float) * 4 * M.n, st>>>(M);
     return cudaGetLastError();

@@ -409,6 +409,7 @@ cudaError_t sort_group(const SortGroup& g, cudaStream_t st) {
     for (int i = 0; i < g.nmat; ++i) n = g.mat[i].n > n ? g.mat[i].n : n;
     launch_chain(sort_rank_kernel, dim3((n + 31) / 32, g.nmat), 1024, 0, st, g);
     if (n <= 32) return cudaGetLastError();
+    ++more_launches;
     launch_chain(sort_gather_kernel, dim3(n < 1024 ? n : 1024, g.nmat), 256, sizeof(float) * n, st, g);
     return cudaGetLastError();
 }
@@ -1196,7 +1197,9 @@ cudaError_t householder_reconstruct(const float* Q, int mp, int k, float* Y, flo
     hh_top_kernel<<<1, 1024, 0, st>>>(Q, k, scratch, Y, T, s);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (mp > k) hh_rows_kernel<<<(mp - k + 7) / 8, 256, 0, st>>>(Q, mp, k, scratch, Y);
+    if (mp <= k) return e;
+    ++more_launches;
+    hh_rows_kernel<<<(mp - k + 7) / 8, 256, 0, st>>>(Q, mp, k, scratch, Y);
     return cudaGetLastError();
 }
 

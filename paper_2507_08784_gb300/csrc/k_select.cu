@@ -493,7 +493,9 @@ cudaError_t select_group(const SelectGroup& g, cudaStream_t st, int stages) {
     int maxmp = 1;
     for (int i = 0; i < g.nmat; ++i) maxmp = g.mat[i].mp > maxmp ? g.mat[i].mp : maxmp;
     cudaError_t e = cudaSuccess;
+    --more_launches;                                       // each of the three adds itself
     if (stages & 1) {
+        ++more_launches;
         launch_chain(lambda_reduce_kernel, dim3((maxmp + 31) / 32, g.nmat), 1024, 0, st, g);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
@@ -504,9 +506,11 @@ cudaError_t select_group(const SelectGroup& g, cudaStream_t st, int stages) {
         const cudaError_t ea = cudaFuncSetAttribute(select_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (ea != cudaSuccess) return ea;
     }
+    ++more_launches;
     launch_chain(select_group_kernel, g.nmat, 1024, smem, st, g);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (g.total_out <= 0) return cudaSuccess;              // every P formed by the caller
+    ++more_launches;
     launch_chain(pr_kernel, (unsigned)((g.total_out + 255) / 256), 256, 0, st, g);
     return cudaGetLastError();
 }

@@ -130,7 +130,7 @@ __global__ void gemm_splitk_reduce(GemmDesc d, int splits) {
 }  // namespace
 
 cudaError_t gemm_f32(const GemmDesc& d, cudaStream_t st) {
-    if (d.M <= 0 || d.N <= 0 || d.batch <= 0) return cudaSuccess;
+    if (d.M <= 0 || d.N <= 0 || d.batch <= 0) { --more_launches; return cudaSuccess; }
     const int tiles = ((d.N + GB_N - 1) / GB_N) * ((d.M + GB_M - 1) / GB_M);
     int splits = 1;
     if (d.batch == 1 && d.ws && tiles < 148 && d.K >= 512) {
@@ -147,6 +147,7 @@ cudaError_t gemm_f32(const GemmDesc& d, cudaStream_t st) {
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         const int64_t total = (int64_t)d.M * d.N;
+        ++more_launches;
         launch_chain(gemm_splitk_reduce, (unsigned)((total + 255) / 256), 256, 0, st, d, splits);
         return cudaGetLastError();
     }
@@ -448,9 +449,12 @@ cudaError_t gemm_group_f32(GemmGroup& g, cudaStream_t st) {
         M.tile0 = g.total_tiles;
         g.total_tiles += tiles * M.splits;
     }
-    if (g.total_tiles <= 0) return cudaSuccess;
+    if (g.total_tiles <= 0) { --more_launches; return cudaSuccess; }
     gemm_group_kernel<<<g.total_tiles, 256, 0, st>>>(g);
-    if (reduce) launch_chain(gemm_group_reduce, dim3(64, g.nmat), 256, 0, st, g);
+    if (reduce) {
+        ++more_launches;
+        launch_chain(gemm_group_reduce, dim3(64, g.nmat), 256, 0, st, g);
+    }
     return cudaGetLastError();
 }
 

@@ -1318,6 +1318,7 @@ cudaError_t launch_pow(TcGroup& g, cudaStream_t st) {
     for (int i = 0; i < g.nmat; ++i)
         if (g.mat[i].splits > 1) { rows = std::max(rows, g.mat[i].rows); kpad = std::max(kpad, g.mat[i].kpad); }
     if (e != cudaSuccess || !rows) return e;
+    ++more_launches;
     launch_chain(pow_reduce_kernel, dim3((rows + 31) / 32, g.nmat, (kpad + 31) / 32), 256, 0, st, g);
     return cudaGetLastError();
 }
@@ -1355,6 +1356,7 @@ __global__ void __launch_bounds__(256) gram_sum_kernel(const __grid_constant__ T
 cudaError_t launch_gram(TcGroup& g, cudaStream_t st) {
     const cudaError_t e = launch<Gram>(g, st);
     if (e != cudaSuccess || g.nmat <= 0) return e;
+    ++more_launches;
     launch_chain(gram_sum_kernel, dim3(64, g.nmat), 256, 0, st, g);
     return cudaGetLastError();
 }

@@ -98,3 +98,63 @@ def test_step_recorded_into_a_graph(m, n, r, k, dtype, opt, t):
     assert torch.equal(Xa, Xb)
     a.close()
     b.close()
+
+
+def _kernel_nodes(run):
+    """Kernels that run() launches on a capturing stream, counted from the graph it leaves."""
+    import ctypes
+    import torch
+    cu = ctypes.CDLL("libcuda.so.1")
+    stream = torch.cuda.Stream()
+    st, graph, n, kind = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t(0), ctypes.c_int(0)
+
+    def check(rc):
+        assert rc == 0, rc
+
+    with torch.cuda.stream(stream):
+        check(cu.cuStreamBeginCapture_v2(st, 2))               # relaxed
+        try:
+            run()
+        finally:
+            rc = cu.cuStreamEndCapture(st, ctypes.byref(graph))
+        check(rc)
+    check(cu.cuGraphGetNodes(graph, None, ctypes.byref(n)))
+    nodes = (ctypes.c_void_p * n.value)()
+    check(cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)))
+    kernels = 0
+    for node in nodes:
+        check(cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)))
+        kernels += kind.value == 0                             # CU_GRAPH_NODE_TYPE_KERNEL
+    check(cu.cuGraphDestroy(graph))
+    return kernels
+
+
+@pytest.mark.parametrize("dtype,opt,mats", [
+    # grouped k <= 32 refreshes beside the larger factors and the eigenproblems' size classes
+    ("f32", "msgd", [(40, 96, 4, 8), (64, 576, 8, 32), (100, 132, 4, 40), (200, 240, 4, 130), (280, 300, 4, 264)]),
+    # no multiple of 4: the unfused step and the ungrouped refresh with K slices; full bases up to and above 256
+    ("f32", "adam", [(65, 131, 4, 12), (63, 777, 5, 20), (129, 65, 3, 0), (300, 310, 4, 0)]),
+    ("f32", "adamw", [(65, 131, 4, 12)]),
+    ("f32", "amsgrad", [(64, 128, 4, 0)]),
+    # tcgen05: whole and sliced products, each class of eigenproblem, Gram matrices of several row chunks
+    ("bf16", "adam", [(136, 264, 16, 20), (200, 328, 16, 68), (256, 4104, 16, 64), (520, 1032, 16, 64), (264, 520, 16, 256)]),
+])
+def test_launch_counts_are_the_kernels_launched(dtype, opt, mats):
+    """glr_stats.launches against the kernel nodes of the recorded step, for a refresh and a compressed step
+    (sizes whose products stay below the library's threshold)."""
+    import torch
+    import paper_2507_08784_gb300 as glr
+    tdt = torch.float32 if dtype == "f32" else torch.bfloat16
+    hs = [glr.GreedyLore(m, n, r, 2, seed=j, basis_rank=k, grad_dtype=dtype, tau=2, optimizer=opt, lr=0.01, beta1=0.9,
+                         beta2=0.99) for j, (m, n, r, k) in enumerate(mats)]
+    X = [torch.zeros(m, n, device="cuda") for m, n, _, _ in mats]
+    G = [[torch.randn(m, n, device="cuda").to(tdt) for _ in range(2)] for m, n, _, _ in mats]
+    for _ in range(2):
+        glr.glr_step_group(hs, G, X)
+    torch.cuda.synchronize()
+    for what in ("refresh", "compressed"):
+        before = sum(h.stats()["launches"] for h in hs)
+        kernels = _kernel_nodes(lambda: glr.glr_step_group(hs, G, X))
+        assert sum(h.stats()["launches"] for h in hs) - before == kernels, what
+    for h in hs:
+        h.close()
