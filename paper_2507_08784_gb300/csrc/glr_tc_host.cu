@@ -178,11 +178,14 @@ bool capturing(cudaStream_t st) {
 }
 
 // Maps copied to the device in stream order.  A copy recorded into a graph reads its source at every
-// replay, long after this call: the handle keeps it.
+// replay, long after this call: the handle keeps it, once for all recordings of the same buffers.
 cudaError_t put_maps(glr_handle* h, CUtensorMap* dst, const CUtensorMap* maps, int n, bool cap, cudaStream_t st) {
     if (cap) {
-        h->captured_maps.emplace_back(maps, maps + n);
-        maps = h->captured_maps.back().data();
+        const size_t bytes = sizeof(CUtensorMap) * n;
+        auto same = [&](const std::vector<CUtensorMap>& v) { return v.size() == (size_t)n && !std::memcmp(v.data(), maps, bytes); };
+        auto kept = std::find_if(h->captured_maps.begin(), h->captured_maps.end(), same);
+        if (kept == h->captured_maps.end()) kept = h->captured_maps.emplace(kept, maps, maps + n);
+        maps = kept->data();
     }
     return cudaMemcpyAsync(dst, maps, sizeof(CUtensorMap) * n, cudaMemcpyHostToDevice, st);
 }

@@ -158,3 +158,32 @@ def test_launch_counts_are_the_kernels_launched(dtype, opt, mats):
         assert sum(h.stats()["launches"] for h in hs) - before == kernels, what
     for h in hs:
         h.close()
+
+
+def test_recording_again_keeps_no_more():
+    """A handle keeps the tile-copy descriptors that recorded steps read (N + 1 of 128 bytes a recording);
+    recordings of the same buffers share them: the process's allocated bytes grow by less than a
+    recording's descriptors."""
+    import ctypes
+    import torch
+    import paper_2507_08784_gb300 as glr
+
+    class Mallinfo2(ctypes.Structure):
+        _fields_ = [(f, ctypes.c_size_t) for f in ("arena", "ordblks", "smblks", "hblks", "hblkhd", "usmblks", "fsmblks",
+                                                   "uordblks", "fordblks", "keepcost")]
+    libc = ctypes.CDLL(None)
+    libc.mallinfo2.restype = Mallinfo2
+    N = 8
+    h = glr.GreedyLore(256, 704, 32, N, seed=1, basis_rank=64, grad_dtype="bf16", tau=1 << 20, optimizer="adam", lr=0.01)
+    X = torch.zeros(256, 704, device="cuda")
+    G = [torch.randn(256, 704, device="cuda").to(torch.bfloat16) for _ in range(N)]
+    for _ in range(2):
+        h.step(G, X)
+    torch.cuda.synchronize()
+    used = []
+    for _ in range(4):
+        for _ in range(250):
+            _kernel_nodes(lambda: h.step(G, X))
+        used.append(libc.mallinfo2().uordblks)
+    h.close()
+    assert min(b - a for a, b in zip(used, used[1:])) < 250 * (N + 1) * 128 / 2
