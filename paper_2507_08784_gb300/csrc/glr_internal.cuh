@@ -353,9 +353,9 @@ cudaError_t jacobi_cluster(const JacobiMat& M, int max_sweeps, cudaStream_t st);
 // Symmetric eigenproblems of the refresh (k_eig.cu), n <= 1024: H (row-major, leading dimension ld,
 // read only) -> eigenvalues (unsorted) and eigenvectors
 // V (row-major n x n, column j for evals[j]); sweeps done in *sweeps.  n <= 128: one CTA a problem
-// (eig_small_group).  Larger n: all problems in one cooperative launch (eig_group) that leaves
-// busy_sms SMs free; ws: eig_ws_floats(n) floats a problem, part: 128 floats a problem, bar: two
-// ints, *err counts a barrier that gave up.
+// (eig_small_group).  Larger n: all problems in one cooperative launch on every SM (eig_group); ws:
+// eig_ws_floats(n) floats a problem, part: 128 floats a problem, bar: two ints, *err counts a barrier
+// that gave up.
 constexpr int kEigSmall = 128;
 constexpr int kEigGroupMax = 64;
 struct EigMat {
@@ -371,7 +371,7 @@ struct EigGroup {
 };
 size_t eig_ws_floats(int n);
 cudaError_t eig_small_group(const EigGroup& g, cudaStream_t st);
-cudaError_t eig_group(EigGroup& g, int busy_sms, cudaStream_t st);
+cudaError_t eig_group(EigGroup& g, cudaStream_t st);
 
 // The blocked Jacobi's round-robin tournament over m blocks of 64 indices (circle method: block 0
 // fixed, the others one slot further each round; slots s and m - 1 - s pair up and are stored at

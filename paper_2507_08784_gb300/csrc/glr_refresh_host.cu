@@ -50,9 +50,8 @@ struct EigItem {
     float* V;
 };
 
-// The eigenproblems: those of n <= 128 on s1, the larger ones in one cooperative launch on s0 (leaving
-// the small ones' SMs free when s1 is another stream).
-int eig_solve(const std::vector<EigItem>& items, cudaStream_t s0, cudaStream_t s1) {
+// The eigenproblems on one stream: those of n <= 128, then the larger ones in one cooperative launch.
+int eig_solve(const std::vector<EigItem>& items, cudaStream_t st) {
     std::vector<const EigItem*> cls[2];
     for (const EigItem& it : items) cls[it.n > kEigSmall ? 1 : 0].push_back(&it);
     for (int big = 0; big < 2; ++big)
@@ -68,8 +67,7 @@ int eig_solve(const std::vector<EigItem>& items, cudaStream_t s0, cudaStream_t s
                 M.H = it.H; M.ld = it.ld; M.V = it.V; M.evals = it.h->evals;
                 M.sweeps = it.h->dflags + 1; M.ws = it.h->eig_ws; M.failed = it.h->dflags + 6;
             }
-            if (big) GLR_LAUNCH(h0, 1, eig_group(g, s0 != s1 ? (int)cls[0].size() : 0, s0));
-            else GLR_LAUNCH(h0, 1, eig_small_group(g, s1));
+            GLR_LAUNCH(h0, 1, big ? eig_group(g, st) : eig_small_group(g, st));
         }
     return GLR_OK;
 }
@@ -112,7 +110,7 @@ int refresh_tails(std::vector<glr_handle*>& hs) {
     }
     {
         PhaseScope ps(h0, GLR_PH_REFRESH, h0->rstream);
-        const int rc = eig_solve(items, h0->rstream, h0->rstream);
+        const int rc = eig_solve(items, h0->rstream);
         if (rc != GLR_OK) return rc;
     }
     GLR_CK(h0, cudaEventRecord(h0->rpow, h0->rstream));
@@ -740,7 +738,7 @@ int refresh_tcl_grouped(std::vector<glr_handle*>& hs) {
     for (glr_handle* h : hs) items.push_back(EigItem{h, h->k, h->gpart, h->kpad, h->Vk});
     {
         PhaseScope ps(h0, GLR_PH_REFRESH, s0);
-        if ((rc = eig_solve(items, s0, s0)) != GLR_OK) return rc;
+        if ((rc = eig_solve(items, s0)) != GLR_OK) return rc;
     }
     // the finish, grouped: sorted Ritz pairs, Q <- Q W, column signs, the Householder WY form,
     // Yt = Y T^T, then Y^T for the W = Y^T Mbar products

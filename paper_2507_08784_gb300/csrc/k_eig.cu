@@ -605,7 +605,7 @@ cudaError_t eig_small_group(const EigGroup& g, cudaStream_t st) {
     return cudaSuccess;
 }
 
-cudaError_t eig_group(EigGroup& g, int busy_sms, cudaStream_t st) {
+cudaError_t eig_group(EigGroup& g, cudaStream_t st) {
     if (g.nmat <= 0) return cudaSuccess;
     int pairs = 0;
     for (int i = 0; i < g.nmat; ++i) {
@@ -620,14 +620,13 @@ cudaError_t eig_group(EigGroup& g, int busy_sms, cudaStream_t st) {
         e = cudaFuncSetAttribute(eig_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGroupSmem);
     if (e == cudaSuccess) e = cudaMemsetAsync(g.bar, 0, 2 * sizeof(int), st);    // arrivals and generation
     if (e != cudaSuccess) return e;
-    const int grid = busy_sms < sms / 2 ? sms - busy_sms : sms;
-    g.parts = 4 * pairs <= grid ? 4 : 1;      // four CTAs a pair where they are to spare (the same bits)
+    g.parts = 4 * pairs <= sms ? 4 : 1;      // four CTAs a pair where they are to spare (the same bits)
     if (!coop) {               // one CTA: the barriers wait for nobody
         eig_group_kernel<<<1, PTHREADS, kGroupSmem, st>>>(g);
         return cudaGetLastError();
     }
     void* args[] = {&g};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(eig_group_kernel), dim3(grid), dim3(PTHREADS), args,
+    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(eig_group_kernel), dim3(sms), dim3(PTHREADS), args,
                                        kGroupSmem, st);
 }
 

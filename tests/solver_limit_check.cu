@@ -44,7 +44,7 @@ static int failures(Solver solver, int n, int max_sweeps, bool nan) {
         EigMat& M = g.mat[0];
         M.n = n; M.tol = tol; M.H = dH; M.ld = n; M.V = V; M.evals = evals; M.sweeps = flags; M.ws = ws; M.failed = flags + 1;
         if (solver == kSmall) CK(eig_small_group(g, nullptr));
-        else CK(eig_group(g, 0, nullptr));
+        else CK(eig_group(g, nullptr));
     } else if (solver == kTail) {
         TailGroup g{};
         g.nmat = 1;
