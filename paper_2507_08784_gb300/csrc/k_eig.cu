@@ -109,9 +109,8 @@ __global__ void __launch_bounds__(8 * LIM, 1) eig_small_kernel(const __grid_cons
         if (t == 0) {
             float o2 = 0.f, t2 = 0.f;
             for (int w = 0; w < NT / 32; ++w) { o2 += red[0][w]; t2 += red[1][w]; }
-            const bool converged = o2 <= M.tol * M.tol * t2;
-            stop = (converged || sweep >= g.max_sweeps) ? 1 : 0;
-            if (stop && !converged && M.failed) atomicAdd(M.failed, 1);
+            stop = (o2 <= M.tol * M.tol * t2 || sweep >= g.max_sweeps) ? 1 : 0;
+            red[0][0] = o2; red[1][0] = t2;                // for the count at the end (kept out of the sweeps' code)
         }
         __syncthreads();
         if (stop) break;
@@ -184,6 +183,7 @@ __global__ void __launch_bounds__(8 * LIM, 1) eig_small_kernel(const __grid_cons
         }
     for (int i = t; i < n; i += NT) M.evals[i] = lam[i];
     if (t == 0 && M.sweeps) *M.sweeps = sweep;
+    if (t == 0 && sweep >= g.max_sweeps && M.failed && !(red[0][0] <= M.tol * M.tol * red[1][0])) atomicAdd(M.failed, 1);
 }
 template <int LIM> constexpr size_t small_smem() {
     return sizeof(float) * (3 * (2 * LIM) * PLD + 2 * 16 * 128 + 2 * 64);

@@ -333,8 +333,7 @@ __global__ void __launch_bounds__(CT, 1) jacobi_cluster_kernel(const __grid_cons
         if (t == 0) {                                   // the same sums, the same decision in every CTA
             float o2 = 0.f, t2 = 0.f;
             for (int c = 0; c < C; ++c) { o2 += peer(part, c)[0]; t2 += peer(part, c)[1]; }
-            stop = (o2 <= M.tol * M.tol * t2 || sweep >= max_sweeps) ? 1 : 0;
-            if (stop && b == 0 && o2 > M.tol * M.tol * t2 && M.failed) atomicAdd(M.failed, 1);
+            stop = o2 <= M.tol * M.tol * t2 ? 1 : sweep < max_sweeps ? 0 : o2 > M.tol * M.tol * t2 ? 2 : 1;
         }
         cluster_sync();                                 // part is read before anyone writes it again
         if (stop) break;
@@ -443,6 +442,7 @@ __global__ void __launch_bounds__(CT, 1) jacobi_cluster_kernel(const __grid_cons
     for (int e = t; e < vrows * n; e += CT) M.V[(size_t)v0 * n + e] = V[e];
     if (b == 0 && t == 0) {
         *M.sweeps = sweep;
+        if (stop == 2 && M.failed) atomicAdd(M.failed, 1);
         if (LOG) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // the log is complete before the CTA ends
     }
 }

@@ -51,8 +51,7 @@ __global__ void __launch_bounds__(1024) jacobi_kernel(float* Hg, int n, float* V
         if (tid == 0) {
             float o2 = 0.f, t2 = 0.f;
             for (int w = 0; w < (nth + 31) / 32; ++w) { o2 += red_off[w]; t2 += red_tot[w]; }
-            done = (o2 <= tol * tol * t2 || sweep >= max_sweeps) ? 1 : 0;
-            if (done && o2 > tol * tol * t2 && failed) atomicAdd(failed, 1);
+            done = o2 <= tol * tol * t2 ? 1 : sweep < max_sweeps ? 0 : o2 > tol * tol * t2 ? 2 : 1;
         }
         __syncthreads();
         if (done) break;
@@ -116,6 +115,7 @@ __global__ void __launch_bounds__(1024) jacobi_kernel(float* Hg, int n, float* V
     if (use_smem)
         for (int e = tid; e < n * n; e += nth) Vg[e] = V[e];
     if (tid == 0 && sweeps_out) *sweeps_out = sweep;
+    if (tid == 0 && done == 2 && failed) atomicAdd(failed, 1);
 }
 
 __device__ __forceinline__ uint32_t float_order(float f) {
@@ -503,7 +503,7 @@ __global__ void __launch_bounds__(1024) chol_inverse_kernel(const float* G, int 
 // ---- blocked factor and inverse of the grouped refreshes, n <= 256 --------------------------------
 // One CTA of 16 warps a matrix, the lower triangle as 32 x 32 blocks in shared memory (block (i, j) at
 // i (i + 1) / 2 + j, pitch 36: rows 16-byte aligned, the products' reads free of bank conflicts),
-// padded to whole blocks with the identity.  A panel: one warp factors the diagonal block with a row
+// padded to whole blocks with a multiple of the identity.  A panel: one warp factors the diagonal block with a row
 // a lane and hands each column on; in the same steps a warp inverts that block and a warp per block
 // below solves against it by substitution; then the trailing blocks are 32 x 32 x 32 products, a
 // warp each.  The inverse goes block column by block column from the last, in place:
@@ -598,12 +598,13 @@ __global__ void __launch_bounds__(CWARPS * 32) chol_group_kernel(const __grid_co
     int attempt = 0;
     for (; attempt < 6; ++attempt) {
         __syncthreads();
+        const float pad = M.tri_only ? 1.f : fmaxf(trace / n, 1e-30f);   // its pivots pass like the matrix's own
 #pragma unroll 4
         for (int q = warp; q < nb * (nb + 1) / 2 * CB; q += CWARPS) {    // a block row a warp
             int i = 0, j = q / CB;                                       // j = i (i + 1) / 2 + block column
             while (j > i) { j -= i + 1; ++i; }
             const int r = i * CB + q % CB, c = j * CB + lane;
-            float v = r == c ? 1.f : 0.f;
+            float v = r == c ? pad : 0.f;
             if (r < n && c < n) {
                 v = c <= r ? entry(r, c) : 0.f;
                 if (r == c && !M.tri_only) v += shift;
@@ -634,7 +635,7 @@ __global__ void __launch_bounds__(CWARPS * 32) chol_group_kernel(const __grid_co
                 float v = 0.f;
                 if (warp == 0) {
                     const float d = __shfl_sync(0xffffffffu, a[0], c);
-                    ok = ok && (d > thresh || p * CB + c >= n);   // the padding's pivots are 1 at any scale
+                    ok = ok && d > thresh;
                     const float l = sqrtf(d);
                     v = lane == c ? l : lane > c ? a[0] / l : 0.f;
                     cb[lane] = v;
@@ -858,9 +859,7 @@ __global__ void __launch_bounds__(512) tail_ritz_kernel(const __grid_constant__ 
         if (tid == 0) {
             float o2 = 0.f, t2 = 0.f;
             for (int w = 0; w < nth / 32; ++w) { o2 += red_off[w]; t2 += red_tot[w]; }
-            const bool converged = o2 <= tol * tol * t2;
-            done = (converged || sweep >= kJacobiSweeps) ? 1 : 0;
-            if (done && !converged && M.failed) atomicAdd(M.failed, 1);
+            done = o2 <= tol * tol * t2 ? 1 : sweep < kJacobiSweeps ? 0 : 2;
         }
         __syncthreads();
         if (done) break;
@@ -927,6 +926,7 @@ __global__ void __launch_bounds__(512) tail_ritz_kernel(const __grid_constant__ 
         M.evals[tid] = ev[tid];
     }
     if (tid == 0 && M.sweeps) *M.sweeps = sweep;
+    if (tid == 0 && done == 2 && M.failed) atomicAdd(M.failed, 1);
     __syncthreads();
     // sorted by descending value (ties by index), unit columns, largest entry positive: a warp a column
     for (int col = warp; col < n; col += blockDim.x >> 5) {
