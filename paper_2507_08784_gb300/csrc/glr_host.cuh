@@ -51,7 +51,7 @@ struct glr_handle {
     // in mn_scratch (m' x n').
     int tc = 0;
     float* mn_scratch = nullptr;
-    float* jwork = nullptr;      // full basis: T^T of the blocked Jacobi above m' = 1024
+    float* jwork = nullptr;      // full basis: the grid-wide Jacobi's second m' x m' buffer, T^T of the blocked one above m' = 1024
     float* jpart = nullptr;      // norm partials of the eigen-solver (used by a group's first handle)
     float* jlog = nullptr;       // full basis up to m' = 512: the Jacobi's rotations (not checkpointed)
     float *eig_ws = nullptr, *sort_ws = nullptr;   // eigen-solver and eigenpair-order scratch (not checkpointed)

@@ -16,14 +16,16 @@
 // CTA and read by another (H, V, the norm partials) is read through L2 (__ldcg), so no stale L1
 // line survives a barrier.
 //
-// For n <= 512 a matrix fits the shared memory of one thread-block cluster and is solved there
-// (jacobi_cluster_kernel): the row pairs of H are spread over up to 16 CTAs, a round's rotations go
+// For n <= 512 a matrix is solved in the shared memory of one thread-block cluster
+// (jacobi_cluster_kernel): the row pairs of H are spread over up to 16 CTAs, one a warp (16 x 16 pairs:
+// hence 512; 76 KB a CTA there, 227 KB would hold n = 896), a round's rotations go
 // to all of them over distributed shared memory; two hardware cluster barriers a round.  The
 // rotations, their order and every product and sum are those of the grid-wide kernel, so the results
 // are the same bits.  A round takes 3.2 us at n = 512 (bound by instruction issue) and 2 us below
 // n = 128 (the rotation's chain of quotients and roots, two cluster barriers); the grid-wide kernel
 // pays 6 us at n = 512 alone and 14 us for the eight matrices of a conv stack, its barrier in global
-// memory and the L2 round trips.
+// memory and the L2 round trips.  Above 512 a warp would take several pairs: tried on one matrix, 5.7 us
+// a round at n = 768 (39 ms; grid-wide 9.1 us, 63 ms) and 7.0 us at 896 (10.6), the same bits; not built in.
 #include <cooperative_groups.h>
 
 #include "glr_internal.cuh"
